@@ -220,38 +220,54 @@ radix_hist_kernel(const uint32_t* __restrict__ keys, int shift, uint32_t mask,
 }
 
 // ---------------------------------------------------------------------------------------
-// pass step 2: per segment, exclusive scan over chunks inside each bin and over the bins
+// pass step 2: per segment and bin, exclusive scan over the chunks; bin totals
+// One CTA takes 32 bins of one segment: a lane per bin (128-byte rows of the histogram), a warp per
+// group of consecutive chunks.  A segment's chunks are summed by 16 warps in 16 CTAs; one CTA per
+// segment walking all of them took 23 us for the 300 to 450 chunks of a single segment.  The scan
+// over the bins is left to the scatter, whose threads have one bin each anyway.
 // ---------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSortMaxBins)
+constexpr int kScanThreads = 512;
+constexpr int kScanWarps = kScanThreads / 32;
+constexpr int kScanBinGroups = kSortMaxBins / 32;
+
+__global__ void __launch_bounds__(kScanThreads)
 radix_scan_kernel(const SortDesc* __restrict__ desc, const int32_t* __restrict__ seg_first,
-                  uint32_t* hist, uint32_t* __restrict__ bin_base) {
+                  uint32_t* hist, uint32_t* __restrict__ bin_total) {
   const int s = blockIdx.x;
   if (s >= desc->n_segments) return;
-  const int d = threadIdx.x;
-  const int c0 = seg_first[s], c1 = seg_first[s + 1];
-  uint32_t run = 0;
+  __shared__ uint32_t part[kScanWarps][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int d = blockIdx.y * 32 + lane;
+  const int c0 = seg_first[s], n_c = seg_first[s + 1] - c0;
+  const int per = (n_c + kScanWarps - 1) / kScanWarps;
+  const int b = c0 + min(n_c, w * per), e = c0 + min(n_c, (w + 1) * per);
+  uint32_t* h = hist + d;
   constexpr int kBatch = 8;
-  for (int c = c0; c < c1; c += kBatch) {
+  uint32_t sum = 0;
+  for (int c = b; c < e; c += kBatch) {
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) sum += c + j < e ? h[(size_t)(c + j) * kSortMaxBins] : 0u;
+  }
+  part[w][lane] = sum;
+  __syncthreads();
+  uint32_t run = 0, total = 0;
+#pragma unroll
+  for (int ww = 0; ww < kScanWarps; ++ww) {
+    const uint32_t t = part[ww][lane];
+    run += ww < w ? t : 0u;
+    total += t;
+  }
+  for (int c = b; c < e; c += kBatch) {
     uint32_t t[kBatch];
 #pragma unroll
-    for (int j = 0; j < kBatch; ++j)
-      t[j] = (c + j < c1) ? hist[(size_t)(c + j) * kSortMaxBins + d] : 0u;
+    for (int j = 0; j < kBatch; ++j) t[j] = c + j < e ? h[(size_t)(c + j) * kSortMaxBins] : 0u;
 #pragma unroll
     for (int j = 0; j < kBatch; ++j) {
-      if (c + j < c1) hist[(size_t)(c + j) * kSortMaxBins + d] = run;
+      if (c + j < e) h[(size_t)(c + j) * kSortMaxBins] = run;
       run += t[j];
     }
   }
-  __shared__ uint32_t tmp[kSortMaxBins];
-  tmp[d] = run;
-  __syncthreads();
-  for (int o = 1; o < kSortMaxBins; o <<= 1) {
-    const uint32_t v = d >= o ? tmp[d - o] : 0u;
-    __syncthreads();
-    tmp[d] += v;
-    __syncthreads();
-  }
-  bin_base[(size_t)s * kSortMaxBins + d] = tmp[d] - run;
+  if (w == 0) bin_total[(size_t)s * kSortMaxBins + d] = total;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -273,7 +289,7 @@ radix_scatter_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __res
                      uint32_t mask, const SortDesc* __restrict__ desc,
                      const int32_t* __restrict__ chunk_seg, const int64_t* __restrict__ seg_bounds,
                      const int64_t* __restrict__ chunk_begin, const int64_t* __restrict__ chunk_end,
-                     const uint32_t* __restrict__ hist, const uint32_t* __restrict__ bin_base,
+                     const uint32_t* __restrict__ hist, const uint32_t* __restrict__ bin_total,
                      const int32_t* __restrict__ seg_first) {
   const int c = blockIdx.x;
   if (c >= desc->n_chunks) return;
@@ -289,12 +305,14 @@ radix_scatter_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __res
   const unsigned lt = (1u << lane) - 1u;
   const int seg = chunk_seg[c];
   const uint32_t seg_begin = (uint32_t)seg_bounds[seg];
+  // where this chunk's entries of every bin start: entries of smaller bins of the segment, then
+  // those of this bin in earlier chunks
+  uint32_t pre = 0, tot = 0;
   if (seg_first) {
     // few chunks (a small input): `hist` holds the raw counts and this CTA sums its segment's
-    // chunks itself - bin totals, the part before its own chunk, the scan over the bins - which
-    // costs a microsecond and saves the scan kernel between the histogram and this one
+    // chunks itself, which costs a microsecond and saves the scan kernel between the histogram
+    // and this one
     const int c0 = seg_first[seg], c1 = seg_first[seg + 1];
-    uint32_t pre = 0, tot = 0;
     for (int cc = c0; cc < c1; cc += 4) {
       uint32_t h[4];
 #pragma unroll
@@ -305,6 +323,11 @@ radix_scatter_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __res
         tot += h[j];
       }
     }
+  } else {
+    pre = hist[(size_t)c * kSortMaxBins + tid];
+    tot = bin_total[(size_t)seg * kSortMaxBins + tid];
+  }
+  {
     uint32_t incl = tot;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -318,8 +341,6 @@ radix_scatter_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __res
     for (int ww = 0; ww < kScatWarps; ++ww) wp += (ww < w) ? warp_tot[ww] : 0u;
     gbase[tid] = seg_begin + (incl - tot + wp) + pre;
     // warp_tot is written again only after the tile loop's barriers (A) and (B)
-  } else {
-    gbase[tid] = seg_begin + bin_base[(size_t)seg * kSortMaxBins + tid] + hist[(size_t)c * kSortMaxBins + tid];
   }
   unsigned short* my_wh = wh + w * kSortMaxBins;
 
@@ -624,7 +645,7 @@ SortLayout sort_layout(int S) {
   L.chunk_begin = o; o = align_up(o + 8 * C);
   L.chunk_end = o;   o = align_up(o + 8 * C);
   L.hist = o;        o = align_up(o + 4 * C * kSortMaxBins);
-  L.bin_base = o;    o = align_up(o + 4 * (size_t)S * kSortMaxBins);
+  L.bin_total = o;   o = align_up(o + 4 * (size_t)S * kSortMaxBins);
   L.chunk_runs = o;  o = align_up(o + 8 * (C * 16 + 1));
   L.bytes = o;
   return L;
@@ -685,7 +706,7 @@ void segsort_run(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* key
   const int64_t* chunk_begin = (const int64_t*)(ws + L.chunk_begin);
   const int64_t* chunk_end = (const int64_t*)(ws + L.chunk_end);
   uint32_t* hist = (uint32_t*)(ws + L.hist);
-  uint32_t* bin_base = (uint32_t*)(ws + L.bin_base);
+  uint32_t* bin_total = (uint32_t*)(ws + L.bin_total);
   const int P = sort_passes(key_bits);
   segsort_prepare_device();
   // spread the bits evenly over the passes
@@ -705,11 +726,11 @@ void segsort_run(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* key
     // with few chunks every scatter CTA scans the counts it needs itself (one launch less)
     const bool fold_scan = chunk_bound(n_cap, L) <= kFoldScanChunks;
     if (!fold_scan)
-      ANTDT_LAUNCH(agg ? "agg_radix_scan" : "radix_scan", radix_scan_kernel, S, kSortMaxBins, 0, s, desc, seg_first, hist,
-                   bin_base);
+      ANTDT_LAUNCH(agg ? "agg_radix_scan" : "radix_scan", radix_scan_kernel, dim3(S, kScanBinGroups),
+                   kScanThreads, 0, s, desc, seg_first, hist, bin_total);
     ANTDT_LAUNCH(agg ? "agg_radix_scatter" : "radix_scatter", radix_scatter_kernel, L.max_chunks, kScatThreads, kScatSmem, s, kin, vin,
                  kout, vout, shift, mask, desc, chunk_seg, seg_bounds, chunk_begin, chunk_end, hist,
-                 bin_base, fold_scan ? seg_first : (const int32_t*)nullptr);
+                 bin_total, fold_scan ? seg_first : (const int32_t*)nullptr);
     kin = kout;
     vin = vout;
     shift += bits;

@@ -44,7 +44,7 @@ struct SortLayout {
   size_t chunk_begin;  // int64 [C]
   size_t chunk_end;    // int64 [C]
   size_t hist;         // uint32 [C * 512]
-  size_t bin_base;     // uint32 [S * 512]
+  size_t bin_total;    // uint32 [S * 512]
   size_t chunk_runs;   // int64 [16 C + 1]  run counts per strip of a chunk (runs pass)
   size_t bytes;        // total
   int max_chunks;      // C
