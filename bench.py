@@ -250,6 +250,11 @@ def scaled_workload(w, scale):
                     name=f"{w.name} scaled x{scale:g}")
 
 
+def row_passes(w):
+    """Passes of a sort by row id (9 bits each)."""
+    return -(-max(1, (w.V - 1).bit_length()) // 9)
+
+
 def algorithmic_bytes(w, nnz, n_bags, sum_u, u):
     """Bytes each kernel of the step has to move per launch (per step for the radix kernels'
     sum), from the counts of the batch: the gathers at full multiplicity, every output once."""
@@ -272,10 +277,15 @@ def algorithmic_bytes(w, nnz, n_bags, sum_u, u):
         "sparse_adagrad": u * (4 + 4 * D) + 2 * u * D * ew + 2 * S * u * D * 4,
         "sparse_adam": u * (4 + 4 * D) + 2 * u * D * ew + 2 * S * u * D * 4,
         "dense_wsum": (w.K + 1) * w.dense_n * 4,
+        # one kernel for the whole sort of a small or mid-sized batch: ids and offsets, a write and a
+        # read of every (id, bag) pair per pass by row id, the bags in sorted order, the lists of
+        # distinct rows and (in a step) the merge order
+        "resident_sort": (4 * nnz + 8 * (n_bags + 1) + 16 * nnz * row_passes(w) + 4 * nnz + 12 * sum_u +
+                          5 * sum_u + 8 * u),
     }
 
 
-def step_bytes(w, nnz, n_bags, sum_u, u, passes_bwd, passes_agg, fused=False):
+def step_bytes(w, nnz, n_bags, sum_u, u, passes_bwd, passes_agg, fused=False, resident=False):
     b = algorithmic_bytes(w, nnz, n_bags, sum_u, u)
     upd = b["sparse_adam"] if w.opt == "adam" else b["sparse_adagrad"]
     if fused and w.K <= 32:   # the one-pass server step: no aggregated gradient in between
@@ -286,6 +296,8 @@ def step_bytes(w, nnz, n_bags, sum_u, u, passes_bwd, passes_agg, fused=False):
     else:
         sort += (passes_agg * (b["agg_radix_hist"] + b["agg_radix_scatter"]) + b["agg_runs_count"] +
                  b["agg_runs_emit"])
+    if resident:        # one kernel instead of the expansion, the sort, the runs and the merge
+        sort = b["resident_sort"] - b["expand_bags"]
     return (b["embbag_fwd"] + b["expand_bags"] + b["seg_reduce_tiles"] + b["agg_reduce"] + upd +
             (b["dense_wsum"] if w.dense_n else 0) + sort)
 
@@ -599,9 +611,9 @@ def run_ours(args):
                         "gathered_GBps": round(ach, 1), "frac_of_l2_gather_peak": round(ach / rate, 4)}
             kern[name]["frac_of_l2_gather_peak"] = l2[name]["frac_of_l2_gather_peak"]
         roof["l2_gather"] = l2.get(top)
-    rowbits = max(1, (w.V - 1).bit_length())
-    passes = -(-rowbits // 9)
-    sb = step_bytes(w, int(nnz_avg), int(bags_avg), sum_u_seen, u_seen, passes, passes, args.fuse_update)
+    passes = row_passes(w)
+    sb = step_bytes(w, int(nnz_avg), int(bags_avg), sum_u_seen, u_seen, passes, passes, args.fuse_update,
+                    "resident_sort" in prof)
     line = {
         "metric": METRIC, "value": samples / (ms * 1e-3), "unit": UNIT, "n_gpus": world,
         "steps": K_steps, "warmup": W, "ms_per_step": ms / K_steps, "higher_is_better": True,

@@ -1,7 +1,9 @@
 // Server aggregation: batch-size weighted sum of the workers' mean gradients.
 //
 // Sparse part, up to 32 workers: the range-partitioned merge of agg_range.cu (no sort).
-// Sparse part, more workers: the workers' row lists (each ascending) are merged by one stable radix sort of
+// Sparse part, small lists and up to 1.8 M entries of 33 to 128 workers: the resident merge
+// (residentsort.cu).
+// Sparse part, more: the workers' row lists (each ascending) are merged by one stable radix sort of
 // (row id, position in the concatenated list); equal rows then sit together in ascending
 // worker order, and the tile-parallel segmented reduction (tile_reduce.cuh) forms each row's
 // weighted sum of its <= K contributions in that fixed order.  Because the sorted positions of
@@ -10,6 +12,7 @@
 // Dense part: a K-way streaming reduction, one 16-byte vector per thread and worker.
 #include "agg_range.cuh"
 #include "opt_math.cuh"
+#include "residentsort.cuh"
 #include "segsort.cuh"
 #include "tile_reduce.cuh"
 
@@ -22,7 +25,7 @@ struct AggLayout {
   SortLayout sort;
   RangeLayout range;
   size_t range_ws;
-  size_t sort_ws, bounds, weights, wuo, cwuo, drop, keys_a, keys_b, src, vals_t, run_start, head_bits,
+  size_t sort_ws, bounds, weights, wuo, cwuo, drop, keys_a, keys_b, src, vals_t, run_start, flags, head_bits,
       tile_first, head_part, tail_part, row_start, src_worker, bytes;
 };
 
@@ -44,6 +47,8 @@ AggLayout agg_layout(int64_t in_cap, int K, int dim) {
   L.run_start = o; o = align_up(o + 8 * (n + 1));
   const size_t tile = (size_t)red_tile_for((int64_t)n);
   const size_t n_tiles = (n + tile - 1) / tile;
+  // what the resident merge wants zeroed lies in one piece: its flag words, head bits, tile_first
+  L.flags = o;      o = align_up(o + 4 * kResFlagWords);
   L.head_bits = o;  o = align_up(o + 4 * head_bits_words((int64_t)n));
   L.tile_first = o; o = align_up(o + 4 * (n_tiles + 1));
   L.head_part = o;  o = align_up(o + 4 * n_tiles * (size_t)dim);
@@ -386,7 +391,7 @@ void sort_merge_order(const antdt_sparse_part* sp, const uint8_t* dropped, bool 
 int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
                        const int64_t* batch_sizes, const uint8_t* dropped, int32_t n_workers,
                        void* ws, size_t ws_bytes, int32_t* dev_status, void* stream,
-                       const FusedUpdate* fu = nullptr, const OrderFork* fork = nullptr) {
+                       const FusedUpdate* fu = nullptr, const OrderFork* fork = nullptr, bool merged = false) {
   const int K = n_workers;
   if (K < 1 || K > kMaxSegments || !batch_sizes || !ws || !aligned16(ws)) return ANTDT_ERR_INVALID_ARG;
   double tot = 0.0;
@@ -423,14 +428,49 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
   float hw[kMaxSegments];
   for (int i = 0; i < K; ++i)
     hw[i] = (dropped && dropped[i]) ? 0.f : (float)((double)batch_sizes[i] / tot);
-  // the range merge (up to 32 workers, sparse part present) carries the weights itself
+  // the two merges carry the weights themselves
+  const bool resident = sp && resident_merge_wanted(K, in_cap, sp->n_rows);
   const bool by_ranges = sp && K <= kRangeMaxWorkers && in_cap > 0;
-  if (!by_ranges) upload_small(hw, 4 * (size_t)K, w8 + L.weights, s);
+  if (!by_ranges && !resident) upload_small(hw, 4 * (size_t)K, w8 + L.weights, s);
 
   if (sp) {
     int64_t* bounds = (int64_t*)(w8 + L.bounds);
     const int64_t agg_cap = sp->out_cap < in_cap ? sp->out_cap : in_cap;
-    if (K <= kRangeMaxWorkers && in_cap > 0) {
+    if (merged) {
+      // the backward's sort made the merge order on the way
+    } else if (resident) {
+      cudaStream_t so = fork ? fork->side : s;
+      if (fork && cudaStreamWaitEvent(so, fork->ids_ready, 0) != cudaSuccess) return ANTDT_ERR_CUDA;
+      ResidentMergeArgs q = {};
+      q.uniq_ids = sp->uniq_ids; q.wuo_in = sp->worker_uniq_offsets; q.in_cap = in_cap; q.n_rows = sp->n_rows;
+      q.n_workers = K; q.agg_ids = sp->agg_ids; q.n_agg = sp->n_agg; q.out_cap = agg_cap;
+      q.wuo_out = (int64_t*)(w8 + L.wuo); q.n_entries = bounds; q.src = (uint32_t*)(w8 + L.src);
+      if (fu && K <= kRangeMaxWorkers) {
+        q.row_start = (uint32_t*)(w8 + L.row_start);
+        q.src_worker = (uint8_t*)(w8 + L.src_worker);
+      } else {
+        q.head_bits = (uint32_t*)(w8 + L.head_bits);
+        q.tile_first = (int32_t*)(w8 + L.tile_first);
+        while ((1 << q.tile_shift) < red_tile_for(in_cap)) ++q.tile_shift;
+      }
+      q.weights_dev = (float*)(w8 + L.weights);
+      for (int i = 0; i < K; ++i) {
+        q.weights[i] = hw[i];
+        if (dropped && dropped[i]) q.dropped[i >> 5] |= 1u << (i & 31);
+      }
+      q.flags = (uint32_t*)(w8 + L.flags); q.zero = q.flags;
+      const size_t zero_bytes = q.head_bits ? L.head_part - L.flags : 4 * kResFlagWords;
+      q.n_zero = (int64_t)(zero_bytes / 4);
+      if (!resident_sort_clears(in_cap) && cudaMemsetAsync(q.zero, 0, zero_bytes, so) != cudaSuccess)
+        return ANTDT_ERR_CUDA;
+      q.pairs = (uint2*)(w8 + L.keys_a);  // keys_a and keys_b lie side by side
+      q.hist = (uint16_t*)(w8 + L.sort_ws + L.sort.hist); q.status = dev_status;
+      const int32_t rc = resident_merge(q, so);
+      if (rc != ANTDT_OK) return rc;
+      if (fork && (cudaEventRecord(fork->order_done, so) != cudaSuccess ||
+                   cudaStreamWaitEvent(s, fork->order_done, 0) != cudaSuccess))
+        return ANTDT_ERR_CUDA;
+    } else if (K <= kRangeMaxWorkers && in_cap > 0) {
       // up to 32 workers: the merge order comes from the range-partitioned pass, no sort
       uint32_t dropped_bits = 0;
       for (int i = 0; i < K; ++i)
@@ -538,7 +578,7 @@ int32_t aggregate_update_forked(const antdt_sparse_part* sp, const antdt_dense_p
                                 int32_t dtype, int32_t opt, float lr, float eps, float beta1,
                                 float beta2, int64_t step, float* state0, float* state1, void* ws,
                                 size_t ws_bytes, int32_t* dev_status, void* stream,
-                                const OrderFork* fork) {
+                                const OrderFork* fork, bool merged) {
   if (!sp || !table || !state0 || step < 1) return ANTDT_ERR_INVALID_ARG;
   if (dtype != ANTDT_F32 && dtype != ANTDT_BF16) return ANTDT_ERR_INVALID_ARG;
   if (sp->dim % (dtype == ANTDT_BF16 ? 8 : 4)) return ANTDT_ERR_INVALID_ARG;
@@ -560,7 +600,31 @@ int32_t aggregate_update_forked(const antdt_sparse_part* sp, const antdt_dense_p
   fu.agg_out = nullptr;
   fu.p = make_opt_params(lr, eps, beta1, beta2, step);
   return aggregate_impl(sp, dp, batch_sizes, nullptr, n_workers, ws, ws_bytes, dev_status, stream, &fu,
-                        fork);
+                        fork, merged);
+}
+
+bool step_merge_targets(const antdt_sparse_part& sp, const int64_t* batch_sizes, int K, int64_t nnz, void* ws,
+                        size_t ws_bytes, StepMerge* m) {
+  if (!batch_sizes || !ws || sp.in_cap < 1 || sp.out_cap < 1 || sp.in_cap >= (1ll << 31) || !sp.agg_ids || !sp.n_agg ||
+      K > kStepMergeWorkers || !resident_sort_fits(K, nnz, sp.n_rows))
+    return false;
+  double tot = 0.0;
+  for (int i = 0; i < K; ++i) {
+    if (batch_sizes[i] < 0) return false;
+    tot += (double)batch_sizes[i];
+  }
+  if (!(tot > 0.0)) return false;
+  const AggLayout L = agg_layout(sp.in_cap, K, sp.dim);
+  if (ws_bytes < L.bytes) return false;
+  char* w8 = static_cast<char*>(ws);
+  m->agg_ids = sp.agg_ids; m->n_agg = sp.n_agg;
+  m->agg_cap = sp.out_cap < sp.in_cap ? sp.out_cap : sp.in_cap;
+  m->n_entries = (int64_t*)(w8 + L.bounds);
+  m->src = (uint32_t*)(w8 + L.src); m->src_worker = (uint8_t*)(w8 + L.src_worker); m->src_cap = sp.in_cap;
+  m->row_start = (uint32_t*)(w8 + L.row_start);
+  m->weights_dev = (float*)(w8 + L.weights);
+  for (int i = 0; i < kStepMergeWorkers; ++i) m->weights[i] = i < K ? (float)((double)batch_sizes[i] / tot) : 0.f;
+  return true;
 }
 }  // namespace antdt
 

@@ -47,6 +47,7 @@ struct PooledArrival {
   const cudaEvent_t* ready;
 };
 
+struct StepMerge;  // residentsort.cuh
 int32_t bwd_dedup_impl(const int32_t* row_ids, int64_t nnz, const int64_t* bag_offsets,
                        int64_t n_bags, int32_t bags_per_sample, const float* d_pooled, int32_t dim,
                        int64_t n_rows, int32_t n_workers, const int64_t* worker_sample_offsets,
@@ -54,8 +55,9 @@ int32_t bwd_dedup_impl(const int32_t* row_ids, int64_t nnz, const int64_t* bag_o
                        int32_t* sorted_occ, float* uniq_grads, int64_t out_cap, void* ws,
                        size_t ws_bytes, int32_t* dev_status, void* stream,
                        const PooledArrival* arrival,
-                       cudaEvent_t ids_done = nullptr);  // embbag_bwd.cu; ids_done: recorded once the
-                                                         // distinct ids and their offsets are written
+                       cudaEvent_t ids_done = nullptr, const StepMerge* merge = nullptr);
+// embbag_bwd.cu; ids_done: recorded once the distinct ids and their offsets are written; merge: the
+// sort also makes the aggregation's merge order (step_merge_targets said that it can)
 
 // A second stream for the aggregation's merge order, which needs the workers' id lists but not
 // their gradients: the order kernels wait for ids_ready on `side`, and the caller's stream waits
@@ -73,7 +75,8 @@ int32_t aggregate_update_forked(const antdt_sparse_part* sp, const antdt_dense_p
                                 int32_t dtype, int32_t opt, float lr, float eps, float beta1,
                                 float beta2, int64_t step, float* state0, float* state1, void* ws,
                                 size_t ws_bytes, int32_t* dev_status, void* stream,
-                                const OrderFork* fork);  // aggregate.cu
+                                const OrderFork* fork, bool merged = false);  // aggregate.cu
+// (merged: the merge order is in the workspace already)
 
 int32_t fwd_impl(const void* table, int32_t dtype, int64_t n_rows, int32_t dim, const int32_t* row_ids,
                  int64_t nnz, const int64_t* bag_offsets, int64_t n_bags, float* pooled,

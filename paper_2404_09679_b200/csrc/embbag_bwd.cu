@@ -1,6 +1,7 @@
 // Worker backward: per-worker dedup of row ids and segmented reduction of d_pooled rows to
 // the worker's mean row gradients.
 //
+// Small and mid-sized inputs: everything up to the runs in one kernel (residentsort.cu).  Otherwise:
 //   prep      occurrence range of every worker (from bag_offsets), 1/b_w scale, offset checks
 //   expand    bag index of every occurrence (the sort's payload)
 //   sort      stable radix sort by row id inside each worker's range     (segsort.cu)
@@ -12,6 +13,7 @@
 // sorted occurrences whatever rows they belong to, so a row that holds 20% of a field's
 // occurrences costs its tiles no more than anyone else's.  Every sum has a fixed order (inside a
 // tile by sorted position, across tiles by tile index), no floating-point atomics anywhere.
+#include "residentsort.cuh"
 #include "segsort.cuh"
 #include "bwd_walk.cuh"
 
@@ -22,7 +24,7 @@ size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct BwdLayout {
   SortLayout sort;
-  size_t sort_ws, wso, occ_bounds, worker_b, keys_a, keys_b, vals_t, head_bits, tile_first,
+  size_t sort_ws, wso, occ_bounds, worker_b, keys_a, keys_b, vals_t, flags_rs, head_bits, tile_first,
       head_part, tail_part, flags, tasks, bytes;
 };
 
@@ -40,13 +42,15 @@ BwdLayout bwd_layout(int64_t nnz, int dim, int K, int tile_len) {
   L.keys_a = o;     o = align_up(o + 4 * n);
   L.keys_b = o;     o = align_up(o + 4 * n);
   L.vals_t = o;     o = align_up(o + 4 * n);
-  L.head_bits = o;  o = align_up(o + 4 * head_bits_words((int64_t)n));
-  L.tile_first = o; o = align_up(o + 4 * (n_tiles + 1));
   const size_t n_str = walk_stretches((int64_t)n, tile_len, dim);
+  // what starts at zero, in one piece: flag words of the resident sort, head bits, task counter
+  L.flags_rs = o;   o = align_up(o + 4 * kResFlagWords);
+  L.head_bits = o;  o = align_up(o + 4 * head_bits_words((int64_t)n));
+  L.tasks = o;      o = align_up(o + 4 * (2 * n_str + 4));
+  L.tile_first = o; o = align_up(o + 4 * (n_tiles + 1));
   L.head_part = o;  o = align_up(o + 4 * n_str * (size_t)dim);
   L.tail_part = o;  o = align_up(o + 4 * n_str * (size_t)dim);
   L.flags = o;      o = align_up(o + n_str);
-  L.tasks = o;      o = align_up(o + 4 * (2 * n_str + 4));
   L.bytes = o;
   return L;
 }
@@ -133,7 +137,7 @@ int32_t bwd_dedup_impl(
     const int64_t* worker_sample_offsets, int32_t* uniq_ids, int64_t* worker_uniq_offsets,
     int64_t* seg_offsets, int32_t* sorted_occ, float* uniq_grads, int64_t out_cap, void* ws,
     size_t ws_bytes, int32_t* dev_status, void* stream, const PooledArrival* arrival,
-    cudaEvent_t ids_done) {
+    cudaEvent_t ids_done, const StepMerge* merge) {
   const int K = n_workers;
   if (nnz < 0 || n_bags < 0 || nnz >= (1ll << 31) || n_bags >= (1ll << 31) || n_rows < 1 ||
       n_rows >= (1ll << 31) || dim < 4 || dim > 1024 || dim % 4 || K < 1 || K > kMaxSegments ||
@@ -169,33 +173,55 @@ int32_t bwd_dedup_impl(
   uint32_t* vals_t = (uint32_t*)(w8 + L.vals_t);
   char* sort_ws = w8 + L.sort_ws;
 
-  // one launch for up to 255 workers; beyond that the offsets travel in pieces
-  if (!segsort_setup_workers(worker_sample_offsets, K, (int)bags_per_sample, bag_offsets, n_bags, nnz,
-                             d_worker_b, sort_ws, L.sort, dev_status, s)) {
-    upload_small(worker_sample_offsets, 8 * ((size_t)K + 1), d_wso, s);
-    ANTDT_LAUNCH("bwd_prep", bwd_prep_kernel, 1, 1024, 0, s, d_wso, K, (int)bags_per_sample,
-                 bag_offsets, n_bags, nnz, d_occ_bounds, d_worker_b, dev_status);
-    segsort_setup(d_occ_bounds, K, nnz, sort_ws, L.sort, s);
-  }
-
   const int key_bits = bits_for(n_rows);
-  const int P = sort_passes(key_bits);
-  // payload ping-pong ends in sorted_occ: start in whichever buffer makes the last pass land there
-  uint32_t* occ_out = reinterpret_cast<uint32_t*>(sorted_occ);
-  uint32_t* expand_to = (P % 2 == 1) ? vals_t : occ_out;
   bool scratch_zeroed = false;
-  if (n_bags > 0 && nnz > 0) {
-    const unsigned grid = (unsigned)((n_bags + 32 * 8 - 1) / (32 * 8));
-    ANTDT_LAUNCH("expand_bags", expand_bags_kernel, grid, 256, 0, s, bag_offsets, n_bags, nnz,
-                 expand_to, dev_status, (uint32_t*)(w8 + L.head_bits), (int64_t)head_bits_words(nnz),
-                 (int32_t*)(w8 + L.tasks));
+  uint32_t* occ_out = reinterpret_cast<uint32_t*>(sorted_occ);
+  if (resident_sort_fits(K, nnz, n_rows)) {
+    const size_t zero_bytes = L.tasks + 8 - L.flags_rs;
+    if (!resident_sort_clears(nnz) && cudaMemsetAsync(w8 + L.flags_rs, 0, zero_bytes, s) != cudaSuccess)
+      return ANTDT_ERR_CUDA;
     scratch_zeroed = true;
+    ResidentSortArgs q = {};
+    q.row_ids = row_ids; q.nnz = nnz; q.bag_offsets = bag_offsets; q.n_bags = n_bags;
+    q.bags_per_sample = bags_per_sample; q.n_rows = n_rows; q.n_workers = K;
+    q.seg_bounds = (int64_t*)(sort_ws + L.sort.seg_bounds); q.worker_b = d_worker_b;
+    q.sorted_occ = occ_out; q.uniq_ids = uniq_ids; q.run_start = seg_offsets;
+    q.seg_runs = worker_uniq_offsets; q.out_cap = out_cap;
+    q.head_bits = (uint32_t*)(w8 + L.head_bits); q.tile_first = (int32_t*)(w8 + L.tile_first);
+    while ((1 << q.tile_shift) < tile_len) ++q.tile_shift;
+    q.flags = (uint32_t*)(w8 + L.flags_rs);
+    q.zero = q.flags; q.n_zero = (int64_t)(zero_bytes / 4);
+    q.pairs = (uint2*)(w8 + L.keys_a);  // keys_a and keys_b lie side by side: 8 bytes per occurrence
+    q.hist = (uint16_t*)(sort_ws + L.sort.hist);
+    q.status = dev_status;
+    const int32_t rc = resident_sort(q, merge, worker_sample_offsets, s);
+    if (rc != ANTDT_OK) return rc;
+  } else {
+    // one launch for up to 255 workers; beyond that the offsets travel in pieces
+    if (!segsort_setup_workers(worker_sample_offsets, K, (int)bags_per_sample, bag_offsets, n_bags, nnz,
+                               d_worker_b, sort_ws, L.sort, dev_status, s)) {
+      upload_small(worker_sample_offsets, 8 * ((size_t)K + 1), d_wso, s);
+      ANTDT_LAUNCH("bwd_prep", bwd_prep_kernel, 1, 1024, 0, s, d_wso, K, (int)bags_per_sample,
+                   bag_offsets, n_bags, nnz, d_occ_bounds, d_worker_b, dev_status);
+      segsort_setup(d_occ_bounds, K, nnz, sort_ws, L.sort, s);
+    }
+
+    const int P = sort_passes(key_bits);
+    // payload ping-pong ends in sorted_occ: start in whichever buffer makes the last pass land there
+    uint32_t* expand_to = (P % 2 == 1) ? vals_t : occ_out;
+    if (n_bags > 0 && nnz > 0) {
+      const unsigned grid = (unsigned)((n_bags + 32 * 8 - 1) / (32 * 8));
+      ANTDT_LAUNCH("expand_bags", expand_bags_kernel, grid, 256, 0, s, bag_offsets, n_bags, nnz,
+                   expand_to, dev_status, (uint32_t*)(w8 + L.head_bits), (int64_t)head_bits_words(nnz),
+                   (int32_t*)(w8 + L.tasks));
+      scratch_zeroed = true;
+    }
+    segsort_run(reinterpret_cast<const uint32_t*>(row_ids), expand_to, keys_a, occ_out, keys_b,
+                vals_t, key_bits, n_rows, nnz, sort_ws, L.sort, dev_status, s);
+    segsort_runs(keys_a, nnz, uniq_ids, seg_offsets, worker_uniq_offsets, nullptr, out_cap,
+                 (uint32_t*)(w8 + L.head_bits), (int32_t*)(w8 + L.tile_first), tile_len, sort_ws,
+                 L.sort, dev_status, s, false, scratch_zeroed);
   }
-  segsort_run(reinterpret_cast<const uint32_t*>(row_ids), expand_to, keys_a, occ_out, keys_b,
-              vals_t, key_bits, n_rows, nnz, sort_ws, L.sort, dev_status, s);
-  segsort_runs(keys_a, nnz, uniq_ids, seg_offsets, worker_uniq_offsets, nullptr, out_cap,
-               (uint32_t*)(w8 + L.head_bits), (int32_t*)(w8 + L.tile_first), tile_len, sort_ws,
-               L.sort, dev_status, s, false, scratch_zeroed);
   if (ids_done && cudaEventRecord(ids_done, s) != cudaSuccess) return ANTDT_ERR_CUDA;
   if (nnz > 0) {
     TileArgs t;

@@ -1,0 +1,882 @@
+// The sort of a small or mid-sized backward by one wave of CTAs that stay for the whole of it.
+//
+// The multi-kernel sort (segsort.cu) is a chain of 8 to 14 short launches; on a small or mid-sized
+// batch each of them is a launch, a ramp and two or three memory round trips.  Here every CTA holds
+// up to 12288 consecutive (row id, bag) pairs in registers:
+//
+//   before      the workers' ranges, the ids, and the bag of every occurrence: first occurrences are
+//               marked in shared memory, a running maximum over the positions spreads the marks
+//   per pass    (by row id) rank inside the warp, digit counters summed over the CTA's warps and
+//               published; a barrier over the CTAs; everybody's counts give the first slot of every
+//               digit; the pairs go to their slots; a second barrier; every CTA takes the pairs of
+//               its own slots
+//   last pass   (by worker) takes everything to the workers' own order.  It ranks the runs of equal
+//               (worker, row) as well as the pairs: a run's rank among the runs of its worker is its
+//               place in the worker's list of distinct rows, so the lists, the run starts, the head
+//               bits and the tiles' first runs are written from here, with nothing left to do
+//
+// All workers are sorted by row as ONE array, so before the last pass the workers of a row stand in
+// ascending order: those runs ARE the aggregation's merge order.  In a step it is written on the way
+// and the merge's four kernels (agg_range.cu) are not needed.
+//
+// What a pass costs is the latency of its steps, 7 us for up to 1500 pairs a CTA, 25 us for 12288; the
+// cost that grows with the square of the CTAs (reading everybody's counts) keeps them to one per SM.  Small inputs
+// (up to 16 CTAs of 2048) run as one thread-block cluster: counts, pairs and barriers go through
+// distributed shared memory (a barrier 0.3 us against 1.3).
+// Measured (in brackets the kernels it replaced: sort, and merge order where a step makes it): 10 k
+// occurrences of 4 workers over 80 k rows 17 us (37 + 35); 426 k of 8 over 26 M 60 us (75 + 62);
+// 1.2 M of one worker over 1 M 99 us (113).
+//
+// The CTAs wait for one another, so the launch is a cluster or a cooperative one (all CTAs resident
+// or none started).  Every wait through memory is bounded all the same (kSpinLimit) and raises
+// ANTDT_ERR_TIMEOUT when it runs out; slots are checked, so even then nothing is written elsewhere.
+#include "residentsort.cuh"
+
+namespace antdt {
+namespace {
+
+constexpr int kThreads = kResThreads;
+constexpr int kWarps = kThreads / 32;
+constexpr int kBins = kSortMaxBins;  // 512 = one bin per thread
+constexpr int kMaxItems = 24;        // pairs per thread
+constexpr int kMinChunk = 1024;
+constexpr int kClusterItems = 4;     // pairs per thread of the cluster form
+constexpr int kMaxCluster = 16;
+constexpr uint32_t kSpinLimit = 1u << 20;
+static_assert(kBins == kThreads, "one digit per thread");
+
+struct Wso { int64_t v[kResMaxWorkers + 1]; };
+
+struct Smem {
+  union {
+    uint32_t mm[kWarps * kBins];          // while ranking: the lanes that hold a digit, per warp
+    uint32_t mark[kMaxItems * kThreads];  // before the sort: first occurrences of the bags
+  };
+  unsigned short wh[kWarps * kBins];      // per-warp digit counters, then their prefix over the warps
+  uint32_t cnt[kBins];                    // a counter's sum over the CTAs
+  uint32_t base[kBins];                   // first slot of every digit for this CTA
+  uint16_t row[kBins];                    // cluster form: this CTA's published counters
+  uint2 pairs[kClusterItems * kThreads];  // cluster form: the pairs of this CTA's slots
+  uint32_t warp_a[kWarps], warp_b[kWarps];
+  uint32_t warp_tot[kWarps];
+  int64_t bound[kResMaxWorkers + 1];      // occurrence range of every worker
+};
+
+// ---- the cluster ----
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// Address of a shared variable as seen in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t remote(const void* p, uint32_t rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ uint32_t ld_remote(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint4 ld_remote4(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_remote2(uint32_t addr, uint32_t x, uint32_t y) {
+  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(x), "r"(y) : "memory");
+}
+
+// Exclusive prefix sum over the block's 512 threads; *total (if not null) receives the sum.
+__device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* warp_tot, uint32_t* total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  uint32_t incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  __syncthreads();  // an earlier scan's readers are done
+  if (lane == 31) warp_tot[w] = incl;
+  __syncthreads();
+  uint32_t pre = 0, tot = 0;
+#pragma unroll
+  for (int i = 0; i < kWarps; ++i) {
+    const uint32_t t = warp_tot[i];
+    pre += i < w ? t : 0u;
+    tot += t;
+  }
+  if (total) *total = tot;
+  return incl - v + pre;
+}
+
+// Stable rank of every valid item among the items of its warp with the same digit; leaves the
+// warp's digit counts in my_wh.  my_mm: a word per digit, the lanes that hold it.  Both zeroed by
+// the caller.  Item i of lane l is element i*32 + l of the warp's `valid` leading elements.
+// The lanes of equal digit find each other by an atomic OR of their lane bits.  match.any does the
+// same in one instruction, but it takes time in proportion to the distinct values it finds, on a
+// unit that the whole SM shares: 62 cycles of the SM per warp instruction for 32 spread digits
+// against 10 for OR, read and clear (6 against 18 when there are only 4 distinct ones); nine votes
+// take 23.
+template <int IPT>
+__device__ __forceinline__ void warp_rank(const uint32_t (&k)[IPT], int valid, int shift, uint32_t mask,
+                                          unsigned short* my_wh, uint32_t* my_mm, unsigned short (&rank)[IPT]) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int i = 0; i < IPT; ++i) {
+    const bool ok = i * 32 + lane < valid;
+    const uint32_t d = (k[i] >> shift) & mask;
+    if (ok) atomicOr(my_mm + d, 1u << lane);
+    __syncwarp();
+    unsigned m = 0;
+    uint32_t old = 0;
+    if (ok) {
+      m = my_mm[d];
+      old = my_wh[d];
+    }
+    __syncwarp();
+    // every peer has read the mask and the counter; the first peer clears the one, bumps the other
+    if (ok && (m & lt) == 0) {
+      my_mm[d] = 0u;
+      my_wh[d] = (unsigned short)(old + __popc(m));
+    }
+    __syncwarp();
+    rank[i] = (unsigned short)(old + __popc(m & lt));
+  }
+}
+
+// Barrier over the CTAs: of the cluster, or `target` arrivals on a counter in memory that only
+// grows.  Orders their memory accesses.
+template <bool CLUSTER>
+__device__ __forceinline__ void all_barrier(uint32_t* counter, uint32_t target, int32_t* status) {
+  if (CLUSTER) {
+    cluster_arrive();
+    cluster_wait();
+    return;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(counter, 1u);
+    uint32_t x = 0;
+    for (uint32_t n = 0; n < kSpinLimit; ++n) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(counter) : "memory");
+      if (x >= target) break;
+    }
+    if (x < target) set_status(status, ANTDT_ERR_TIMEOUT);
+  }
+  __syncthreads();
+}
+
+// Sums of the C published rows of counters and of those before `rank`, per counter (the
+// returned values are those of counter threadIdx.x).  rows: 16-bit counters, kBins to a row, of
+// which the first nb are used.  A thread takes eight counters (one 16-byte load) of every 64th (or
+// 32nd, ...) part of the rows: this is the one step whose cost grows with the square of the CTAs.
+template <bool CLUSTER>
+__device__ __forceinline__ void sum_rows(Smem& S, const uint16_t* rows, uint32_t nb, int rank, int C,
+                                         uint32_t& total, uint32_t& before) {
+  const int tid = threadIdx.x;
+  const int q = nb >= 16 ? (int)(nb >> 3) : 2;  // a power of two: 16-byte columns of a row
+  const int col = tid & (q - 1), grp = tid / q, groups = kThreads / q;
+  S.cnt[tid] = 0u;
+  S.base[tid] = 0u;
+  __syncthreads();
+  uint32_t t[8], b[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) t[j] = b[j] = 0u;
+  const uint4* p = reinterpret_cast<const uint4*>(rows) + col;
+  constexpr int kRow = kBins / 8;  // uint4 per row
+  for (int c0 = grp; c0 < C; c0 += 4 * groups) {
+    uint4 x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      x[i] = c0 + i * groups >= C ? make_uint4(0u, 0u, 0u, 0u)
+             : CLUSTER ? ld_remote4(remote(S.row, (uint32_t)(c0 + i * groups)) + 16u * col)
+                       : __ldcg(p + (size_t)(c0 + i * groups) * kRow);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t on = c0 + i * groups < rank ? 0xffffffffu : 0u;
+      const uint32_t y[4] = {x[i].x, x[i].y, x[i].z, x[i].w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        t[2 * j] += y[j] & 0xffffu; t[2 * j + 1] += y[j] >> 16;
+        b[2 * j] += y[j] & 0xffffu & on; b[2 * j + 1] += (y[j] >> 16) & on;
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {  // counter col*8 + j at [j][col]: neighbouring lanes, neighbouring banks
+    if (t[j]) atomicAdd(&S.cnt[j * q + col], t[j]);
+    if (b[j]) atomicAdd(&S.base[j * q + col], b[j]);
+  }
+  __syncthreads();
+  const bool in = tid < 8 * q;
+  total = in ? S.cnt[(tid & 7) * q + (tid >> 3)] : 0u;
+  before = in ? S.base[(tid & 7) * q + (tid >> 3)] : 0u;
+}
+
+// First slot of every digit for this CTA: everybody's counts of smaller digits, then those of this
+// digit in CTAs of smaller rank.
+template <bool CLUSTER>
+__device__ __forceinline__ void digit_bases(Smem& S, const uint16_t* rows, uint32_t nb, int rank, int C) {
+  uint32_t total, before;
+  sum_rows<CLUSTER>(S, rows, nb, rank, C, total, before);
+  const uint32_t ex = block_scan(threadIdx.x < nb ? total : 0u, S.warp_tot, nullptr);  // barriers inside
+  S.base[threadIdx.x] = ex + before;
+}
+
+// The bag of every occurrence of this CTA's chunk [g0, g0 + n_mine), which lies in the occurrences
+// [beg, end) of the bags [bag0, bag1); CTA `rank` of the C that share these bags checks a share of
+// their offsets.  S.mark must be zero over the chunk.
+template <int IPT>
+__device__ __forceinline__ void chunk_bags(Smem& S, const ResidentSortArgs& a, int64_t bag0, int64_t bag1,
+                                           int64_t beg, int64_t end, int64_t g0, int n_mine, int rank, int C,
+                                           uint32_t (&v)[IPT]) {
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const int wbase = wp * 32 * IPT, valid = min(max(n_mine - wbase, 0), 32 * IPT);
+  {
+    // the offsets ascend: each CTA checks a share
+    const int64_t share = (bag1 - bag0 + C - 1) / C;
+    const int64_t b_end = min(bag1, bag0 + (rank + 1) * share);
+    bool bad = false;
+    for (int64_t b = bag0 + rank * share + tid; b < b_end; b += kThreads) {
+      const int64_t lo = __ldg(a.bag_offsets + b), hi = __ldg(a.bag_offsets + b + 1);
+      bad |= lo < beg || hi < lo || hi > end;
+    }
+    if (bad) set_status(a.status, ANTDT_ERR_BAD_OFFSETS);
+
+    // last bag that begins at or before the chunk: near where bags of equal length would put it,
+    // else by a search that looks at 512 offsets at a time
+    int64_t lo_b = bag0, hi_b = bag1;  // offset(lo_b) <= g0 < offset(hi_b) for ascending offsets
+    {
+      const int64_t guess = bag0 + (int64_t)((double)(bag1 - bag0) * (double)(g0 - beg) / (double)(end - beg));
+      const int64_t wl = max(bag0, min(guess - kThreads / 2, bag1 - kThreads));
+      const int64_t b = min(wl + tid, bag1);
+      const int c = __syncthreads_count(__ldg(a.bag_offsets + b) <= g0);
+      if (c > 0 && c < kThreads) { lo_b = wl + c - 1; hi_b = lo_b + 1; }
+      else if (c == 0) hi_b = wl;
+      else lo_b = min(wl + kThreads - 1, bag1 - 1);
+    }
+    while (hi_b - lo_b > 1) {  // uniform over the block
+      const int64_t step = (hi_b - lo_b + kThreads - 1) / kThreads;
+      const int64_t b = min(lo_b + step * tid, hi_b);
+      const int c = __syncthreads_count(b < hi_b && __ldg(a.bag_offsets + b) <= g0);
+      lo_b = lo_b + step * max(c - 1, 0);
+      hi_b = min(hi_b, lo_b + step);
+    }
+    constexpr int kBatch = 4;
+    for (int64_t b0 = lo_b; b0 < bag1; b0 += kBatch * kThreads) {
+      int64_t lo[kBatch], hi[kBatch];
+      bool past = false;
+#pragma unroll
+      for (int t = 0; t < kBatch; ++t) {
+        const int64_t b = min(b0 + t * kThreads + tid, bag1 - 1);
+        lo[t] = __ldg(a.bag_offsets + b);
+        hi[t] = __ldg(a.bag_offsets + b + 1);
+      }
+#pragma unroll
+      for (int t = 0; t < kBatch; ++t) {
+        const int64_t b = b0 + t * kThreads + tid;
+        const int64_t from = max(lo[t], g0);
+        past |= lo[t] >= g0 + n_mine;
+        if (b < bag1 && from < min(hi[t], g0 + n_mine)) S.mark[from - g0] = (uint32_t)(b - bag0) + 1u;
+      }
+      if (__syncthreads_or(past ? 1 : 0)) break;
+    }
+    __syncthreads();
+    uint32_t carry = 0;
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) {
+      uint32_t x = i * 32 + lane < valid ? S.mark[wbase + i * 32 + lane] : 0u;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) x = max(x, __shfl_up_sync(0xffffffffu, x, o));
+      x = max(x, carry);
+      v[i] = x;
+      carry = __shfl_sync(0xffffffffu, x, 31);
+    }
+    if (lane == 0) S.warp_tot[wp] = carry;
+    __syncthreads();
+    uint32_t pre = 1;
+#pragma unroll
+    for (int i = 0; i < kWarps; ++i) pre = max(pre, i < wp ? S.warp_tot[i] : 0u);
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) v[i] = (uint32_t)bag0 + max(v[i], pre) - 1u;
+  }
+}
+
+// Ranks of the CTA's items among those of equal digit: inside the warp (rk), the prefix over the
+// warps (S.wh), and the CTA's count of every digit, stored to my_row.
+template <int IPT>
+__device__ __forceinline__ void rank_and_publish(Smem& S, const uint32_t (&k)[IPT], int valid, int shift, uint32_t nb,
+                                                 uint16_t* my_row, unsigned short (&rk)[IPT]) {
+  const int tid = threadIdx.x, wp = tid >> 5;
+  __syncthreads();  // marks, counters and bases of the step before have been read
+  for (uint32_t i = tid; i < kWarps * nb / 2; i += kThreads) reinterpret_cast<uint32_t*>(S.wh)[i] = 0u;
+  for (uint32_t i = tid; i < kWarps * nb; i += kThreads) S.mm[i] = 0u;
+  __syncthreads();
+  warp_rank<IPT>(k, valid, shift, nb - 1u, S.wh + wp * nb, S.mm + wp * nb, rk);
+  __syncthreads();
+  uint32_t sum = 0;
+  if (tid < nb) {
+    uint32_t t[kWarps];
+#pragma unroll
+    for (int i = 0; i < kWarps; ++i) t[i] = S.wh[i * nb + tid];
+#pragma unroll
+    for (int i = 0; i < kWarps; ++i) {
+      S.wh[i * nb + tid] = (unsigned short)sum;
+      sum += t[i];
+    }
+  }
+  my_row[tid] = (uint16_t)sum;
+}
+
+// The passes by row id (the low key_bits of the keys) over the n pairs that C CTAs hold, ce to a CTA.
+// Leaves this CTA with the pairs of its own slots; the pairs of all slots can be read (until the next
+// barrier) in `pairs`, or in the CTAs' S.pairs.  Returns the arrivals on the barrier's counter.
+template <int IPT, bool CLUSTER>
+__device__ __forceinline__ uint32_t sort_passes_by_row(Smem& S, uint32_t (&k)[IPT], uint32_t (&v)[IPT], int key_bits,
+                                                       int64_t n, int64_t g0, int n_mine, int ce, int cta, int C,
+                                                       uint2* pairs, uint16_t* hist, uint32_t* counter,
+                                                       int32_t* status) {
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int wbase = wp * 32 * IPT, valid = min(max(n_mine - wbase, 0), 32 * IPT);
+  const int P = sort_passes(key_bits);
+  uint16_t* const my_row = CLUSTER ? S.row : hist + (size_t)cta * kBins;
+  // every CTA of a cluster arrives, but of the others only the C that hold pairs
+  uint32_t arrivals = 0;
+  int shift = 0;
+  for (int p = 0; p < P; ++p) {
+    const int bits = (key_bits - shift + (P - p) - 1) / (P - p);
+    const uint32_t nb = 1u << bits, dmask = nb - 1u;
+    unsigned short rk[IPT];
+    rank_and_publish<IPT>(S, k, valid, shift, nb, my_row, rk);
+    arrivals += C;
+    all_barrier<CLUSTER>(counter, arrivals, status);
+    digit_bases<CLUSTER>(S, hist, nb, cta, C);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) {
+      if (i * 32 + lane < valid) {
+        const uint32_t d = (k[i] >> shift) & dmask;
+        const uint32_t q = S.base[d] + S.wh[wp * nb + d] + rk[i];
+        if (CLUSTER) {
+          const uint32_t c = q / (uint32_t)ce;
+          if (c < (uint32_t)C) st_remote2(remote(S.pairs + (q - c * (uint32_t)ce), c), k[i], v[i]);
+        } else if (q < (uint32_t)n) {
+          __stcg(pairs + q, make_uint2(k[i], v[i]));
+        }
+      }
+    }
+    arrivals += C;
+    all_barrier<CLUSTER>(counter, arrivals, status);
+    shift += bits;
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) {
+      if (i * 32 + lane < valid) {
+        const uint2 kv = CLUSTER ? S.pairs[wbase + i * 32 + lane] : __ldcg(pairs + g0 + wbase + i * 32 + lane);
+        k[i] = kv.x;
+        v[i] = kv.y;
+      }
+    }
+  }
+  return arrivals;
+}
+
+// The pair before this warp's first slot (one lane asks).
+template <bool CLUSTER>
+__device__ __forceinline__ uint2 pair_before(Smem& S, const uint2* pairs, int64_t g0, int wbase, int ce, int cta) {
+  if (!CLUSTER) return __ldcg(pairs + g0 + wbase - 1);
+  if (wbase > 0) return S.pairs[wbase - 1];
+  const uint32_t at = remote(&S.pairs[ce - 1], (uint32_t)cta - 1u);
+  return make_uint2(ld_remote(at), ld_remote(at + 4));
+}
+
+// Keys are worker << key_bits | row; a row id outside the table becomes n_rows (key_bits holds it),
+// which every reader skips.
+template <int IPT, bool CLUSTER>
+__global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 2 : 1))
+resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_constant__ StepMerge m,
+                     const __grid_constant__ Wso wso) {
+  extern __shared__ __align__(16) unsigned char res_smem[];
+  Smem& S = *reinterpret_cast<Smem*>(res_smem);
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const int K = a.n_workers, F = a.bags_per_sample, cta = blockIdx.x, ce = a.chunk;
+  const bool merge = m.agg_ids != nullptr;
+
+  for (int i = tid; i < ce; i += kThreads) S.mark[i] = 0u;
+  if (CLUSTER) {  // (otherwise the flag words had to be cleared before the launch anyway)
+    for (int64_t i = (int64_t)cta * kThreads + tid; i < a.n_zero; i += (int64_t)gridDim.x * kThreads) a.zero[i] = 0u;
+  }
+  {  // the workers' ranges: ascending, inside [0, nnz], whatever the offsets hold
+    if (wp == 0) {
+      int64_t carry = 0;
+      for (int i0 = 0; i0 <= K; i0 += 32) {
+        const int i = i0 + lane;
+        const int64_t raw = i <= K ? __ldg(a.bag_offsets + wso.v[i] * (int64_t)F) : 0;
+        if (cta == 0 && ((i == 0 && raw != 0) || (i == K && raw != a.nnz)))
+          set_status(a.status, ANTDT_ERR_BAD_OFFSETS);
+        int64_t x = max(raw, carry);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int64_t t = __shfl_up_sync(0xffffffffu, x, o);
+          if (lane >= o) x = max(x, t);
+        }
+        carry = __shfl_sync(0xffffffffu, x, 31);
+        if (i <= K) S.bound[i] = min(x, a.nnz);
+      }
+    }
+    __syncthreads();
+  }
+  const int64_t n = S.bound[K];
+  const int C = (int)((n + ce - 1) / ce);
+  if (cta == 0) {
+    if (tid <= K) a.seg_bounds[tid] = S.bound[tid];
+    if (tid < K) a.worker_b[tid] = 1.0f / (float)(wso.v[tid + 1] - wso.v[tid]);  // inf for an empty worker: unused
+    if (merge && tid < K) m.weights_dev[tid] = m.weights[tid];
+    if (C == 0) {
+      if (tid <= K) a.seg_runs[tid] = 0;
+      if (tid == 0) {
+        a.run_start[0] = 0;
+        if (merge) { *m.n_agg = 0; m.n_entries[0] = 0; m.n_entries[1] = 0; }
+      }
+    }
+  }
+  // A CTA without pairs leaves, but a cluster's CTAs all stay (its barriers count every one).
+  if (CLUSTER ? C == 0 : cta >= C) return;
+  const int64_t g0 = (int64_t)cta * ce;
+  const int n_mine = (int)max((int64_t)0, min((int64_t)ce, n - g0));
+  const int wbase = wp * 32 * IPT;
+  const int valid = min(max(n_mine - wbase, 0), 32 * IPT);
+  uint32_t* const counter = a.flags;
+
+  uint32_t k[IPT], v[IPT];
+  {
+    const int32_t* ids = a.row_ids + g0 + wbase;
+    bool bad_id = false;
+    int w = 0;
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) {
+      k[i] = 0u;
+      v[i] = 0u;
+      if (i * 32 + lane < valid) {
+        uint32_t id = (uint32_t)__ldg(ids + i * 32 + lane);
+        if (id >= (uint32_t)a.n_rows) {
+          bad_id = true;
+          id = (uint32_t)a.n_rows;
+        }
+        const int64_t g = g0 + wbase + i * 32 + lane;
+        while (w < K - 1 && g >= S.bound[w + 1]) ++w;  // positions ascend
+        k[i] = ((uint32_t)w << a.key_bits) | id;
+      }
+    }
+    if (bad_id) set_status(a.status, ANTDT_ERR_ID_OUT_OF_RANGE);
+  }
+  if (n_mine > 0) chunk_bags<IPT>(S, a, 0, a.n_bags, 0, n, g0, n_mine, cta, C, v);
+
+  uint16_t* const my_row = CLUSTER ? S.row : a.hist + (size_t)cta * kBins;
+  uint32_t arrivals = sort_passes_by_row<IPT, CLUSTER>(S, k, v, a.key_bits, n, g0, n_mine, ce, cta, C, a.pairs, a.hist,
+                                                       counter, a.status);
+
+  // ---- runs of (row, worker) and of rows, in merge order ----
+  const uint32_t row_mask = a.key_bits < 32 ? (1u << a.key_bits) - 1u : 0xffffffffu;
+  uint32_t head_m = 0, row_m = 0;  // bit i: this lane's item i starts a run / a row
+  uint32_t heads_warp = 0, rows_warp = 0;  // of the whole warp
+  {
+    uint32_t left = 0;
+    if (lane == 0 && valid > 0 && g0 + wbase > 0) left = pair_before<CLUSTER>(S, a.pairs, g0, wbase, ce, cta).x;
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) {
+      uint32_t prev = __shfl_up_sync(0xffffffffu, k[i], 1);
+      if (lane == 0) prev = left;
+      left = __shfl_sync(0xffffffffu, k[i], 31);
+      const bool in = i * 32 + lane < valid, start = g0 + wbase + i * 32 + lane == 0;
+      const bool h = in && (start || prev != k[i]), r = in && (start || ((prev ^ k[i]) & row_mask) != 0u);
+      head_m |= (h ? 1u : 0u) << i;
+      row_m |= (r ? 1u : 0u) << i;
+      heads_warp += __popc(__ballot_sync(0xffffffffu, h));
+      rows_warp += __popc(__ballot_sync(0xffffffffu, r));
+    }
+  }
+  // ---- by worker: ranks of the pairs and of the runs among those of their worker ----
+  // counters of this pass: pairs of worker w at w, its runs at Kp + w; published besides: all runs, all rows
+  const uint32_t Kp = 1u << a.worker_bits, kB = 2u * Kp;
+  unsigned short rk[IPT], hk[IPT];
+  __syncthreads();
+  for (uint32_t i = tid; i < kWarps * kB / 2; i += kThreads) reinterpret_cast<uint32_t*>(S.wh)[i] = 0u;
+  for (uint32_t i = tid; i < kWarps * kB; i += kThreads) S.mm[i] = 0u;
+  __syncthreads();
+  {
+    const unsigned lt = (1u << lane) - 1u;
+    unsigned short* wh = S.wh + wp * kB;
+    uint32_t* mm = S.mm + wp * kB;
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) {
+      const bool ok = i * 32 + lane < valid, h = (head_m >> i) & 1u;
+      const uint32_t d = ok ? (uint32_t)((uint64_t)k[i] >> a.key_bits) : 0u;
+      if (ok) atomicOr(mm + d, 1u << lane);
+      const unsigned heads = __ballot_sync(0xffffffffu, h);
+      unsigned peers = 0;
+      uint32_t old = 0, old_h = 0;
+      if (ok) {
+        peers = mm[d];
+        old = wh[d];
+        old_h = wh[Kp + d];
+      }
+      __syncwarp();
+      if (ok && (peers & lt) == 0) {
+        mm[d] = 0u;
+        wh[d] = (unsigned short)(old + __popc(peers));
+        wh[Kp + d] = (unsigned short)(old_h + __popc(peers & heads));
+      }
+      __syncwarp();
+      rk[i] = (unsigned short)(old + __popc(peers & lt));
+      hk[i] = (unsigned short)(old_h + __popc(peers & heads & lt) + (h ? 1u : 0u));  // runs up to and with this item's
+    }
+  }
+  if (lane == 0) { S.warp_a[wp] = heads_warp; S.warp_b[wp] = rows_warp; }
+  __syncthreads();
+  uint32_t heads_pre = 0, rows_pre = 0, heads_cta = 0, rows_cta = 0;
+#pragma unroll
+  for (int i = 0; i < kWarps; ++i) {
+    heads_pre += i < wp ? S.warp_a[i] : 0u; heads_cta += S.warp_a[i];
+    rows_pre += i < wp ? S.warp_b[i] : 0u; rows_cta += S.warp_b[i];
+  }
+  if (tid < (int)kB) {
+    uint32_t sum = 0;
+    uint32_t t[kWarps];
+#pragma unroll
+    for (int i = 0; i < kWarps; ++i) t[i] = S.wh[i * kB + tid];
+#pragma unroll
+    for (int i = 0; i < kWarps; ++i) {
+      S.wh[i * kB + tid] = (unsigned short)sum;
+      sum += t[i];
+    }
+    my_row[tid] = (uint16_t)sum;
+  } else {
+    my_row[tid] = (uint16_t)(tid == (int)kB ? heads_cta : (tid == (int)kB + 1 ? rows_cta : 0u));
+  }
+  arrivals += C;
+  all_barrier<CLUSTER>(counter, arrivals, a.status);
+  {
+    uint32_t total, before;
+    sum_rows<CLUSTER>(S, a.hist, 2u * kB, cta, C, total, before);
+    if (CLUSTER) cluster_arrive();  // the last look at another CTA's memory; nobody leaves before the wait
+    // prefix over the workers' pairs, then over their runs (behind all n pairs)
+    const uint32_t ex = block_scan(tid < (int)kB ? total : 0u, S.warp_tot, nullptr);
+    const uint32_t own = tid < (int)Kp ? ex : ex - (uint32_t)n;
+    S.base[tid] = tid < (int)kB ? own + before : before;
+    S.cnt[tid] = tid < (int)kB ? own : total;
+    __syncthreads();
+  }
+  const uint32_t n_runs = S.cnt[kB], n_rows_all = S.cnt[kB + 1];
+  if (cta == 0) {
+    if (tid < K) a.seg_runs[tid] = S.cnt[Kp + tid];
+    if (tid == 0) {
+      a.seg_runs[K] = n_runs;
+      a.run_start[min((int64_t)n_runs, a.out_cap)] = n;
+      if (n_runs > a.out_cap) set_status(a.status, ANTDT_ERR_CAPACITY);
+      if (merge) {
+        *m.n_agg = n_rows_all;
+        m.n_entries[0] = 0;
+        m.n_entries[1] = n_runs;
+        if (n_rows_all > m.agg_cap) set_status(a.status, ANTDT_ERR_CAPACITY);
+      }
+    }
+  }
+  uint32_t mrun = S.base[kB] + heads_pre, mrow = S.base[kB + 1] + rows_pre;  // runs / rows before the warp
+  const uint32_t tile_mask = (1u << a.tile_shift) - 1u;
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int i = 0; i < IPT; ++i) {
+    const bool in = i * 32 + lane < valid, h = (head_m >> i) & 1u, r = (row_m >> i) & 1u;
+    const unsigned hb = __ballot_sync(0xffffffffu, h), rb = __ballot_sync(0xffffffffu, r);
+    if (in) {
+      const uint32_t w = (uint32_t)((uint64_t)k[i] >> a.key_bits), row = k[i] & row_mask;
+      const uint32_t q = S.base[w] + S.wh[wp * kB + w] + rk[i];
+      const uint32_t u = S.base[Kp + w] + S.wh[wp * kB + Kp + w] + hk[i] - 1u;  // this item's run in its worker's list
+      if (q < (uint32_t)n) {
+        a.sorted_occ[q] = v[i];
+        if ((q & tile_mask) == 0) a.tile_first[q >> a.tile_shift] = (int32_t)u;
+        if (h) {
+          atomicOr(a.head_bits + (q >> 5), 1u << (q & 31));
+          const uint32_t slot = mrun + __popc(hb & lt);
+          if (u < a.out_cap) {
+            a.uniq_ids[u] = (int32_t)row;
+            a.run_start[u] = q;
+          }
+          if (merge && slot < m.src_cap) {
+            m.src[slot] = u;
+            m.src_worker[slot] = (uint8_t)w;
+            if (r) {
+              const uint32_t x = mrow + __popc(rb & lt);
+              if (x < m.agg_cap) {
+                m.agg_ids[x] = (int32_t)row;
+                m.row_start[x] = slot;
+              }
+            }
+          }
+        }
+      }
+    }
+    mrun += __popc(hb);
+    mrow += __popc(rb);
+  }
+  if (CLUSTER) cluster_wait();
+}
+
+// The merge order of the workers' row lists by the same passes: (row id, position in the concatenated
+// lists) sorted by row id.  Positions are worker-major, so a row's entries stand in ascending worker
+// order.  An entry of a dropped worker or with an id outside the table gets the key n_rows, sorts
+// behind everything and counts for nothing.
+// It serves small lists (a cluster: 9 k entries of 5 workers 16 us against 30 for the range merge's
+// four kernels and two memsets) and lists of more than 32 workers.
+template <int IPT, bool CLUSTER>
+__global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 2 : 1))
+resident_merge_kernel(const __grid_constant__ ResidentMergeArgs a) {
+  extern __shared__ __align__(16) unsigned char res_smem[];
+  Smem& S = *reinterpret_cast<Smem*>(res_smem);
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const int K = a.n_workers, cta = blockIdx.x, ce = a.chunk;
+  if (CLUSTER)
+    for (int64_t i = (int64_t)cta * kThreads + tid; i < a.n_zero; i += (int64_t)gridDim.x * kThreads) a.zero[i] = 0u;
+  if (wp == 0) {  // ascending and inside [0, in_cap], whatever came in
+    int64_t carry = 0;
+    for (int i0 = 0; i0 <= K; i0 += 32) {
+      const int i = i0 + lane;
+      const int64_t raw = i <= K ? __ldg(a.wuo_in + i) : 0;
+      if (cta == 0 && i == K && (raw < 0 || raw > a.in_cap)) set_status(a.status, ANTDT_ERR_CAPACITY);
+      int64_t x = max(raw, carry);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int64_t t = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x = max(x, t);
+      }
+      carry = __shfl_sync(0xffffffffu, x, 31);
+      if (i <= K) S.bound[i] = min(x, a.in_cap);
+    }
+  }
+  __syncthreads();
+  const int64_t n = S.bound[K];
+  const int C = (int)((n + ce - 1) / ce);
+  if (cta == 0) {
+    for (int i = tid; i <= K; i += kThreads) a.wuo_out[i] = S.bound[i];
+    for (int i = tid; i < K; i += kThreads) a.weights_dev[i] = a.weights[i];
+    if (C == 0 && tid == 0) { *a.n_agg = 0; a.n_entries[0] = 0; a.n_entries[1] = 0; }
+  }
+  if (CLUSTER ? C == 0 : cta >= C) return;
+  const int64_t g0 = (int64_t)cta * ce;
+  const int n_mine = (int)max((int64_t)0, min((int64_t)ce, n - g0));
+  const int wbase = wp * 32 * IPT, valid = min(max(n_mine - wbase, 0), 32 * IPT);
+  uint32_t k[IPT], v[IPT];
+  {
+    bool bad_id = false;
+    int w = 0;
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) {
+      k[i] = 0u;
+      v[i] = 0u;
+      if (i * 32 + lane < valid) {
+        const int64_t g = g0 + wbase + i * 32 + lane;
+        uint32_t id = (uint32_t)__ldg(a.uniq_ids + g);
+        if (i == 0) w = min(interval_of(S.bound, K + 1, g), K - 1);
+        while (w < K - 1 && g >= S.bound[w + 1]) ++w;
+        const bool dropped = (a.dropped[w >> 5] >> (w & 31)) & 1u;
+        bad_id |= !dropped && id >= (uint32_t)a.n_rows;
+        k[i] = dropped || id >= (uint32_t)a.n_rows ? (uint32_t)a.n_rows : id;
+        v[i] = (uint32_t)g;
+      }
+    }
+    if (bad_id) set_status(a.status, ANTDT_ERR_ID_OUT_OF_RANGE);
+  }
+  uint32_t arrivals = sort_passes_by_row<IPT, CLUSTER>(S, k, v, a.key_bits, n, g0, n_mine, ce, cta, C, a.pairs, a.hist,
+                                                       a.flags, a.status);
+  // ---- rows; entries that count ----
+  uint32_t row_m = 0, rows_warp = 0, kept_warp = 0;
+  {
+    uint2 left = make_uint2(0u, 0u);
+    if (lane == 0 && valid > 0 && g0 + wbase > 0) left = pair_before<CLUSTER>(S, a.pairs, g0, wbase, ce, cta);
+    bool repeats = false;
+#pragma unroll
+    for (int i = 0; i < IPT; ++i) {
+      uint32_t pk = __shfl_up_sync(0xffffffffu, k[i], 1), pv = __shfl_up_sync(0xffffffffu, v[i], 1);
+      if (lane == 0) { pk = left.x; pv = left.y; }
+      left = make_uint2(__shfl_sync(0xffffffffu, k[i], 31), __shfl_sync(0xffffffffu, v[i], 31));
+      const bool in = i * 32 + lane < valid && k[i] < (uint32_t)a.n_rows;
+      const bool start = g0 + wbase + i * 32 + lane == 0, r = in && (start || pk != k[i]);
+      // the same row twice in one worker's list
+      if (in && !r) repeats |= interval_of(S.bound, K + 1, pv) == interval_of(S.bound, K + 1, v[i]);
+      row_m |= (r ? 1u : 0u) << i;
+      rows_warp += __popc(__ballot_sync(0xffffffffu, r));
+      kept_warp += __popc(__ballot_sync(0xffffffffu, in));
+    }
+    if (repeats) set_status(a.status, ANTDT_ERR_BAD_OFFSETS);
+  }
+  if (lane == 0) { S.warp_a[wp] = kept_warp; S.warp_b[wp] = rows_warp; }
+  __syncthreads();
+  uint32_t rows_pre = 0, kept_cta = 0, rows_cta = 0;
+#pragma unroll
+  for (int i = 0; i < kWarps; ++i) {
+    kept_cta += S.warp_a[i];
+    rows_pre += i < wp ? S.warp_b[i] : 0u;
+    rows_cta += S.warp_b[i];
+  }
+  uint16_t* const my_row = CLUSTER ? S.row : a.hist + (size_t)cta * kBins;
+  if (tid < 16) my_row[tid] = (uint16_t)(tid == 0 ? kept_cta : (tid == 1 ? rows_cta : 0u));
+  arrivals += C;
+  all_barrier<CLUSTER>(a.flags, arrivals, a.status);
+  {
+    uint32_t total, before;
+    sum_rows<CLUSTER>(S, a.hist, 16u, cta, C, total, before);
+    if (CLUSTER) cluster_arrive();  // the last look at another CTA's memory; nobody leaves before the wait
+    __syncthreads();
+    if (tid < 2) { S.cnt[tid] = total; S.base[tid] = before; }
+    __syncthreads();
+  }
+  if (cta == 0 && tid == 0) {
+    *a.n_agg = S.cnt[1];
+    a.n_entries[0] = 0;
+    a.n_entries[1] = S.cnt[0];
+    if (S.cnt[1] > a.out_cap) set_status(a.status, ANTDT_ERR_CAPACITY);
+  }
+  uint32_t mrow = S.base[1] + rows_pre;  // rows before the warp
+  const uint32_t tile_mask = (1u << a.tile_shift) - 1u;
+  const unsigned le = 0xffffffffu >> (31 - lane);
+#pragma unroll
+  for (int i = 0; i < IPT; ++i) {
+    const bool r = (row_m >> i) & 1u;
+    const unsigned rb = __ballot_sync(0xffffffffu, r);
+    if (i * 32 + lane < valid && k[i] < (uint32_t)a.n_rows) {
+      const uint32_t slot = (uint32_t)(g0 + wbase + i * 32 + lane);
+      const uint32_t x = mrow + __popc(rb & le) - 1u;  // index of this entry's row
+      a.src[slot] = v[i];
+      if (a.src_worker) a.src_worker[slot] = (uint8_t)min(interval_of(S.bound, K + 1, v[i]), K - 1);
+      if (r) {
+        if (x < a.out_cap) {
+          a.agg_ids[x] = (int32_t)k[i];
+          if (a.row_start) a.row_start[x] = slot;
+        }
+        if (a.head_bits) atomicOr(a.head_bits + (slot >> 5), 1u << (slot & 31));
+      }
+      if (a.tile_first && (slot & tile_mask) == 0) a.tile_first[slot >> a.tile_shift] = (int32_t)x;
+    }
+    mrow += __popc(rb);
+  }
+  if (CLUSTER) cluster_wait();
+}
+
+// The form a sort of nnz occurrences takes: one cluster of up to 16 CTAs, or one CTA per SM.
+struct Form { int ctas, chunk; bool cluster; };
+#define RESIDENT_DISPATCH(GO)                                   \
+  do {                                                          \
+    const int ipt = (f.chunk + kThreads - 1) / kThreads;        \
+    if (f.cluster && ipt <= 2) GO(2, true);                     \
+    if (f.cluster) GO(4, true);                                 \
+    if (ipt <= 4) GO(4, false);                                 \
+    if (ipt <= 8) GO(8, false);                                 \
+    if (ipt <= 16) GO(16, false);                               \
+    GO(24, false);                                              \
+  } while (0)
+Form form_for(int64_t nnz) {
+  Form f;
+  f.cluster = nnz <= (int64_t)kMaxCluster * kClusterItems * kThreads;
+  const int64_t most = f.cluster ? kMaxCluster : kNumSM;
+  int64_t c = (nnz + most - 1) / most;
+  c = (c + 31) & ~(int64_t)31;
+  f.chunk = (int)(c < kMinChunk ? kMinChunk : c);
+  f.ctas = (int)((nnz + f.chunk - 1) / f.chunk);
+  if (f.cluster)
+    while (f.ctas & (f.ctas - 1)) ++f.ctas;  // cluster sizes are powers of two; spare CTAs hold nothing
+  return f;
+}
+
+template <typename... P, typename... A>
+int32_t launch_one(const char* name, void (*kernel)(P...), const Form& f, cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)f.ctas);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = sizeof(Smem);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  if (f.cluster) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)f.ctas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const int tok = prof_begin(name, s);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  prof_end(tok, s);
+  return e == cudaSuccess ? ANTDT_OK : ANTDT_ERR_CUDA;
+}
+
+}  // namespace
+
+void resident_sort_prepare_device() {
+  static bool done[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (done[dev & 63]) return;
+  auto opt_in = [](auto* k, bool cluster) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
+    if (cluster) cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  };
+#define OPT_IN(IPT, CLUSTER)                            \
+  opt_in(resident_sort_kernel<IPT, CLUSTER>, CLUSTER);  \
+  opt_in(resident_merge_kernel<IPT, CLUSTER>, CLUSTER)
+  OPT_IN(2, true);
+  OPT_IN(4, true);
+  OPT_IN(4, false);
+  OPT_IN(8, false);
+  OPT_IN(16, false);
+  OPT_IN(24, false);
+#undef OPT_IN
+  done[dev & 63] = true;
+}
+
+bool resident_sort_fits(int K, int64_t nnz, int64_t n_rows) {
+  // worker and row in 32 bits; at most one CTA per SM
+  return nnz > 0 && K <= kResMaxWorkers && bits_for(K) + bits_for(n_rows + 1) <= 32 &&
+         nnz <= (int64_t)kNumSM * kThreads * kMaxItems;
+}
+
+bool resident_sort_clears(int64_t nnz) { return form_for(nnz).cluster; }
+
+int32_t resident_sort(const ResidentSortArgs& args, const StepMerge* merge, const int64_t* wso_host, cudaStream_t s) {
+  ResidentSortArgs a = args;
+  const Form f = form_for(a.nnz);
+  a.key_bits = bits_for(a.n_rows + 1);
+  a.worker_bits = a.n_workers <= 32 ? 5 : bits_for(a.n_workers);
+  a.chunk = f.chunk;
+  resident_sort_prepare_device();
+  Wso wso;
+  for (int i = 0; i <= kResMaxWorkers; ++i) wso.v[i] = wso_host[i < a.n_workers ? i : a.n_workers];
+  const StepMerge m = merge ? *merge : StepMerge{};
+#define SORT_GO(IPT, CLUSTER) \
+  return launch_one("resident_sort", resident_sort_kernel<IPT, CLUSTER>, f, s, a, m, wso)
+  RESIDENT_DISPATCH(SORT_GO);
+#undef SORT_GO
+}
+
+bool resident_merge_wanted(int K, int64_t in_cap, int64_t n_rows) {
+  // Small lists, whatever the workers; else the range merge is as fast or faster up to 32 workers.
+  return in_cap > 0 && K <= kResMaxWorkers && n_rows < (1ll << 31) - 1 &&
+         (form_for(in_cap).cluster || (K > 32 && in_cap <= (int64_t)kNumSM * kThreads * kMaxItems));
+}
+
+int32_t resident_merge(const ResidentMergeArgs& args, cudaStream_t s) {
+  ResidentMergeArgs a = args;
+  const Form f = form_for(a.in_cap);
+  a.key_bits = bits_for(a.n_rows + 1);
+  a.chunk = f.chunk;
+  resident_sort_prepare_device();
+#define MERGE_GO(IPT, CLUSTER) return launch_one("resident_merge", resident_merge_kernel<IPT, CLUSTER>, f, s, a)
+  RESIDENT_DISPATCH(MERGE_GO);
+#undef MERGE_GO
+}
+
+}  // namespace antdt

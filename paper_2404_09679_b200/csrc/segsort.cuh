@@ -52,7 +52,7 @@ struct SortLayout {
 };
 SortLayout sort_layout(int n_segments);
 
-inline int sort_passes(int key_bits) { return (key_bits + kSortMaxBits - 1) / kSortMaxBits; }
+__host__ __device__ inline int sort_passes(int key_bits) { return (key_bits + kSortMaxBits - 1) / kSortMaxBits; }
 // Words of the head-bit mask of n elements; readers look one tile past the last element.
 inline size_t head_bits_words(int64_t n) { return (size_t)(n / 32) + 4; }
 inline int bits_for(int64_t n_values) {  // bits needed for values in [0, n_values)

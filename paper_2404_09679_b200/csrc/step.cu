@@ -6,18 +6,38 @@
 
 #include "agg_range.cuh"
 #include "common.cuh"
+#include "residentsort.cuh"
 #include "segsort.cuh"
 
 namespace antdt {
+static antdt_sparse_part sparse_part_of(const antdt_step_desc* d) {
+  antdt_sparse_part sp;
+  sp.dim = d->dim; sp.n_rows = d->n_rows; sp.uniq_ids = d->d_uniq_ids;
+  sp.worker_uniq_offsets = d->d_worker_uniq_offsets; sp.uniq_grads = d->d_uniq_grads;
+  sp.in_cap = d->uniq_cap; sp.agg_ids = d->d_agg_ids; sp.agg_grads = d->d_agg_grads;
+  sp.n_agg = d->d_n_agg; sp.out_cap = d->agg_cap;
+  return sp;
+}
+
+// Whether this step's sort makes the aggregation's merge order on the way (small and mid-sized
+// batches with the one-pass server step), and where it puts it.  ws_skip: the backward's part of
+// the workspace, see fork_ws_skip.
+static bool step_merge_of(const antdt_step_desc* d, size_t ws_skip, StepMerge* m) {
+  if (ws_skip == 0 || !d->fuse_update || (d->opt != ANTDT_OPT_ADAGRAD && d->opt != ANTDT_OPT_ADAM)) return false;
+  return step_merge_targets(sparse_part_of(d), d->batch_sizes, d->n_workers, d->nnz,
+                            static_cast<char*>(d->ws) + ws_skip, d->ws_bytes - ws_skip, m);
+}
+
 // The server half of a step: aggregate, then update; in one pass when the descriptor asks for it.
 static int32_t server_step(const antdt_step_desc* d, antdt_sparse_part* sp, const antdt_dense_part* dp,
-                           void* stream, const OrderFork* fork = nullptr, size_t ws_skip = 0) {
+                           void* stream, const OrderFork* fork = nullptr, size_t ws_skip = 0,
+                           bool merged = false) {
   if (d->fuse_update && (d->opt == ANTDT_OPT_ADAGRAD || d->opt == ANTDT_OPT_ADAM)) {
     if (d->n_workers <= kRangeMaxWorkers) sp->agg_grads = nullptr;  // not materialised
     return aggregate_update_forked(sp, dp, d->batch_sizes, d->n_workers, d->table, d->dtype, d->opt,
                                    d->lr, d->eps, d->beta1, d->beta2, d->step, d->state0, d->state1,
                                    static_cast<char*>(d->ws) + ws_skip, d->ws_bytes - ws_skip,
-                                   d->d_status, stream, fork);
+                                   d->d_status, stream, fork, merged);
   }
   // a forked step keeps the aggregation's scratch behind the backward's (both are live at once)
   int32_t rc = weighted_aggregate_forked(sp, dp, d->batch_sizes, d->n_workers,
@@ -38,7 +58,7 @@ struct StepStreams {
   cudaStream_t in = nullptr, out = nullptr;
   cudaStream_t side_fwd = nullptr, side_order = nullptr;  // branches of a forked device step
   cudaEvent_t start, ids, dense, fwd, done, outdone;
-  cudaEvent_t fork, fwd_done, ids_done, order_done;
+  cudaEvent_t fwd_done, ids_done, order_done;
   cudaEvent_t piece[kMaxPieces];
 };
 StepStreams g_ss[64];
@@ -55,7 +75,7 @@ StepStreams* step_streams() {
     if (cudaStreamCreateWithFlags(&ss.side_fwd, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
     if (cudaStreamCreateWithFlags(&ss.side_order, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
     cudaEvent_t* ev[] = {&ss.start, &ss.ids, &ss.dense, &ss.fwd, &ss.done, &ss.outdone,
-                         &ss.fork, &ss.fwd_done, &ss.ids_done, &ss.order_done};
+                         &ss.fwd_done, &ss.ids_done, &ss.order_done};
     for (cudaEvent_t* e : ev)
       if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     for (cudaEvent_t& e : ss.piece)
@@ -63,6 +83,23 @@ StepStreams* step_streams() {
     ss.ready = true;
   }
   return &ss;
+}
+}  // namespace
+
+namespace {
+// Small and mid-sized steps keep the aggregation's scratch behind the backward's instead of on top of
+// it: the merge order is made beside the backward, by its sort or on a branch of the graph.
+constexpr int64_t kForkMaxNnz = (int64_t)1 << 22;
+
+size_t fork_ws_skip(const antdt_step_desc* d) { // 0: no room for it, or too large a step
+  if (d->nnz < 1 || d->nnz > kForkMaxNnz || d->n_workers > antdt::kRangeMaxWorkers ||
+      d->uniq_cap < 1)
+    return 0;
+  const size_t b = antdt_embbag_bwd_dedup_workspace_bytes(d->nnz, d->n_bags, d->dim, d->n_workers);
+  const size_t a = antdt_weighted_aggregate_workspace_bytes(d->uniq_cap, d->dim, d->n_workers);
+  const size_t skip = (b + 255) / 256 * 256;
+  if (b == 0 || a == 0 || d->ws_bytes < skip + a) return 0;
+  return skip;
 }
 }  // namespace
 
@@ -151,22 +188,23 @@ extern "C" int32_t antdt_bsp_step_host(const antdt_step_desc* d, void* stream) {
   if (d->h_pooled && d->n_bags > 0)
     CK(cudaMemcpyAsync(d->h_pooled, d->d_pooled_out, 4 * (size_t)d->n_bags * D,
                        cudaMemcpyDeviceToHost, ss->out));
+  size_t ws_skip = fork_ws_skip(d);
+  antdt::StepMerge merge;
+  const bool merged = antdt::step_merge_of(d, ws_skip, &merge);
+  if (!merged) ws_skip = 0;
   antdt::PooledArrival arrival{n_pieces, piece_entry_end, ss->piece};
   rc = antdt::bwd_dedup_impl(d->d_row_ids, d->nnz, d->d_bag_offsets, d->n_bags, d->bags_per_sample,
                               d->d_d_pooled, d->dim, d->n_rows, d->n_workers,
                               d->worker_sample_offsets, d->d_uniq_ids, d->d_worker_uniq_offsets,
                               d->d_seg_offsets, d->d_sorted_occ, d->d_uniq_grads, d->uniq_cap, d->ws,
-                              d->ws_bytes, d->d_status, stream, n_pieces > 0 ? &arrival : nullptr);
+                              d->ws_bytes, d->d_status, stream, n_pieces > 0 ? &arrival : nullptr, nullptr,
+                              merged ? &merge : nullptr);
   if (rc != ANTDT_OK) return rc;
   CK(cudaStreamWaitEvent(s, ss->dense, 0));
-  antdt_sparse_part sp;
-  sp.dim = d->dim; sp.n_rows = d->n_rows; sp.uniq_ids = d->d_uniq_ids;
-  sp.worker_uniq_offsets = d->d_worker_uniq_offsets; sp.uniq_grads = d->d_uniq_grads;
-  sp.in_cap = d->uniq_cap; sp.agg_ids = d->d_agg_ids; sp.agg_grads = d->d_agg_grads;
-  sp.n_agg = d->d_n_agg; sp.out_cap = d->agg_cap;
+  antdt_sparse_part sp = antdt::sparse_part_of(d);
   antdt_dense_part dp;
   dp.grads = d->d_dense_grads; dp.n = d->dense_n; dp.stride = d->dense_n; dp.out = d->d_dense_out;
-  rc = antdt::server_step(d, &sp, dense ? &dp : nullptr, stream);
+  rc = antdt::server_step(d, &sp, dense ? &dp : nullptr, stream, nullptr, ws_skip, merged);
   if (rc != ANTDT_OK) return rc;
   CK(cudaEventRecord(ss->done, s));
 
@@ -193,19 +231,6 @@ extern "C" int32_t antdt_bsp_step_host(const antdt_step_desc* d, void* stream) {
 // and the step time is the length of the dependency chain; it needs the aggregation's scratch
 // behind the backward's instead of on top of it.
 namespace {
-constexpr int64_t kForkMaxNnz = (int64_t)1 << 22;
-
-size_t fork_ws_skip(const antdt_step_desc* d) {  // 0: no room (or no reason) to fork
-  if (d->nnz < 1 || d->nnz > kForkMaxNnz || d->n_workers > antdt::kRangeMaxWorkers ||
-      d->uniq_cap < 1)
-    return 0;
-  const size_t b = antdt_embbag_bwd_dedup_workspace_bytes(d->nnz, d->n_bags, d->dim, d->n_workers);
-  const size_t a = antdt_weighted_aggregate_workspace_bytes(d->uniq_cap, d->dim, d->n_workers);
-  const size_t skip = (b + 255) / 256 * 256;
-  if (b == 0 || a == 0 || d->ws_bytes < skip + a) return 0;
-  return skip;
-}
-
 int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
   if (!d || d->nnz < 0 || d->n_bags < 0 || d->dim < 1 || !d->d_bag_offsets || !d->d_n_agg)
     return ANTDT_ERR_INVALID_ARG;
@@ -213,39 +238,47 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
   if (dense && !d->d_dense_out) return ANTDT_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   StepStreams* ss = nullptr;
-  size_t ws_skip = 0;
-  if (forked && (ws_skip = fork_ws_skip(d)) > 0) ss = step_streams();
-  if (!ss) ws_skip = 0;
+  size_t ws_skip = fork_ws_skip(d);
+  antdt::StepMerge merge;
+  const bool merged = antdt::step_merge_of(d, ws_skip, &merge);
+  if (forked && ws_skip > 0) ss = step_streams();
+  if (!ss && !merged) ws_skip = 0;
 #define CK(x) do { if ((x) != cudaSuccess) return ANTDT_ERR_CUDA; } while (0)
-  void* fwd_stream = stream;
-  if (ss) {
-    CK(cudaEventRecord(ss->fork, s));
-    CK(cudaStreamWaitEvent(ss->side_fwd, ss->fork, 0));
-    fwd_stream = ss->side_fwd;
+  auto forward = [&](void* st) {
+    return antdt::fwd_impl(d->table, d->dtype, d->n_rows, d->dim, d->d_row_ids, d->nnz, d->d_bag_offsets,
+                           d->n_bags, d->d_pooled_out, d->d_status, st, d->bags_per_sample);
+  };
+  auto backward = [&]() {
+    return antdt::bwd_dedup_impl(d->d_row_ids, d->nnz, d->d_bag_offsets, d->n_bags, d->bags_per_sample,
+                                 d->d_d_pooled, d->dim, d->n_rows, d->n_workers, d->worker_sample_offsets,
+                                 d->d_uniq_ids, d->d_worker_uniq_offsets, d->d_seg_offsets, d->d_sorted_occ,
+                                 d->d_uniq_grads, d->uniq_cap, d->ws, d->ws_bytes, d->d_status, stream, nullptr,
+                                 ss ? ss->ids_done : nullptr, merged ? &merge : nullptr);
+  };
+  int32_t rc;
+  if (!ss) {
+    rc = forward(stream);
+    if (rc == ANTDT_OK) rc = backward();
+    if (rc != ANTDT_OK) return rc;
+  } else {
+    // The forward waits for the sort although it needs nothing from it: started beside the sort
+    // it takes the SMs that the sort (the head of the longest chain) waits for.
+    CK(cudaEventRecord(ss->ids_done, s));  // recorded again behind the run detection
+    rc = backward();
+    CK(cudaStreamWaitEvent(ss->side_fwd, ss->ids_done, 0));
+    const int32_t rf = forward(ss->side_fwd);
+    CK(cudaEventRecord(ss->fwd_done, ss->side_fwd));  // joined even after an error
+    CK(cudaStreamWaitEvent(s, ss->fwd_done, 0));      // the update writes the table the forward reads
+    if (rf != ANTDT_OK) return rf;
+    if (rc != ANTDT_OK) return rc;
   }
-  int32_t rc = antdt::fwd_impl(d->table, d->dtype, d->n_rows, d->dim, d->d_row_ids, d->nnz,
-                               d->d_bag_offsets, d->n_bags, d->d_pooled_out, d->d_status, fwd_stream,
-                               d->bags_per_sample);
-  if (ss) CK(cudaEventRecord(ss->fwd_done, ss->side_fwd));  // joined below even after an error
-  if (rc == ANTDT_OK)
-    rc = antdt::bwd_dedup_impl(d->d_row_ids, d->nnz, d->d_bag_offsets, d->n_bags, d->bags_per_sample,
-                               d->d_d_pooled, d->dim, d->n_rows, d->n_workers,
-                               d->worker_sample_offsets, d->d_uniq_ids, d->d_worker_uniq_offsets,
-                               d->d_seg_offsets, d->d_sorted_occ, d->d_uniq_grads, d->uniq_cap, d->ws,
-                               d->ws_bytes, d->d_status, stream, nullptr, ss ? ss->ids_done : nullptr);
-  // the update writes the table the forward reads
-  if (ss) CK(cudaStreamWaitEvent(s, ss->fwd_done, 0));
-  if (rc != ANTDT_OK) return rc;
-  antdt_sparse_part sp;
-  sp.dim = d->dim; sp.n_rows = d->n_rows; sp.uniq_ids = d->d_uniq_ids;
-  sp.worker_uniq_offsets = d->d_worker_uniq_offsets; sp.uniq_grads = d->d_uniq_grads;
-  sp.in_cap = d->uniq_cap; sp.agg_ids = d->d_agg_ids; sp.agg_grads = d->d_agg_grads;
-  sp.n_agg = d->d_n_agg; sp.out_cap = d->agg_cap;
+  antdt_sparse_part sp = antdt::sparse_part_of(d);
   antdt_dense_part dp;
   dp.grads = d->d_dense_grads; dp.n = d->dense_n; dp.stride = d->dense_n; dp.out = d->d_dense_out;
   antdt::OrderFork fork;
   if (ss) fork = antdt::OrderFork{ss->side_order, ss->ids_done, ss->order_done};
-  return antdt::server_step(d, &sp, dense ? &dp : nullptr, stream, ss ? &fork : nullptr, ws_skip);
+  return antdt::server_step(d, &sp, dense ? &dp : nullptr, stream, ss && !merged ? &fork : nullptr, ws_skip,
+                            merged);
 #undef CK
 }
 }  // namespace
@@ -346,6 +379,7 @@ extern "C" int32_t antdt_bsp_step_graph(const antdt_step_desc* d, void* stream) 
 
   // miss: capture the four calls
   antdt::segsort_prepare_device();
+  antdt::resident_sort_prepare_device();
   antdt::range_prepare_device();
   if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     cudaGetLastError();  // e.g. the legacy default stream cannot be captured: plain launches
