@@ -55,9 +55,11 @@ int32_t bwd_dedup_impl(const int32_t* row_ids, int64_t nnz, const int64_t* bag_o
                        int32_t* sorted_occ, float* uniq_grads, int64_t out_cap, void* ws,
                        size_t ws_bytes, int32_t* dev_status, void* stream,
                        const PooledArrival* arrival,
-                       cudaEvent_t ids_done = nullptr, const StepMerge* merge = nullptr);
+                       cudaEvent_t ids_done = nullptr, const StepMerge* merge = nullptr,
+                       cudaEvent_t sort_started = nullptr);
 // embbag_bwd.cu; ids_done: recorded once the distinct ids and their offsets are written; merge: the
-// sort also makes the aggregation's merge order (step_merge_targets said that it can)
+// sort also makes the aggregation's merge order (step_merge_targets said that it can); sort_started:
+// recorded when the CTAs of the resident sort have begun
 
 // A second stream for the aggregation's merge order, which needs the workers' id lists but not
 // their gradients: the order kernels wait for ids_ready on `side`, and the caller's stream waits

@@ -137,7 +137,7 @@ int32_t bwd_dedup_impl(
     const int64_t* worker_sample_offsets, int32_t* uniq_ids, int64_t* worker_uniq_offsets,
     int64_t* seg_offsets, int32_t* sorted_occ, float* uniq_grads, int64_t out_cap, void* ws,
     size_t ws_bytes, int32_t* dev_status, void* stream, const PooledArrival* arrival,
-    cudaEvent_t ids_done, const StepMerge* merge) {
+    cudaEvent_t ids_done, const StepMerge* merge, cudaEvent_t sort_started) {
   const int K = n_workers;
   if (nnz < 0 || n_bags < 0 || nnz >= (1ll << 31) || n_bags >= (1ll << 31) || n_rows < 1 ||
       n_rows >= (1ll << 31) || dim < 4 || dim > 1024 || dim % 4 || K < 1 || K > kMaxSegments ||
@@ -194,7 +194,7 @@ int32_t bwd_dedup_impl(
     q.pairs = (uint2*)(w8 + L.keys_a);  // keys_a and keys_b lie side by side: 8 bytes per occurrence
     q.hist = (uint16_t*)(sort_ws + L.sort.hist);
     q.status = dev_status;
-    const int32_t rc = resident_sort(q, merge, worker_sample_offsets, s);
+    const int32_t rc = resident_sort(q, merge, worker_sample_offsets, s, sort_started);
     if (rc != ANTDT_OK) return rc;
   } else {
     // one launch for up to 255 workers; beyond that the offsets travel in pieces

@@ -790,13 +790,14 @@ Form form_for(int64_t nnz) {
 }
 
 template <typename... P, typename... A>
-int32_t launch_one(const char* name, void (*kernel)(P...), const Form& f, cudaStream_t s, const A&... args) {
+int32_t launch_one(const char* name, cudaEvent_t started, void (*kernel)(P...), const Form& f, cudaStream_t s,
+                   const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)f.ctas);
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = sizeof(Smem);
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   if (f.cluster) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)f.ctas;
@@ -808,6 +809,12 @@ int32_t launch_one(const char* name, void (*kernel)(P...), const Form& f, cudaSt
   }
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  if (started) {
+    at[1].id = cudaLaunchAttributeLaunchCompletionEvent;
+    at[1].val.launchCompletionEvent.event = started;
+    at[1].val.launchCompletionEvent.flags = 0;
+    cfg.numAttrs = 2;
+  }
   const int tok = prof_begin(name, s);
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
   prof_end(tok, s);
@@ -846,7 +853,8 @@ bool resident_sort_fits(int K, int64_t nnz, int64_t n_rows) {
 
 bool resident_sort_clears(int64_t nnz) { return form_for(nnz).cluster; }
 
-int32_t resident_sort(const ResidentSortArgs& args, const StepMerge* merge, const int64_t* wso_host, cudaStream_t s) {
+int32_t resident_sort(const ResidentSortArgs& args, const StepMerge* merge, const int64_t* wso_host, cudaStream_t s,
+                      cudaEvent_t started) {
   ResidentSortArgs a = args;
   const Form f = form_for(a.nnz);
   a.key_bits = bits_for(a.n_rows + 1);
@@ -857,7 +865,7 @@ int32_t resident_sort(const ResidentSortArgs& args, const StepMerge* merge, cons
   for (int i = 0; i <= kResMaxWorkers; ++i) wso.v[i] = wso_host[i < a.n_workers ? i : a.n_workers];
   const StepMerge m = merge ? *merge : StepMerge{};
 #define SORT_GO(IPT, CLUSTER) \
-  return launch_one("resident_sort", resident_sort_kernel<IPT, CLUSTER>, f, s, a, m, wso)
+  return launch_one("resident_sort", started, resident_sort_kernel<IPT, CLUSTER>, f, s, a, m, wso)
   RESIDENT_DISPATCH(SORT_GO);
 #undef SORT_GO
 }
@@ -874,7 +882,7 @@ int32_t resident_merge(const ResidentMergeArgs& args, cudaStream_t s) {
   a.key_bits = bits_for(a.n_rows + 1);
   a.chunk = f.chunk;
   resident_sort_prepare_device();
-#define MERGE_GO(IPT, CLUSTER) return launch_one("resident_merge", resident_merge_kernel<IPT, CLUSTER>, f, s, a)
+#define MERGE_GO(IPT, CLUSTER) return launch_one("resident_merge", (cudaEvent_t)nullptr, resident_merge_kernel<IPT, CLUSTER>, f, s, a)
   RESIDENT_DISPATCH(MERGE_GO);
 #undef MERGE_GO
 }

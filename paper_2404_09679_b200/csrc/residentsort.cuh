@@ -47,7 +47,9 @@ bool step_merge_targets(const antdt_sparse_part& sp, const int64_t* batch_sizes,
 bool resident_sort_fits(int n_workers, int64_t nnz, int64_t n_rows);
 bool resident_sort_clears(int64_t nnz);
 void resident_sort_prepare_device();  // kernel attributes; before a stream capture
-int32_t resident_sort(const ResidentSortArgs& a, const StepMerge* merge, const int64_t* wso_host, cudaStream_t s);
+// started: recorded once every CTA of the sort has begun (best effort), or nullptr
+int32_t resident_sort(const ResidentSortArgs& a, const StepMerge* merge, const int64_t* wso_host, cudaStream_t s,
+                      cudaEvent_t started = nullptr);
 
 // The merge order of the workers' row lists alone (the arrays of agg_range.cuh), for small lists and
 // for lists of 33 to 128 workers.

@@ -51,14 +51,16 @@ static int32_t server_step(const antdt_step_desc* d, antdt_sparse_part* sp, cons
 }  // namespace antdt
 
 namespace {
-// Side streams and events of the host-buffer step, created on first use for each device.
+// Side streams and events of the steps, created on first use for each device.  An event's wait must
+// follow its record with no other step's record in between, so a step holds `mu` while it is issued.
 constexpr int kMaxPieces = 16;  // the d_pooled copy is cut into at most this many pieces
 struct StepStreams {
+  std::mutex mu;
   bool ready = false;
   cudaStream_t in = nullptr, out = nullptr;
   cudaStream_t side_fwd = nullptr, side_order = nullptr;  // branches of a forked device step
   cudaEvent_t start, ids, dense, fwd, done, outdone;
-  cudaEvent_t fwd_done, ids_done, order_done;
+  cudaEvent_t fwd_done, ids_done, order_done, sort_started;
   cudaEvent_t piece[kMaxPieces];
 };
 StepStreams g_ss[64];
@@ -75,7 +77,7 @@ StepStreams* step_streams() {
     if (cudaStreamCreateWithFlags(&ss.side_fwd, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
     if (cudaStreamCreateWithFlags(&ss.side_order, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
     cudaEvent_t* ev[] = {&ss.start, &ss.ids, &ss.dense, &ss.fwd, &ss.done, &ss.outdone,
-                         &ss.fwd_done, &ss.ids_done, &ss.order_done};
+                         &ss.fwd_done, &ss.ids_done, &ss.order_done, &ss.sort_started};
     for (cudaEvent_t* e : ev)
       if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     for (cudaEvent_t& e : ss.piece)
@@ -119,6 +121,7 @@ extern "C" int32_t antdt_bsp_step_host(const antdt_step_desc* d, void* stream) {
   if (dense && (!d->d_dense_grads || !d->d_dense_out || !d->h_dense_out)) return ANTDT_ERR_INVALID_ARG;
   StepStreams* ss = step_streams();
   if (!ss) return ANTDT_ERR_CUDA;
+  std::lock_guard<std::mutex> lk(ss->mu);
 
 #define CK(x) do { if ((x) != cudaSuccess) return ANTDT_ERR_CUDA; } while (0)
   // inputs: everything earlier on the caller's stream first (the staging buffers are reused),
@@ -241,8 +244,14 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
   size_t ws_skip = fork_ws_skip(d);
   antdt::StepMerge merge;
   const bool merged = antdt::step_merge_of(d, ws_skip, &merge);
-  if (forked && ws_skip > 0) ss = step_streams();
+  // The resident sort leaves half of every SM to others and waits for latencies most of the time, so
+  // the forward runs beside it, started once the sort's CTAs are in place (before them it would take
+  // the SMs that they wait for).
+  const bool beside = antdt::resident_sort_fits(d->n_workers, d->nnz, d->n_rows);
+  if (beside || (forked && ws_skip > 0)) ss = step_streams();
   if (!ss && !merged) ws_skip = 0;
+  std::unique_lock<std::mutex> lk;
+  if (ss) lk = std::unique_lock<std::mutex>(ss->mu);
 #define CK(x) do { if ((x) != cudaSuccess) return ANTDT_ERR_CUDA; } while (0)
   auto forward = [&](void* st) {
     return antdt::fwd_impl(d->table, d->dtype, d->n_rows, d->dim, d->d_row_ids, d->nnz, d->d_bag_offsets,
@@ -253,7 +262,8 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
                                  d->d_d_pooled, d->dim, d->n_rows, d->n_workers, d->worker_sample_offsets,
                                  d->d_uniq_ids, d->d_worker_uniq_offsets, d->d_seg_offsets, d->d_sorted_occ,
                                  d->d_uniq_grads, d->uniq_cap, d->ws, d->ws_bytes, d->d_status, stream, nullptr,
-                                 ss ? ss->ids_done : nullptr, merged ? &merge : nullptr);
+                                 ss ? ss->ids_done : nullptr, merged ? &merge : nullptr,
+                                 ss && beside ? ss->sort_started : nullptr);
   };
   int32_t rc;
   if (!ss) {
@@ -261,12 +271,18 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
     if (rc == ANTDT_OK) rc = backward();
     if (rc != ANTDT_OK) return rc;
   } else {
-    // The forward waits for the sort although it needs nothing from it: started beside the sort
-    // it takes the SMs that the sort (the head of the longest chain) waits for.
-    CK(cudaEventRecord(ss->ids_done, s));  // recorded again behind the run detection
+    cudaEvent_t after = beside ? ss->sort_started : ss->ids_done;
+    CK(cudaEventRecord(after, s));  // recorded again by the backward
+    int32_t rf = ANTDT_OK;
+    if (!beside) {
+      CK(cudaStreamWaitEvent(ss->side_fwd, after, 0));
+      rf = forward(ss->side_fwd);
+    }
     rc = backward();
-    CK(cudaStreamWaitEvent(ss->side_fwd, ss->ids_done, 0));
-    const int32_t rf = forward(ss->side_fwd);
+    if (beside) {
+      CK(cudaStreamWaitEvent(ss->side_fwd, after, 0));
+      rf = forward(ss->side_fwd);
+    }
     CK(cudaEventRecord(ss->fwd_done, ss->side_fwd));  // joined even after an error
     CK(cudaStreamWaitEvent(s, ss->fwd_done, 0));      // the update writes the table the forward reads
     if (rf != ANTDT_OK) return rf;
@@ -276,8 +292,9 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
   antdt_dense_part dp;
   dp.grads = d->d_dense_grads; dp.n = d->dense_n; dp.stride = d->dense_n; dp.out = d->d_dense_out;
   antdt::OrderFork fork;
-  if (ss) fork = antdt::OrderFork{ss->side_order, ss->ids_done, ss->order_done};
-  return antdt::server_step(d, &sp, dense ? &dp : nullptr, stream, ss && !merged ? &fork : nullptr, ws_skip,
+  const bool order_fork = ss && forked && ws_skip > 0 && !merged;
+  if (order_fork) fork = antdt::OrderFork{ss->side_order, ss->ids_done, ss->order_done};
+  return antdt::server_step(d, &sp, dense ? &dp : nullptr, stream, order_fork ? &fork : nullptr, ws_skip,
                             merged);
 #undef CK
 }
