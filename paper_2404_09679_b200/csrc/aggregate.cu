@@ -45,7 +45,7 @@ AggLayout agg_layout(int64_t in_cap, int K, int dim) {
   L.src = o;       o = align_up(o + 4 * n);
   L.vals_t = o;    o = align_up(o + 4 * n);
   L.run_start = o; o = align_up(o + 8 * (n + 1));
-  const size_t tile = (size_t)red_tile_for((int64_t)n);
+  const size_t tile = (size_t)red_tile_for((int64_t)n, dim);
   const size_t n_tiles = (n + tile - 1) / tile;
   // what the resident merge wants zeroed lies in one piece: its flag words, head bits, tile_first
   L.flags = o;      o = align_up(o + 4 * kResFlagWords);
@@ -385,7 +385,7 @@ void sort_merge_order(const antdt_sparse_part* sp, const uint8_t* dropped, bool 
                 (uint32_t*)(w8 + L.vals_t), key_bits, 0, in_cap, sort_ws, L.sort, dev_status, s, true);
     segsort_runs(keys_a, in_cap, sp->agg_ids, (int64_t*)(w8 + L.run_start), nullptr, sp->n_agg,
                  agg_cap, (uint32_t*)(w8 + L.head_bits),
-                 (int32_t*)(w8 + L.tile_first), red_tile_for(in_cap > 0 ? in_cap : 1), sort_ws, L.sort, dev_status, s, true);
+                 (int32_t*)(w8 + L.tile_first), red_tile_for(in_cap > 0 ? in_cap : 1, sp->dim), sort_ws, L.sort, dev_status, s, true);
 }
 
 int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
@@ -451,7 +451,7 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
       } else {
         q.head_bits = (uint32_t*)(w8 + L.head_bits);
         q.tile_first = (int32_t*)(w8 + L.tile_first);
-        while ((1 << q.tile_shift) < red_tile_for(in_cap)) ++q.tile_shift;
+        while ((1 << q.tile_shift) < red_tile_for(in_cap, sp->dim)) ++q.tile_shift;
       }
       q.weights_dev = (float*)(w8 + L.weights);
       for (int i = 0; i < K; ++i) {
@@ -481,7 +481,7 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
       range_merge_order(sp->uniq_ids, sp->worker_uniq_offsets, in_cap, sp->n_rows, K, dropped_bits,
                         sp->agg_ids, sp->n_agg, agg_cap, (int64_t*)(w8 + L.wuo), bounds,
                         (uint32_t*)(w8 + L.src), fu ? nullptr : (uint32_t*)(w8 + L.head_bits),
-                        fu ? nullptr : (int32_t*)(w8 + L.tile_first), red_tile_for(in_cap),
+                        fu ? nullptr : (int32_t*)(w8 + L.tile_first), red_tile_for(in_cap, sp->dim),
                         fu ? (uint32_t*)(w8 + L.row_start) : nullptr,
                         fu ? (uint8_t*)(w8 + L.src_worker) : nullptr, hw, (float*)(w8 + L.weights),
                         w8 + L.range_ws, L.range, dev_status, so);
@@ -516,7 +516,7 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
       t.payload = (const uint32_t*)(w8 + L.src);
       t.head_bits = (const uint32_t*)(w8 + L.head_bits);
       t.tile_first = (const int32_t*)(w8 + L.tile_first);
-      t.tile = red_tile_for(in_cap);
+      t.tile = red_tile_for(in_cap, sp->dim);
       t.rows = sp->uniq_grads;
       t.dim = sp->dim;
       t.n_host = in_cap;

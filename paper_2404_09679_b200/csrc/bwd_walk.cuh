@@ -48,10 +48,7 @@ struct WalkScratch {
   bool tasks_zeroed = false;  // the caller has cleared the list's counter on this stream already
 };
 inline int walk_tiles_per_stretch(int dim) {  // = lane groups per CTA, see launch_bwd_walk
-  const int nvec = dim / 4;
-  int g = 1;
-  while (g < nvec && g < 32) g <<= 1;
-  return kRedThreads / g;
+  return kRedThreads / red_group(dim);
 }
 inline size_t walk_stretches(int64_t n, int tile, int dim) {
   const int64_t n_tiles = (n + tile - 1) / tile;

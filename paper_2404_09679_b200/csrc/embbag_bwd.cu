@@ -117,7 +117,7 @@ extern "C" size_t antdt_embbag_bwd_dedup_workspace_bytes(int64_t nnz, int64_t n_
                                                          int32_t n_workers) {
   (void)n_bags;
   if (nnz < 0 || dim < 1 || n_workers < 1 || n_workers > antdt::kMaxSegments) return 0;
-  return antdt::bwd_layout(nnz, dim, n_workers, antdt::red_tile_for(nnz)).bytes;
+  return antdt::bwd_layout(nnz, dim, n_workers, antdt::red_tile_for(nnz, dim)).bytes;
 }
 
 extern "C" size_t antdt_embbag_bwd_dedup_min_workspace_bytes(int64_t nnz, int64_t n_bags, int32_t dim,
@@ -155,7 +155,7 @@ int32_t bwd_dedup_impl(
   if (worker_sample_offsets[K] * (int64_t)bags_per_sample != n_bags) return ANTDT_ERR_INVALID_ARG;
   // short reduction tiles for a small input when the workspace has room for their partial sums,
   // the long tiles (the minimum workspace) otherwise
-  int tile_len = red_tile_for(nnz);
+  int tile_len = red_tile_for(nnz, dim);
   BwdLayout L = bwd_layout(nnz, dim, K, tile_len);
   if (ws_bytes < L.bytes && tile_len != kRedTile) {
     tile_len = kRedTile;

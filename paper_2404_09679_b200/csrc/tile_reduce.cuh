@@ -22,9 +22,20 @@ namespace antdt {
 constexpr int kRedTile = 64;       // sorted entries per reduction tile of a large input
 constexpr int kRedTileSmall = 16;  // ... of a small one: a tile is walked serially, so a small input
                                    // needs short tiles to fill the machine and to end soon
-constexpr int64_t kRedSmallN = (int64_t)1 << 20;
+// Lanes that share a tile: a 16-byte vector of the row each.
+inline int red_group(int dim) {
+  int g = 1;
+  while (g < dim / 4 && g < 32) g <<= 1;
+  return g;
+}
 // Tile length for an input of at most n entries (n: the host-side bound the launch is sized by).
-inline int red_tile_for(int64_t n) { return n <= kRedSmallN ? kRedTileSmall : kRedTile; }
+// Long tiles mean fewer partial sums, but they have to make two full waves of warps (4 CTAs of 8
+// warps per SM): 2.4 M entries of 16 floats are one wave of 64-entry tiles (walk 63 us, aggregation
+// 58) and four of 16-entry ones (48, 42); 1.2 M of 96 floats are four waves of the long ones (80 us
+// against 95).
+inline int red_tile_for(int64_t n, int dim) {
+  return n * red_group(dim) <= (int64_t)kRedTile * 32 * 2 * kNumSM * 32 ? kRedTileSmall : kRedTile;
+}
 constexpr int kRedThreads = 256;
 constexpr int kRedUnroll = 4;
 
