@@ -6,6 +6,7 @@ Device buffers are torch CUDA tensors (torch is used for device memory and strea
 """
 from __future__ import annotations
 
+import array
 import ctypes as C
 import os
 from typing import Optional, Sequence
@@ -172,21 +173,40 @@ def _check(rc: int, where: str):
         raise AntdtError(rc, where)
 
 
+# A call on a small batch costs its marshalling, so that part is kept to what ctypes takes as it is:
+# plain integers for pointers, the raw stream handle, typed arrays built in one go.
 def _dp(t: Optional[torch.Tensor]):
-    """Device (or pinned host) tensor -> raw pointer; None -> NULL."""
+    """Device (or pinned host) tensor -> address; None -> NULL."""
     if t is None:
         return None
     assert t.is_contiguous()
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
-def _i64s(xs: Sequence[int]):
-    return (C.c_int64 * len(xs))(*[int(x) for x in xs])
+class _i64s:
+    """Host int64 array; passes as its address."""
+    __slots__ = ("_a", "_as_parameter_")
+
+    def __init__(self, xs: Sequence[int]):
+        try:
+            self._a = array.array("q", xs)
+        except TypeError:  # not all integers
+            self._a = array.array("q", [int(x) for x in xs])
+        self._as_parameter_ = self._a.buffer_info()[0]
+
+
+def fill_i64s(dst, xs: Sequence[int]):
+    """Host int64 ctypes array <- sequence of the same length."""
+    try:
+        dst[:] = xs
+    except TypeError:
+        dst[:] = [int(x) for x in xs]
 
 
 def _f64s(xs: Sequence[float]):

@@ -108,8 +108,8 @@ class DeviceStep:
         d.d_d_pooled = d_pooled.data_ptr()
         d.d_dense_grads = None if dense_grads is None else dense_grads.data_ptr()
         d.dense_n = 0 if dense_grads is None else dense_grads.shape[1]
-        self._wso[:] = [int(x) for x in worker_sample_offsets]
-        self._bsz[:] = [int(x) for x in batch_sizes]
+        B.fill_i64s(self._wso, worker_sample_offsets)
+        B.fill_i64s(self._bsz, batch_sizes)
         if graph:
             B.antdt_bsp_step_graph(d, stream)
         else:
@@ -161,8 +161,8 @@ class HostStep:
         d.bags_per_sample = bags_per_sample
         d.h_d_pooled, d.h_dense_grads = p(h_d_pooled), p(h_dense_grads)
         d.dense_n = 0 if h_dense_grads is None else h_dense_grads.shape[1]
-        self._inner._wso[:] = [int(x) for x in worker_sample_offsets]
-        self._inner._bsz[:] = [int(x) for x in batch_sizes]
+        B.fill_i64s(self._inner._wso, worker_sample_offsets)
+        B.fill_i64s(self._inner._bsz, batch_sizes)
         d.d_row_ids, d.d_bag_offsets, d.d_d_pooled = p(st.d_row_ids), p(st.d_bag_offsets), p(st.d_d_pooled)
         d.d_dense_grads, d.d_pooled_out, d.d_dense_out = p(st.d_dense_grads), p(st.d_pooled_out), p(st.d_dense_out)
         d.d_n_agg, d.d_status = p(st.d_n_agg), p(st.d_status)
