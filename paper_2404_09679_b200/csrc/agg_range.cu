@@ -357,11 +357,13 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
                  });
 }
 
-size_t emit_smem(int r_log2, int K) {  // tables, small arrays, head bits of up to R*K slots
+// Tables, small arrays, and the head bits of up to R*K slots for a reader that wants them (without
+// them an SM works on 6 ranges of 32 workers at once instead of 4: 278 -> 249 us on 16.2 M entries).
+size_t emit_smem(int r_log2, int K, bool head_bits) {
   const size_t R = (size_t)1 << r_log2;
   const EmitShape e = emit_shape(r_log2, K);
   return 4 * (R >> e.mask_lg) + (e.fc16 ? 2 : 4) * R + 8 + 4 * (256 + 256 + 32 + 33 + 16) +
-         4 * (R * (size_t)K / 32 + 2) + 12;
+         (head_bits ? 4 * (R * (size_t)K / 32 + 2) : 0) + 12;
 }
 
 }  // namespace
@@ -384,7 +386,7 @@ void range_prepare_device() {
   bool& done = attr_set[dev_id & 63];
   if (done) return;
   cudaFuncSetAttribute(range_emit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)emit_smem(kRangeMaxLog2, kRangeMaxWorkers));
+                       (int)emit_smem(kRangeMaxLog2, kRangeMaxWorkers, true));
   done = true;
 }
 
@@ -416,7 +418,8 @@ void range_merge_order(const int32_t* uniq_ids, const int64_t* wuo_in, int64_t i
   if (head_bits) cudaMemsetAsync(head_bits, 0, head_bits_words(in_cap) * 4, s);
   // every tile's entry is written unless ids were skipped as invalid: start from a valid index
   if (tile_first) cudaMemsetAsync(tile_first, 0, 4 * ((size_t)((in_cap + tile - 1) >> tile_shift) + 1), s);
-  ANTDT_LAUNCH("agg_range_emit", range_emit_kernel, (unsigned)P, kRaThreads, emit_smem(r_log2, K), s,
+  ANTDT_LAUNCH("agg_range_emit", range_emit_kernel, (unsigned)P, kRaThreads,
+               emit_smem(r_log2, K, head_bits != nullptr), s,
                uniq_ids, bnd, wuo_out, K, P, r_log2, n_rows, dropped_bits, base, agg_ids, out_cap, src,
                head_bits, tile_first, tile_shift, row_start, src_worker, status);
 }
