@@ -450,13 +450,16 @@ radix_scatter_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __res
 constexpr int kRunThreads = 512;
 constexpr int kRunStrips = kRunThreads / 32;  // 16
 
-struct Strip { int64_t s0, lo, hi; };  // 128-aligned start, clipped [lo, hi)
+// Positions are 32-bit (fewer than 2^31 elements): at 64 bits the emit walk took 62 registers, so the
+// sort's 444 chunks ran as one and a half waves of two CTAs per SM; three fit now.
+struct Strip { uint32_t s0, lo, hi; };  // 128-aligned start, clipped [lo, hi)
 
-__device__ __forceinline__ Strip strip_of(int64_t b, int64_t e, int w) {
-  const int64_t ab = b & ~(int64_t)127;
-  const int64_t len = (((e - ab) + kRunStrips - 1) / kRunStrips + 127) & ~(int64_t)127;
+__device__ __forceinline__ Strip strip_of(int64_t b64, int64_t e64, int w) {
+  const uint32_t b = (uint32_t)b64, e = (uint32_t)e64;
+  const uint32_t ab = b & ~127u;
+  const uint32_t len = (((e - ab) + kRunStrips - 1) / kRunStrips + 127u) & ~127u;
   Strip st;
-  st.s0 = ab + (int64_t)w * len;
+  st.s0 = ab + (uint32_t)w * len;
   st.lo = max(st.s0, b);
   st.hi = min(e, st.s0 + len);
   return st;
@@ -464,7 +467,7 @@ __device__ __forceinline__ Strip strip_of(int64_t b, int64_t e, int w) {
 
 // The 4 keys [i, i+4) of a lane (i is a multiple of 4; the key buffers are 16-byte aligned).
 // Keys outside [lo, hi) are not loaded.
-__device__ __forceinline__ void load4(const uint32_t* __restrict__ keys, int64_t i, const Strip& st,
+__device__ __forceinline__ void load4(const uint32_t* __restrict__ keys, uint32_t i, const Strip& st,
                                       uint32_t (&k)[4]) {
   if (i >= st.lo && i + 4 <= st.hi) {
     const uint4 v = __ldg(reinterpret_cast<const uint4*>(keys + i));
@@ -477,14 +480,14 @@ __device__ __forceinline__ void load4(const uint32_t* __restrict__ keys, int64_t
 
 // 4-bit mask: bit j set iff key i+j is inside the strip and starts a run.  prev_k3 is the last
 // key of the lane to the left (meaningful when that key lies inside the strip).
-__device__ __forceinline__ unsigned heads4(const uint32_t* __restrict__ keys, int64_t i, const Strip& st,
-                                           int64_t seg_begin, const uint32_t (&k)[4], uint32_t prev_k3,
+__device__ __forceinline__ unsigned heads4(const uint32_t* __restrict__ keys, uint32_t i, const Strip& st,
+                                           uint32_t seg_begin, const uint32_t (&k)[4], uint32_t prev_k3,
                                            int lane) {
   unsigned m = 0;
   uint32_t prev = prev_k3;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const int64_t e = i + j;
+    const uint32_t e = i + j;
     if (e >= st.lo && e < st.hi) {
       bool h;
       if (e == seg_begin) h = true;
@@ -499,7 +502,7 @@ __device__ __forceinline__ unsigned heads4(const uint32_t* __restrict__ keys, in
   return m;
 }
 
-__global__ void __launch_bounds__(kRunThreads)
+__global__ void __launch_bounds__(kRunThreads, kSortCtasPerSM)
 runs_count_kernel(const uint32_t* __restrict__ keys, const SortDesc* __restrict__ desc,
                   const int32_t* __restrict__ chunk_seg, const int64_t* __restrict__ seg_bounds,
                   const int64_t* __restrict__ chunk_begin, const int64_t* __restrict__ chunk_end,
@@ -508,11 +511,11 @@ runs_count_kernel(const uint32_t* __restrict__ keys, const SortDesc* __restrict_
   if (c >= desc->n_chunks) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const Strip st = strip_of(chunk_begin[c], chunk_end[c], w);
-  const int64_t seg_begin = seg_bounds[chunk_seg[c]];
+  const uint32_t seg_begin = (uint32_t)seg_bounds[chunk_seg[c]];
   int cnt = 0;
-  for (int64_t j0 = st.s0; j0 < st.hi; j0 += 256) {
+  for (uint32_t j0 = st.s0; j0 < st.hi; j0 += 256) {
     uint32_t ka[4], kb[4];
-    const int64_t ia = j0 + lane * 4, ib = ia + 128;
+    const uint32_t ia = j0 + lane * 4, ib = ia + 128;
     load4(keys, ia, st, ka);
     load4(keys, ib, st, kb);
     const uint32_t pa = __shfl_up_sync(0xffffffffu, ka[3], 1);
@@ -557,25 +560,25 @@ runs_scan_kernel(const SortDesc* __restrict__ desc, const int32_t* __restrict__ 
 }
 
 // One warp step of the emit walk: the 128 keys [i0, i0+128), 4 per lane.
-__device__ __forceinline__ void emit_step(const uint32_t* __restrict__ keys, int64_t i0, const Strip& st,
-                                          int64_t b, int64_t e, int64_t seg_begin, const uint32_t (&k)[4],
-                                          int lane, int64_t& running, int32_t* __restrict__ uniq_keys,
-                                          int64_t* __restrict__ run_start, int64_t out_cap,
+__device__ __forceinline__ void emit_step(const uint32_t* __restrict__ keys, uint32_t i0, const Strip& st,
+                                          uint32_t b, uint32_t e, uint32_t seg_begin, const uint32_t (&k)[4],
+                                          int lane, uint32_t& running, int32_t* __restrict__ uniq_keys,
+                                          int64_t* __restrict__ run_start, uint32_t out_cap,
                                           uint32_t* head_bits, int32_t* __restrict__ tile_first,
                                           int tile_shift) {
-  const int64_t i = i0 + lane * 4;
+  const uint32_t i = i0 + lane * 4;
   const uint32_t prev = __shfl_up_sync(0xffffffffu, k[3], 1);
   const unsigned m = heads4(keys, i, st, seg_begin, k, prev, lane);
   // heads in the lanes to the left: inclusive warp scan of the per-lane counts
-  const int mine = __popc(m);
-  int incl = mine;
+  const uint32_t mine = __popc(m);
+  uint32_t incl = mine;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += t;
   }
-  int64_t r = running + (incl - mine);  // runs that start before this lane's first key
-  if (tile_first && i >= st.lo && i < st.hi && (i & (((int64_t)1 << tile_shift) - 1)) == 0)
+  uint32_t r = running + (incl - mine);  // runs that start before this lane's first key
+  if (tile_first && i >= st.lo && i < st.hi && (i & ((1u << tile_shift) - 1u)) == 0)
     tile_first[i >> tile_shift] = (int32_t)(r + (m & 1u) - 1);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
@@ -595,7 +598,7 @@ __device__ __forceinline__ void emit_step(const uint32_t* __restrict__ keys, int
     word |= __shfl_xor_sync(0xffffffffu, word, 2);
     word |= __shfl_xor_sync(0xffffffffu, word, 4);
     if ((lane & 7) == 0 && word) {
-      const int64_t w0 = i0 + (lane >> 3) * 32;
+      const uint32_t w0 = i0 + (lane >> 3) * 32;
       if (w0 >= b && w0 + 32 <= e) head_bits[w0 >> 5] = word;
       else atomicOr(&head_bits[w0 >> 5], word);
     }
@@ -603,21 +606,21 @@ __device__ __forceinline__ void emit_step(const uint32_t* __restrict__ keys, int
   running += __shfl_sync(0xffffffffu, incl, 31);
 }
 
-__global__ void __launch_bounds__(kRunThreads)
+__global__ void __launch_bounds__(kRunThreads, kSortCtasPerSM)
 runs_emit_kernel(const uint32_t* __restrict__ keys, const SortDesc* __restrict__ desc,
                  const int32_t* __restrict__ chunk_seg, const int64_t* __restrict__ seg_bounds,
                  const int64_t* __restrict__ chunk_begin, const int64_t* __restrict__ chunk_end,
                  const int64_t* __restrict__ strip_runs, int32_t* __restrict__ uniq_keys,
-                 int64_t* __restrict__ run_start, int64_t out_cap, uint32_t* head_bits,
+                 int64_t* __restrict__ run_start, uint32_t out_cap, uint32_t* head_bits,
                  int32_t* __restrict__ tile_first, int tile_shift) {
   const int c = blockIdx.x;
   if (c >= desc->n_chunks) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t b = chunk_begin[c], e = chunk_end[c];
+  const uint32_t b = (uint32_t)chunk_begin[c], e = (uint32_t)chunk_end[c];
   const Strip st = strip_of(b, e, w);
-  const int64_t seg_begin = seg_bounds[chunk_seg[c]];
-  int64_t running = strip_runs[(size_t)c * kRunStrips + w];  // runs that start before this strip
-  for (int64_t j0 = st.s0; j0 < st.hi; j0 += 256) {
+  const uint32_t seg_begin = (uint32_t)seg_bounds[chunk_seg[c]];
+  uint32_t running = (uint32_t)strip_runs[(size_t)c * kRunStrips + w];  // runs that start before this strip
+  for (uint32_t j0 = st.s0; j0 < st.hi; j0 += 256) {
     uint32_t ka[4], kb[4];
     load4(keys, j0 + lane * 4, st, ka);
     load4(keys, j0 + 128 + lane * 4, st, kb);
@@ -757,7 +760,7 @@ void segsort_runs(const uint32_t* sorted_keys, int64_t n_cap, int32_t* uniq_keys
                n_runs_out, run_start, out_cap, status);
   ANTDT_LAUNCH(agg ? "agg_runs_emit" : "runs_emit", runs_emit_kernel, L.max_chunks, kRunThreads, 0, s, sorted_keys, desc,
                chunk_seg, seg_bounds, chunk_begin, chunk_end, chunk_runs, uniq_keys, run_start,
-               out_cap, head_bits, tile_first, tile_shift);
+               (uint32_t)(out_cap < (1ll << 31) ? out_cap : (1ll << 31)), head_bits, tile_first, tile_shift);
 }
 
 }  // namespace antdt
