@@ -712,13 +712,14 @@ void segsort_run(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* key
   uint32_t* bin_total = (uint32_t*)(ws + L.bin_total);
   const int P = sort_passes(key_bits);
   segsort_prepare_device();
-  // spread the bits evenly over the passes
+  // Spread the bits evenly over the passes, the wider digits last: the first pass sees the keys in
+  // random order, so its writes are the most scattered (25 bits as 8+8+9 instead of 9+8+8).
   int shift = 0;
   const uint32_t* kin = keys_in;
   const uint32_t* vin = vals_in;
   const int S = L.n_segments;
   for (int p = 0; p < P; ++p) {
-    const int bits = (key_bits - shift + (P - p) - 1) / (P - p);
+    const int bits = (key_bits - shift) / (P - p);
     const uint32_t mask = (1u << bits) - 1u;
     // the last pass lands in the output buffers, the one before in the temporaries, ...
     const bool to_out = ((P - 1 - p) % 2) == 0;
