@@ -70,43 +70,75 @@ bwd_prep_kernel(const int64_t* __restrict__ wso, int K, int F, const int64_t* __
   }
 }
 
-// One warp expands 32 consecutive bags: lane l holds the end offset of bag b0+l, every
-// occurrence of the warp's range finds its bag by a 5-step search over the lanes' values.
+// One warp expands kExpandGroups x 32 consecutive bags: lane l holds the end offset of bag l of every
+// group, all requested at once (the kernel is one dependent load and a stream of stores).
+// A lane finds the bag of one occurrence by a 5-step search over the lanes' ends and walks on from
+// there for the three that follow: one 16-byte store (the first and last few occurrences of a group,
+// off the 16-byte grid, go one by one).
+// 5.2 M bags, 105 M occurrences: 129 us, were 162 with one group per warp and a search and a 4-byte
+// store per occurrence.
+constexpr int kExpandGroups = 4;
 __global__ void __launch_bounds__(256)
 expand_bags_kernel(const int64_t* __restrict__ bag_offsets, int64_t n_bags, int64_t nnz,
                    uint32_t* __restrict__ occ_bag, int32_t* status, uint32_t* __restrict__ zero_words,
                    int64_t n_zero_words, int32_t* __restrict__ zero_pair) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int64_t first_bag = warp * (32 * kExpandGroups);
+  int64_t at[kExpandGroups + 1];  // offset of bag 32 g + lane (past the last bag: the end)
+#pragma unroll
+  for (int g = 0; g <= kExpandGroups; ++g)
+    at[g] = __ldg(bag_offsets + min(first_bag + 32 * g + (g < kExpandGroups ? lane : 0), n_bags));
   // scratch that later kernels of the call expect zeroed (the run heads' bit mask, the fix-up's
   // task counter): cleared here, on the way, instead of by two memsets in the chain of launches
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_zero_words;
        i += (int64_t)gridDim.x * blockDim.x)
     zero_words[i] = 0u;
   if (blockIdx.x == 0 && threadIdx.x < 2 && zero_pair) zero_pair[threadIdx.x] = 0;
-  const int lane = threadIdx.x & 31;
-  const int64_t b0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
-  if (b0 >= n_bags) return;
-  const int64_t b = min(b0 + lane, n_bags - 1);
-  const int64_t lo = bag_offsets[b], hi = bag_offsets[b + 1];
-  const bool bad = lo < 0 || hi < lo || hi > nnz;
-  if (__any_sync(0xffffffffu, bad)) {  // skip the whole group; readers bound-check bag indices
-    if (lane == 0) set_status(status, ANTDT_ERR_BAD_OFFSETS);
-    return;
-  }
-  const int64_t first = __shfl_sync(0xffffffffu, lo, 0);
-  const int64_t last = __shfl_sync(0xffffffffu, hi, 31);  // lanes past n_bags repeat the last bag
-  const int64_t span = last - first;
-  if (span >= (1ll << 31)) return;  // cannot happen: nnz < 2^31
-  const int my_end = (int)(hi - first);  // ascending over the lanes
-  for (int64_t base = 0; base < span; base += 32) {
-    const int o = (int)base + lane;
-    // first lane whose end is > o
-    int l = 0;
 #pragma unroll
-    for (int step = 16; step > 0; step >>= 1) {
-      const int e = __shfl_sync(0xffffffffu, my_end, l + step - 1);
-      if (e <= o) l += step;
+  for (int g = 0; g < kExpandGroups; ++g) {
+    const int64_t b0 = first_bag + 32 * g;
+    if (b0 >= n_bags) return;
+    const int64_t lo = at[g], next = __shfl_sync(0xffffffffu, at[g + 1], 0);
+    int64_t hi = __shfl_down_sync(0xffffffffu, lo, 1);
+    if (lane == 31) hi = next;
+    const bool bad = lo < 0 || hi < lo || hi > nnz;
+    if (__any_sync(0xffffffffu, bad)) {  // skip the whole group; readers bound-check bag indices
+      if (lane == 0) set_status(status, ANTDT_ERR_BAD_OFFSETS);
+      continue;
     }
-    if (o < span) occ_bag[first + o] = (uint32_t)min(b0 + l, n_bags - 1);
+    const int64_t first = __shfl_sync(0xffffffffu, lo, 0);
+    const int span = (int)(next - first);  // < 2^31: offsets lie in [0, nnz]
+    const int my_end = (int)(hi - first);  // ascending over the lanes
+    // the group's range starts this far into an aligned group of four
+    const int skew = (int)(((reinterpret_cast<uintptr_t>(occ_bag) >> 2) + (uint64_t)first) & 3);
+    for (int base = -skew; base < span; base += 128) {
+      const int o = base + 4 * lane;
+      int l = 0;  // first lane whose end is > max(o, 0)
+#pragma unroll
+      for (int step = 16; step > 0; step >>= 1) {
+        const int e = __shfl_sync(0xffffffffu, my_end, l + step - 1);
+        if (e <= max(o, 0)) l += step;
+      }
+      uint32_t q[4];
+      int end = __shfl_sync(0xffffffffu, my_end, l & 31);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        // on to the bag that holds o + j (empty bags are stepped over; the vote keeps the lanes together)
+        while (__any_sync(0xffffffffu, o + j >= end && l < 31)) {
+          if (o + j >= end && l < 31) ++l;
+          end = __shfl_sync(0xffffffffu, my_end, l & 31);
+        }
+        q[j] = (uint32_t)min(b0 + l, n_bags - 1);
+      }
+      if (o >= 0 && o + 4 <= span) {
+        *reinterpret_cast<uint4*>(occ_bag + first + o) = make_uint4(q[0], q[1], q[2], q[3]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (o + j >= 0 && o + j < span) occ_bag[first + o + j] = q[j];
+      }
+    }
   }
 }
 
@@ -210,7 +242,8 @@ int32_t bwd_dedup_impl(
     // payload ping-pong ends in sorted_occ: start in whichever buffer makes the last pass land there
     uint32_t* expand_to = (P % 2 == 1) ? vals_t : occ_out;
     if (n_bags > 0 && nnz > 0) {
-      const unsigned grid = (unsigned)((n_bags + 32 * 8 - 1) / (32 * 8));
+      const int64_t per_cta = 32 * 8 * kExpandGroups;
+      const unsigned grid = (unsigned)((n_bags + per_cta - 1) / per_cta);
       ANTDT_LAUNCH("expand_bags", expand_bags_kernel, grid, 256, 0, s, bag_offsets, n_bags, nnz,
                    expand_to, dev_status, (uint32_t*)(w8 + L.head_bits), (int64_t)head_bits_words(nnz),
                    (int32_t*)(w8 + L.tasks));
