@@ -191,12 +191,14 @@ struct FusedUpdate {
 // after it without the prefetch 2.42, loaded before it 2.58); 32 waves 2.58;
 // 8 waves 2.62; 4 waves 2.74; 2 waves 2.88; 1 wave 2.95; one row per lane group and no stride
 // 3.30; 6 CTAs/SM 3.05; 2 rows in flight 3.5-4.1; 4 rows 5.0.  Adam (fp32 rows, 16 and 32
-// workers): 2.91 / 1.96 ms against 3.22 / 2.20 for the two kernels; at 6 CTAs/SM 3.26 / 2.30.
+// workers): 2.91 / 1.96 ms against 3.22 / 2.20 for the two kernels; at 6 CTAs/SM 3.26 / 2.30; the
+// grid of 64 waves instead of 16: 2655 -> 2588 and 1769 -> 1746 us (32 waves 2611 / 1745, 8 waves
+// 2732 / 1818), where Adagrad on the bf16 table goes 1619 -> 1653.
 __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 constexpr int kFusedRows = 1;
-constexpr int kFusedWaves = 16;
+constexpr int kFusedWaves = 16, kFusedWavesAdam = 64;
 constexpr int kFusedCtas = 8;
 template <int G, int VPL, bool ADAM, bool BF16>
 __global__ void __launch_bounds__(256, (VPL == 1 ? kFusedCtas : 1))
@@ -321,7 +323,7 @@ void launch_agg_update(const FusedUpdate& fu, const uint32_t* row_start, const u
   const int64_t want = (out_cap + gpb - 1) / gpb;
   const size_t smem = 4 * (size_t)K;
   const bool adam = fu.opt == ANTDT_OPT_ADAM, bf16 = fu.dtype == ANTDT_BF16;
-  const int64_t cap = (int64_t)kNumSM * kFusedCtas * kFusedWaves;
+  const int64_t cap = (int64_t)kNumSM * kFusedCtas * (adam ? kFusedWavesAdam : kFusedWaves);
   const unsigned grid = (unsigned)(want > cap ? cap : (want < 1 ? 1 : want));
 #define FU_GO(A, B)                                                                              \
   ANTDT_LAUNCH("agg_update", (agg_update_kernel<G, VPL, A, B>), grid, 256, smem, s, row_start, src, \
