@@ -66,12 +66,17 @@ struct StepStreams {
 StepStreams g_ss[64];
 std::mutex g_ss_mu;
 
-StepStreams* step_streams() {
+StepStreams* step_streams(cudaStream_t s) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
   std::lock_guard<std::mutex> lk(g_ss_mu);
   StepStreams& ss = g_ss[dev];
   if (!ss.ready) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;  // nothing is created during a capture
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      return nullptr;
+    }
     if (cudaStreamCreateWithFlags(&ss.in, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
     if (cudaStreamCreateWithFlags(&ss.out, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
     if (cudaStreamCreateWithFlags(&ss.side_fwd, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
@@ -119,7 +124,7 @@ extern "C" int32_t antdt_bsp_step_host(const antdt_step_desc* d, void* stream) {
     return ANTDT_ERR_INVALID_ARG;
   const bool dense = d->h_dense_grads && d->dense_n > 0;
   if (dense && (!d->d_dense_grads || !d->d_dense_out || !d->h_dense_out)) return ANTDT_ERR_INVALID_ARG;
-  StepStreams* ss = step_streams();
+  StepStreams* ss = step_streams(s);
   if (!ss) return ANTDT_ERR_CUDA;
   std::lock_guard<std::mutex> lk(ss->mu);
 
@@ -252,7 +257,7 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
   // the forward runs beside it, started once the sort's CTAs are in place (before them it would take
   // the SMs that they wait for).
   const bool beside = antdt::resident_sort_fits(d->n_workers, d->nnz, d->n_rows);
-  if (beside || (forked && ws_skip > 0)) ss = step_streams();
+  if (beside || (forked && ws_skip > 0)) ss = step_streams(s);
   if (!ss && !merged) ws_skip = 0;
   std::unique_lock<std::mutex> lk;
   if (ss) lk = std::unique_lock<std::mutex>(ss->mu);
@@ -269,10 +274,17 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
                                  ss ? ss->ids_done : nullptr, merged ? &merge : nullptr,
                                  ss && beside ? ss->sort_started : nullptr);
   };
+  antdt_dense_part dp;
+  dp.grads = d->d_dense_grads; dp.n = d->dense_n; dp.stride = d->dense_n; dp.out = d->d_dense_out;
   int32_t rc;
   if (!ss) {
     rc = forward(stream);
-    if (rc == ANTDT_OK) rc = backward();
+    if (rc != ANTDT_OK) return rc;
+  }
+  // the dense sum runs under the sort
+  antdt::DenseBeside beside_sort(dense ? &dp : nullptr, d->batch_sizes, nullptr, d->n_workers, d->d_status, s);
+  if (!ss) {
+    rc = backward();
     if (rc != ANTDT_OK) return rc;
   } else {
     cudaEvent_t after = beside ? ss->sort_started : ss->ids_done;
@@ -293,12 +305,10 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
     if (rc != ANTDT_OK) return rc;
   }
   antdt_sparse_part sp = antdt::sparse_part_of(d);
-  antdt_dense_part dp;
-  dp.grads = d->d_dense_grads; dp.n = d->dense_n; dp.stride = d->dense_n; dp.out = d->d_dense_out;
   antdt::OrderFork fork;
   const bool order_fork = ss && forked && ws_skip > 0 && !merged;
   if (order_fork) fork = antdt::OrderFork{ss->side_order, ss->ids_done, ss->order_done};
-  return antdt::server_step(d, &sp, dense ? &dp : nullptr, stream, order_fork ? &fork : nullptr, ws_skip,
+  return antdt::server_step(d, &sp, dense && !beside_sort.issued() ? &dp : nullptr, stream, order_fork ? &fork : nullptr, ws_skip,
                             merged);
 #undef CK
 }
@@ -401,6 +411,8 @@ extern "C" int32_t antdt_bsp_step_graph(const antdt_step_desc* d, void* stream) 
   // miss: capture the four calls
   antdt::segsort_prepare_device();
   antdt::resident_sort_prepare_device();
+  antdt::aggregate_prepare_device(s);
+  step_streams(s);
   antdt::range_prepare_device();
   if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     cudaGetLastError();  // e.g. the legacy default stream cannot be captured: plain launches
