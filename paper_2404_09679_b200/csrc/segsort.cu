@@ -4,7 +4,7 @@
 // Work decomposition: every segment is cut into chunks of chunk_elems consecutive elements
 // (about kSortChunksTarget chunks in all, one CTA each, so a pass is a single wave on 148 SMs
 // at 4 CTAs per SM).  One pass = histogram per chunk -> exclusive scan over (bin, chunk) inside
-// each segment -> scatter.  The scatter ranks a 4096-pair tile with warp match/ballot
+// each segment -> scatter.  The scatter ranks a 4096-pair tile with warp votes or match
 // (stable: tile order is warp-striped), reorders the tile in shared memory by bin and writes
 // each bin's run with consecutive threads, so global stores are as coalesced as the digit
 // distribution allows.
@@ -283,6 +283,27 @@ constexpr int kScatItems = kSortTile / kScatThreads;  // 8
 constexpr int kScatWarps = kScatThreads / 32;         // 16
 constexpr size_t kScatSmem = 3 * kSortMaxBins * 4 + kScatWarps * kSortMaxBins * 2 + 2 * kSortTile * 4 + 64;
 
+// Lanes of the warp whose digit (BITS wide) equals this lane's: one vote per bit.
+template <int BITS>
+__device__ __forceinline__ unsigned digit_peers(uint32_t d) {
+  unsigned m = 0xffffffffu;
+#pragma unroll
+  for (int b = 0; b < BITS; ++b) {
+    const unsigned one = (d >> b) & 1u;
+    m &= __ballot_sync(0xffffffffu, one != 0u) ^ (one - 1u);
+  }
+  return m;
+}
+
+// How the lanes of equal digit find each other.  match.any takes time in proportion to the distinct
+// values it finds, on a unit that the whole SM shares (62 cycles for 32 spread digits, 6 for 4): it
+// was busy nine cycles in ten of a first pass over 8-bit digits.  Votes take 20 to 23 whatever the
+// digits.  So the last pass, where the repeats of a hot row stand together, goes by match (VOTES = 0),
+// the others by votes: first pass 651 -> 582 us (65 M pairs, 24-bit ids), 940 -> 889 (105 M, 25 bits),
+// 390 -> 370 (35 M, 26 bits), second 590 -> 570, 783 -> 829, 474 -> 458; votes in the last pass
+// 428 -> 517, 670 -> 823, 322 -> 335.  A choice per warp by the distinct digits of the tile before
+// spilled and lost what it gained.
+template <int VOTES>
 __global__ void __launch_bounds__(kScatThreads, kSortCtasPerSM)
 radix_scatter_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in,
                      uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out, int shift,
@@ -366,25 +387,39 @@ radix_scatter_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __res
     }
     __syncthreads();  // (A) also: the previous tile's write-out is over
 
-    // peer masks of all items first (independent, their latencies overlap), counters after
-    unsigned pm[kScatItems];
+    if (VOTES > 0) {
 #pragma unroll
-    for (int i = 0; i < kScatItems; ++i) {
-      const bool valid = wbase + i * 32 < tile_n;
-      const uint32_t d = valid ? ((k[i] >> shift) & mask) : (uint32_t)kSortMaxBins;
-      pm[i] = __match_any_sync(0xffffffffu, d);
-    }
+      for (int i = 0; i < kScatItems; ++i) {
+        const bool valid = wbase + i * 32 < tile_n;
+        const uint32_t d = (k[i] >> shift) & mask;
+        const unsigned m = digit_peers<(VOTES > 0 ? VOTES : 1)>(d) & __ballot_sync(0xffffffffu, valid);
+        // every peer reads the counter (one broadcast), the first peer then bumps it
+        const uint32_t old = valid ? my_wh[d] : 0u;
+        __syncwarp();
+        if (valid && (m & lt) == 0) my_wh[d] = (unsigned short)(old + __popc(m));
+        __syncwarp();
+        rank[i] = (unsigned short)(old + __popc(m & lt));
+      }
+    } else {
+      // peer masks of all items first (independent, their latencies overlap), counters after
+      unsigned pm[kScatItems];
 #pragma unroll
-    for (int i = 0; i < kScatItems; ++i) {
-      const bool valid = wbase + i * 32 < tile_n;
-      const uint32_t d = (k[i] >> shift) & mask;
-      const unsigned m = pm[i];
-      // every peer reads the counter (one broadcast), the first peer then bumps it
-      const uint32_t old = valid ? my_wh[d] : 0u;
-      __syncwarp();
-      if (valid && (m & lt) == 0) my_wh[d] = (unsigned short)(old + __popc(m));
-      __syncwarp();
-      rank[i] = (unsigned short)(old + __popc(m & lt));
+      for (int i = 0; i < kScatItems; ++i) {
+        const bool valid = wbase + i * 32 < tile_n;
+        const uint32_t d = valid ? ((k[i] >> shift) & mask) : (uint32_t)kSortMaxBins;
+        pm[i] = __match_any_sync(0xffffffffu, d);
+      }
+#pragma unroll
+      for (int i = 0; i < kScatItems; ++i) {
+        const bool valid = wbase + i * 32 < tile_n;
+        const uint32_t d = (k[i] >> shift) & mask;
+        const unsigned m = pm[i];
+          const uint32_t old = valid ? my_wh[d] : 0u;
+        __syncwarp();
+        if (valid && (m & lt) == 0) my_wh[d] = (unsigned short)(old + __popc(m));
+        __syncwarp();
+        rank[i] = (unsigned short)(old + __popc(m & lt));
+      }
     }
     __syncthreads();  // (B)
 
@@ -684,10 +719,13 @@ void segsort_prepare_device() {
   cudaGetDevice(&dev_id);
   bool& done = attr_set[dev_id & 63];
   if (done) return;
-  cudaFuncSetAttribute(radix_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)kScatSmem);
-  cudaFuncSetAttribute(radix_scatter_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                       cudaSharedmemCarveoutMaxShared);
+  auto opt_in = [](auto* k) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatSmem);
+    cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  };
+  opt_in(radix_scatter_kernel<0>);
+  opt_in(radix_scatter_kernel<8>);
+  opt_in(radix_scatter_kernel<9>);
   done = true;
 }
 
@@ -732,9 +770,14 @@ void segsort_run(const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* key
     if (!fold_scan)
       ANTDT_LAUNCH(agg ? "agg_radix_scan" : "radix_scan", radix_scan_kernel, dim3(S, kScanBinGroups),
                    kScanThreads, 0, s, desc, seg_first, hist, bin_total);
-    ANTDT_LAUNCH(agg ? "agg_radix_scatter" : "radix_scatter", radix_scatter_kernel, L.max_chunks, kScatThreads, kScatSmem, s, kin, vin,
-                 kout, vout, shift, mask, desc, chunk_seg, seg_bounds, chunk_begin, chunk_end, hist,
-                 bin_total, fold_scan ? seg_first : (const int32_t*)nullptr);
+#define SCATTER_GO(VOTES)                                                                                       \
+  ANTDT_LAUNCH(agg ? "agg_radix_scatter" : "radix_scatter", radix_scatter_kernel<VOTES>, L.max_chunks, kScatThreads, \
+               kScatSmem, s, kin, vin, kout, vout, shift, mask, desc, chunk_seg, seg_bounds, chunk_begin, chunk_end, \
+               hist, bin_total, fold_scan ? seg_first : (const int32_t*)nullptr)
+    if (p + 1 == P) SCATTER_GO(0);
+    else if (bits <= 8) SCATTER_GO(8);
+    else SCATTER_GO(9);
+#undef SCATTER_GO
     kin = kout;
     vin = vout;
     shift += bits;
