@@ -6,7 +6,7 @@
 // rows; there is no contraction here and so no tensor-core work.  Three kernels:
 //   embbag_fwd_flat_kernel    rows of up to 512 bytes, one bag per group: every lane reads the ids
 //                             itself, four rows in flight, 32 registers -> 64 warps per SM
-//   embbag_fwd_stride_kernel  the same for short bags: capped grid, groups stride over the bags
+//   embbag_fwd_stride_kernel  the same for many bags: capped grid, groups stride over the bags
 //                             and read the next bag's offsets ahead
 //   embbag_fwd_kernel         wider rows (VPL vectors per lane): ids staged through the group's
 //                             registers G at a time (one coalesced load, then shuffles)
@@ -123,7 +123,23 @@ embbag_fwd_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
 constexpr int kFlatThreads = 256;
 constexpr int kFlatUnroll = 4;
 constexpr int kFlatCtas = 8;     // CTAs per SM
-constexpr int kFlatWaves = 32;   // grid cap of the striding form, in resident waves
+
+// Whether bags of avg ids are strided over (embbag_fwd_stride_kernel) and by how many resident waves of
+// CTAs; 0: one bag per lane group.  W: waves that one bag per lane group would make.
+// Reading the next bag's offsets ahead pays once a lane group has several turns, and the more of a
+// bag's time its offsets are: for rows of 16 vectors and more always, for 8 vectors below 8 ids, for
+// less below 3.  Measured, one bag per group -> striding: 128 floats x 10 ids, W 39 / 157: 206 -> 196,
+// 778 -> 701 us; 64 x 10, W 79: 440 -> 411; 64 x 4.5, W 20 / 327: 79 -> 70, 1175 -> 958; 32 x 1, W 39:
+// 105 -> 89; against it 32 x 10, W 39: 265 -> 284, 16 x 4.5, W 20: 104 -> 112, 32 x 1, W 2.5: the same.
+// About ten turns per group are best: fewer waves unbalance the SMs (W 327 in 1 / 4 / 16 waves: 1127 /
+// 1039 / 958 us), more waste the reading ahead (W 39 in 4 / 16 / 32 waves: 119 / 128 / 140).
+inline int stride_waves(int G, int64_t n_bags, int64_t nnz) {
+  const int64_t per_wave = (int64_t)kNumSM * kFlatCtas * (kFlatThreads / G);
+  const int64_t W = n_bags / per_wave;
+  if (W < 8 || (G < 16 && nnz >= (G == 8 ? 8 : 3) * n_bags)) return 0;
+  const int64_t waves = (W + 5) / 10;
+  return waves < 1 ? 1 : (waves > 16 ? 16 : (int)waves);
+}
 
 // One bag: this lane's 16 bytes of the sum of the rows that ids[0..len) name, as packed fp32 pairs.
 // (The output address is formed by the caller after the loop: at 32 registers every 64-bit value
@@ -211,8 +227,7 @@ embbag_fwd_flat_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
   if (lg < nvec) flat_store<BF16>(pooled + bag * (int64_t)dim + (size_t)lg * EPV, acc);
 }
 
-// Short bags (a few ids each): the chain offsets -> ids -> rows is most of a bag's time, so the
-// grid is capped, every lane group strides over its bags (bag order), and the NEXT bag's offsets
+// Where the chain offsets -> ids -> rows is much of a bag's time (stride_waves): the grid is capped, every lane group strides over its bags (bag order), and the NEXT bag's offsets
 // are read before the current bag's rows are requested (30 fields x 4.5 ids x 128-byte rows:
 // 1.06 -> 0.84 ms).  The loop is written out in one piece on purpose: at 32 registers the form of
 // the source decides what the compiler keeps in flight, and two tidier versions of this same loop
@@ -298,7 +313,7 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
 template <int G, int VPL, bool BF16>
 void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_ids, int64_t nnz,
                 const int64_t* bag_offsets, int64_t n_bags, float* pooled, int32_t* status,
-                cudaStream_t s, int fields, bool short_bags) {
+                cudaStream_t s, int fields) {
   constexpr bool flat = VPL == 1;  // rows of up to 512 bytes
   const int64_t gpb = (flat ? kFlatThreads : kFwdThreads) / G;
   int64_t grid = (n_bags + gpb - 1) / gpb, sample_blocks = 0;
@@ -308,10 +323,9 @@ void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_i
   } else {
     fields = 0;
   }
-  if (flat && short_bags) {
-    const int64_t cap = (int64_t)kNumSM * kFlatCtas * kFlatWaves;
-    grid = (n_bags + gpb - 1) / gpb;
-    ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_stride_kernel<G, BF16>), (unsigned)(grid < cap ? grid : cap),
+  const int waves = flat && fields == 0 ? stride_waves(G, n_bags, nnz) : 0;
+  if (waves > 0) {
+    ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_stride_kernel<G, BF16>), (unsigned)(kNumSM * kFlatCtas * waves),
                  kFlatThreads, 0, s, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status);
   } else if (flat && fields > 0) {
     ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_flat_kernel<G, BF16, true>), (unsigned)grid, kFlatThreads, 0, s,
@@ -331,10 +345,10 @@ void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_i
 template <bool BF16>
 int32_t dispatch_fwd(int nvec, const void* table, int64_t n_rows, int dim, const int32_t* row_ids,
                      int64_t nnz, const int64_t* bag_offsets, int64_t n_bags, float* pooled,
-                     int32_t* status, cudaStream_t s, int fields, bool short_bags) {
+                     int32_t* status, cudaStream_t s, int fields) {
 #define FWD_CASE(G, VPL)                                                                      \
   launch_fwd<G, VPL, BF16>(table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled,     \
-                           status, s, fields, short_bags);                                    \
+                           status, s, fields);                                                \
   return ANTDT_OK;
   if (nvec <= 1) { FWD_CASE(1, 1) }
   if (nvec <= 2) { FWD_CASE(2, 1) }
@@ -369,15 +383,14 @@ int32_t fwd_impl(const void* table, int32_t dtype, int64_t n_rows, int32_t dim, 
   // Field-major order pays when a bag's id list fills a 32-byte sector (eight ids or more on
   // average): measured -12% on 100 fields x 10 ids x 256-byte rows, -2% on 40 x 20 x 128-byte rows,
   // but +8% on 30 fields x 4.5 ids, where the scattered id reads cost more than the rows gain.
-  const bool short_bags = nnz < 8 * n_bags;
-  const int fields = (bags_per_sample > 1 && !short_bags) ? bags_per_sample : 0;
+  const int fields = (bags_per_sample > 1 && nnz >= 8 * n_bags) ? bags_per_sample : 0;
   int32_t rc;
   if (dtype == ANTDT_BF16)
     rc = dispatch_fwd<true>(dim / 8, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled,
-                            dev_status, s, fields, short_bags);
+                            dev_status, s, fields);
   else
     rc = dispatch_fwd<false>(dim / 4, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags,
-                             pooled, dev_status, s, fields, short_bags);
+                             pooled, dev_status, s, fields);
   if (rc != ANTDT_OK) return rc;
   return cuda_ok();
 }
