@@ -31,6 +31,7 @@ range_split_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ 
                    int64_t* __restrict__ wuo_out, int64_t* __restrict__ n_entries,
                    int32_t* __restrict__ bnd, const WeightBlob weights, float* __restrict__ weights_out,
                    int32_t* status) {
+  pdl_sync();
   __shared__ int64_t s_wuo[kRangeMaxWorkers + 1];
   if (blockIdx.x == 0 && weights_out && threadIdx.x < K) weights_out[threadIdx.x] = weights.w[threadIdx.x];
   if (threadIdx.x == 0) {  // ascending and inside [0, in_cap], whatever came in
@@ -173,6 +174,7 @@ __global__ void __launch_bounds__(kRaThreads)
 range_count_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ bnd,
                    const int64_t* __restrict__ wuo, int K, int64_t P, int r_log2, int64_t n_rows,
                    uint32_t dropped, int32_t* __restrict__ distinct, int32_t* status) {
+  pdl_sync();
   __shared__ uint32_t pres[(1 << kRangeMaxLog2) / 32];
   __shared__ int64_t s_before;
   __shared__ int32_t s_beg[32], s_off[33], s_tmp[2 * kRaWarps];
@@ -198,6 +200,7 @@ range_count_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ 
 __global__ void __launch_bounds__(1024)
 range_scan_kernel(const int32_t* __restrict__ distinct, int64_t P, int64_t* __restrict__ base,
                   int64_t* __restrict__ n_agg, int64_t out_cap, int32_t* status) {
+  pdl_sync();
   __shared__ int64_t warp_tot[32];
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   const int64_t per = (P + 1023) / 1024;
@@ -266,6 +269,7 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
                   int64_t out_cap, uint32_t* __restrict__ src, uint32_t* head_bits,
                   int32_t* __restrict__ tile_first, int tile_shift, uint32_t* __restrict__ row_start,
                   uint8_t* __restrict__ src_worker, int32_t* status) {
+  pdl_sync();
   extern __shared__ __align__(16) unsigned char ra_smem[];
   const int R = 1 << r_log2;
   const int nW = R / 32;  // presence words: at most 256 = one per thread

@@ -70,6 +70,7 @@ AggLayout agg_layout(int64_t in_cap, int K, int dim) {
 __global__ void agg_prep_kernel(const int64_t* __restrict__ wuo_in, int K, int64_t in_cap,
                                 int64_t* __restrict__ bounds, int64_t* __restrict__ wuo,
                                 int32_t* status) {
+  pdl_sync();
   const int tid = threadIdx.x;
   for (int i = tid; i <= K; i += blockDim.x) {
     int64_t v = wuo_in[i];
@@ -96,6 +97,7 @@ __global__ void agg_prep_backup_kernel(const int64_t* __restrict__ wuo_in, const
                                        int K, int64_t in_cap, int64_t* __restrict__ bounds,
                                        int64_t* __restrict__ wuo, int64_t* __restrict__ cwuo,
                                        int32_t* status) {
+  pdl_sync();
   if (threadIdx.x != 0) return;
   int64_t prev = 0, acc = 0;
   for (int i = 0; i <= K; ++i) {  // K <= 1024: a serial pass is enough
@@ -119,6 +121,7 @@ __global__ void __launch_bounds__(256)
 agg_compact_kernel(const int32_t* __restrict__ uniq_ids, const int64_t* __restrict__ wuo,
                    const int64_t* __restrict__ cwuo, const uint32_t* __restrict__ drop, int K,
                    uint32_t* __restrict__ keys_c, uint32_t* __restrict__ vals_c) {
+  pdl_sync();
   extern __shared__ int64_t s_cw[];  // wuo [K+1], cwuo [K+1], then K drop flags
   int64_t* s_wuo = s_cw;
   int64_t* s_cwuo = s_cw + (K + 1);
@@ -146,6 +149,7 @@ __global__ void __launch_bounds__(256, 4)
 dense_wsum_kernel(const float* __restrict__ grads, int64_t n4, int64_t stride,
                   const float* __restrict__ weights, const __grid_constant__ DenseWeights blob, int K,
                   float* __restrict__ out) {
+  pdl_sync();
   extern __shared__ float s_wd[];
   for (int i = threadIdx.x; i < K; i += blockDim.x) s_wd[i] = weights ? weights[i] : blob.w[i];
   __syncthreads();
@@ -205,6 +209,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 __global__ void __launch_bounds__(kBulkThreads, 16)
 dense_wsum_bulk_kernel(const float* __restrict__ grads, uint32_t n, int64_t stride,
                        const __grid_constant__ DenseWeights blob, int K, float* __restrict__ out, int32_t* status) {
+  pdl_sync();
   extern __shared__ __align__(128) float s_ring[];  // [slots][group][elems]
   __shared__ __align__(8) uint64_t s_full[kBulkSlots], s_empty[kBulkSlots];
   __shared__ float s_wt[kDenseBlobWorkers];
@@ -314,6 +319,7 @@ agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __rest
                   const uint8_t* __restrict__ src_worker, const float* __restrict__ weights, int K,
                   void* table, int64_t n_rows, int dim, OptParams p, float* state0, float* state1,
                   float* __restrict__ agg_out) {
+  pdl_sync();
   extern __shared__ float s_w[];  // the K weights
   for (int i = threadIdx.x; i < K; i += blockDim.x) s_w[i] = weights[i];
   __syncthreads();
@@ -586,6 +592,7 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
   if (!by_ranges && !resident) upload_small(hw, 4 * (size_t)K, w8 + L.weights, s);
   // the dense part runs beside the sparse one where there is enough of it
   DenseBeside beside(sp && in_cap > 0 ? dp : nullptr, batch_sizes, dropped, K, dev_status, s);
+  PdlScope pdl(!beside.issued() && in_cap <= kPdlMaxItems);
 
   if (sp) {
     int64_t* bounds = (int64_t*)(w8 + L.bounds);

@@ -83,6 +83,7 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
                 const uint32_t* __restrict__ head_bits, const int32_t* __restrict__ tile_first,
                 const float* __restrict__ rows, float* __restrict__ out, const WalkScratch ws,
                 const int payload_vec) {
+  pdl_sync();
   constexpr int TPS = kRedThreads / G;  // tiles per stretch
   constexpr int CH = WalkChunk<VPL>::value;
   constexpr unsigned kFull = 0xffffffffu;
@@ -304,6 +305,7 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
 template <int G, int VPL, int TILE>
 __global__ void __launch_bounds__(kRedThreads)
 bwd_fixup_kernel(const TileArgs a, const WalkScratch ws) {
+  pdl_sync();
   constexpr int TPS = kRedThreads / G;
   constexpr int64_t SPAN = (int64_t)TPS * TILE;  // entries of a stretch
   const int n_tasks = ws.tasks[0];

@@ -20,12 +20,53 @@ void prof_untimed(bool on);
 // Adds n to the launch counter: kernels that ran as nodes of a replayed graph.
 void count_launches(int64_t n);
 
+// Programmatic dependent launch: a kernel's CTAs may be scheduled once every CTA of the kernel before
+// it on the stream has begun, so its launch is over by the time that kernel ends (3.1 -> 2.1 us a
+// kernel in a chain of short ones, 1.2 -> 1.1 in a graph).  Every kernel therefore begins with a
+// wait for the kernel before it to be complete and its writes visible, and does nothing before.
+// pdl_sync also lets the next kernel be scheduled; a kernel that must keep room on its SMs for
+// another stream only waits.  Off (PdlScope) for large inputs, where a microsecond a kernel is nothing
+// and CTAs that wait take room, and while the dense part runs on its side stream.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_sync() {
+  pdl_wait();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+inline thread_local bool t_pdl = false;  // this thread's launches carry the attribute
+class PdlScope {
+ public:
+  explicit PdlScope(bool on) : was_(t_pdl) { t_pdl = on; }
+  ~PdlScope() { t_pdl = was_; }
+
+ private:
+  bool was_;
+};
+constexpr int64_t kPdlMaxItems = (int64_t)1 << 24;  // occurrences, bags or rows of a call
+inline cudaLaunchAttribute pdl_attribute() {
+  cudaLaunchAttribute a;
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
+}
+template <typename... P, typename... A>
+void launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at = pdl_attribute();
+  cfg.attrs = &at;
+  cfg.numAttrs = t_pdl ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Launch `kernel` and account for it (launch counter; CUDA-event bracket when profiling is on).
-#define ANTDT_LAUNCH(name, kernel, grid, block, smem, stream, ...)        \
-  do {                                                                    \
-    int _tok = antdt::prof_begin(name, stream);                           \
-    kernel<<<(grid), (block), (smem), (stream)>>>(__VA_ARGS__);           \
-    antdt::prof_end(_tok, stream);                                        \
+#define ANTDT_LAUNCH(name, kernel, grid, block, smem, stream, ...)                   \
+  do {                                                                               \
+    int _tok = antdt::prof_begin(name, stream);                                      \
+    antdt::launch_kernel(kernel, dim3(grid), dim3(block), (smem), (stream), __VA_ARGS__); \
+    antdt::prof_end(_tok, stream);                                                   \
   } while (0)
 
 static inline int32_t cuda_ok() {
@@ -58,7 +99,7 @@ int32_t bwd_dedup_impl(const int32_t* row_ids, int64_t nnz, const int64_t* bag_o
                        size_t ws_bytes, int32_t* dev_status, void* stream,
                        const PooledArrival* arrival,
                        cudaEvent_t ids_done = nullptr, const StepMerge* merge = nullptr,
-                       cudaEvent_t sort_started = nullptr);
+                       cudaEvent_t sort_started = nullptr, bool pdl_allowed = true);
 // embbag_bwd.cu; ids_done: recorded once the distinct ids and their offsets are written; merge: the
 // sort also makes the aggregation's merge order (step_merge_targets said that it can); sort_started:
 // recorded when the CTAs of the resident sort have begun
@@ -105,7 +146,8 @@ class DenseBeside {
 
 int32_t fwd_impl(const void* table, int32_t dtype, int64_t n_rows, int32_t dim, const int32_t* row_ids,
                  int64_t nnz, const int64_t* bag_offsets, int64_t n_bags, float* pooled,
-                 int32_t* dev_status, void* stream, int32_t bags_per_sample);  // embbag_fwd.cu
+                 int32_t* dev_status, void* stream, int32_t bags_per_sample,
+                 bool beside = false);  // embbag_fwd.cu; beside: runs beside the kernel that the stream depends on
 
 constexpr int kNumSM = 148;  // B200: 2 dies x 74 SMs; grids are sized in multiples of this
 

@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(1024)
 bwd_prep_kernel(const int64_t* __restrict__ wso, int K, int F, const int64_t* __restrict__ bag_offsets,
                 int64_t n_bags, int64_t nnz, int64_t* __restrict__ occ_bounds,
                 float* __restrict__ worker_b, int32_t* status) {
+  pdl_sync();
   const int tid = threadIdx.x;
   if (tid == 0 && (bag_offsets[0] != 0 || bag_offsets[n_bags] != nnz))
     set_status(status, ANTDT_ERR_BAD_OFFSETS);
@@ -82,6 +83,7 @@ __global__ void __launch_bounds__(256)
 expand_bags_kernel(const int64_t* __restrict__ bag_offsets, int64_t n_bags, int64_t nnz,
                    uint32_t* __restrict__ occ_bag, int32_t* status, uint32_t* __restrict__ zero_words,
                    int64_t n_zero_words, int32_t* __restrict__ zero_pair) {
+  pdl_sync();
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int64_t first_bag = warp * (32 * kExpandGroups);
@@ -169,7 +171,7 @@ int32_t bwd_dedup_impl(
     const int64_t* worker_sample_offsets, int32_t* uniq_ids, int64_t* worker_uniq_offsets,
     int64_t* seg_offsets, int32_t* sorted_occ, float* uniq_grads, int64_t out_cap, void* ws,
     size_t ws_bytes, int32_t* dev_status, void* stream, const PooledArrival* arrival,
-    cudaEvent_t ids_done, const StepMerge* merge, cudaEvent_t sort_started) {
+    cudaEvent_t ids_done, const StepMerge* merge, cudaEvent_t sort_started, bool pdl_allowed) {
   const int K = n_workers;
   if (nnz < 0 || n_bags < 0 || nnz >= (1ll << 31) || n_bags >= (1ll << 31) || n_rows < 1 ||
       n_rows >= (1ll << 31) || dim < 4 || dim > 1024 || dim % 4 || K < 1 || K > kMaxSegments ||
@@ -196,6 +198,7 @@ int32_t bwd_dedup_impl(
   if (ws_bytes < L.bytes) return ANTDT_ERR_WORKSPACE_TOO_SMALL;
 
   cudaStream_t s = (cudaStream_t)stream;
+  PdlScope pdl(pdl_allowed && nnz <= kPdlMaxItems);
   char* w8 = static_cast<char*>(ws);
   int64_t* d_wso = (int64_t*)(w8 + L.wso);
   int64_t* d_occ_bounds = (int64_t*)(w8 + L.occ_bounds);

@@ -23,7 +23,8 @@ __global__ void __launch_bounds__(kFwdThreads, (VPL == 1 ? 12 : 1))
 embbag_fwd_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
                   const int32_t* __restrict__ row_ids, int64_t nnz,
                   const int64_t* __restrict__ bag_offsets, int64_t n_bags,
-                  float* __restrict__ pooled, int32_t* status, int fields, int64_t sample_blocks) {
+                  float* __restrict__ pooled, int32_t* status, int fields, int64_t sample_blocks, bool chained) {
+  if (chained) pdl_sync();  // (beside a kernel that it depends on the start of, it must not wait for its end)
   constexpr int EPV = BF16 ? 8 : 4;   // elements per 16-byte vector
   constexpr int PAIRS = EPV / 2;      // packed fp32 pairs per vector
   constexpr int U = (G < kFwdUnroll) ? G : kFwdUnroll;
@@ -205,7 +206,8 @@ __global__ void __launch_bounds__(kFlatThreads, kFlatCtas)
 embbag_fwd_flat_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
                        const int32_t* __restrict__ row_ids, int64_t nnz,
                        const int64_t* __restrict__ bag_offsets, int64_t n_bags,
-                       float* __restrict__ pooled, int32_t* status, int fields, int64_t sample_blocks) {
+                       float* __restrict__ pooled, int32_t* status, int fields, int64_t sample_blocks, bool chained) {
+  if (chained) pdl_sync();  // (beside a kernel that it depends on the start of, it must not wait for its end)
   constexpr int EPV = BF16 ? 8 : 4;
   const int lg = threadIdx.x & (G - 1);
   int64_t bag;
@@ -237,7 +239,8 @@ __global__ void __launch_bounds__(kFlatThreads, kFlatCtas)
 embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
                          const int32_t* __restrict__ row_ids, int64_t nnz,
                          const int64_t* __restrict__ bag_offsets, int64_t n_bags,
-                         float* __restrict__ pooled, int32_t* status) {
+                         float* __restrict__ pooled, int32_t* status, bool chained) {
+  if (chained) pdl_sync();  // (beside a kernel that it depends on the start of, it must not wait for its end)
   constexpr int EPV = BF16 ? 8 : 4;
   constexpr int PAIRS = EPV / 2;
   constexpr int GPB = kFlatThreads / G;  // groups (bags) per CTA and turn
@@ -313,7 +316,7 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
 template <int G, int VPL, bool BF16>
 void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_ids, int64_t nnz,
                 const int64_t* bag_offsets, int64_t n_bags, float* pooled, int32_t* status,
-                cudaStream_t s, int fields) {
+                cudaStream_t s, int fields, bool chained) {
   constexpr bool flat = VPL == 1;  // rows of up to 512 bytes
   const int64_t gpb = (flat ? kFlatThreads : kFwdThreads) / G;
   int64_t grid = (n_bags + gpb - 1) / gpb, sample_blocks = 0;
@@ -326,29 +329,29 @@ void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_i
   const int waves = flat && fields == 0 ? stride_waves(G, n_bags, nnz) : 0;
   if (waves > 0) {
     ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_stride_kernel<G, BF16>), (unsigned)(kNumSM * kFlatCtas * waves),
-                 kFlatThreads, 0, s, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status);
+                 kFlatThreads, 0, s, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, chained);
   } else if (flat && fields > 0) {
     ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_flat_kernel<G, BF16, true>), (unsigned)grid, kFlatThreads, 0, s,
-                 table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, fields, sample_blocks);
+                 table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, fields, sample_blocks, chained);
   } else if (flat) {
     ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_flat_kernel<G, BF16, false>), (unsigned)grid, kFlatThreads, 0, s,
-                 table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, fields, sample_blocks);
+                 table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, fields, sample_blocks, chained);
   } else if (fields > 0) {
     ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_kernel<G, VPL, BF16, true>), (unsigned)grid, kFwdThreads, 0, s,
-                 table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, fields, sample_blocks);
+                 table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, fields, sample_blocks, chained);
   } else {
     ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_kernel<G, VPL, BF16, false>), (unsigned)grid, kFwdThreads, 0, s,
-                 table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, fields, sample_blocks);
+                 table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, fields, sample_blocks, chained);
   }
 }
 
 template <bool BF16>
 int32_t dispatch_fwd(int nvec, const void* table, int64_t n_rows, int dim, const int32_t* row_ids,
                      int64_t nnz, const int64_t* bag_offsets, int64_t n_bags, float* pooled,
-                     int32_t* status, cudaStream_t s, int fields) {
+                     int32_t* status, cudaStream_t s, int fields, bool chained) {
 #define FWD_CASE(G, VPL)                                                                      \
   launch_fwd<G, VPL, BF16>(table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled,     \
-                           status, s, fields);                                                \
+                           status, s, fields, chained);                                       \
   return ANTDT_OK;
   if (nvec <= 1) { FWD_CASE(1, 1) }
   if (nvec <= 2) { FWD_CASE(2, 1) }
@@ -370,7 +373,7 @@ namespace antdt {
 // The entry point's body; bags_per_sample > 0 (the step knows it) selects the field-major order.
 int32_t fwd_impl(const void* table, int32_t dtype, int64_t n_rows, int32_t dim, const int32_t* row_ids,
                  int64_t nnz, const int64_t* bag_offsets, int64_t n_bags, float* pooled,
-                 int32_t* dev_status, void* stream, int32_t bags_per_sample) {
+                 int32_t* dev_status, void* stream, int32_t bags_per_sample, bool beside) {
   if (n_bags < 0 || nnz < 0 || n_rows < 1 || n_rows >= (1ll << 31) || nnz >= (1ll << 31) ||
       n_bags >= (1ll << 31) || dim < 1 || dim > 1024)
     return ANTDT_ERR_INVALID_ARG;
@@ -380,6 +383,7 @@ int32_t fwd_impl(const void* table, int32_t dtype, int64_t n_rows, int32_t dim, 
   if (!table || !bag_offsets || !pooled || (nnz > 0 && !row_ids)) return ANTDT_ERR_INVALID_ARG;
   if (!aligned16(table) || !aligned16(pooled)) return ANTDT_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
+  PdlScope pdl(!beside && nnz <= kPdlMaxItems && n_bags <= kPdlMaxItems);
   // Field-major order pays when a bag's id list fills a 32-byte sector (eight ids or more on
   // average): measured -12% on 100 fields x 10 ids x 256-byte rows, -2% on 40 x 20 x 128-byte rows,
   // but +8% on 30 fields x 4.5 ids, where the scattered id reads cost more than the rows gain.
@@ -387,10 +391,10 @@ int32_t fwd_impl(const void* table, int32_t dtype, int64_t n_rows, int32_t dim, 
   int32_t rc;
   if (dtype == ANTDT_BF16)
     rc = dispatch_fwd<true>(dim / 8, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled,
-                            dev_status, s, fields);
+                            dev_status, s, fields, !beside);
   else
     rc = dispatch_fwd<false>(dim / 4, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags,
-                             pooled, dev_status, s, fields);
+                             pooled, dev_status, s, fields, !beside);
   if (rc != ANTDT_OK) return rc;
   return cuda_ok();
 }

@@ -21,6 +21,7 @@ __global__ void __launch_bounds__(kOptThreads)
 sparse_opt_kernel(void* table, int64_t n_rows, int dim, const int32_t* __restrict__ ids,
                   const float* __restrict__ grads, const int64_t* __restrict__ n_ids_dev,
                   int64_t max_ids, OptParams p, float* state0, float* state1, int32_t* status) {
+  pdl_sync();
   const int lg = threadIdx.x & (G - 1);
   const int nvec = dim / 4;
   const int64_t n = min(*n_ids_dev, max_ids);
@@ -77,6 +78,7 @@ __global__ void __launch_bounds__(kOptThreads)
 rowwise_adagrad_kernel(void* table, int64_t n_rows, int dim, const int32_t* __restrict__ ids,
                        const float* __restrict__ grads, const int64_t* __restrict__ n_ids_dev,
                        int64_t max_ids, OptParams p, float* state0, int32_t* status) {
+  pdl_sync();
   const int lg = threadIdx.x & (G - 1);
   const int nvec = dim / 4;
   const unsigned gmask = group_mask<G>();
@@ -124,6 +126,7 @@ template <bool ADAM>
 __global__ void __launch_bounds__(kOptThreads)
 dense_opt_kernel(float* __restrict__ params, const float* __restrict__ grad, int64_t n4, OptParams p,
                  float* __restrict__ state0, float* __restrict__ state1) {
+  pdl_sync();
   const int64_t stride = (int64_t)gridDim.x * kOptThreads;
   for (int64_t e = (int64_t)blockIdx.x * kOptThreads + threadIdx.x; e < n4; e += stride) {
     const float4 g = ldg_f4(grad + 4 * e);
@@ -200,6 +203,7 @@ extern "C" int32_t antdt_sparse_opt_update(void* table, int32_t dtype, int64_t n
     return ANTDT_ERR_INVALID_ARG;
   const OptParams p = make_opt_params(lr, eps, beta1, beta2, step);
   const bool adam = opt == ANTDT_OPT_ADAM, bf16 = dtype == ANTDT_BF16;
+  PdlScope pdl(max_ids <= kPdlMaxItems);
   cudaStream_t s = (cudaStream_t)stream;
   const int nvec = dim / 4;
   if (opt == ANTDT_OPT_ROWWISE_ADAGRAD) {
@@ -245,6 +249,7 @@ extern "C" int32_t antdt_dense_opt_update(float* params, const float* grad, int6
     return ANTDT_ERR_INVALID_ARG;
   const OptParams p = make_opt_params(lr, eps, beta1, beta2, step);
   const int64_t n4 = n / 4;
+  PdlScope pdl(n4 <= kPdlMaxItems);
   const int64_t want = (n4 + kOptThreads - 1) / kOptThreads;
   const int64_t cap = (int64_t)kNumSM * 16;
   const unsigned grid = (unsigned)(want > cap ? cap : want);

@@ -397,6 +397,7 @@ template <int IPT, bool CLUSTER>
 __global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 2 : 1))
 resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_constant__ StepMerge m,
                      const __grid_constant__ Wso wso) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char res_smem[];
   Smem& S = *reinterpret_cast<Smem*>(res_smem);
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
@@ -633,6 +634,7 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
 template <int IPT, bool CLUSTER>
 __global__ void __launch_bounds__(kThreads, (IPT <= 8 ? 2 : 1))
 resident_merge_kernel(const __grid_constant__ ResidentMergeArgs a) {
+  pdl_sync();
   extern __shared__ __align__(16) unsigned char res_smem[];
   Smem& S = *reinterpret_cast<Smem*>(res_smem);
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
@@ -797,7 +799,7 @@ int32_t launch_one(const char* name, cudaEvent_t started, void (*kernel)(P...), 
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = sizeof(Smem);
   cfg.stream = s;
-  cudaLaunchAttribute at[2];
+  cudaLaunchAttribute at[3];
   if (f.cluster) {
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)f.ctas;
@@ -810,11 +812,12 @@ int32_t launch_one(const char* name, cudaEvent_t started, void (*kernel)(P...), 
   cfg.attrs = at;
   cfg.numAttrs = 1;
   if (started) {
-    at[1].id = cudaLaunchAttributeLaunchCompletionEvent;
-    at[1].val.launchCompletionEvent.event = started;
-    at[1].val.launchCompletionEvent.flags = 0;
-    cfg.numAttrs = 2;
+    cudaLaunchAttribute& e = at[cfg.numAttrs++];
+    e.id = cudaLaunchAttributeLaunchCompletionEvent;
+    e.val.launchCompletionEvent.event = started;
+    e.val.launchCompletionEvent.flags = 0;
   }
+  if (f.cluster && t_pdl) at[cfg.numAttrs++] = pdl_attribute();
   const int tok = prof_begin(name, s);
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
   prof_end(tok, s);

@@ -46,6 +46,7 @@ namespace antdt {
 namespace {
 struct SmallBlob { uint32_t w[512]; };
 __global__ void upload_small_kernel(SmallBlob blob, int n_words, uint32_t* dst) {
+  pdl_sync();
   for (int i = threadIdx.x; i < n_words; i += blockDim.x) dst[i] = blob.w[i];
 }
 }  // namespace
@@ -59,6 +60,7 @@ template <int G>
 __global__ void __launch_bounds__(256)
 probe_gather_kernel(const float4* __restrict__ rows, uint32_t n_rows, const int32_t* __restrict__ idx,
                     int64_t n_out, int per_out, float4* __restrict__ out) {
+  pdl_sync();
   const int lg = threadIdx.x & (G - 1);
   const int64_t o = ((int64_t)blockIdx.x * 256 + threadIdx.x) / G;
   if (o >= n_out) return;

@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(1024)
 segsort_setup_kernel(const int64_t* __restrict__ bounds_in, int S, int64_t n_cap, SortDesc* desc,
                      int64_t* seg_bounds, int32_t* seg_first, int32_t* chunk_seg,
                      int64_t* chunk_begin, int64_t* chunk_end, int max_chunks) {
+  pdl_sync();
   segsort_setup_body(bounds_in, S, n_cap, desc, seg_bounds, seg_first, chunk_seg, chunk_begin, chunk_end,
                      max_chunks);
 }
@@ -134,6 +135,7 @@ bwd_setup_kernel(const WorkerBlob blob, int K, int F, const int64_t* __restrict_
                  int64_t n_bags, int64_t nnz, float* __restrict__ worker_b, SortDesc* desc,
                  int64_t* seg_bounds, int32_t* seg_first, int32_t* chunk_seg, int64_t* chunk_begin,
                  int64_t* chunk_end, int max_chunks, int32_t* status) {
+  pdl_sync();
   __shared__ int64_t s_occ[kSetupMaxWorkers + 1];
   const int tid = threadIdx.x;
   if (tid == 0 && (bag_offsets[0] != 0 || bag_offsets[n_bags] != nnz))
@@ -177,6 +179,7 @@ radix_hist_kernel(const uint32_t* __restrict__ keys, int shift, uint32_t mask,
                   const SortDesc* __restrict__ desc, const int64_t* __restrict__ chunk_begin,
                   const int64_t* __restrict__ chunk_end, uint32_t* __restrict__ hist,
                   int64_t check_rows, int32_t* status) {
+  pdl_sync();
   const int c = blockIdx.x;
   if (c >= desc->n_chunks) return;
   __shared__ uint32_t sh[kSortMaxBins];
@@ -247,6 +250,7 @@ constexpr int kScanBinGroups = kSortMaxBins / 32;
 __global__ void __launch_bounds__(kScanThreads)
 radix_scan_kernel(const SortDesc* __restrict__ desc, const int32_t* __restrict__ seg_first,
                   uint32_t* hist, uint32_t* __restrict__ bin_total) {
+  pdl_sync();
   const int s = blockIdx.x;
   if (s >= desc->n_segments) return;
   __shared__ uint32_t part[kScanWarps][32];
@@ -326,6 +330,7 @@ radix_scatter_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __res
                      const int64_t* __restrict__ chunk_begin, const int64_t* __restrict__ chunk_end,
                      const uint32_t* __restrict__ hist, const uint32_t* __restrict__ bin_total,
                      const int32_t* __restrict__ seg_first) {
+  pdl_sync();
   const int c = blockIdx.x;
   if (c >= desc->n_chunks) return;
   extern __shared__ __align__(16) unsigned char scat_smem[];
@@ -556,6 +561,7 @@ runs_count_kernel(const uint32_t* __restrict__ keys, const SortDesc* __restrict_
                   const int32_t* __restrict__ chunk_seg, const int64_t* __restrict__ seg_bounds,
                   const int64_t* __restrict__ chunk_begin, const int64_t* __restrict__ chunk_end,
                   int64_t* __restrict__ strip_runs) {
+  pdl_sync();
   const int c = blockIdx.x;
   if (c >= desc->n_chunks) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -581,6 +587,7 @@ __global__ void __launch_bounds__(1024)
 runs_scan_kernel(const SortDesc* __restrict__ desc, const int32_t* __restrict__ seg_first,
                  int64_t* strip_runs, int64_t* seg_runs, int64_t* n_runs_out, int64_t* run_start,
                  int64_t out_cap, int32_t* status) {
+  pdl_sync();
   __shared__ int64_t warp_tot[32];
   __shared__ int64_t total;
   const int n = desc->n_chunks * kRunStrips;
@@ -662,6 +669,7 @@ runs_emit_kernel(const uint32_t* __restrict__ keys, const SortDesc* __restrict__
                  const int64_t* __restrict__ strip_runs, int32_t* __restrict__ uniq_keys,
                  int64_t* __restrict__ run_start, uint32_t out_cap, uint32_t* head_bits,
                  int32_t* __restrict__ tile_first, int tile_shift) {
+  pdl_sync();
   const int c = blockIdx.x;
   if (c >= desc->n_chunks) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;

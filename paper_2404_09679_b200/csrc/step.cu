@@ -262,29 +262,29 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
   std::unique_lock<std::mutex> lk;
   if (ss) lk = std::unique_lock<std::mutex>(ss->mu);
 #define CK(x) do { if ((x) != cudaSuccess) return ANTDT_ERR_CUDA; } while (0)
-  auto forward = [&](void* st) {
+  auto forward = [&](void* st, bool side) {
     return antdt::fwd_impl(d->table, d->dtype, d->n_rows, d->dim, d->d_row_ids, d->nnz, d->d_bag_offsets,
-                           d->n_bags, d->d_pooled_out, d->d_status, st, d->bags_per_sample);
+                           d->n_bags, d->d_pooled_out, d->d_status, st, d->bags_per_sample, side);
   };
-  auto backward = [&]() {
+  auto backward = [&](bool pdl_allowed) {
     return antdt::bwd_dedup_impl(d->d_row_ids, d->nnz, d->d_bag_offsets, d->n_bags, d->bags_per_sample,
                                  d->d_d_pooled, d->dim, d->n_rows, d->n_workers, d->worker_sample_offsets,
                                  d->d_uniq_ids, d->d_worker_uniq_offsets, d->d_seg_offsets, d->d_sorted_occ,
                                  d->d_uniq_grads, d->uniq_cap, d->ws, d->ws_bytes, d->d_status, stream, nullptr,
                                  ss ? ss->ids_done : nullptr, merged ? &merge : nullptr,
-                                 ss && beside ? ss->sort_started : nullptr);
+                                 ss && beside ? ss->sort_started : nullptr, pdl_allowed);
   };
   antdt_dense_part dp;
   dp.grads = d->d_dense_grads; dp.n = d->dense_n; dp.stride = d->dense_n; dp.out = d->d_dense_out;
   int32_t rc;
   if (!ss) {
-    rc = forward(stream);
+    rc = forward(stream, false);
     if (rc != ANTDT_OK) return rc;
   }
   // the dense sum runs under the sort
   antdt::DenseBeside beside_sort(dense ? &dp : nullptr, d->batch_sizes, nullptr, d->n_workers, d->d_status, s);
   if (!ss) {
-    rc = backward();
+    rc = backward(!beside_sort.issued());
     if (rc != ANTDT_OK) return rc;
   } else {
     cudaEvent_t after = beside ? ss->sort_started : ss->ids_done;
@@ -292,12 +292,12 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
     int32_t rf = ANTDT_OK;
     if (!beside) {
       CK(cudaStreamWaitEvent(ss->side_fwd, after, 0));
-      rf = forward(ss->side_fwd);
+      rf = forward(ss->side_fwd, true);
     }
-    rc = backward();
+    rc = backward(!beside_sort.issued());
     if (beside) {
       CK(cudaStreamWaitEvent(ss->side_fwd, after, 0));
-      rf = forward(ss->side_fwd);
+      rf = forward(ss->side_fwd, true);
     }
     CK(cudaEventRecord(ss->fwd_done, ss->side_fwd));  // joined even after an error
     CK(cudaStreamWaitEvent(s, ss->fwd_done, 0));      // the update writes the table the forward reads

@@ -73,6 +73,7 @@ tile_reduce_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
                    const uint32_t* __restrict__ head_bits, const int32_t* __restrict__ tile_first,
                    const float* __restrict__ rows, float* __restrict__ out,
                    float* __restrict__ head_part, float* __restrict__ tail_part) {
+  pdl_sync();
   extern __shared__ int64_t s_bounds[];  // payload range of every worker [K+1], then K weights
   float* s_w = reinterpret_cast<float*>(s_bounds + (a.K + 1));
   const int K = a.K;
@@ -198,6 +199,7 @@ __device__ __forceinline__ bool head_at(const uint32_t* __restrict__ hb, int64_t
 template <int G, int VPL, int TILE>
 __global__ void __launch_bounds__(kRedThreads)
 tile_fixup_kernel(const TileArgs a) {
+  pdl_sync();
   const int64_t n = a.n_dev ? min(*a.n_dev, a.n_host) : a.n_host;
   const int lg = threadIdx.x & (G - 1);
   const int64_t tile = (int64_t)blockIdx.x * (kRedThreads / G) + threadIdx.x / G;
