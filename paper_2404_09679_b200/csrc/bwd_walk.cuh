@@ -44,9 +44,11 @@ struct WalkScratch {
   float* head_part;   // [n_stretches, dim]
   float* tail_part;   // [n_stretches, dim]
   uint8_t* flags;     // [n_stretches]
-  int32_t* tasks;     // [2 n_stretches + 4]
+  int32_t* tasks;     // [2 n_stretches + 4]; word 1: CTAs of the walk that have ended
+  bool inline_fixup = false;  // set by the launch: the walk's last CTA does the tasks
   bool tasks_zeroed = false;  // the caller has cleared the list's counter on this stream already
 };
+constexpr int64_t kInlineFixStretches = 24;
 inline int walk_tiles_per_stretch(int dim) {  // = lane groups per CTA, see launch_bwd_walk
   return kRedThreads / red_group(dim);
 }
@@ -75,6 +77,72 @@ __device__ __forceinline__ void put_row(float* row, const float4 (&acc)[VPL], fl
     if (lg + k * G < nvec)
       reinterpret_cast<float4*>(row)[lg + k * G] =
           make_float4(acc[k].x * s, acc[k].y * s, acc[k].z * s, acc[k].w * s);
+}
+
+// Fix-up: one lane group per task, see the head of this file; CTA `cta` of `ctas` takes its share.
+// (Loads past L1: the partials may have been written by other SMs while this kernel ran.)
+template <int G, int VPL, int TILE>
+__device__ __forceinline__ void fixup_tasks(const TileArgs& a, const WalkScratch& ws, int cta, int ctas) {
+  constexpr int TPS = kRedThreads / G;
+  constexpr int64_t SPAN = (int64_t)TPS * TILE;  // entries of a stretch
+  const int n_tasks = __ldcg(ws.tasks);
+  const int64_t n = a.n_host;
+  const int64_t last = (n - 1) / SPAN;  // the last stretch; n >= 1 here
+  const int lg = threadIdx.x & (G - 1);
+  const int glane0 = (threadIdx.x & 31) & ~(G - 1);  // first lane of this group in its warp
+  const unsigned gmask = group_mask<G>();
+  const int dim = a.dim;
+  const int nvec = dim / 4;
+  for (int t = cta * TPS + threadIdx.x / G; t < n_tasks; t += ctas * TPS) {
+    const int64_t s0 = __ldcg(ws.tasks + 2 + 2 * (size_t)t);
+    const int64_t u = __ldcg(ws.tasks + 3 + 2 * (size_t)t);
+    float4 tot[VPL];
+#pragma unroll
+    for (int k = 0; k < VPL; ++k) tot[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    {
+      const float4* tail = reinterpret_cast<const float4*>(ws.tail_part + (size_t)s0 * dim);
+#pragma unroll
+      for (int k = 0; k < VPL; ++k)
+        if (lg + k * G < nvec) tot[k] = __ldcg(tail + lg + k * G);
+    }
+    int w = interval_of(a.bounds, a.K + 1, min(n, (s0 + 1) * SPAN) - 1);  // worker of the run's entries
+    if (w > a.K - 1) w = a.K - 1;
+    const float scale = a.scales[w];
+    int64_t j = s0 + 1;  // next stretch whose leading piece may belong to the run
+    for (;;) {
+      // lane l: does the run stop in stretch j+l?  (a run end inside it; the last stretch has one)
+      const int64_t mine = j + lg;
+      const uint8_t f = mine <= last ? __ldcg(ws.flags + mine) : (uint8_t)(kCloses | kStartsRun);
+      const unsigned stops = (__ballot_sync(gmask, (f & kCloses) != 0) >> glane0) &
+                             ((G == 32) ? 0xffffffffu : ((1u << (G & 31)) - 1u));
+      const int fs = stops ? __ffs((int)stops) - 1 : G;  // stretches j .. j+fs-1 lie inside the run
+      const int f_end = __shfl_sync(gmask, (int)f, fs < G ? fs : 0, G);
+      const int take = fs + ((fs < G && !(f_end & kStartsRun)) ? 1 : 0);  // pieces to add, in order
+      for (int i0 = 0; i0 < take; i0 += 4) {
+        float4 x[4][VPL];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int k = 0; k < VPL; ++k) {
+            const int vi = lg + k * G;
+            x[i][k] = (i0 + i < take && vi < nvec)
+                          ? __ldcg(reinterpret_cast<const float4*>(ws.head_part + (size_t)(j + i0 + i) * dim) + vi)
+                          : make_float4(0.f, 0.f, 0.f, 0.f);
+          }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int k = 0; k < VPL; ++k) {
+            if (i0 + i < take) {
+              tot[k].x += x[i][k].x; tot[k].y += x[i][k].y; tot[k].z += x[i][k].z; tot[k].w += x[i][k].w;
+            }
+          }
+      }
+      if (fs < G) break;
+      j += G;
+    }
+    if (u < a.out_cap) put_row<G, VPL>(a.out + (size_t)u * dim, tot, scale, lg, nvec);
+  }
 }
 
 template <int G, int VPL, int TILE>
@@ -263,8 +331,7 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
   if (lg == 0)
     s_flag[grp] = in_range ? (uint8_t)((closes ? kCloses : 0) | (started ? kStartsRun : 0)) : (uint8_t)kNoTile;
   __syncthreads();
-  if (!in_range) return;
-  if (grp == 0) {
+  if (in_range && grp == 0) {
     // the stretch's own record: its flag byte and, if a run enters it, that run's piece in it
     bool any_close = false;
     float4 tot[VPL];
@@ -279,7 +346,7 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
     if (!started) put_row<G, VPL>(ws.head_part + (size_t)stretch * dim, tot, 1.f, lg, nvec);
     if (lg == 0) ws.flags[stretch] = (uint8_t)((any_close ? kCloses : 0) | (started ? kStartsRun : 0));
   }
-  if (open_tail && (started || closes)) {
+  if (in_range && open_tail && (started || closes)) {
     // the run that is open at this tile's end started here: collect what follows
     bool done = false;
     for (int g = grp + 1; g < TPS && !done; ++g) {
@@ -299,73 +366,25 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
       }
     }
   }
-}
-
-// Fix-up: one lane group per task, see the head of this file.
-template <int G, int VPL, int TILE>
-__global__ void __launch_bounds__(kRedThreads)
-bwd_fixup_kernel(const TileArgs a, const WalkScratch ws) {
-  pdl_sync();
-  constexpr int TPS = kRedThreads / G;
-  constexpr int64_t SPAN = (int64_t)TPS * TILE;  // entries of a stretch
-  const int n_tasks = ws.tasks[0];
-  const int64_t n = a.n_host;
-  const int64_t last = (n - 1) / SPAN;  // the last stretch; n >= 1 here
-  const int lg = threadIdx.x & (G - 1);
-  const int glane0 = (threadIdx.x & 31) & ~(G - 1);  // first lane of this group in its warp
-  const unsigned gmask = group_mask<G>();
-  const int dim = a.dim;
-  const int nvec = dim / 4;
-  const int groups = gridDim.x * TPS;
-  for (int t = blockIdx.x * TPS + threadIdx.x / G; t < n_tasks; t += groups) {
-    const int64_t s0 = ws.tasks[2 + 2 * (size_t)t];
-    const int64_t u = ws.tasks[3 + 2 * (size_t)t];
-    float4 tot[VPL];
-#pragma unroll
-    for (int k = 0; k < VPL; ++k) tot[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    add_row<G, VPL>(tot, ws.tail_part + (size_t)s0 * dim, lg, nvec);
-    int w = interval_of(a.bounds, a.K + 1, min(n, (s0 + 1) * SPAN) - 1);  // worker of the run's entries
-    if (w > a.K - 1) w = a.K - 1;
-    const float scale = a.scales[w];
-    int64_t j = s0 + 1;  // next stretch whose leading piece may belong to the run
-    for (;;) {
-      // lane l: does the run stop in stretch j+l?  (a run end inside it; the last stretch has one)
-      const int64_t mine = j + lg;
-      const uint8_t f = mine <= last ? ws.flags[mine] : (uint8_t)(kCloses | kStartsRun);
-      const unsigned stops = (__ballot_sync(gmask, (f & kCloses) != 0) >> glane0) &
-                             ((G == 32) ? 0xffffffffu : ((1u << (G & 31)) - 1u));
-      const int fs = stops ? __ffs((int)stops) - 1 : G;  // stretches j .. j+fs-1 lie inside the run
-      const int f_end = __shfl_sync(gmask, (int)f, fs < G ? fs : 0, G);
-      const int take = fs + ((fs < G && !(f_end & kStartsRun)) ? 1 : 0);  // pieces to add, in order
-      for (int i0 = 0; i0 < take; i0 += 4) {
-        float4 x[4][VPL];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int k = 0; k < VPL; ++k) {
-            const int vi = lg + k * G;
-            x[i][k] = (i0 + i < take && vi < nvec)
-                          ? reinterpret_cast<const float4*>(ws.head_part + (size_t)(j + i0 + i) * dim)[vi]
-                          : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int k = 0; k < VPL; ++k) {
-            if (i0 + i < take) {
-              tot[k].x += x[i][k].x; tot[k].y += x[i][k].y; tot[k].z += x[i][k].z; tot[k].w += x[i][k].w;
-            }
-          }
-      }
-      if (fs < G) break;
-      j += G;
+  // A small input's few tasks are done by the CTA that ends last, instead of by another launch.
+  if (TILE == kRedTileSmall && ws.inline_fixup) {
+    __threadfence();
+    if (__syncthreads_or(threadIdx.x == 0 && atomicAdd(ws.tasks + 1, 1) == (int)gridDim.x - 1)) {
+      __threadfence();
+      fixup_tasks<G, VPL, TILE>(a, ws, 0, 1);
     }
-    if (u < a.out_cap) put_row<G, VPL>(a.out + (size_t)u * dim, tot, scale, lg, nvec);
   }
 }
 
 template <int G, int VPL, int TILE>
-void launch_bwd_walk_t(const TileArgs& a_in, const WalkScratch& ws, const char* name_tiles,
+__global__ void __launch_bounds__(kRedThreads)
+bwd_fixup_kernel(const TileArgs a, const WalkScratch ws) {
+  pdl_sync();
+  fixup_tasks<G, VPL, TILE>(a, ws, blockIdx.x, gridDim.x);
+}
+
+template <int G, int VPL, int TILE>
+void launch_bwd_walk_t(const TileArgs& a_in, const WalkScratch& ws_in, const char* name_tiles,
                        const char* name_fixup, cudaStream_t s) {
   constexpr int TPS = kRedThreads / G;
   const int64_t n_tiles = (a_in.n_host + TILE - 1) / TILE;
@@ -373,6 +392,11 @@ void launch_bwd_walk_t(const TileArgs& a_in, const WalkScratch& ws, const char* 
   if (a.tile_begin < 0) a.tile_begin = 0;
   if (a.tile_end < 0 || a.tile_end > n_tiles) a.tile_end = n_tiles;
   a.tile_begin = a.tile_begin / TPS * TPS;  // a launch covers whole stretches (callers cut there)
+  WalkScratch ws = ws_in;
+  // 10 k occurrences as a graph 34.9 -> 32.9 us; from about 30 stretches on one CTA takes as long for
+  // the tasks as the launch, at 256 it takes 5 us longer.
+  ws.inline_fixup = TILE == kRedTileSmall && a.walk && a.fixup && a.tile_begin == 0 && a.tile_end == n_tiles && n_tiles > TPS &&
+                    n_tiles <= kInlineFixStretches * TPS;
   const size_t smem = 2 * (size_t)TPS * a.dim * 4 + 8 * ((size_t)a.K + 1) + TPS;
   if (smem > 48 * 1024) {  // rows of 1024 floats: more than the default dynamic shared memory
     static bool attr_set[64] = {};
@@ -391,7 +415,7 @@ void launch_bwd_walk_t(const TileArgs& a_in, const WalkScratch& ws, const char* 
     ANTDT_LAUNCH(name_tiles, (bwd_walk_kernel<G, VPL, TILE>), grid, kRedThreads, smem, s, a, a.payload,
                  a.head_bits, a.tile_first, a.rows, a.out, ws, vec);
   }
-  if (a.fixup && n_tiles > TPS) {
+  if (a.fixup && n_tiles > TPS && !ws.inline_fixup) {
     const int64_t want = ((n_tiles + TPS - 1) / TPS + TPS - 1) / TPS;
     const unsigned grid = (unsigned)(want < 8 * kNumSM ? want : 8 * kNumSM);
     ANTDT_LAUNCH(name_fixup, (bwd_fixup_kernel<G, VPL, TILE>), grid, kRedThreads, 0, s, a, ws);
