@@ -353,9 +353,10 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
                    const int64_t u = u0 + t;
                    src[dest] = (uint32_t)j;
                    if (src_worker) src_worker[dest] = (uint8_t)w;  // saves the reader a search
-                   if (slot == 0 && u < out_cap) {
-                     agg_ids[u] = (int32_t)id;
-                     if (row_start) row_start[u] = (uint32_t)dest;  // the row's first merge slot
+                   if (slot == 0) {
+                     if (u < out_cap) agg_ids[u] = (int32_t)id;
+                     // the row's first merge slot (one more than rows: it ends the last one)
+                     if (row_start && u <= out_cap) row_start[u] = (uint32_t)dest;
                    }
                    if (tile_first && (dest & tile_mask) == 0) tile_first[dest >> tile_shift] = (int32_t)u;
                  });

@@ -49,7 +49,7 @@ void range_prepare_device();
 //   tile_first          index into agg_ids of the row that slot t*tile belongs to
 //                       (head_bits and tile_first may both be nullptr: a reader that goes by
 //                       row_start needs neither)
-//   row_start [out_cap] merge slot of the first contribution of each row of agg_ids, or nullptr
+//   row_start [out_cap+1] merge slot of the first contribution of each row of agg_ids, or nullptr
 //   src_worker [in_cap] the worker of every merge slot (one byte), or nullptr
 //   weights_host [K]    the workers' weights; the first kernel carries them to weights_dev [K]
 //                       as a parameter (nullptr: the caller has put them there already)

@@ -288,6 +288,9 @@ dense_wsum_bulk_kernel(const float* __restrict__ grads, uint32_t n, int64_t stri
 // is formed in that fixed order and goes straight into the Adagrad / Adam arithmetic, so the
 // aggregated gradient is never written to or read back from memory (agg_out, if given, receives
 // it all the same).  No partial sums, no second pass: a row has at most K contributions.
+// Without a table (UPDATE false) it forms the sums alone, for lists so short that the tile reduction's
+// second launch counts: 9 k entries of 5 workers 64.5 -> 57 us for a step of four calls.  (For long ones the
+// tile reduction is faster, 129 against 170 us on 1.9 M entries x 64.)
 struct FusedUpdate {
   void* table; int dtype; int opt; OptParams p; float* state0; float* state1; float* agg_out;
 };
@@ -310,7 +313,7 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 constexpr int kFusedRows = 1;
 constexpr int kFusedWaves = 16, kFusedWavesAdam = 64;
 constexpr int kFusedCtas = 8;
-template <int G, int VPL, bool ADAM, bool BF16>
+template <int G, int VPL, bool UPDATE, bool ADAM, bool BF16>
 __global__ void __launch_bounds__(256, (VPL == 1 ? kFusedCtas : 1))
 agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __restrict__ src,
                   const int32_t* __restrict__ agg_ids, const int64_t* __restrict__ n_agg_dev,
@@ -329,6 +332,9 @@ agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __rest
   // 32-bit row numbers and slots (fewer than 2^31 of each): the kernel is bound by its instruction
   // stream and by the registers that live across the chain of loads
   const uint32_t n = (uint32_t)min(*n_agg_dev, out_cap);
+  // where the capacity cuts rows off, the next row's start still ends the last one (the update, whose
+  // result is flagged then, does without: it has no register to spare)
+  const uint32_t n_starts = UPDATE ? n : (uint32_t)*n_agg_dev;
   const uint32_t total = (uint32_t)min(n_entries[1], in_cap);
   const uint32_t stride = gridDim.x * (256 / G);
   for (uint32_t u0 = blockIdx.x * (256 / G) + threadIdx.x / G; u0 < n; u0 += R * stride) {
@@ -340,7 +346,7 @@ agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __rest
       const uint32_t u = u0 + r * stride;
       ok[r] = u < n;
       s0[r] = ok[r] ? __ldg(row_start + u) : 0u;
-      s1[r] = ok[r] ? (u + 1 < n ? __ldg(row_start + u + 1) : total) : 0u;
+      s1[r] = ok[r] ? (u + 1 < n_starts ? __ldg(row_start + u + 1) : total) : 0u;
       row[r] = ok[r] ? __ldg(agg_ids + u) : -1;
     }
     uint32_t longest = 0;
@@ -362,7 +368,7 @@ agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __rest
       for (int r = 0; r < R; ++r) {
         at[r] = (size_t)(ok[r] ? row[r] : 0) * dim + 4 * (size_t)vi;
         g[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (ok[r]) {  // towards L2 now (costs no register), into registers after the sum
+        if (UPDATE && ok[r]) {  // towards L2 now (costs no register), into registers after the sum
           prefetch_l2(static_cast<const char*>(table) + at[r] * (BF16 ? 2 : 4));
           prefetch_l2(state0 + at[r]);
           if (ADAM) prefetch_l2(state1 + at[r]);
@@ -401,7 +407,7 @@ agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __rest
       // (to overlap their latency with it) costs registers that the 64 warps per SM do not have
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        if (ok[r]) {
+        if (UPDATE && ok[r]) {
           w[r] = load_row4(table, BF16, at[r]);
           a0[r] = *reinterpret_cast<const float4*>(state0 + at[r]);
           if (ADAM) a1[r] = *reinterpret_cast<const float4*>(state1 + at[r]);
@@ -410,7 +416,8 @@ agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __rest
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         if (!ok[r]) continue;
-        if (agg_out) reinterpret_cast<float4*>(agg_out + (size_t)(u0 + r * stride) * dim)[vi] = g[r];
+        if (!UPDATE || agg_out) reinterpret_cast<float4*>(agg_out + (size_t)(u0 + r * stride) * dim)[vi] = g[r];
+        if (!UPDATE) continue;
         if (ADAM) {
           w[r].x = adam1(a0[r].x, a1[r].x, g[r].x, w[r].x, p); w[r].y = adam1(a0[r].y, a1[r].y, g[r].y, w[r].y, p);
           w[r].z = adam1(a0[r].z, a1[r].z, g[r].z, w[r].z, p); w[r].w = adam1(a0[r].w, a1[r].w, g[r].w, w[r].w, p);
@@ -436,8 +443,14 @@ void launch_agg_update(const FusedUpdate& fu, const uint32_t* row_start, const u
   const bool adam = fu.opt == ANTDT_OPT_ADAM, bf16 = fu.dtype == ANTDT_BF16;
   const int64_t cap = (int64_t)kNumSM * kFusedCtas * (adam ? kFusedWavesAdam : kFusedWaves);
   const unsigned grid = (unsigned)(want > cap ? cap : (want < 1 ? 1 : want));
+  if (!fu.table) {  // the sums alone
+    ANTDT_LAUNCH("agg_reduce", (agg_update_kernel<G, VPL, false, false, false>), grid, 256, smem, s, row_start, src,
+                 sp->agg_ids, sp->n_agg, out_cap, n_entries, sp->uniq_grads, sp->in_cap, src_worker, weights, K,
+                 nullptr, sp->n_rows, sp->dim, fu.p, nullptr, nullptr, fu.agg_out);
+    return;
+  }
 #define FU_GO(A, B)                                                                              \
-  ANTDT_LAUNCH("agg_update", (agg_update_kernel<G, VPL, A, B>), grid, 256, smem, s, row_start, src, \
+  ANTDT_LAUNCH("agg_update", (agg_update_kernel<G, VPL, true, A, B>), grid, 256, smem, s, row_start, src, \
                sp->agg_ids, sp->n_agg, out_cap, n_entries, sp->uniq_grads, sp->in_cap, src_worker, weights, K, \
                fu.table, sp->n_rows, sp->dim, fu.p, fu.state0, fu.state1, fu.agg_out)
   if (adam) { if (bf16) FU_GO(true, true); else FU_GO(true, false); }
@@ -589,6 +602,8 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
   // the two merges carry the weights themselves
   const bool resident = sp && resident_merge_wanted(K, in_cap, sp->n_rows);
   const bool by_ranges = sp && K <= kRangeMaxWorkers && in_cap > 0;
+  // a lane group per row: the one-pass update, and the sums of short lists
+  const bool by_rows = sp && in_cap > 0 && ((fu && K <= kRangeMaxWorkers) || (!fu && resident && resident_sort_clears(in_cap)));
   if (!by_ranges && !resident) upload_small(hw, 4 * (size_t)K, w8 + L.weights, s);
   // the dense part runs beside the sparse one where there is enough of it
   DenseBeside beside(sp && in_cap > 0 ? dp : nullptr, batch_sizes, dropped, K, dev_status, s);
@@ -606,7 +621,7 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
       q.uniq_ids = sp->uniq_ids; q.wuo_in = sp->worker_uniq_offsets; q.in_cap = in_cap; q.n_rows = sp->n_rows;
       q.n_workers = K; q.agg_ids = sp->agg_ids; q.n_agg = sp->n_agg; q.out_cap = agg_cap;
       q.wuo_out = (int64_t*)(w8 + L.wuo); q.n_entries = bounds; q.src = (uint32_t*)(w8 + L.src);
-      if (fu && K <= kRangeMaxWorkers) {
+      if (by_rows) {
         q.row_start = (uint32_t*)(w8 + L.row_start);
         q.src_worker = (uint8_t*)(w8 + L.src_worker);
       } else {
@@ -652,9 +667,9 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
     } else {
       sort_merge_order(sp, dropped, any_dropped, K, in_cap, agg_cap, w8, L, dev_status, s);
     }
-    if (fu && K <= kRangeMaxWorkers && in_cap > 0) {
+    if (by_rows) {
       // one pass: every aggregated row is summed and applied by the lane group that owns it
-      FusedUpdate f = *fu;
+      FusedUpdate f = fu ? *fu : FusedUpdate{};
       f.agg_out = sp->agg_grads;
       const uint32_t* rs = (const uint32_t*)(w8 + L.row_start);
       const uint32_t* src = (const uint32_t*)(w8 + L.src);

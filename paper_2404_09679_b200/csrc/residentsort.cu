@@ -610,10 +610,8 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
             m.src_worker[slot] = (uint8_t)w;
             if (r) {
               const uint32_t x = mrow + __popc(rb & lt);
-              if (x < m.agg_cap) {
-                m.agg_ids[x] = (int32_t)row;
-                m.row_start[x] = slot;
-              }
+              if (x < m.agg_cap) m.agg_ids[x] = (int32_t)row;
+              if (x <= m.agg_cap) m.row_start[x] = slot;  // one more than rows: it ends the last one
             }
           }
         }
@@ -753,10 +751,8 @@ resident_merge_kernel(const __grid_constant__ ResidentMergeArgs a) {
       a.src[slot] = v[i];
       if (a.src_worker) a.src_worker[slot] = (uint8_t)min(interval_of(S.bound, K + 1, v[i]), K - 1);
       if (r) {
-        if (x < a.out_cap) {
-          a.agg_ids[x] = (int32_t)k[i];
-          if (a.row_start) a.row_start[x] = slot;
-        }
+        if (x < a.out_cap) a.agg_ids[x] = (int32_t)k[i];
+        if (a.row_start && x <= a.out_cap) a.row_start[x] = slot;  // one more than rows: it ends the last one
         if (a.head_bits) atomicOr(a.head_bits + (slot >> 5), 1u << (slot & 31));
       }
       if (a.tile_first && (slot & tile_mask) == 0) a.tile_first[slot >> a.tile_shift] = (int32_t)x;

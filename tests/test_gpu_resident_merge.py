@@ -59,3 +59,18 @@ def test_dropped_workers_and_foreign_ids(K):
     uid[wuo[1] - 1] = V + 3      # the last id of worker 0 lies outside the table: skipped and flagged
     ids, _, _, _, code = G.gpu_aggregate(uid, wuo, g, bsz, V)
     assert code == B.ERR_ID_OUT_OF_RANGE and ids.max() < V
+
+
+@pytest.mark.parametrize("K,D", [(1, 4), (5, 20), (40, 64), (128, 200)])
+def test_sums_by_rows_at_the_capacity(K, D):
+    """Short lists are summed row by row: every row kept must be right when the capacity cuts the rest."""
+    rng = np.random.default_rng(K)
+    uid, wuo = _lists(rng, K, 500, [150] * K)
+    g = rng.normal(size=(len(uid), D)).astype(np.float32)
+    bsz = rng.integers(1, 9, size=K)
+    want_ids, want = oracle.aggregate_sparse(uid, wuo, g, bsz.astype(np.int64))
+    for cap in (1, len(want_ids) - 1, len(want_ids)):
+        ids, agg, n, _, code = G.gpu_aggregate(uid, wuo, g, bsz, 500, out_cap=cap)
+        assert n == len(want_ids) and code == (B.ERR_CAPACITY if cap < n else 0)
+        assert np.array_equal(ids, want_ids[:cap])
+        G.close(agg, want[:cap])
