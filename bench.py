@@ -455,7 +455,7 @@ def run_ours(args):
     # the device calls behind one C call; --fuse-update: aggregate and update in one pass
     dstep = DeviceStep(buf, table, state0, state1, oc, w.K, fuse_update=args.fuse_update)
 
-    # Launch form of the timed steps.  A step is 30-40 launches; on the small configurations
+    # Launch form of the timed steps.  A step is 4 to 25 launches; on the small configurations
     # they, not the kernels, are the step time, so there the step is replayed as one CUDA graph.
     # (auto: wherever the entry point can replay a graph, i.e. not for Adam, whose step number
     # changes kernel parameters every step; on the large configurations it saves the launch gaps.)

@@ -220,11 +220,12 @@ int32_t antdt_embbag_fwd(const void* table, int32_t dtype, int64_t n_rows, int32
  *   out_cap              capacity in rows; nnz always suffices; CAPACITY -> dev_status
  *   ws, ws_bytes         device scratch.  antdt_embbag_bwd_dedup_workspace_bytes(...) is the size
  *                        to allocate; antdt_embbag_bwd_dedup_min_workspace_bytes(...) is the least
- *                        the call accepts (WORKSPACE_TOO_SMALL below it).  The two differ for up to
- *                        2^20 occurrences only: with the larger one the reduction walks 16-entry
- *                        tiles, which keeps a small input spread over the whole GPU; with less it
- *                        walks the 64-entry tiles of large inputs.  Results are the same up to the
- *                        order of the floating-point sums (both orders are fixed). */
+ *                        the call accepts (WORKSPACE_TOO_SMALL below it).  The two differ only
+ *                        for inputs that long tiles would not spread over the whole GPU (up to
+ *                        1.2 M occurrences at dim 64, 4.8 M at dim 16): with the larger one their
+ *                        reduction walks 16-entry tiles; with less it walks the 64-entry tiles of
+ *                        large inputs.  Results are the same up to the order of the
+ *                        floating-point sums (both orders are fixed). */
 size_t antdt_embbag_bwd_dedup_workspace_bytes(int64_t nnz, int64_t n_bags, int32_t dim,
                                               int32_t n_workers);
 size_t antdt_embbag_bwd_dedup_min_workspace_bytes(int64_t nnz, int64_t n_bags, int32_t dim,
@@ -248,8 +249,7 @@ int32_t antdt_embbag_bwd_dedup(const int32_t* row_ids, int64_t nnz, const int64_
  *   - Arguments and results are those of antdt_embbag_bwd_dedup without ws / ws_bytes; inputs and
  *     outputs are still the caller's buffers.
  *   - Limit: antdt_embbag_bwd_dedup_min_workspace_bytes(nnz, n_bags, dim, n_workers) must not exceed
- *     ANTDT_STATIC_SCRATCH_BYTES (24 MiB: roughly 1.1 million occurrences at dim 64, 1.7 million at
- *     dim 16, with up to 64 workers).  Beyond it the call returns ANTDT_ERR_CAPACITY and launches
+ *     ANTDT_STATIC_SCRATCH_BYTES (24 MiB: roughly 1.8 million occurrences with up to 64 workers).  Beyond it the call returns ANTDT_ERR_CAPACITY and launches
  *     nothing.
  *   - The call itself makes no cudaMalloc / cudaFree and no allocating library call.  The first
  *     call on each device looks up the array's device address (cudaGetSymbolAddress, with that
@@ -416,7 +416,7 @@ int32_t antdt_bsp_step_host(const antdt_step_desc* d, void* stream);
  * call instead of four: for small batches the per-call host cost is the step time. */
 int32_t antdt_bsp_step_device(const antdt_step_desc* d, void* stream);
 /* The same device-resident step (Section II's iteration: local gradients, aggregation, update),
- * replayed as ONE CUDA graph launch.  A step is 30-40 short kernels; on small batches their
+ * replayed as ONE CUDA graph launch.  A step is 4 to 25 kernels; on small batches their
  * launches, not their run time, are the step time.  The first call with a given descriptor
  * captures antdt_bsp_step_device on `stream` (thread-local capture mode), instantiates the graph
  * and launches it; later calls whose descriptor is equal launch the kept executable graph.
@@ -441,16 +441,20 @@ int32_t antdt_bsp_step_device(const antdt_step_desc* d, void* stream);
  *   - Per-kernel event timing (antdt_profile_enable) does not see kernels inside a graph;
  *     antdt_launch_count counts a replay's kernel nodes.
  *   - Small batches (at most 2^22 occurrences, at most 32 workers) are captured
- *     as three branches when the workspace has room: the forward beside the backward, and the
+ *     as branches when the workspace has room: the forward beside the backward, and the
  *     aggregation's merge order (which needs the workers' id lists, not their gradients) beside
- *     the backward's sums.  No kernel fills the device there, so the step time is the length of
- *     the dependency chain.  The results are those of the one-chain step.  Room means ws_bytes
+ *     the backward's sums, unless the backward's sort makes it on the way (up to about 1.8 M
+ *     occurrences, fuse_update).  No kernel fills the device there, so the step time is the length
+ *     of the dependency chain.  The results are those of the one-chain step.  Room means ws_bytes
  *     >= antdt_bsp_step_workspace_bytes(...): the aggregation's scratch then sits behind the
  *     backward's instead of on top of it.  The branches use two library-owned side streams.
+ *     antdt_bsp_step_device uses one of them too, for the forward of a batch that the backward
+ *     sorts in one kernel, and a third carries a large dense part beside the sort or the merge;
+ *     the caller's stream waits for all of them.
  * Returns ANTDT_OK, an argument error, or ANTDT_ERR_CUDA. */
 int32_t antdt_bsp_step_graph(const antdt_step_desc* d, void* stream);
 /* Workspace of a step: the larger of the backward's and the aggregation's figures; their sum
- * (the backward's rounded up to 256 bytes) for a batch small enough for the three-branch graph.
+ * (the backward's rounded up to 256 bytes) for a batch small enough for both to be live at once (2^22 occurrences).
  * 0 for arguments either figure rejects. */
 size_t antdt_bsp_step_workspace_bytes(int64_t nnz, int64_t n_bags, int32_t dim, int32_t n_workers,
                                       int64_t uniq_cap);

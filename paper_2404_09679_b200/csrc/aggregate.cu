@@ -9,7 +9,8 @@
 // weighted sum of its <= K contributions in that fixed order.  Because the sorted positions of
 // one worker ascend with the row id, the gather of the workers' gradient rows is K
 // forward-moving streams, not a random walk.
-// Dense part: a K-way streaming reduction, one 16-byte vector per thread and worker.
+// Dense part: a K-way streaming reduction, one 16-byte vector per thread and worker; a large one
+// beside a sort or a merge order takes a kernel that fits between their CTAs (dense_wsum_bulk_kernel).
 #include <mutex>
 
 #include "agg_range.cuh"

@@ -236,12 +236,15 @@ extern "C" int32_t antdt_bsp_step_host(const antdt_step_desc* d, void* stream) {
 // The same four calls for a batch that is already resident in device memory: nothing is copied,
 // the status word is left as the caller set it.
 //
-// forked: the step as three chains instead of one.  The forward needs nothing from the backward,
-// and the aggregation's merge order needs the workers' id lists but not their gradients, so both
-// run on side streams beside the backward (fork and join by events; in a capture they become
-// parallel branches of the graph).  It pays on small batches, where no kernel fills the device
-// and the step time is the length of the dependency chain; it needs the aggregation's scratch
-// behind the backward's instead of on top of it.
+// What runs beside what (fork and join by events; in a capture, parallel branches of the graph):
+//   dense sum     a large one beside the sort, on its own side stream (DenseBeside, aggregate.cu)
+//   forward       beside the resident sort (residentsort.cu) wherever the backward takes that one;
+//                 beside the whole backward in a forked step
+//   merge order   (needs the workers' id lists but not their gradients) made by the resident sort on
+//                 the way; else, in a forked step, beside the backward's sums
+// forked: a small step inside a graph, where no kernel fills the device and the step time is the
+// length of the dependency chain.  It needs the aggregation's scratch behind the backward's instead
+// of on top of it.
 namespace {
 int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
   if (!d || d->nnz < 0 || d->n_bags < 0 || d->dim < 1 || !d->d_bag_offsets || !d->d_n_agg)
@@ -329,7 +332,7 @@ extern "C" size_t antdt_bsp_step_workspace_bytes(int64_t nnz, int64_t n_bags, in
 
 // ---------------------------------------------------------------------------------------
 // The device-resident step replayed as a CUDA graph.
-// A step is 30-40 short launches; on small batches the launches, not the kernels, are the step
+// A step is 4 to 25 short launches; on small batches the launches, not the kernels, are the step
 // time.  The four calls are captured once per distinct descriptor and replayed with a single
 // graph launch.  Everything a captured launch depends on is in the key: every scalar and device
 // pointer of the descriptor and the CONTENTS of the two host arrays (they reach the device as
