@@ -8,7 +8,8 @@
 //               marked in shared memory, a running maximum over the positions spreads the marks
 //   per pass    (by row id) rank inside the warp, digit counters summed over the CTA's warps and
 //               published; a barrier over the CTAs; everybody's counts give the first slot of every
-//               digit; the pairs go to their slots; a second barrier; every CTA takes the pairs of
+//               digit; the pairs go to their slots, put in the order of their digits in shared memory
+//               first so that a warp stores to a few lines; a second barrier; every CTA takes the pairs of
 //               its own slots
 //   last pass   (by worker) takes everything to the workers' own order.  It ranks the runs of equal
 //               (worker, row) as well as the pairs: a run's rank among the runs of its worker is its
@@ -25,7 +26,7 @@
 // distributed shared memory (a barrier 0.3 us against 1.3).
 // Measured (in brackets the kernels it replaced: sort, and merge order where a step makes it): 10 k
 // occurrences of 4 workers over 80 k rows 17 us (37 + 35); 426 k of 8 over 26 M 60 us (75 + 62);
-// 1.2 M of one worker over 1 M 99 us (113).
+// 1.2 M of one worker over 1 M 74 us (113).
 //
 // The CTAs wait for one another, so the launch is a cluster or a cooperative one (all CTAs resident
 // or none started).  Every wait through memory is bounded all the same (kSpinLimit) and raises
@@ -42,25 +43,43 @@ constexpr int kMaxItems = 24;        // pairs per thread
 constexpr int kMinChunk = 1024;
 constexpr int kClusterItems = 4;     // pairs per thread of the cluster form
 constexpr int kMaxCluster = 16;
+constexpr int kMatchWorkers = 8;     // see the pass by worker
 constexpr uint32_t kSpinLimit = 1u << 20;
 static_assert(kBins == kThreads, "one digit per thread");
 
+// Pairs per thread: every warp of a CTA takes an equal share of its chunk.
+__host__ __device__ constexpr int items_per_thread(int chunk) { return (chunk + kThreads - 1) / kThreads; }
+
 struct Wso { int64_t v[kResMaxWorkers + 1]; };
 
-struct Smem {
-  union {
-    uint32_t mm[kWarps * kBins];          // while ranking: the lanes that hold a digit, per warp
-    uint32_t mark[kMaxItems * kThreads];  // before the sort: first occurrences of the bags
-  };
+struct __align__(16) Smem {
   unsigned short wh[kWarps * kBins];      // per-warp digit counters, then their prefix over the warps
   uint32_t cnt[kBins];                    // a counter's sum over the CTAs
   uint32_t base[kBins];                   // first slot of every digit for this CTA
+  uint32_t loc[kBins];                    // pairs of smaller digits in this CTA
   uint16_t row[kBins];                    // cluster form: this CTA's published counters
-  uint2 pairs[kClusterItems * kThreads];  // cluster form: the pairs of this CTA's slots
   uint32_t warp_a[kWarps], warp_b[kWarps];
   uint32_t warp_tot[kWarps];
   int64_t bound[kResMaxWorkers + 1];      // occurrence range of every worker
+
+  // Behind the struct (smem_bytes), one after the other in the same place:
+  __device__ uint32_t* mm() { return reinterpret_cast<uint32_t*>(this + 1); }    // while ranking: the lanes that
+                                                                                 // hold a digit, per warp [kWarps * kBins]
+  __device__ uint32_t* mark() { return reinterpret_cast<uint32_t*>(this + 1); }  // before the sort: first occurrences
+                                                                                 // of the bags [chunk]
+  __device__ uint2* stage() { return reinterpret_cast<uint2*>(this + 1); }       // after ranking: the pairs in the
+                                                                                 // order of their digits; after the
+                                                                                 // passes: this CTA's own [chunk]
+  // cluster form, behind mm: the pairs of this CTA's slots [kClusterItems * kThreads]
+  __device__ uint2* pairs() { return reinterpret_cast<uint2*>(mm() + kWarps * kBins); }
 };
+size_t smem_bytes(int chunk, bool cluster) {
+  // the pass by worker: pairs, a word per pair, its masks (two times 128 workers at most)
+  const size_t mm = 4 * (size_t)kWarps * kBins, tail = 12 * (size_t)chunk + 4 * (size_t)kWarps * 2 * kResMaxWorkers;
+  return sizeof(Smem) + (cluster ? mm + 8 * (size_t)kClusterItems * kThreads : (tail > mm ? tail : mm));
+}
+static_assert(4 * kClusterItems * kThreads + 4 * kWarps * 2 * kResMaxWorkers <= 4 * kWarps * kBins,
+              "cluster form: marks, or a word per pair and the masks of the pass by worker, end before pairs");
 
 // ---- the cluster ----
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
@@ -124,6 +143,7 @@ __device__ __forceinline__ void warp_rank(const uint32_t (&k)[IPT], int valid, i
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
   for (int i = 0; i < IPT; ++i) {
+    if (IPT > 4 && i % 4 == 0 && i * 32 >= valid) break;
     const bool ok = i * 32 + lane < valid;
     const uint32_t d = (k[i] >> shift) & mask;
     if (ok) atomicOr(my_mm + d, 1u << lane);
@@ -147,17 +167,15 @@ __device__ __forceinline__ void warp_rank(const uint32_t (&k)[IPT], int valid, i
 
 // Barrier over the CTAs: of the cluster, or `target` arrivals on a counter in memory that only
 // grows.  Orders their memory accesses.
-template <bool CLUSTER>
-__device__ __forceinline__ void all_barrier(uint32_t* counter, uint32_t target, int32_t* status) {
-  if (CLUSTER) {
-    cluster_arrive();
-    cluster_wait();
-    return;
-  }
+__device__ __forceinline__ void grid_arrive(uint32_t* counter) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(counter, 1u);
+  }
+}
+__device__ __forceinline__ void grid_wait(uint32_t* counter, uint32_t target, int32_t* status) {
+  if (threadIdx.x == 0) {
     uint32_t x = 0;
     for (uint32_t n = 0; n < kSpinLimit; ++n) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(counter) : "memory");
@@ -166,6 +184,16 @@ __device__ __forceinline__ void all_barrier(uint32_t* counter, uint32_t target, 
     if (x < target) set_status(status, ANTDT_ERR_TIMEOUT);
   }
   __syncthreads();
+}
+template <bool CLUSTER>
+__device__ __forceinline__ void all_barrier(uint32_t* counter, uint32_t target, int32_t* status) {
+  if (CLUSTER) {
+    cluster_arrive();
+    cluster_wait();
+  } else {
+    grid_arrive(counter);
+    grid_wait(counter, target, status);
+  }
 }
 
 // Sums of the C published rows of counters and of those before `rank`, per counter (the
@@ -254,7 +282,7 @@ template <int IPT>
 __device__ __forceinline__ void chunk_bags(Smem& S, const ResidentSortArgs& a, const BagWindow& win, int64_t end,
                                            int64_t g0, int n_mine, uint32_t (&v)[IPT]) {
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
-  const int wbase = wp * 32 * IPT, valid = min(max(n_mine - wbase, 0), 32 * IPT);
+  const int per = items_per_thread(a.chunk), wbase = wp * 32 * per, valid = min(max(n_mine - wbase, 0), 32 * per);
   const int32_t c0 = (int32_t)g0, c1 = (int32_t)g0 + n_mine;
   bool covered = true;  // the window holds every bag of the chunk
   if (tid == 0) covered = win.first == 0 || win.lo[0] <= c0;
@@ -264,7 +292,7 @@ __device__ __forceinline__ void chunk_bags(Smem& S, const ResidentSortArgs& a, c
     for (int t = 0; t < kWindowTurns; ++t) {
       const int64_t b = win.first + t * kThreads + tid;
       const int32_t from = max(win.lo[t], c0);
-      if (b < a.n_bags && from < min(win.hi[t], c1)) S.mark[from - c0] = (uint32_t)b + 1u;
+      if (b < a.n_bags && from < min(win.hi[t], c1)) S.mark()[from - c0] = (uint32_t)b + 1u;
     }
   } else {
     // last bag that begins at or before the chunk: near where bags of equal length would put it,
@@ -301,7 +329,7 @@ __device__ __forceinline__ void chunk_bags(Smem& S, const ResidentSortArgs& a, c
         const int64_t b = b0 + t * kThreads + tid;
         const int64_t from = max(lo[t], g0);
         past |= lo[t] >= g0 + n_mine;
-        if (b < a.n_bags && from < min(hi[t], g0 + n_mine)) S.mark[from - g0] = (uint32_t)b + 1u;
+        if (b < a.n_bags && from < min(hi[t], g0 + n_mine)) S.mark()[from - g0] = (uint32_t)b + 1u;
       }
       if (__syncthreads_or(past ? 1 : 0)) break;
     }
@@ -311,12 +339,14 @@ __device__ __forceinline__ void chunk_bags(Smem& S, const ResidentSortArgs& a, c
     uint32_t carry = 0;
 #pragma unroll
     for (int i = 0; i < IPT; ++i) {
-      uint32_t x = i * 32 + lane < valid ? S.mark[wbase + i * 32 + lane] : 0u;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) x = max(x, __shfl_up_sync(0xffffffffu, x, o));
-      x = max(x, carry);
-      v[i] = x;
-      carry = __shfl_sync(0xffffffffu, x, 31);
+      if (IPT > 4 && i % 4 == 0 && i * 32 >= valid) break;
+      // marks ascend, so the running maximum is the last mark so far
+      const uint32_t x = i * 32 + lane < valid ? S.mark()[wbase + i * 32 + lane] : 0u;
+      const unsigned marked = __ballot_sync(0xffffffffu, x != 0u), upto = marked & (0xffffffffu >> (31 - lane));
+      const uint32_t own = __shfl_sync(0xffffffffu, x, 31 - __clz(upto | 1u));
+      const uint32_t last = __shfl_sync(0xffffffffu, x, 31 - __clz(marked | 1u));
+      v[i] = upto ? own : carry;
+      carry = marked ? last : carry;
     }
     if (lane == 0) S.warp_tot[wp] = carry;
     __syncthreads();
@@ -324,21 +354,24 @@ __device__ __forceinline__ void chunk_bags(Smem& S, const ResidentSortArgs& a, c
 #pragma unroll
     for (int i = 0; i < kWarps; ++i) pre = max(pre, i < wp ? S.warp_tot[i] : 0u);
 #pragma unroll
-    for (int i = 0; i < IPT; ++i) v[i] = max(v[i], pre) - 1u;
+    for (int i = 0; i < IPT; ++i) {
+      if (IPT > 4 && i % 4 == 0 && i * 32 >= valid) break;
+      v[i] = max(v[i], pre) - 1u;
+    }
   }
 }
 
 // Ranks of the CTA's items among those of equal digit: inside the warp (rk), the prefix over the
-// warps (S.wh), and the CTA's count of every digit, stored to my_row.
+// warps (S.wh), and the CTA's count of every digit, stored to my_row and returned (thread's digit).
 template <int IPT>
-__device__ __forceinline__ void rank_and_publish(Smem& S, const uint32_t (&k)[IPT], int valid, int shift, uint32_t nb,
+__device__ __forceinline__ uint32_t rank_and_publish(Smem& S, const uint32_t (&k)[IPT], int valid, int shift, uint32_t nb,
                                                  uint16_t* my_row, unsigned short (&rk)[IPT]) {
   const int tid = threadIdx.x, wp = tid >> 5;
   __syncthreads();  // marks, counters and bases of the step before have been read
   for (uint32_t i = tid; i < kWarps * nb / 2; i += kThreads) reinterpret_cast<uint32_t*>(S.wh)[i] = 0u;
-  for (uint32_t i = tid; i < kWarps * nb; i += kThreads) S.mm[i] = 0u;
+  for (uint32_t i = tid; i < kWarps * nb; i += kThreads) S.mm()[i] = 0u;
   __syncthreads();
-  warp_rank<IPT>(k, valid, shift, nb - 1u, S.wh + wp * nb, S.mm + wp * nb, rk);
+  warp_rank<IPT>(k, valid, shift, nb - 1u, S.wh + wp * nb, S.mm() + wp * nb, rk);
   __syncthreads();
   uint32_t sum = 0;
   if (tid < nb) {
@@ -352,18 +385,19 @@ __device__ __forceinline__ void rank_and_publish(Smem& S, const uint32_t (&k)[IP
     }
   }
   my_row[tid] = (uint16_t)sum;
+  return sum;
 }
 
 // The passes by row id (the low key_bits of the keys) over the n pairs that C CTAs hold, ce to a CTA.
-// Leaves this CTA with the pairs of its own slots; the pairs of all slots can be read (until the next
-// barrier) in `pairs`, or in the CTAs' S.pairs.  Returns the arrivals on the barrier's counter.
+// Leaves this CTA with the pairs of its own slots in S.stage(), or in S.pairs(); the pairs of all slots can
+// be read in `pairs`, or in the CTAs' S.pairs().  Returns the arrivals on the barrier's counter.
 template <int IPT, bool CLUSTER>
 __device__ __forceinline__ uint32_t sort_passes_by_row(Smem& S, uint32_t (&k)[IPT], uint32_t (&v)[IPT], int key_bits,
                                                        int64_t n, int64_t g0, int n_mine, int ce, int cta, int C,
                                                        uint2* pairs, uint16_t* hist, uint32_t* counter,
                                                        int32_t* status) {
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  const int wbase = wp * 32 * IPT, valid = min(max(n_mine - wbase, 0), 32 * IPT);
+  const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const int per = items_per_thread(ce), wbase = wp * 32 * per, valid = min(max(n_mine - wbase, 0), 32 * per);
   const int P = sort_passes(key_bits);
   uint16_t* const my_row = CLUSTER ? S.row : hist + (size_t)cta * kBins;
   // every CTA of a cluster arrives, but of the others only the C that hold pairs
@@ -373,45 +407,77 @@ __device__ __forceinline__ uint32_t sort_passes_by_row(Smem& S, uint32_t (&k)[IP
     const int bits = (key_bits - shift + (P - p) - 1) / (P - p);
     const uint32_t nb = 1u << bits, dmask = nb - 1u;
     unsigned short rk[IPT];
-    rank_and_publish<IPT>(S, k, valid, shift, nb, my_row, rk);
+    const uint32_t count = rank_and_publish<IPT>(S, k, valid, shift, nb, my_row, rk);
     arrivals += C;
-    all_barrier<CLUSTER>(counter, arrivals, status);
-    digit_bases<CLUSTER>(S, hist, nb, cta, C);
-    __syncthreads();
+    if (CLUSTER) {
+      all_barrier<CLUSTER>(counter, arrivals, status);
+      digit_bases<CLUSTER>(S, hist, nb, cta, C);
+      __syncthreads();
 #pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      if (i * 32 + lane < valid) {
-        const uint32_t d = (k[i] >> shift) & dmask;
-        const uint32_t q = S.base[d] + S.wh[wp * nb + d] + rk[i];
-        if (CLUSTER) {
+      for (int i = 0; i < IPT; ++i) {
+        if (IPT > 4 && i % 4 == 0 && i * 32 >= valid) break;
+        if (i * 32 + lane < valid) {
+          const uint32_t d = (k[i] >> shift) & dmask;
+          const uint32_t q = S.base[d] + S.wh[wp * nb + d] + rk[i];
           const uint32_t c = q / (uint32_t)ce;
-          if (c < (uint32_t)C) st_remote2(remote(S.pairs + (q - c * (uint32_t)ce), c), k[i], v[i]);
-        } else if (q < (uint32_t)n) {
-          __stcg(pairs + q, make_uint2(k[i], v[i]));
+          if (c < (uint32_t)C) st_remote2(remote(S.pairs() + (q - c * (uint32_t)ce), c), k[i], v[i]);
         }
+      }
+    } else {
+      // While the others' counts arrive the pairs are put in the order of their digits in shared
+      // memory, so that consecutive threads store to consecutive slots: a store of a warp touches the
+      // lines of a few digits instead of 32.
+      grid_arrive(counter);
+      const uint32_t loc = block_scan(tid < (int)nb ? count : 0u, S.warp_tot, nullptr);
+      S.loc[tid] = loc;
+      __syncthreads();
+      uint2* const stage = S.stage();
+#pragma unroll
+      for (int i = 0; i < IPT; ++i) {
+        if (IPT > 4 && i % 4 == 0 && i * 32 >= valid) break;
+        if (i * 32 + lane < valid) {
+          const uint32_t d = (k[i] >> shift) & dmask;
+          stage[S.loc[d] + S.wh[wp * nb + d] + rk[i]] = make_uint2(k[i], v[i]);
+        }
+      }
+      grid_wait(counter, arrivals, status);
+      digit_bases<CLUSTER>(S, hist, nb, cta, C);
+      S.base[tid] -= loc;
+      __syncthreads();
+#pragma unroll 4
+      for (int j = tid; j < n_mine; j += kThreads) {
+        const uint2 kv = stage[j];
+        const uint32_t q = S.base[(kv.x >> shift) & dmask] + (uint32_t)j;
+        if (q < (uint32_t)n) __stcg(pairs + q, kv);
       }
     }
     arrivals += C;
     all_barrier<CLUSTER>(counter, arrivals, status);
     shift += bits;
+    if (p + 1 == P) break;
 #pragma unroll
     for (int i = 0; i < IPT; ++i) {
+      if (IPT > 4 && i % 4 == 0 && i * 32 >= valid) break;
       if (i * 32 + lane < valid) {
-        const uint2 kv = CLUSTER ? S.pairs[wbase + i * 32 + lane] : __ldcg(pairs + g0 + wbase + i * 32 + lane);
+        const uint2 kv = CLUSTER ? S.pairs()[wbase + i * 32 + lane] : __ldcg(pairs + g0 + wbase + i * 32 + lane);
         k[i] = kv.x;
         v[i] = kv.y;
       }
     }
   }
+  if (!CLUSTER) {
+#pragma unroll 8
+    for (int j = tid; j < n_mine; j += kThreads) S.stage()[j] = __ldcg(pairs + g0 + j);
+  }
+  __syncthreads();
   return arrivals;
 }
 
-// The pair before this warp's first slot (one lane asks).
+// The pair before the CTA's first slot, g0 > 0 (for the one thread that has the first pair).
 template <bool CLUSTER>
-__device__ __forceinline__ uint2 pair_before(Smem& S, const uint2* pairs, int64_t g0, int wbase, int ce, int cta) {
-  if (!CLUSTER) return __ldcg(pairs + g0 + wbase - 1);
-  if (wbase > 0) return S.pairs[wbase - 1];
-  const uint32_t at = remote(&S.pairs[ce - 1], (uint32_t)cta - 1u);
+__device__ __forceinline__ uint2 pair_before(Smem& S, const uint2* pairs, int64_t g0, int ce, int cta) {
+  if (!CLUSTER) return __ldcg(pairs + g0 - 1);
+  const uint32_t at = remote(&S.pairs()[ce - 1], (uint32_t)cta - 1u);
   return make_uint2(ld_remote(at), ld_remote(at + 4));
 }
 
@@ -428,7 +494,7 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
   const int K = a.n_workers, F = a.bags_per_sample, cta = blockIdx.x, ce = a.chunk;
   const bool merge = m.agg_ids != nullptr;
   const int64_t g0 = (int64_t)cta * ce;
-  const int wbase = wp * 32 * IPT;
+  const int per = items_per_thread(ce), wbase = wp * 32 * per;
 
   // Everything whose address does not depend on the workers' ranges is requested at once: the kernel's
   // beginning is a chain of round trips to memory (backward of 1.2 M occurrences 189 -> 177 us, of 500 k
@@ -436,6 +502,7 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
   uint32_t k[IPT], v[IPT];
 #pragma unroll
   for (int i = 0; i < IPT; ++i) {
+    if (IPT > 4 && i % 4 == 0 && i >= per) break;
     const int64_t g = g0 + wbase + i * 32 + lane;
     k[i] = g < a.nnz ? (uint32_t)__ldg(a.row_ids + g) : 0u;
   }
@@ -453,7 +520,7 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
     }
     if (bad) set_status(a.status, ANTDT_ERR_BAD_OFFSETS);
   }
-  for (int i = tid; i < ce; i += kThreads) S.mark[i] = 0u;
+  for (int i = tid; i < ce; i += kThreads) S.mark()[i] = 0u;
   if (CLUSTER) {  // (otherwise the flag words had to be cleared before the launch anyway)
     for (int64_t i = (int64_t)cta * kThreads + tid; i < a.n_zero; i += (int64_t)gridDim.x * kThreads) a.zero[i] = 0u;
   }
@@ -494,13 +561,14 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
   // A CTA without pairs leaves, but a cluster's CTAs all stay (its barriers count every one).
   if (CLUSTER ? C == 0 : cta >= C) return;
   const int n_mine = (int)max((int64_t)0, min((int64_t)ce, n - g0));
-  const int valid = min(max(n_mine - wbase, 0), 32 * IPT);
+  const int valid = min(max(n_mine - wbase, 0), 32 * per);
   uint32_t* const counter = a.flags;
   {
     bool bad_id = false;
     int w = valid > 0 ? min(interval_of(S.bound, K + 1, g0 + wbase), K - 1) : 0;
 #pragma unroll
     for (int i = 0; i < IPT; ++i) {
+      if (IPT > 4 && i % 4 == 0 && i * 32 >= valid) break;
       uint32_t id = k[i];
       k[i] = 0u;
       v[i] = 0u;
@@ -522,60 +590,69 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
   uint32_t arrivals = sort_passes_by_row<IPT, CLUSTER>(S, k, v, a.key_bits, n, g0, n_mine, ce, cta, C, a.pairs, a.hist,
                                                        counter, a.status);
 
-  // ---- runs of (row, worker) and of rows, in merge order ----
-  const uint32_t row_mask = a.key_bits < 32 ? (1u << a.key_bits) - 1u : 0xffffffffu;
-  uint32_t head_m = 0, row_m = 0;  // bit i: this lane's item i starts a run / a row
-  uint32_t heads_warp = 0, rows_warp = 0;  // of the whole warp
-  {
-    uint32_t left = 0;
-    if (lane == 0 && valid > 0 && g0 + wbase > 0) left = pair_before<CLUSTER>(S, a.pairs, g0, wbase, ce, cta).x;
-#pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      uint32_t prev = __shfl_up_sync(0xffffffffu, k[i], 1);
-      if (lane == 0) prev = left;
-      left = __shfl_sync(0xffffffffu, k[i], 31);
-      const bool in = i * 32 + lane < valid, start = g0 + wbase + i * 32 + lane == 0;
-      const bool h = in && (start || prev != k[i]), r = in && (start || ((prev ^ k[i]) & row_mask) != 0u);
-      head_m |= (h ? 1u : 0u) << i;
-      row_m |= (r ? 1u : 0u) << i;
-      heads_warp += __popc(__ballot_sync(0xffffffffu, h));
-      rows_warp += __popc(__ballot_sync(0xffffffffu, r));
-    }
-  }
-  // ---- by worker: ranks of the pairs and of the runs among those of their worker ----
+  // ---- runs of (row, worker) and of rows in merge order; by worker: ranks of the pairs and of the runs
+  // among those of their worker ----
+  // From here on everything is done once, so its code is short loops over the pairs in shared memory:
+  // unrolled over pairs in registers it waited for its own instructions (1.2 M occurrences of one worker:
+  // ranking by worker 29 k cycles where a second turn took 8 k; backward 167 -> 152 us).
   // counters of this pass: pairs of worker w at w, its runs at Kp + w; published besides: all runs, all rows
+  const uint32_t row_mask = a.key_bits < 32 ? (1u << a.key_bits) - 1u : 0xffffffffu;
   const uint32_t Kp = 1u << a.worker_bits, kB = 2u * Kp;
-  unsigned short rk[IPT], hk[IPT];
-  __syncthreads();
+  const uint2* const kv = CLUSTER ? S.pairs() : S.stage();
+  uint32_t* const ranks = CLUSTER ? S.mm() : reinterpret_cast<uint32_t*>(S.stage() + ce);  // a pair's | its run's << 16
+  uint32_t* const masks = ranks + ce;
+  const unsigned lt = (1u << lane) - 1u;
+  const uint32_t before_cta = tid == 0 && n_mine > 0 && g0 > 0 ? pair_before<CLUSTER>(S, a.pairs, g0, ce, cta).x : 0u;
+  // pair j of this CTA: its key, whether it starts a run, whether it starts a row
+  auto look = [&](int j, bool in, uint32_t& key, bool& head, bool& first) {
+    key = in ? kv[j].x : 0u;
+    const uint32_t prev = in && j > 0 ? kv[j - 1].x : before_cta;
+    head = in && (g0 + j == 0 || prev != key);
+    first = in && (g0 + j == 0 || ((prev ^ key) & row_mask) != 0u);
+  };
+  uint32_t heads_warp = 0, rows_warp = 0;
   for (uint32_t i = tid; i < kWarps * kB / 2; i += kThreads) reinterpret_cast<uint32_t*>(S.wh)[i] = 0u;
-  for (uint32_t i = tid; i < kWarps * kB; i += kThreads) S.mm[i] = 0u;
+  if (K > kMatchWorkers)
+    for (uint32_t i = tid; i < kWarps * kB; i += kThreads) masks[i] = 0u;
   __syncthreads();
   {
-    const unsigned lt = (1u << lane) - 1u;
-    unsigned short* wh = S.wh + wp * kB;
-    uint32_t* mm = S.mm + wp * kB;
-#pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      const bool ok = i * 32 + lane < valid, h = (head_m >> i) & 1u;
-      const uint32_t d = ok ? (uint32_t)((uint64_t)k[i] >> a.key_bits) : 0u;
-      if (ok) atomicOr(mm + d, 1u << lane);
-      const unsigned heads = __ballot_sync(0xffffffffu, h);
+    unsigned short* const wh = S.wh + wp * kB;
+    uint32_t* const mm = masks + wp * kB;
+#pragma unroll 1
+    for (int i = 0; i * 32 < valid; ++i) {
+      const int j = wbase + i * 32 + lane;
+      const bool ok = i * 32 + lane < valid;
+      uint32_t key;
+      bool h, r;
+      look(j, ok, key, h, r);
+      const uint32_t d = (uint32_t)((uint64_t)key >> a.key_bits);
+      const unsigned heads = __ballot_sync(0xffffffffu, h), all = __ballot_sync(0xffffffffu, ok);
+      heads_warp += __popc(heads);
+      rows_warp += __popc(__ballot_sync(0xffffffffu, r));
       unsigned peers = 0;
       uint32_t old = 0, old_h = 0;
+      if (K == 1) {
+        peers = all;
+      } else if (K <= kMatchWorkers) {  // few distinct values: match is the cheaper one, see warp_rank
+        if (ok) peers = __match_any_sync(all, d);
+      } else {
+        if (ok) atomicOr(mm + d, 1u << lane);
+        __syncwarp();
+        if (ok) peers = mm[d];
+      }
       if (ok) {
-        peers = mm[d];
         old = wh[d];
         old_h = wh[Kp + d];
       }
       __syncwarp();
       if (ok && (peers & lt) == 0) {
-        mm[d] = 0u;
+        if (K > kMatchWorkers) mm[d] = 0u;
         wh[d] = (unsigned short)(old + __popc(peers));
         wh[Kp + d] = (unsigned short)(old_h + __popc(peers & heads));
       }
       __syncwarp();
-      rk[i] = (unsigned short)(old + __popc(peers & lt));
-      hk[i] = (unsigned short)(old_h + __popc(peers & heads & lt) + (h ? 1u : 0u));  // runs up to and with this item's
+      // (runs: up to and with this pair's)
+      if (ok) ranks[j] = (old + __popc(peers & lt)) | (old_h + __popc(peers & heads & lt) + (h ? 1u : 0u)) << 16;
     }
   }
   if (lane == 0) { S.warp_a[wp] = heads_warp; S.warp_b[wp] = rows_warp; }
@@ -630,20 +707,24 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
   }
   uint32_t mrun = S.base[kB] + heads_pre, mrow = S.base[kB + 1] + rows_pre;  // runs / rows before the warp
   const uint32_t tile_mask = (1u << a.tile_shift) - 1u;
-  const unsigned lt = (1u << lane) - 1u;
-#pragma unroll
-  for (int i = 0; i < IPT; ++i) {
-    const bool in = i * 32 + lane < valid, h = (head_m >> i) & 1u, r = (row_m >> i) & 1u;
+#pragma unroll 1
+  for (int i = 0; i * 32 < valid; ++i) {
+    const int j = wbase + i * 32 + lane;
+    const bool in = i * 32 + lane < valid;
+    uint32_t key;
+    bool h, r;
+    look(j, in, key, h, r);
     const unsigned hb = __ballot_sync(0xffffffffu, h), rb = __ballot_sync(0xffffffffu, r);
     if (in) {
-      const uint32_t w = (uint32_t)((uint64_t)k[i] >> a.key_bits), row = k[i] & row_mask;
-      const uint32_t q = S.base[w] + S.wh[wp * kB + w] + rk[i];
-      const uint32_t u = S.base[Kp + w] + S.wh[wp * kB + Kp + w] + hk[i] - 1u;  // this item's run in its worker's list
+      const uint32_t w = (uint32_t)((uint64_t)key >> a.key_bits), row = key & row_mask, rank = ranks[j];
+      const uint32_t q = S.base[w] + S.wh[wp * kB + w] + (rank & 0xffffu);
+      const uint32_t u = S.base[Kp + w] + S.wh[wp * kB + Kp + w] + (rank >> 16) - 1u;  // its run in its worker's list
       if (q < (uint32_t)n) {
-        a.sorted_occ[q] = v[i];
+        a.sorted_occ[q] = kv[j].y;
         if ((q & tile_mask) == 0) a.tile_first[q >> a.tile_shift] = (int32_t)u;
+        if (K == 1 && lane == 0) a.head_bits[q >> 5] = hb;  // q is the place in the row order: a whole word
         if (h) {
-          atomicOr(a.head_bits + (q >> 5), 1u << (q & 31));
+          if (K > 1) atomicOr(a.head_bits + (q >> 5), 1u << (q & 31));
           const uint32_t slot = mrun + __popc(hb & lt);
           if (u < a.out_cap) {
             a.uniq_ids[u] = (int32_t)row;
@@ -684,10 +765,11 @@ resident_merge_kernel(const __grid_constant__ ResidentMergeArgs a) {
   if (CLUSTER)
     for (int64_t i = (int64_t)cta * kThreads + tid; i < a.n_zero; i += (int64_t)gridDim.x * kThreads) a.zero[i] = 0u;
   const int64_t g0 = (int64_t)cta * ce;
-  const int wbase = wp * 32 * IPT;
+  const int per = items_per_thread(ce), wbase = wp * 32 * per;
   uint32_t k[IPT], v[IPT];
 #pragma unroll
   for (int i = 0; i < IPT; ++i) {  // on their way while the bounds are read (past the lists' end: not used)
+    if (IPT > 4 && i % 4 == 0 && i >= per) break;
     const int64_t g = g0 + wbase + i * 32 + lane;
     k[i] = g < a.in_cap ? (uint32_t)__ldg(a.uniq_ids + g) : 0u;
   }
@@ -717,12 +799,13 @@ resident_merge_kernel(const __grid_constant__ ResidentMergeArgs a) {
   }
   if (CLUSTER ? C == 0 : cta >= C) return;
   const int n_mine = (int)max((int64_t)0, min((int64_t)ce, n - g0));
-  const int valid = min(max(n_mine - wbase, 0), 32 * IPT);
+  const int valid = min(max(n_mine - wbase, 0), 32 * per);
   {
     bool bad_id = false;
     int w = 0;
 #pragma unroll
     for (int i = 0; i < IPT; ++i) {
+      if (IPT > 4 && i % 4 == 0 && i * 32 >= valid) break;
       const uint32_t id = k[i];
       k[i] = 0u;
       v[i] = 0u;
@@ -741,21 +824,20 @@ resident_merge_kernel(const __grid_constant__ ResidentMergeArgs a) {
   uint32_t arrivals = sort_passes_by_row<IPT, CLUSTER>(S, k, v, a.key_bits, n, g0, n_mine, ce, cta, C, a.pairs, a.hist,
                                                        a.flags, a.status);
   // ---- rows; entries that count ----
-  uint32_t row_m = 0, rows_warp = 0, kept_warp = 0;
+  const uint2* const kv = CLUSTER ? S.pairs() : S.stage();  // short loops, as in the sort
+  const uint2 before_cta = tid == 0 && n_mine > 0 && g0 > 0 ? pair_before<CLUSTER>(S, a.pairs, g0, ce, cta)
+                                                            : make_uint2(0u, 0u);
+  uint32_t rows_warp = 0, kept_warp = 0;
   {
-    uint2 left = make_uint2(0u, 0u);
-    if (lane == 0 && valid > 0 && g0 + wbase > 0) left = pair_before<CLUSTER>(S, a.pairs, g0, wbase, ce, cta);
     bool repeats = false;
-#pragma unroll
-    for (int i = 0; i < IPT; ++i) {
-      uint32_t pk = __shfl_up_sync(0xffffffffu, k[i], 1), pv = __shfl_up_sync(0xffffffffu, v[i], 1);
-      if (lane == 0) { pk = left.x; pv = left.y; }
-      left = make_uint2(__shfl_sync(0xffffffffu, k[i], 31), __shfl_sync(0xffffffffu, v[i], 31));
-      const bool in = i * 32 + lane < valid && k[i] < (uint32_t)a.n_rows;
-      const bool start = g0 + wbase + i * 32 + lane == 0, r = in && (start || pk != k[i]);
+#pragma unroll 1
+    for (int i = 0; i * 32 < valid; ++i) {
+      const int j = wbase + i * 32 + lane;
+      const bool ok = i * 32 + lane < valid;
+      const uint2 x = ok ? kv[j] : make_uint2(0u, 0u), p = ok && j > 0 ? kv[j - 1] : before_cta;
+      const bool in = ok && x.x < (uint32_t)a.n_rows, r = in && (g0 + j == 0 || p.x != x.x);
       // the same row twice in one worker's list
-      if (in && !r) repeats |= interval_of(S.bound, K + 1, pv) == interval_of(S.bound, K + 1, v[i]);
-      row_m |= (r ? 1u : 0u) << i;
+      if (in && !r) repeats |= interval_of(S.bound, K + 1, p.y) == interval_of(S.bound, K + 1, x.y);
       rows_warp += __popc(__ballot_sync(0xffffffffu, r));
       kept_warp += __popc(__ballot_sync(0xffffffffu, in));
     }
@@ -791,17 +873,21 @@ resident_merge_kernel(const __grid_constant__ ResidentMergeArgs a) {
   uint32_t mrow = S.base[1] + rows_pre;  // rows before the warp
   const uint32_t tile_mask = (1u << a.tile_shift) - 1u;
   const unsigned le = 0xffffffffu >> (31 - lane);
-#pragma unroll
-  for (int i = 0; i < IPT; ++i) {
-    const bool r = (row_m >> i) & 1u;
+#pragma unroll 1
+  for (int i = 0; i * 32 < valid; ++i) {
+    const int j = wbase + i * 32 + lane;
+    const bool ok = i * 32 + lane < valid;
+    const uint2 e = ok ? kv[j] : make_uint2(0u, 0u);
+    const uint32_t prev = ok && j > 0 ? kv[j - 1].x : before_cta.x;
+    const bool in = ok && e.x < (uint32_t)a.n_rows, r = in && (g0 + j == 0 || prev != e.x);
     const unsigned rb = __ballot_sync(0xffffffffu, r);
-    if (i * 32 + lane < valid && k[i] < (uint32_t)a.n_rows) {
-      const uint32_t slot = (uint32_t)(g0 + wbase + i * 32 + lane);
+    if (in) {
+      const uint32_t slot = (uint32_t)(g0 + j);
       const uint32_t x = mrow + __popc(rb & le) - 1u;  // index of this entry's row
-      a.src[slot] = v[i];
-      if (a.src_worker) a.src_worker[slot] = (uint8_t)min(interval_of(S.bound, K + 1, v[i]), K - 1);
+      a.src[slot] = e.y;
+      if (a.src_worker) a.src_worker[slot] = (uint8_t)min(interval_of(S.bound, K + 1, e.y), K - 1);
       if (r) {
-        if (x < a.out_cap) a.agg_ids[x] = (int32_t)k[i];
+        if (x < a.out_cap) a.agg_ids[x] = (int32_t)e.x;
         if (a.row_start && x <= a.out_cap) a.row_start[x] = slot;  // one more than rows: it ends the last one
         if (a.head_bits) atomicOr(a.head_bits + (slot >> 5), 1u << (slot & 31));
       }
@@ -816,7 +902,7 @@ resident_merge_kernel(const __grid_constant__ ResidentMergeArgs a) {
 struct Form { int ctas, chunk; bool cluster; };
 #define RESIDENT_DISPATCH(GO)                                   \
   do {                                                          \
-    const int ipt = (f.chunk + kThreads - 1) / kThreads;        \
+    const int ipt = items_per_thread(f.chunk);                  \
     if (f.cluster && ipt <= 2) GO(2, true);                     \
     if (f.cluster) GO(4, true);                                 \
     if (ipt <= 4) GO(4, false);                                 \
@@ -843,7 +929,7 @@ int32_t launch_one(const char* name, cudaEvent_t started, void (*kernel)(P...), 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)f.ctas);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = sizeof(Smem);
+  cfg.dynamicSmemBytes = smem_bytes(f.chunk, f.cluster);
   cfg.stream = s;
   cudaLaunchAttribute at[3];
   if (f.cluster) {
@@ -877,13 +963,14 @@ void resident_sort_prepare_device() {
   int dev = 0;
   cudaGetDevice(&dev);
   if (done[dev & 63]) return;
-  auto opt_in = [](auto* k, bool cluster) {
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
+  auto opt_in = [](auto* k, int items, bool cluster) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem_bytes(items * kThreads, cluster));
     if (cluster) cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   };
 #define OPT_IN(IPT, CLUSTER)                            \
-  opt_in(resident_sort_kernel<IPT, CLUSTER>, CLUSTER);  \
-  opt_in(resident_merge_kernel<IPT, CLUSTER>, CLUSTER)
+  opt_in(resident_sort_kernel<IPT, CLUSTER>, IPT, CLUSTER);  \
+  opt_in(resident_merge_kernel<IPT, CLUSTER>, IPT, CLUSTER)
   OPT_IN(2, true);
   OPT_IN(4, true);
   OPT_IN(4, false);

@@ -62,3 +62,14 @@ def test_the_largest_input_and_the_one_after_it(extra):
     lens = np.full(n // 8, 8, np.int64)
     lens[0] += n - lens.sum()
     _check(lens, [0, len(lens) // 3, len(lens)], 1, 40_000, 4, rng, hot=0.05)
+
+
+@pytest.mark.parametrize("K,n", [(1, 148 * 512 * 24), (8, 148 * 512 * 17 + 31), (9, 148 * 512 * 9 - 33), (2, 148 * 512 * 4 + 1)])
+def test_shares_of_the_warps_and_ways_to_rank_by_worker(K, n):
+    rng = np.random.default_rng(n)
+    lens = rng.integers(0, 5, size=n // 2)
+    lens[-1] += max(0, n - lens.sum())
+    lens[np.cumsum(lens) > n] = 0
+    lens[0] += n - lens.sum()
+    cuts = np.sort(rng.integers(0, len(lens) + 1, size=K - 1))
+    _check(lens, np.concatenate([[0], cuts, [len(lens)]]), 1, 300_000, 4, rng, hot=0.1)
