@@ -366,10 +366,13 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
       }
     }
   }
-  // A small input's few tasks are done by the CTA that ends last, instead of by another launch.
+  // A small input's few tasks are done by the CTA that ends last, instead of by another launch.  A CTA
+  // counts itself as ended behind a barrier: its partials, flags and tasks come from several warps.
   if (TILE == kRedTileSmall && ws.inline_fixup) {
     __threadfence();
-    if (__syncthreads_or(threadIdx.x == 0 && atomicAdd(ws.tasks + 1, 1) == (int)gridDim.x - 1)) {
+    __syncthreads();
+    const bool last_cta = threadIdx.x == 0 && atomicAdd(ws.tasks + 1, 1) == (int)gridDim.x - 1;
+    if (__syncthreads_or(last_cta ? 1 : 0)) {
       __threadfence();
       fixup_tasks<G, VPL, TILE>(a, ws, 0, 1);
     }
