@@ -1,0 +1,20 @@
+// Index arithmetic of the kernels that must stay in bounds whatever memory holds, and up to the limits
+// of what the entry points accept.  Plain C++ as well, so that its edges are tested on the host.
+#pragma once
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define ANTDT_HD __host__ __device__ __forceinline__
+#else
+#define ANTDT_HD inline
+#endif
+
+namespace antdt {
+
+// Worker of a resident-sort key (worker << key_bits | row id).  Below 2^worker_bits for every key: after
+// a wait that ran out a CTA can read slots that nobody has written, and indexes its tables by this.
+ANTDT_HD uint32_t key_worker(uint32_t key, int key_bits, int worker_bits) {
+  return (uint32_t)((uint64_t)key >> key_bits) & ((1u << worker_bits) - 1u);
+}
+
+}  // namespace antdt

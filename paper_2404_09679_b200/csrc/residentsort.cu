@@ -29,8 +29,12 @@
 // 1.2 M of one worker over 1 M 74 us (113).
 //
 // The CTAs wait for one another, so the launch is a cluster or a cooperative one (all CTAs resident
-// or none started).  Every wait through memory is bounded all the same (kSpinLimit) and raises
-// ANTDT_ERR_TIMEOUT when it runs out; slots are checked, so even then nothing is written elsewhere.
+// or none started).  A wait through memory is bounded all the same (kSpinLimit) and raises
+// ANTDT_ERR_TIMEOUT when it runs out.  What a CTA reads then may be anything, so every index that comes
+// out of memory is masked or checked: digits and workers by their masks, slots, runs and rows by the
+// lengths of the arrays.  A cluster's barrier is the hardware's, without a limit; every CTA of the
+// cluster arrives at each of them.
+#include "index_math.cuh"
 #include "residentsort.cuh"
 
 namespace antdt {
@@ -625,7 +629,7 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
       uint32_t key;
       bool h, r;
       look(j, ok, key, h, r);
-      const uint32_t d = (uint32_t)((uint64_t)key >> a.key_bits);
+      const uint32_t d = key_worker(key, a.key_bits, a.worker_bits);
       const unsigned heads = __ballot_sync(0xffffffffu, h), all = __ballot_sync(0xffffffffu, ok);
       heads_warp += __popc(heads);
       rows_warp += __popc(__ballot_sync(0xffffffffu, r));
@@ -716,7 +720,7 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
     look(j, in, key, h, r);
     const unsigned hb = __ballot_sync(0xffffffffu, h), rb = __ballot_sync(0xffffffffu, r);
     if (in) {
-      const uint32_t w = (uint32_t)((uint64_t)key >> a.key_bits), row = key & row_mask, rank = ranks[j];
+      const uint32_t w = key_worker(key, a.key_bits, a.worker_bits), row = key & row_mask, rank = ranks[j];
       const uint32_t q = S.base[w] + S.wh[wp * kB + w] + (rank & 0xffffu);
       const uint32_t u = S.base[Kp + w] + S.wh[wp * kB + Kp + w] + (rank >> 16) - 1u;  // its run in its worker's list
       if (q < (uint32_t)n) {

@@ -1,0 +1,41 @@
+"""Index arithmetic shared by the kernels (csrc/index_math.cuh), compiled for the host: values that stale
+memory can hold and sizes at the limit of what the entry points accept."""
+import ctypes as C
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2404_09679_b200", "csrc")
+PROBE = r"""
+#include "index_math.cuh"
+using namespace antdt;
+extern "C" void key_workers(const uint32_t* key, int n, int key_bits, int worker_bits, uint32_t* out) {
+  for (int i = 0; i < n; ++i) out[i] = key_worker(key[i], key_bits, worker_bits);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("index_math")
+    src, so = str(d / "probe.cpp"), str(d / "probe.so")
+    open(src, "w").write(PROBE)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-fsanitize=undefined", "-fno-sanitize-recover",
+                    "-static-libubsan", "-fPIC", "-shared", "-I", CSRC, src, "-o", so], check=True)
+    return C.CDLL(so)
+
+
+@pytest.mark.parametrize("key_bits,worker_bits", [(1, 5), (17, 5), (27, 5), (31, 5), (24, 7), (25, 7)])
+def test_worker_of_any_key_is_an_index_into_the_worker_tables(lib, key_bits, worker_bits):
+    keys = np.concatenate([np.random.default_rng(0).integers(0, 1 << 32, size=1000, dtype=np.uint64),
+                           [0, 1, (1 << 32) - 1, 1 << 31]]).astype(np.uint32)
+    out = np.zeros_like(keys)
+    lib.key_workers(C.c_void_p(keys.ctypes.data), keys.size, key_bits, worker_bits, C.c_void_p(out.ctypes.data))
+    assert out.max() < 1 << worker_bits
+    w = np.arange(min(1 << worker_bits, 1 << (32 - key_bits)), dtype=np.uint64)      # and it is the worker of a good key
+    good = (w << np.uint64(key_bits) | np.uint64((1 << key_bits) - 1)).astype(np.uint32)
+    out = np.zeros_like(good)
+    lib.key_workers(C.c_void_p(good.ctypes.data), good.size, key_bits, worker_bits, C.c_void_p(out.ctypes.data))
+    assert np.array_equal(out, w)
