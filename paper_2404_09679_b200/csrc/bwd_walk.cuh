@@ -199,7 +199,7 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
       started = (heads & 1ull) != 0;
     }
     if (last_tile) ends = (ends & ((1ull << (nv - 1)) - 1ull)) | (1ull << (nv - 1));  // array end closes
-    u = tile_first[tile];
+    u = run_index(tile_first[tile], o_begin);
     w = interval_of(s_bounds, K + 1, o_begin);
     if (w > K - 1) w = K - 1;
   }

@@ -17,4 +17,12 @@ ANTDT_HD uint32_t key_worker(uint32_t key, int key_bits, int worker_bits) {
   return (uint32_t)((uint64_t)key >> key_bits) & ((1u << worker_bits) - 1u);
 }
 
+// Run index with which a reduction tile that begins at entry o_begin goes on (first: what the sort left in
+// tile_first).  Nobody writes it for tiles behind the last sorted entry, which exist when the offsets are bad:
+// at most one run starts per entry, so a value above o_begin (a negative one too) is not one, and the
+// indices that follow it inside the tile stay below 2^31.
+ANTDT_HD int32_t run_index(int32_t first, int64_t o_begin) {
+  return (uint32_t)first < (uint32_t)o_begin ? first : (int32_t)o_begin;
+}
+
 }  // namespace antdt

@@ -16,6 +16,7 @@
 // offsets, done once per lane and broadcast).
 #pragma once
 #include "common.cuh"
+#include "index_math.cuh"
 
 namespace antdt {
 
@@ -110,7 +111,7 @@ tile_reduce_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
   }
   if (last_tile) ends = (ends & ((1ull << (nv - 1)) - 1ull)) | (1ull << (nv - 1));  // array end closes
 
-  int64_t u = tile_first[tile];
+  int64_t u = run_index(tile_first[tile], o_begin);
   float4 acc[VPL];
 #pragma unroll
   for (int k = 0; k < VPL; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -216,7 +217,7 @@ tile_fixup_kernel(const TileArgs a) {
   const uint64_t cur = tile_heads<TILE>(a.head_bits, o_begin);
   const uint64_t nxt_heads = tile_heads<TILE>(a.head_bits, o_end);
   const bool after = head_at(a.head_bits, o_end + TILE);
-  const int32_t first_run = __ldg(a.tile_first + tile);
+  const int32_t first_run = run_index(__ldg(a.tile_first + tile), o_begin);
   float4 tot[VPL], nxt[VPL];
 #pragma unroll
   for (int k = 0; k < VPL; ++k) {

@@ -14,6 +14,7 @@ using namespace antdt;
 extern "C" void key_workers(const uint32_t* key, int n, int key_bits, int worker_bits, uint32_t* out) {
   for (int i = 0; i < n; ++i) out[i] = key_worker(key[i], key_bits, worker_bits);
 }
+extern "C" int32_t run_index_of(int32_t first, int64_t o_begin) { return run_index(first, o_begin); }
 """
 
 
@@ -39,3 +40,12 @@ def test_worker_of_any_key_is_an_index_into_the_worker_tables(lib, key_bits, wor
     out = np.zeros_like(good)
     lib.key_workers(C.c_void_p(good.ctypes.data), good.size, key_bits, worker_bits, C.c_void_p(out.ctypes.data))
     assert np.array_equal(out, w)
+
+
+@pytest.mark.parametrize("o_begin", [0, 16, 64, 4096, (1 << 31) - 64])
+def test_run_index_of_a_tile_is_never_outside_what_precedes_it(lib, o_begin):
+    f = lambda first: lib.run_index_of(C.c_int32(first), C.c_int64(o_begin))  # noqa: E731
+    for good in {0, o_begin // 2, o_begin}:
+        assert f(good) == good
+    for stale in (-1, -(1 << 31), -2, (1 << 31) - 1, o_begin + 1):
+        assert 0 <= f(stale) <= o_begin
