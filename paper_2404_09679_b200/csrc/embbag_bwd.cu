@@ -13,6 +13,7 @@
 // sorted occurrences whatever rows they belong to, so a row that holds 20% of a field's
 // occurrences costs its tiles no more than anyone else's.  Every sum has a fixed order (inside a
 // tile by sorted position, across tiles by tile index), no floating-point atomics anywhere.
+#include "index_math.cuh"
 #include "residentsort.cuh"
 #include "segsort.cuh"
 #include "bwd_walk.cuh"
@@ -110,35 +111,36 @@ expand_bags_kernel(const int64_t* __restrict__ bag_offsets, int64_t n_bags, int6
       continue;
     }
     const int64_t first = __shfl_sync(0xffffffffu, lo, 0);
-    const int span = (int)(next - first);  // < 2^31: offsets lie in [0, nnz]
-    const int my_end = (int)(hi - first);  // ascending over the lanes
-    // the group's range starts this far into an aligned group of four
-    const int skew = (int)(((reinterpret_cast<uintptr_t>(occ_bag) >> 2) + (uint64_t)first) & 3);
-    for (int base = -skew; base < span; base += 128) {
-      const int o = base + 4 * lane;
-      int l = 0;  // first lane whose end is > max(o, 0)
+    // the group's range starts this far into an aligned group of four; slots are counted from there
+    const uint32_t skew = (uint32_t)(((reinterpret_cast<uintptr_t>(occ_bag) >> 2) + (uint64_t)first) & 3);
+    const BagSpan span((uint32_t)(next - first), skew);         // offsets lie in [0, nnz]
+    const uint32_t my_end = (uint32_t)(hi - first) + span.skew;  // ascending over the lanes
+    uint32_t* const out = occ_bag + (first - (int64_t)skew);     // slot 0, on the 16-byte grid
+    for (uint32_t base = 0; base < span.total; base += kSpanTurn) {
+      const uint32_t x = base + 4 * lane;
+      int l = 0;  // first lane whose end is > max(x, skew)
 #pragma unroll
       for (int step = 16; step > 0; step >>= 1) {
-        const int e = __shfl_sync(0xffffffffu, my_end, l + step - 1);
-        if (e <= max(o, 0)) l += step;
+        const uint32_t e = __shfl_sync(0xffffffffu, my_end, l + step - 1);
+        if (e <= max(x, span.skew)) l += step;
       }
       uint32_t q[4];
-      int end = __shfl_sync(0xffffffffu, my_end, l & 31);
+      uint32_t end = __shfl_sync(0xffffffffu, my_end, l & 31);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        // on to the bag that holds o + j (empty bags are stepped over; the vote keeps the lanes together)
-        while (__any_sync(0xffffffffu, o + j >= end && l < 31)) {
-          if (o + j >= end && l < 31) ++l;
+        // on to the bag that holds x + j (empty bags are stepped over; the vote keeps the lanes together)
+        while (__any_sync(0xffffffffu, x + j >= end && l < 31)) {
+          if (x + j >= end && l < 31) ++l;
           end = __shfl_sync(0xffffffffu, my_end, l & 31);
         }
         q[j] = (uint32_t)min(b0 + l, n_bags - 1);
       }
-      if (o >= 0 && o + 4 <= span) {
-        *reinterpret_cast<uint4*>(occ_bag + first + o) = make_uint4(q[0], q[1], q[2], q[3]);
+      if (span.whole(x)) {
+        *reinterpret_cast<uint4*>(out + x) = make_uint4(q[0], q[1], q[2], q[3]);
       } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (o + j >= 0 && o + j < span) occ_bag[first + o + j] = q[j];
+          if (span.holds(x + j)) out[x + j] = q[j];
       }
     }
   }

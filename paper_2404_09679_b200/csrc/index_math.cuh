@@ -25,4 +25,15 @@ ANTDT_HD int32_t run_index(int32_t first, int64_t o_begin) {
   return (uint32_t)first < (uint32_t)o_begin ? first : (int32_t)o_begin;
 }
 
+// The slots that a group of bags fills: span of them (fewer than 2^31), skew (0 to 3) behind the start of an
+// aligned group of four.  Slots are counted from there in unsigned 32 bits, four to a lane and 128 to a
+// turn: the turn after the last slot of an array of 2^31 - 1 occurrences does not wrap.
+constexpr uint32_t kSpanTurn = 128;
+struct BagSpan {
+  uint32_t skew, total;  // slots skew .. total - 1 are the group's
+  ANTDT_HD BagSpan(uint32_t span, uint32_t skew_) : skew(skew_), total(span + skew_) {}
+  ANTDT_HD bool holds(uint32_t x) const { return x >= skew && x < total; }
+  ANTDT_HD bool whole(uint32_t x) const { return x >= skew && x + 4 <= total; }  // x .. x + 3
+};
+
 }  // namespace antdt

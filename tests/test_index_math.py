@@ -15,6 +15,17 @@ extern "C" void key_workers(const uint32_t* key, int n, int key_bits, int worker
   for (int i = 0; i < n; ++i) out[i] = key_worker(key[i], key_bits, worker_bits);
 }
 extern "C" int32_t run_index_of(int32_t first, int64_t o_begin) { return run_index(first, o_begin); }
+// slots that the turns of a group cover (a turn inside the group by its first and last lane); -1: the turns do not end
+extern "C" int64_t covered(uint32_t span, uint32_t skew) {
+  const BagSpan s(span, skew);
+  int64_t n = 0, turns = 0;
+  for (uint32_t base = 0; base < s.total; base += kSpanTurn) {
+    if (++turns > (1ll << 24) + 1) return -1;
+    if (s.whole(base) && s.whole(base + kSpanTurn - 4)) { n += kSpanTurn; continue; }
+    for (uint32_t x = base; x < base + kSpanTurn; ++x) n += s.holds(x);
+  }
+  return n;
+}
 """
 
 
@@ -49,3 +60,11 @@ def test_run_index_of_a_tile_is_never_outside_what_precedes_it(lib, o_begin):
         assert f(good) == good
     for stale in (-1, -(1 << 31), -2, (1 << 31) - 1, o_begin + 1):
         assert 0 <= f(stale) <= o_begin
+
+
+@pytest.mark.parametrize("skew", [0, 1, 2, 3])
+def test_turns_of_a_group_of_bags_cover_its_slots_once(lib, skew):
+    lib.covered.restype = C.c_int64
+    for span in [0, 1, 2, 3, 4, 5, 124, 125, 127, 128, 129, 1000, (1 << 31) - 129, (1 << 31) - 128, (1 << 31) - 4,
+                 (1 << 31) - 1]:
+        assert lib.covered(C.c_uint32(span), C.c_uint32(skew)) == span
