@@ -366,7 +366,8 @@ int32_t antdt_dense_opt_update(float* params, const float* grad, int64_t n, int3
 /* One whole step from HOST buffers: copies the step's inputs to the caller's device staging
  * buffers, runs fwd, bwd_dedup, aggregate and update in order on `stream`, and copies the
  * results (pooled, dense_out, n_agg, status) back.  The copies run on two internal side
- * streams (created on the first call on a device) so that they overlap the kernels; `stream`
+ * streams (created on the first call on a device, shared by all host-buffer steps of that device:
+ * their copies run in the order of the calls) so that they overlap the kernels; `stream`
  * waits for all of them before the call's work on it ends, so synchronising `stream` (or an
  * event recorded on it after the call) is enough.  Host buffers should be page-locked for the
  * copies to overlap.  Every pointer of the descriptor is described beside its field.
@@ -447,10 +448,14 @@ int32_t antdt_bsp_step_device(const antdt_step_desc* d, void* stream);
  *     occurrences, fuse_update).  No kernel fills the device there, so the step time is the length
  *     of the dependency chain.  The results are those of the one-chain step.  Room means ws_bytes
  *     >= antdt_bsp_step_workspace_bytes(...): the aggregation's scratch then sits behind the
- *     backward's instead of on top of it.  The branches use two library-owned side streams.
- *     antdt_bsp_step_device uses one of them too, for the forward of a batch that the backward
- *     sorts in one kernel, and a third carries a large dense part beside the sort or the merge;
- *     the caller's stream waits for all of them.
+ *     backward's instead of on top of it.
+ *   - Side streams.  The branches of a capture are streams of the library that join it until it
+ *     ends.  antdt_bsp_step_device uses such streams too, for the forward of a batch that the
+ *     backward sorts in one kernel and for a large dense part beside the sort or the merge (as does
+ *     antdt_weighted_aggregate); the caller's stream waits for all of them.  They are created on
+ *     first use, up to 16 per device.  A call takes only streams that no other caller's work is on,
+ *     and does without (everything in order on `stream`) where there are none: steps on different
+ *     streams of a device do not wait for each other.
  * Returns ANTDT_OK, an argument error, or ANTDT_ERR_CUDA. */
 int32_t antdt_bsp_step_graph(const antdt_step_desc* d, void* stream);
 /* Workspace of a step: the larger of the backward's and the aggregation's figures; their sum
@@ -458,7 +463,7 @@ int32_t antdt_bsp_step_graph(const antdt_step_desc* d, void* stream);
  * 0 for arguments either figure rejects. */
 size_t antdt_bsp_step_workspace_bytes(int64_t nnz, int64_t n_bags, int32_t dim, int32_t n_workers,
                                       int64_t uniq_cap);
-/* Destroys the executable graphs kept for the current device. */
+/* Destroys the executable graphs and the idle side streams kept for the current device. */
 int32_t antdt_bsp_step_graph_reset(void);
 
 /* ---- helpers ------------------------------------------------------------------------ */

@@ -11,8 +11,6 @@
 // forward-moving streams, not a random walk.
 // Dense part: a K-way streaming reduction, one 16-byte vector per thread and worker; a large one
 // beside a sort or a merge order takes a kernel that fits between their CTAs (dense_wsum_bulk_kernel).
-#include <mutex>
-
 #include "agg_range.cuh"
 #include "opt_math.cuh"
 #include "residentsort.cuh"
@@ -471,35 +469,8 @@ extern "C" size_t antdt_weighted_aggregate_workspace_bytes(int64_t in_cap, int32
 
 namespace antdt {
 namespace {
-// Side stream of the dense part, created on first use for each device.  An event's wait must follow
-// its record with no other call's record in between, so a call holds `mu` while it is issued.
-struct DenseSide {
-  std::mutex mu;
-  bool ready = false;
-  cudaStream_t stream = nullptr;
-  cudaEvent_t start = nullptr, done = nullptr;
-};
-DenseSide* dense_side(cudaStream_t s) {
-  static DenseSide sides[64];
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
-  DenseSide& d = sides[dev];
-  std::lock_guard<std::mutex> lk(d.mu);
-  if (!d.ready) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;  // nothing is created during a capture
-    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
-        cudaStreamCreateWithFlags(&d.stream, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&d.start, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&d.done, cudaEventDisableTiming) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    d.ready = true;
-  }
-  return &d;
-}
-
 constexpr int64_t kDenseBesideBytes = 8 << 20;  // below, the fork and join cost what they hide
+enum { kDenseStart = 0, kDenseDone = 1 };  // events of the dense part's side set
 constexpr int kBulkSmem = 4 * kBulkSlots * kBulkGroup * kBulkElems;
 
 bool dense_valid(const antdt_dense_part& d) {
@@ -715,7 +686,7 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
 }
 }  // namespace
 
-void aggregate_prepare_device(cudaStream_t s) {
+void aggregate_prepare_device() {
   static bool done[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
@@ -723,7 +694,6 @@ void aggregate_prepare_device(cudaStream_t s) {
     cudaFuncSetAttribute(dense_wsum_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBulkSmem);
     done[dev & 63] = true;
   }
-  dense_side(s);
 }
 
 // 2.2 GB (32 workers x 16.8 M) beside the sort of 35 M occurrences: 1.19 ms instead of 0.34 alone, the
@@ -736,31 +706,27 @@ DenseBeside::DenseBeside(const antdt_dense_part* dp, const int64_t* batch_sizes,
     return;
   float hw[kDenseBlobWorkers];
   if (!worker_weights(batch_sizes, dropped, K, hw)) return;
-  aggregate_prepare_device(s);
-  DenseSide* d = dense_side(s);
-  if (!d) return;
-  lk_ = std::unique_lock<std::mutex>(d->mu);
-  if (cudaEventRecord(d->start, s) != cudaSuccess || cudaStreamWaitEvent(d->stream, d->start, 0) != cudaSuccess) {
+  aggregate_prepare_device();
+  if (!side_.take(s)) return;
+  if (cudaEventRecord(side_->event[kDenseStart], s) != cudaSuccess ||
+      cudaStreamWaitEvent(side_->stream[0], side_->event[kDenseStart], 0) != cudaSuccess) {
     cudaGetLastError();
-    lk_.unlock();
+    side_.release();
     return;
   }
   DenseWeights blob = {};
   for (int i = 0; i < K; ++i) blob.w[i] = hw[i];
   const int64_t tiles = (dp->n + kBulkElems - 1) / kBulkElems;
   ANTDT_LAUNCH("dense_wsum", dense_wsum_bulk_kernel, (unsigned)(tiles < kNumSM ? tiles : kNumSM), kBulkThreads,
-               kBulkSmem, d->stream, dp->grads, (uint32_t)dp->n, dp->stride, blob, K, dp->out, dev_status);
+               kBulkSmem, side_->stream[0], dp->grads, (uint32_t)dp->n, dp->stride, blob, K, dp->out, dev_status);
   issued_ = true;
-  side_ = d->stream;
-  done_ = d->done;
 }
 
 void DenseBeside::join() {
   if (!side_) return;
-  cudaEventRecord(done_, side_);
-  cudaStreamWaitEvent(main_, done_, 0);
-  side_ = nullptr;
-  lk_.unlock();
+  cudaEventRecord(side_->event[kDenseDone], side_->stream[0]);
+  cudaStreamWaitEvent(main_, side_->event[kDenseDone], 0);
+  side_.release();
 }
 
 int32_t weighted_aggregate_forked(const antdt_sparse_part* sp, const antdt_dense_part* dp,

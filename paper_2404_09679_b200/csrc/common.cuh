@@ -5,9 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <mutex>
-
 #include "antdt.h"
+#include "side_streams.cuh"
 
 namespace antdt {
 
@@ -123,12 +122,12 @@ int32_t aggregate_update_forked(const antdt_sparse_part* sp, const antdt_dense_p
                                 const OrderFork* fork, bool merged = false);  // aggregate.cu
 // (merged: the merge order is in the workspace already)
 
-// aggregate.cu: the side stream and kernel attributes of the dense part; before a capture of s.
-void aggregate_prepare_device(cudaStream_t s);
+// aggregate.cu: kernel attributes of the dense part; before a capture.
+void aggregate_prepare_device();
 // The aggregation's dense part on a side stream, beside what the caller issues on `s` until join()
 // (or the end of this object): it streams at the memory's rate with one small CTA per SM, and the sort
 // and the merge order are chains of latencies that leave the memory idle.  Not issued for a small
-// or invalid part, more than 128 workers, or inside a capture on a device not prepared yet.
+// or invalid part, more than 128 workers, or where no side stream is free.
 class DenseBeside {
  public:
   DenseBeside(const antdt_dense_part* dp, const int64_t* batch_sizes, const uint8_t* dropped, int n_workers,
@@ -139,9 +138,8 @@ class DenseBeside {
 
  private:
   bool issued_ = false;
-  cudaStream_t main_, side_ = nullptr;
-  cudaEvent_t done_ = nullptr;
-  std::unique_lock<std::mutex> lk_;  // the side stream's events are one call's at a time
+  cudaStream_t main_;
+  SideLease side_;
 };
 
 int32_t fwd_impl(const void* table, int32_t dtype, int64_t n_rows, int32_t dim, const int32_t* row_ids,

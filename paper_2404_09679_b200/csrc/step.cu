@@ -8,6 +8,7 @@
 #include "common.cuh"
 #include "residentsort.cuh"
 #include "segsort.cuh"
+#include "side_streams.cuh"
 
 namespace antdt {
 static antdt_sparse_part sparse_part_of(const antdt_step_desc* d) {
@@ -51,16 +52,14 @@ static int32_t server_step(const antdt_step_desc* d, antdt_sparse_part* sp, cons
 }  // namespace antdt
 
 namespace {
-// Side streams and events of the steps, created on first use for each device.  An event's wait must
-// follow its record with no other step's record in between, so a step holds `mu` while it is issued.
+// Copy streams and events of the host-buffer steps, created on first use for each device.  An event's wait
+// must follow its record with no other step's record in between, so a step holds `mu` while it is issued.
 constexpr int kMaxPieces = 16;  // the d_pooled copy is cut into at most this many pieces
 struct StepStreams {
   std::mutex mu;
   bool ready = false;
   cudaStream_t in = nullptr, out = nullptr;
-  cudaStream_t side_fwd = nullptr, side_order = nullptr;  // branches of a forked device step
   cudaEvent_t start, ids, dense, fwd, done, outdone;
-  cudaEvent_t fwd_done, ids_done, order_done, sort_started;
   cudaEvent_t piece[kMaxPieces];
 };
 StepStreams g_ss[64];
@@ -79,10 +78,7 @@ StepStreams* step_streams(cudaStream_t s) {
     }
     if (cudaStreamCreateWithFlags(&ss.in, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
     if (cudaStreamCreateWithFlags(&ss.out, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
-    if (cudaStreamCreateWithFlags(&ss.side_fwd, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
-    if (cudaStreamCreateWithFlags(&ss.side_order, cudaStreamNonBlocking) != cudaSuccess) return nullptr;
-    cudaEvent_t* ev[] = {&ss.start, &ss.ids, &ss.dense, &ss.fwd, &ss.done, &ss.outdone,
-                         &ss.fwd_done, &ss.ids_done, &ss.order_done, &ss.sort_started};
+    cudaEvent_t* ev[] = {&ss.start, &ss.ids, &ss.dense, &ss.fwd, &ss.done, &ss.outdone};
     for (cudaEvent_t* e : ev)
       if (cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     for (cudaEvent_t& e : ss.piece)
@@ -246,13 +242,16 @@ extern "C" int32_t antdt_bsp_step_host(const antdt_step_desc* d, void* stream) {
 // length of the dependency chain.  It needs the aggregation's scratch behind the backward's instead
 // of on top of it.
 namespace {
+enum { kSideFwd = 0, kSideOrder = 1 };                                // streams of a step's side set
+enum { kFwdDone = 0, kIdsDone = 1, kOrderDone = 2, kSortStarted = 3 };  // its events
+
 int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
   if (!d || d->nnz < 0 || d->n_bags < 0 || d->dim < 1 || !d->d_bag_offsets || !d->d_n_agg)
     return ANTDT_ERR_INVALID_ARG;
   const bool dense = d->d_dense_grads && d->dense_n > 0;
   if (dense && !d->d_dense_out) return ANTDT_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  StepStreams* ss = nullptr;
+  antdt::SideLease side;
   size_t ws_skip = fork_ws_skip(d);
   antdt::StepMerge merge;
   const bool merged = antdt::step_merge_of(d, ws_skip, &merge);
@@ -260,57 +259,55 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
   // the forward runs beside it, started once the sort's CTAs are in place (before them it would take
   // the SMs that they wait for).
   const bool beside = antdt::resident_sort_fits(d->n_workers, d->nnz, d->n_rows);
-  if (beside || (forked && ws_skip > 0)) ss = step_streams(s);
-  if (!ss && !merged) ws_skip = 0;
-  std::unique_lock<std::mutex> lk;
-  if (ss) lk = std::unique_lock<std::mutex>(ss->mu);
+  if (beside || (forked && ws_skip > 0)) side.take(s);
+  if (!side && !merged) ws_skip = 0;
 #define CK(x) do { if ((x) != cudaSuccess) return ANTDT_ERR_CUDA; } while (0)
-  auto forward = [&](void* st, bool side) {
+  auto forward = [&](void* st, bool on_side) {
     return antdt::fwd_impl(d->table, d->dtype, d->n_rows, d->dim, d->d_row_ids, d->nnz, d->d_bag_offsets,
-                           d->n_bags, d->d_pooled_out, d->d_status, st, d->bags_per_sample, side);
+                           d->n_bags, d->d_pooled_out, d->d_status, st, d->bags_per_sample, on_side);
   };
   auto backward = [&](bool pdl_allowed) {
     return antdt::bwd_dedup_impl(d->d_row_ids, d->nnz, d->d_bag_offsets, d->n_bags, d->bags_per_sample,
                                  d->d_d_pooled, d->dim, d->n_rows, d->n_workers, d->worker_sample_offsets,
                                  d->d_uniq_ids, d->d_worker_uniq_offsets, d->d_seg_offsets, d->d_sorted_occ,
                                  d->d_uniq_grads, d->uniq_cap, d->ws, d->ws_bytes, d->d_status, stream, nullptr,
-                                 ss ? ss->ids_done : nullptr, merged ? &merge : nullptr,
-                                 ss && beside ? ss->sort_started : nullptr, pdl_allowed);
+                                 side ? side->event[kIdsDone] : nullptr, merged ? &merge : nullptr,
+                                 side && beside ? side->event[kSortStarted] : nullptr, pdl_allowed);
   };
   antdt_dense_part dp;
   dp.grads = d->d_dense_grads; dp.n = d->dense_n; dp.stride = d->dense_n; dp.out = d->d_dense_out;
   int32_t rc;
-  if (!ss) {
+  if (!side) {
     rc = forward(stream, false);
     if (rc != ANTDT_OK) return rc;
   }
   // the dense sum runs under the sort
   antdt::DenseBeside beside_sort(dense ? &dp : nullptr, d->batch_sizes, nullptr, d->n_workers, d->d_status, s);
-  if (!ss) {
+  if (!side) {
     rc = backward(!beside_sort.issued());
     if (rc != ANTDT_OK) return rc;
   } else {
-    cudaEvent_t after = beside ? ss->sort_started : ss->ids_done;
+    cudaEvent_t after = side->event[beside ? kSortStarted : kIdsDone];
     CK(cudaEventRecord(after, s));  // recorded again by the backward
     int32_t rf = ANTDT_OK;
     if (!beside) {
-      CK(cudaStreamWaitEvent(ss->side_fwd, after, 0));
-      rf = forward(ss->side_fwd, true);
+      CK(cudaStreamWaitEvent(side->stream[kSideFwd], after, 0));
+      rf = forward(side->stream[kSideFwd], true);
     }
     rc = backward(!beside_sort.issued());
     if (beside) {
-      CK(cudaStreamWaitEvent(ss->side_fwd, after, 0));
-      rf = forward(ss->side_fwd, true);
+      CK(cudaStreamWaitEvent(side->stream[kSideFwd], after, 0));
+      rf = forward(side->stream[kSideFwd], true);
     }
-    CK(cudaEventRecord(ss->fwd_done, ss->side_fwd));  // joined even after an error
-    CK(cudaStreamWaitEvent(s, ss->fwd_done, 0));      // the update writes the table the forward reads
+    CK(cudaEventRecord(side->event[kFwdDone], side->stream[kSideFwd]));  // joined even after an error
+    CK(cudaStreamWaitEvent(s, side->event[kFwdDone], 0));  // the update writes the table the forward reads
     if (rf != ANTDT_OK) return rf;
     if (rc != ANTDT_OK) return rc;
   }
   antdt_sparse_part sp = antdt::sparse_part_of(d);
   antdt::OrderFork fork;
-  const bool order_fork = ss && forked && ws_skip > 0 && !merged;
-  if (order_fork) fork = antdt::OrderFork{ss->side_order, ss->ids_done, ss->order_done};
+  const bool order_fork = side && forked && ws_skip > 0 && !merged;
+  if (order_fork) fork = antdt::OrderFork{side->stream[kSideOrder], side->event[kIdsDone], side->event[kOrderDone]};
   return antdt::server_step(d, &sp, dense && !beside_sort.issued() ? &dp : nullptr, stream, order_fork ? &fork : nullptr, ws_skip,
                             merged);
 #undef CK
@@ -414,8 +411,8 @@ extern "C" int32_t antdt_bsp_step_graph(const antdt_step_desc* d, void* stream) 
   // miss: capture the four calls
   antdt::segsort_prepare_device();
   antdt::resident_sort_prepare_device();
-  antdt::aggregate_prepare_device(s);
-  step_streams(s);
+  antdt::aggregate_prepare_device();
+  antdt::side_streams_prepare(2);  // a step's own and one for its dense part
   antdt::range_prepare_device();
   if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
     cudaGetLastError();  // e.g. the legacy default stream cannot be captured: plain launches
@@ -476,5 +473,6 @@ extern "C" int32_t antdt_bsp_step_graph_reset(void) {
   for (GraphEntry& e : g_gc[dev].entries)
     if (e.exec) cudaGraphExecDestroy(e.exec);
   g_gc[dev].entries.clear();
+  antdt::side_streams_free();
   return ANTDT_OK;
 }
