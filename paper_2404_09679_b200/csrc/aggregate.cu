@@ -572,11 +572,12 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
   char* w8 = static_cast<char*>(ws);
 
   // the two merges carry the weights themselves
-  const bool resident = sp && resident_merge_wanted(K, in_cap, sp->n_rows);
+  bool resident = sp && !merged && resident_merge_wanted(K, in_cap, sp->n_rows);
   const bool by_ranges = sp && K <= kRangeMaxWorkers && in_cap > 0;
   // a lane group per row: the one-pass update, and the sums of short lists
-  const bool by_rows = sp && in_cap > 0 && ((fu && K <= kRangeMaxWorkers) || (!fu && resident && resident_sort_clears(in_cap)));
-  if (!by_ranges && !resident) upload_small(hw, 4 * (size_t)K, w8 + L.weights, s);
+  bool by_rows = sp && in_cap > 0 && ((fu && K <= kRangeMaxWorkers) || (!fu && resident && resident_sort_clears(in_cap)));
+  auto upload_weights = [&] { upload_small(hw, 4 * (size_t)K, w8 + L.weights, s); };
+  if (!by_ranges && !resident) upload_weights();
   // the dense part runs beside the sparse one where there is enough of it
   DenseBeside beside(sp && in_cap > 0 ? dp : nullptr, batch_sizes, dropped, K, dev_status, s);
   PdlScope pdl(!beside.issued() && in_cap <= kPdlMaxItems);
@@ -584,9 +585,7 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
   if (sp) {
     int64_t* bounds = (int64_t*)(w8 + L.bounds);
     const int64_t agg_cap = sp->out_cap < in_cap ? sp->out_cap : in_cap;
-    if (merged) {
-      // the backward's sort made the merge order on the way
-    } else if (resident) {
+    if (resident) {
       cudaStream_t so = fork ? fork->side : s;
       if (fork && cudaStreamWaitEvent(so, fork->ids_ready, 0) != cudaSuccess) return ANTDT_ERR_CUDA;
       ResidentMergeArgs q = {};
@@ -614,11 +613,19 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
       q.pairs = (uint2*)(w8 + L.keys_a);  // keys_a and keys_b lie side by side
       q.hist = (uint16_t*)(w8 + L.sort_ws + L.sort.hist); q.status = dev_status;
       const int32_t rc = resident_merge(q, so);
-      if (rc != ANTDT_OK) return rc;
+      if (rc != ANTDT_OK && rc != kResidentRefused) return rc;
       if (fork && (cudaEventRecord(fork->order_done, so) != cudaSuccess ||
                    cudaStreamWaitEvent(s, fork->order_done, 0) != cudaSuccess))
         return ANTDT_ERR_CUDA;
-    } else if (K <= kRangeMaxWorkers && in_cap > 0) {
+      if (rc == kResidentRefused) {
+        resident = false;
+        by_rows = fu && K <= kRangeMaxWorkers;
+        if (!by_ranges) upload_weights();
+      }
+    }
+    if (merged || resident) {
+      // the merge order is there: the backward's sort made it on the way, or the resident merge
+    } else if (by_ranges) {
       // up to 32 workers: the merge order comes from the range-partitioned pass, no sort
       uint32_t dropped_bits = 0;
       for (int i = 0; i < K; ++i)

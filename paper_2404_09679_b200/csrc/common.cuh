@@ -13,6 +13,7 @@ namespace antdt {
 // ---- launch bookkeeping (runtime.cu) --------------------------------------------------
 int prof_begin(const char* name, cudaStream_t s);
 void prof_end(int token, cudaStream_t s);
+void prof_refused(int token);  // behind prof_end: the launch was refused, it does not count
 // While on, this thread's launches are counted but not bracketed by events (a stream that is
 // being captured cannot time its nodes).
 void prof_untimed(bool on);
@@ -98,10 +99,10 @@ int32_t bwd_dedup_impl(const int32_t* row_ids, int64_t nnz, const int64_t* bag_o
                        size_t ws_bytes, int32_t* dev_status, void* stream,
                        const PooledArrival* arrival,
                        cudaEvent_t ids_done = nullptr, const StepMerge* merge = nullptr,
-                       cudaEvent_t sort_started = nullptr, bool pdl_allowed = true);
+                       bool* merge_made = nullptr, cudaEvent_t sort_started = nullptr, bool pdl_allowed = true);
 // embbag_bwd.cu; ids_done: recorded once the distinct ids and their offsets are written; merge: the
-// sort also makes the aggregation's merge order (step_merge_targets said that it can); sort_started:
-// recorded when the CTAs of the resident sort have begun
+// sort also makes the aggregation's merge order (step_merge_targets said that it can), merge_made: that
+// it has; sort_started: recorded when the CTAs of the resident sort have begun
 
 // A second stream for the aggregation's merge order, which needs the workers' id lists but not
 // their gradients: the order kernels wait for ids_ready on `side`, and the caller's stream waits

@@ -173,7 +173,7 @@ int32_t bwd_dedup_impl(
     const int64_t* worker_sample_offsets, int32_t* uniq_ids, int64_t* worker_uniq_offsets,
     int64_t* seg_offsets, int32_t* sorted_occ, float* uniq_grads, int64_t out_cap, void* ws,
     size_t ws_bytes, int32_t* dev_status, void* stream, const PooledArrival* arrival,
-    cudaEvent_t ids_done, const StepMerge* merge, cudaEvent_t sort_started, bool pdl_allowed) {
+    cudaEvent_t ids_done, const StepMerge* merge, bool* merge_made, cudaEvent_t sort_started, bool pdl_allowed) {
   const int K = n_workers;
   if (nnz < 0 || n_bags < 0 || nnz >= (1ll << 31) || n_bags >= (1ll << 31) || n_rows < 1 ||
       n_rows >= (1ll << 31) || dim < 4 || dim > 1024 || dim % 4 || K < 1 || K > kMaxSegments ||
@@ -213,11 +213,11 @@ int32_t bwd_dedup_impl(
   const int key_bits = bits_for(n_rows);
   bool scratch_zeroed = false;
   uint32_t* occ_out = reinterpret_cast<uint32_t*>(sorted_occ);
-  if (resident_sort_fits(K, nnz, n_rows)) {
+  bool resident = resident_sort_fits(K, nnz, n_rows);
+  if (resident) {
     const size_t zero_bytes = L.tasks + 8 - L.flags_rs;
     if (!resident_sort_clears(nnz) && cudaMemsetAsync(w8 + L.flags_rs, 0, zero_bytes, s) != cudaSuccess)
       return ANTDT_ERR_CUDA;
-    scratch_zeroed = true;
     ResidentSortArgs q = {};
     q.row_ids = row_ids; q.nnz = nnz; q.bag_offsets = bag_offsets; q.n_bags = n_bags;
     q.bags_per_sample = bags_per_sample; q.n_rows = n_rows; q.n_workers = K;
@@ -232,8 +232,11 @@ int32_t bwd_dedup_impl(
     q.hist = (uint16_t*)(sort_ws + L.sort.hist);
     q.status = dev_status;
     const int32_t rc = resident_sort(q, merge, worker_sample_offsets, s, sort_started);
-    if (rc != ANTDT_OK) return rc;
-  } else {
+    if (rc != ANTDT_OK && rc != kResidentRefused) return rc;
+    resident = scratch_zeroed = rc == ANTDT_OK;
+  }
+  if (merge_made) *merge_made = resident && merge;
+  if (!resident) {
     // one launch for up to 255 workers; beyond that the offsets travel in pieces
     if (!segsort_setup_workers(worker_sample_offsets, K, (int)bags_per_sample, bag_offsets, n_bags, nnz,
                                d_worker_b, sort_ws, L.sort, dev_status, s)) {

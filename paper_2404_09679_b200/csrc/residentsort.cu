@@ -34,6 +34,9 @@
 // out of memory is masked or checked: digits and workers by their masks, slots, runs and rows by the
 // lengths of the arrays.  A cluster's barrier is the hardware's, without a limit; every CTA of the
 // cluster arrives at each of them.
+#include <algorithm>
+#include <mutex>
+
 #include "index_math.cuh"
 #include "residentsort.cuh"
 
@@ -43,16 +46,10 @@ namespace {
 constexpr int kThreads = kResThreads;
 constexpr int kWarps = kThreads / 32;
 constexpr int kBins = kSortMaxBins;  // 512 = one bin per thread
-constexpr int kMaxItems = 24;        // pairs per thread
-constexpr int kMinChunk = 1024;
-constexpr int kClusterItems = 4;     // pairs per thread of the cluster form
-constexpr int kMaxCluster = 16;
+constexpr int kClusterItems = kResClusterItems;
 constexpr int kMatchWorkers = 8;     // see the pass by worker
 constexpr uint32_t kSpinLimit = 1u << 20;
 static_assert(kBins == kThreads, "one digit per thread");
-
-// Pairs per thread: every warp of a CTA takes an equal share of its chunk.
-__host__ __device__ constexpr int items_per_thread(int chunk) { return (chunk + kThreads - 1) / kThreads; }
 
 struct Wso { int64_t v[kResMaxWorkers + 1]; };
 
@@ -902,8 +899,6 @@ resident_merge_kernel(const __grid_constant__ ResidentMergeArgs a) {
   if (CLUSTER) cluster_wait();
 }
 
-// The form a sort of nnz occurrences takes: one cluster of up to 16 CTAs, or one CTA per SM.
-struct Form { int ctas, chunk; bool cluster; };
 #define RESIDENT_DISPATCH(GO)                                   \
   do {                                                          \
     const int ipt = items_per_thread(f.chunk);                  \
@@ -914,21 +909,10 @@ struct Form { int ctas, chunk; bool cluster; };
     if (ipt <= 16) GO(16, false);                               \
     GO(24, false);                                              \
   } while (0)
-Form form_for(int64_t nnz) {
-  Form f;
-  f.cluster = nnz <= (int64_t)kMaxCluster * kClusterItems * kThreads;
-  const int64_t most = f.cluster ? kMaxCluster : kNumSM;
-  int64_t c = (nnz + most - 1) / most;
-  c = (c + 31) & ~(int64_t)31;
-  f.chunk = (int)(c < kMinChunk ? kMinChunk : c);
-  f.ctas = (int)((nnz + f.chunk - 1) / f.chunk);
-  if (f.cluster)
-    while (f.ctas & (f.ctas - 1)) ++f.ctas;  // cluster sizes are powers of two; spare CTAs hold nothing
-  return f;
-}
+static_assert(kResSMs == kNumSM, "one CTA per SM");
 
 template <typename... P, typename... A>
-int32_t launch_one(const char* name, cudaEvent_t started, void (*kernel)(P...), const Form& f, cudaStream_t s,
+int32_t launch_one(const char* name, cudaEvent_t started, void (*kernel)(P...), const ResidentForm& f, cudaStream_t s,
                    const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)f.ctas);
@@ -957,46 +941,102 @@ int32_t launch_one(const char* name, cudaEvent_t started, void (*kernel)(P...), 
   const int tok = prof_begin(name, s);
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
   prof_end(tok, s);
-  return e == cudaSuccess ? ANTDT_OK : ANTDT_ERR_CUDA;
+  if (e == cudaSuccess) return ANTDT_OK;
+  // The limits are those of the process; a stream may have fewer SMs (a green context's).
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize || e == cudaErrorLaunchOutOfResources ||
+      e == cudaErrorInvalidConfiguration || e == cudaErrorNotSupported) {
+    cudaGetLastError();
+    prof_refused(tok);
+    return kResidentRefused;
+  }
+  return ANTDT_ERR_CUDA;
+}
+
+bool went_well(cudaError_t e) {
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess;
+}
+// CTAs of the largest cluster of `kernel` that can be launched; of a cooperative launch.
+template <typename... P>
+int most_in_cluster(void (*kernel)(P...), int items) {
+  const size_t smem = smem_bytes(items * kThreads, true);
+  if (!went_well(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return 0;
+  const bool wide = went_well(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  for (int ctas = wide ? kResMaxCluster : 8; ctas > 0; ctas /= 2) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (went_well(cudaOccupancyMaxActiveClusters(&n, kernel, &cfg)) && n > 0) return ctas;
+  }
+  return 0;
+}
+template <typename... P>
+int most_at_once(void (*kernel)(P...), int items, int sms) {
+  const size_t smem = smem_bytes(items * kThreads, false);
+  int per_sm = 0;
+  if (!went_well(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) ||
+      !went_well(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem)))
+    return 0;
+  return per_sm * sms;
+}
+
+ResidentLimits query_limits(int dev) {
+  ResidentLimits lim = {};
+  int sms = 0, coop = 0;
+  if (went_well(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) &&
+      went_well(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev))) {
+    lim.cluster = std::min(std::min(most_in_cluster(resident_sort_kernel<2, true>, 2), most_in_cluster(resident_sort_kernel<4, true>, 4)),
+                           std::min(most_in_cluster(resident_merge_kernel<2, true>, 2), most_in_cluster(resident_merge_kernel<4, true>, 4)));
+#define FORM_LIMIT(I, IPT)                                                                   \
+  static_assert(kResFormItems[I] == IPT, "the dispatch below");                              \
+  if (coop) lim.ctas[I] = std::min(most_at_once(resident_sort_kernel<IPT, false>, IPT, sms), \
+                                   most_at_once(resident_merge_kernel<IPT, false>, IPT, sms))
+    FORM_LIMIT(0, 4);
+    FORM_LIMIT(1, 8);
+    FORM_LIMIT(2, 16);
+    FORM_LIMIT(3, 24);
+#undef FORM_LIMIT
+  }
+  return lim;
+}
+
+// Kernel attributes and limits of the current device, found on first use.
+const ResidentLimits& resident_limits() {
+  static std::once_flag once[64];
+  static ResidentLimits lim[64];
+  static const ResidentLimits none = {};
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    return none;
+  }
+  std::call_once(once[dev], [dev] { lim[dev] = query_limits(dev); });
+  return lim[dev];
 }
 
 }  // namespace
 
-void resident_sort_prepare_device() {
-  static bool done[64] = {};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (done[dev & 63]) return;
-  auto opt_in = [](auto* k, int items, bool cluster) {
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem_bytes(items * kThreads, cluster));
-    if (cluster) cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  };
-#define OPT_IN(IPT, CLUSTER)                            \
-  opt_in(resident_sort_kernel<IPT, CLUSTER>, IPT, CLUSTER);  \
-  opt_in(resident_merge_kernel<IPT, CLUSTER>, IPT, CLUSTER)
-  OPT_IN(2, true);
-  OPT_IN(4, true);
-  OPT_IN(4, false);
-  OPT_IN(8, false);
-  OPT_IN(16, false);
-  OPT_IN(24, false);
-#undef OPT_IN
-  done[dev & 63] = true;
-}
+void resident_sort_prepare_device() { resident_limits(); }
 
 bool resident_sort_fits(int K, int64_t nnz, int64_t n_rows) {
-  // worker and row in 32 bits; at most one CTA per SM
-  return nnz > 0 && K <= kResMaxWorkers && bits_for(K) + bits_for(n_rows + 1) <= 32 &&
-         nnz <= (int64_t)kNumSM * kThreads * kMaxItems;
+  // worker and row in 32 bits
+  return K <= kResMaxWorkers && bits_for(K) + bits_for(n_rows + 1) <= 32 && resident_holds(resident_limits(), nnz);
 }
 
-bool resident_sort_clears(int64_t nnz) { return form_for(nnz).cluster; }
+bool resident_sort_clears(int64_t nnz) { return resident_form(nnz).cluster; }
 
 int32_t resident_sort(const ResidentSortArgs& args, const StepMerge* merge, const int64_t* wso_host, cudaStream_t s,
                       cudaEvent_t started) {
   ResidentSortArgs a = args;
-  const Form f = form_for(a.nnz);
+  const ResidentForm f = resident_form(a.nnz);
   a.key_bits = bits_for(a.n_rows + 1);
   a.worker_bits = a.n_workers <= 32 ? 5 : bits_for(a.n_workers);
   a.chunk = f.chunk;
@@ -1012,13 +1052,13 @@ int32_t resident_sort(const ResidentSortArgs& args, const StepMerge* merge, cons
 
 bool resident_merge_wanted(int K, int64_t in_cap, int64_t n_rows) {
   // Small lists, whatever the workers; else the range merge is as fast or faster up to 32 workers.
-  return in_cap > 0 && K <= kResMaxWorkers && n_rows < (1ll << 31) - 1 &&
-         (form_for(in_cap).cluster || (K > 32 && in_cap <= (int64_t)kNumSM * kThreads * kMaxItems));
+  return in_cap > 0 && K <= kResMaxWorkers && n_rows < (1ll << 31) - 1 && (K > 32 || resident_form(in_cap).cluster) &&
+         resident_holds(resident_limits(), in_cap);
 }
 
 int32_t resident_merge(const ResidentMergeArgs& args, cudaStream_t s) {
   ResidentMergeArgs a = args;
-  const Form f = form_for(a.in_cap);
+  const ResidentForm f = resident_form(a.in_cap);
   a.key_bits = bits_for(a.n_rows + 1);
   a.chunk = f.chunk;
   resident_sort_prepare_device();

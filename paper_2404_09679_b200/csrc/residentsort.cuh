@@ -3,11 +3,11 @@
 // id check, stable sort by row id inside each worker, distinct rows, run starts, head bits, first
 // run of each reduction tile), and on request the merge order of the aggregation.
 #pragma once
+#include "resident_form.cuh"
 #include "segsort.cuh"
 
 namespace antdt {
 
-constexpr int kResThreads = 512;
 constexpr int kResMaxWorkers = 128;
 
 struct ResidentSortArgs {
@@ -43,11 +43,14 @@ struct StepMerge {
 bool step_merge_targets(const antdt_sparse_part& sp, const int64_t* batch_sizes, int n_workers, int64_t nnz,
                         void* ws, size_t ws_bytes, StepMerge* m);
 
-// Whether an input is one for this kernel, and whether it zeroes `zero` itself.
+// Whether an input is one for this kernel on the current device, and whether it zeroes `zero` itself.
 bool resident_sort_fits(int n_workers, int64_t nnz, int64_t n_rows);
 bool resident_sort_clears(int64_t nnz);
 void resident_sort_prepare_device();  // kernel attributes; before a stream capture
-// started: recorded once every CTA of the sort has begun (best effort), or nullptr
+// started: recorded once every CTA of the sort has begun (best effort), or nullptr.
+// kResidentRefused: the launch was refused and nothing runs (the stream has fewer SMs than the device); the
+// caller takes the kernels of segsort.cuh or agg_range.cuh.
+constexpr int32_t kResidentRefused = -1;
 int32_t resident_sort(const ResidentSortArgs& a, const StepMerge* merge, const int64_t* wso_host, cudaStream_t s,
                       cudaEvent_t started = nullptr);
 

@@ -31,7 +31,7 @@ cudaEvent_t get_event() {
 void drain_locked() {
   for (Pending& p : g_pending) {
     float ms = 0.f;
-    if (p.a && p.b && cudaEventSynchronize(p.b) == cudaSuccess &&
+    if (p.slot >= 0 && p.a && p.b && cudaEventSynchronize(p.b) == cudaSuccess &&
         cudaEventElapsedTime(&ms, p.a, p.b) == cudaSuccess) {
       g_slots[p.slot].ms += ms;
     }
@@ -125,6 +125,14 @@ void prof_end(int token, cudaStream_t s) {
   if (token < 0) return;
   std::lock_guard<std::mutex> lk(g_mu);
   if (token < (int)g_pending.size() && g_pending[token].b) cudaEventRecord(g_pending[token].b, s);
+}
+
+void prof_refused(int token) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  --g_launches;
+  if (token < 0 || token >= (int)g_pending.size()) return;
+  g_slots[g_pending[token].slot].launches -= 1;
+  g_pending[token].slot = -1;
 }
 }  // namespace antdt
 

@@ -198,7 +198,7 @@ extern "C" int32_t antdt_bsp_step_host(const antdt_step_desc* d, void* stream) {
                        cudaMemcpyDeviceToHost, ss->out));
   size_t ws_skip = fork_ws_skip(d);
   antdt::StepMerge merge;
-  const bool merged = antdt::step_merge_of(d, ws_skip, &merge);
+  bool merged = antdt::step_merge_of(d, ws_skip, &merge);
   if (!merged) ws_skip = 0;
   antdt::PooledArrival arrival{n_pieces, piece_entry_end, ss->piece};
   rc = antdt::bwd_dedup_impl(d->d_row_ids, d->nnz, d->d_bag_offsets, d->n_bags, d->bags_per_sample,
@@ -206,7 +206,7 @@ extern "C" int32_t antdt_bsp_step_host(const antdt_step_desc* d, void* stream) {
                               d->worker_sample_offsets, d->d_uniq_ids, d->d_worker_uniq_offsets,
                               d->d_seg_offsets, d->d_sorted_occ, d->d_uniq_grads, d->uniq_cap, d->ws,
                               d->ws_bytes, d->d_status, stream, n_pieces > 0 ? &arrival : nullptr, nullptr,
-                              merged ? &merge : nullptr);
+                              merged ? &merge : nullptr, &merged);
   if (rc != ANTDT_OK) return rc;
   CK(cudaStreamWaitEvent(s, ss->dense, 0));
   antdt_sparse_part sp = antdt::sparse_part_of(d);
@@ -254,7 +254,7 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
   antdt::SideLease side;
   size_t ws_skip = fork_ws_skip(d);
   antdt::StepMerge merge;
-  const bool merged = antdt::step_merge_of(d, ws_skip, &merge);
+  bool merged = antdt::step_merge_of(d, ws_skip, &merge);
   // The resident sort leaves half of every SM to others and waits for latencies most of the time, so
   // the forward runs beside it, started once the sort's CTAs are in place (before them it would take
   // the SMs that they wait for).
@@ -271,7 +271,7 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
                                  d->d_d_pooled, d->dim, d->n_rows, d->n_workers, d->worker_sample_offsets,
                                  d->d_uniq_ids, d->d_worker_uniq_offsets, d->d_seg_offsets, d->d_sorted_occ,
                                  d->d_uniq_grads, d->uniq_cap, d->ws, d->ws_bytes, d->d_status, stream, nullptr,
-                                 side ? side->event[kIdsDone] : nullptr, merged ? &merge : nullptr,
+                                 side ? side->event[kIdsDone] : nullptr, merged ? &merge : nullptr, &merged,
                                  side && beside ? side->event[kSortStarted] : nullptr, pdl_allowed);
   };
   antdt_dense_part dp;
