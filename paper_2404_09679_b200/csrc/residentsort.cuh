@@ -47,7 +47,8 @@ bool step_merge_targets(const antdt_sparse_part& sp, const int64_t* batch_sizes,
 bool resident_sort_fits(int n_workers, int64_t nnz, int64_t n_rows);
 bool resident_sort_clears(int64_t nnz);
 void resident_sort_prepare_device();  // kernel attributes; before a stream capture
-// started: recorded once every CTA of the sort has begun (best effort), or nullptr.
+// started: recorded once every CTA of the sort has begun (best effort), or nullptr.  That can be before the
+// work ahead of the sort on s is over (programmatic dependent launch): whoever goes by it waits for that too.
 // kResidentRefused: the launch was refused and nothing runs (the stream has fewer SMs than the device); the
 // caller takes the kernels of segsort.cuh or agg_range.cuh.
 constexpr int32_t kResidentRefused = -1;

@@ -16,7 +16,7 @@ constexpr int kSideSets = 8;
 
 struct SideSet {
   cudaStream_t stream[2];
-  cudaEvent_t event[4];  // an event's wait follows its record inside one lease
+  cudaEvent_t event[5];  // an event's wait follows its record inside one lease
 };
 
 class SideLease {

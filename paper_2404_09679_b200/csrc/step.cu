@@ -243,7 +243,7 @@ extern "C" int32_t antdt_bsp_step_host(const antdt_step_desc* d, void* stream) {
 // of on top of it.
 namespace {
 enum { kSideFwd = 0, kSideOrder = 1 };                                // streams of a step's side set
-enum { kFwdDone = 0, kIdsDone = 1, kOrderDone = 2, kSortStarted = 3 };  // its events
+enum { kBefore = 0, kFwdDone = 1, kIdsDone = 2, kOrderDone = 3, kSortStarted = 4 };  // its events
 
 int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
   if (!d || d->nnz < 0 || d->n_bags < 0 || d->dim < 1 || !d->d_bag_offsets || !d->d_n_agg)
@@ -287,17 +287,19 @@ int32_t device_step(const antdt_step_desc* d, void* stream, bool forked) {
     rc = backward(!beside_sort.issued());
     if (rc != ANTDT_OK) return rc;
   } else {
-    cudaEvent_t after = side->event[beside ? kSortStarted : kIdsDone];
-    CK(cudaEventRecord(after, s));  // recorded again by the backward
+    // The forward waits for what is ahead of the step on s, and beside the resident sort for its CTAs to
+    // have begun.  The second does not imply the first: the sort is a dependent launch, its CTAs may begin
+    // while the kernel ahead (the update of the step before) still runs.
+    cudaStream_t sf = side->stream[kSideFwd];
+    CK(cudaEventRecord(side->event[kBefore], s));
+    CK(cudaStreamWaitEvent(sf, side->event[kBefore], 0));
     int32_t rf = ANTDT_OK;
-    if (!beside) {
-      CK(cudaStreamWaitEvent(side->stream[kSideFwd], after, 0));
-      rf = forward(side->stream[kSideFwd], true);
-    }
+    if (beside) CK(cudaEventRecord(side->event[kSortStarted], s));  // recorded again by the sort
+    else rf = forward(sf, true);
     rc = backward(!beside_sort.issued());
     if (beside) {
-      CK(cudaStreamWaitEvent(side->stream[kSideFwd], after, 0));
-      rf = forward(side->stream[kSideFwd], true);
+      CK(cudaStreamWaitEvent(sf, side->event[kSortStarted], 0));
+      rf = forward(sf, true);
     }
     CK(cudaEventRecord(side->event[kFwdDone], side->stream[kSideFwd]));  // joined even after an error
     CK(cudaStreamWaitEvent(s, side->event[kFwdDone], 0));  // the update writes the table the forward reads
