@@ -150,9 +150,12 @@ extern "C" int32_t antdt_bsp_step_host(const antdt_step_desc* d, void* stream) {
     const int64_t F = d->bags_per_sample;
     const size_t row_bytes = 4 * D;
     // A cut costs the link about 26 us while the read-back runs the other way (54 MB: 1242 us as one
-    // copy, 1450 us in 8 pieces), what it hides is the reduction of the pieces before the last
-    // (20 us for those 54 MB): pieces of 64 MB at least.
-    const size_t most = (size_t)d->n_bags * row_bytes >> 26;
+    // copy, 1450 us in 8 pieces), what it hides is the reduction of the pieces before the last.  Pieces of
+    // 256 MB at least: 1 / 2 / 4 / 8 / 16 pieces of 256 MB in all take 5774 / 5825 / 6072 / 6296 / 6537 us with
+    // one id per bag and 6757 / 6739 / 6868 / 6927 / 7279 with ten; of 512 MB 11660 / 11809 / 11854 / 11993 /
+    // 12470 and 13272 / 13277 / 13231 / 13434 / 13817; of 1 GB 23629 / 23767 / 23292 / 23476 / 24145 and 27288 /
+    // 26517 / 26324 / 26474 / 26964 (two runs of one kind differ by up to 3%).
+    const size_t most = (size_t)d->n_bags * row_bytes >> 28;
     int want = K < kMaxPieces ? K : kMaxPieces;
     if ((size_t)want > most) want = (int)most;
     if (want < 1 || F < 1 || !d->worker_sample_offsets) want = 1;

@@ -11,10 +11,10 @@ from tests.step_harness import make_batch, plan_steps
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("counts", [[4096] * 4, [16_000, 0, 0, 384], [0, 5000, 11_384, 0]])
+@pytest.mark.parametrize("counts", [[16_384] * 4, [64_000, 0, 0, 1536], [0, 20_000, 45_536, 0]])
 def test_host_step_in_pieces_equals_the_device_step(counts):
-    w = synth.WORKLOADS[3].scaled(K=4, B=16_384, F=48, V=300_000, dense_n=0, len_mean=3.0, speed_kind="equal")
-    assert w.B * w.F * w.D * 4 >= 3 << 26       # three pieces of 64 MB or more
+    w = synth.WORKLOADS[3].scaled(K=4, B=65_536, F=48, V=300_000, dense_n=0, len_mean=3.0, speed_kind="equal")
+    assert w.B * w.F * w.D * 4 >= 3 << 28       # three pieces of 256 MB or more
     b = make_batch(synth.BatchMaker(w, "cuda"), plan_steps(w, 1)[0], 0)
     wso = [sum(counts[:i]) for i in range(5)]
     nnz, n_bags = b["row_ids"].numel(), b["bag_offsets"].numel() - 1
