@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 import oracle
+from paper_2404_09679_b200 import binding as B
 from tests import gpu_util as G
 
 pytestmark = pytest.mark.gpu
@@ -58,10 +59,14 @@ def test_unequal_workers_and_table_sizes(V):
 @pytest.mark.parametrize("extra", [0, 1])
 def test_the_largest_input_and_the_one_after_it(extra):
     rng = np.random.default_rng(9)
-    n = 148 * 512 * 16 + extra
+    n = 148 * 512 * 24 + extra                 # one more goes to the multi-kernel sort
     lens = np.full(n // 8, 8, np.int64)
     lens[0] += n - lens.sum()
+    B.antdt_profile_enable(True)
     _check(lens, [0, len(lens) // 3, len(lens)], 1, 40_000, 4, rng, hot=0.05)
+    ran = set(B.antdt_profile_get())
+    B.antdt_profile_enable(False)
+    assert ("resident_sort" in ran) == (extra == 0) and ("radix_scatter" in ran) == (extra == 1)
 
 
 @pytest.mark.parametrize("K,n", [(1, 148 * 512 * 24), (8, 148 * 512 * 17 + 31), (9, 148 * 512 * 9 - 33), (2, 148 * 512 * 4 + 1)])
