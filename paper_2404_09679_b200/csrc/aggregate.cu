@@ -703,9 +703,11 @@ void aggregate_prepare_device() {
   }
 }
 
-// 2.2 GB (32 workers x 16.8 M) beside the sort of 35 M occurrences: 1.19 ms instead of 0.34 alone, the
-// sort's kernels 0.15 ms slower, the step 5472 -> 5305 us; with the full-size kernel at 2 CTAs per SM
-// beside the merge order 5380.  Alone with the merge order (117 MB of 16 workers): 601 -> 580 us.
+// 2.2 GB (32 workers x 16.8 M) beside the sort of 35 M occurrences: 1.03 - 1.19 ms instead of 0.34 alone, the
+// sort's kernels 0.15 ms slower, the step 5426 - 5554 -> 5269 - 5419 us (6 runs of each in turn); with the
+// full-size kernel at 2 CTAs per SM beside the merge order 5380.  285 MB of 16 workers in the step of 65 M
+// occurrences: 9507 - 9647 -> 9279 - 9600, hardly more than the runs differ.  117 MB beside the merge order of a
+// server alone: 618 - 627 -> 555 - 558 us.
 DenseBeside::DenseBeside(const antdt_dense_part* dp, const int64_t* batch_sizes, const uint8_t* dropped, int K,
                          int32_t* dev_status, cudaStream_t s) : main_(s) {
   if (!dp || !batch_sizes || K < 1 || K > kDenseBlobWorkers || !dense_valid(*dp) || dp->n * 4 * (K + 1) < kDenseBesideBytes ||

@@ -44,8 +44,8 @@ extern "C" int32_t antdt_embbag_bwd_dedup_static(
     scratch = g_scratch_ptr[dev];
   }
   // The array keeps the previous call's contents.  The shared implementation writes every part
-  // of its scratch before reading it and zeroes the one part that is accumulated into (the
-  // run-head bit mask) with a memset on the stream, so no extra clearing is needed here.
+  // of its scratch before reading it and zeroes what it accumulates into (run-head bits, counters) on
+  // the stream, so no extra clearing is needed here.
   return antdt_embbag_bwd_dedup(row_ids, nnz, bag_offsets, n_bags, bags_per_sample, d_pooled, dim,
                                 n_rows, n_workers, worker_sample_offsets, uniq_ids,
                                 worker_uniq_offsets, seg_offsets, sorted_occ, uniq_grads, out_cap,

@@ -125,19 +125,32 @@ constexpr int kFlatThreads = 256;
 constexpr int kFlatUnroll = 4;
 constexpr int kFlatCtas = 8;     // CTAs per SM
 
-// Whether bags of avg ids are strided over (embbag_fwd_stride_kernel) and by how many resident waves of
-// CTAs; 0: one bag per lane group.  W: waves that one bag per lane group would make.
-// Reading the next bag's offsets ahead pays once a lane group has several turns, and the more of a
-// bag's time its offsets are: for rows of 16 vectors and more always, for 8 vectors below 8 ids, for
-// less below 3.  Measured, one bag per group -> striding: 128 floats x 10 ids, W 39 / 157: 206 -> 196,
-// 778 -> 701 us; 64 x 10, W 79: 440 -> 411; 64 x 4.5, W 20 / 327: 79 -> 70, 1175 -> 958; 32 x 1, W 39:
-// 105 -> 89; against it 32 x 10, W 39: 265 -> 284, 16 x 4.5, W 20: 104 -> 112, 32 x 1, W 2.5: the same.
+// Whether bags are strided over (embbag_fwd_stride_kernel) and by how many resident waves of CTAs; 0: one bag
+// per lane group.  W: waves that one bag per lane group would make.
+// Reading the next bag's offsets ahead pays once a lane group has several turns, and the more of a bag's time
+// its offsets are: the shorter its list and the wider its rows.  Above a length that depends on both, the
+// fewer lane groups at work cost more than the offsets.  One bag per group -> striding, us, by ids per bag:
+//   fp32, 32 vectors, W 39    1: 93 -> 79    3: 116 -> 99    10: 200 -> 191   20: 321 -> 325   40: 560 -> 584
+//         16 vectors, W 39    1: 96 -> 82    3: 127 -> 108   10: 224 -> 217   20: 361 -> 367   40: 632 -> 688
+//          8 vectors, W 39    1: 100 -> 88   4.5: 169 -> 158   5.5: 186 -> 182   6: 194 -> 194   7: 211 -> 219
+//                     W 130   4.5: 551 -> 488   6.5: 660 -> 614
+//          4 vectors, W 19    1.5: 58 -> 53   2: 67 -> 62    2.5: 71 -> 71    3: 82 -> 84      4.5: 103 -> 119
+//          2 vectors, W 32    1.5: 104 -> 104   2: 123 -> 128   3: 155 -> 175
+//   bf16, 32 vectors, W 78    1: 217 -> 189   4.5: 319 -> 296   10: 480 -> 479   20: 772 -> 817
+//         16 vectors, W 39    1: 114 -> 100   3: 153 -> 145   4.5: 180 -> 177   10: 275 -> 292
+//          8 vectors, W 19    1: 62 -> 56    3: 91 -> 88     4.5: 107 -> 107   10: 165 -> 175
+//          4 vectors, W 19    1.5: 70 -> 71   3: 103 -> 103
+// Few turns: W 7, 16 vectors, 4.5 ids 34 -> 31; W 8, 32 vectors, 10 ids 47 -> 47; W 2.5, 8 vectors, 1 id the same.
 // About ten turns per group are best: fewer waves unbalance the SMs (W 327 in 1 / 4 / 16 waves: 1127 /
 // 1039 / 958 us), more waste the reading ahead (W 39 in 4 / 16 / 32 waves: 119 / 128 / 140).
-inline int stride_waves(int G, int64_t n_bags, int64_t nnz) {
+inline int stride_below(int G, bool bf16) {  // ids per bag
+  if (bf16) return G >= 32 ? 8 : (G == 16 ? 5 : (G == 8 ? 4 : 0));
+  return G >= 16 ? 16 : (G == 8 ? 6 : (G == 4 ? 3 : 0));
+}
+inline int stride_waves(int G, bool bf16, int64_t n_bags, int64_t nnz) {
   const int64_t per_wave = (int64_t)kNumSM * kFlatCtas * (kFlatThreads / G);
   const int64_t W = n_bags / per_wave;
-  if (W < 8 || (G < 16 && nnz >= (G == 8 ? 8 : 3) * n_bags)) return 0;
+  if (W < 8 || nnz >= stride_below(G, bf16) * n_bags) return 0;
   const int64_t waves = (W + 5) / 10;
   return waves < 1 ? 1 : (waves > 16 ? 16 : (int)waves);
 }
@@ -229,9 +242,9 @@ embbag_fwd_flat_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
   if (lg < nvec) flat_store<BF16>(pooled + bag * (int64_t)dim + (size_t)lg * EPV, acc);
 }
 
-// Where the chain offsets -> ids -> rows is much of a bag's time (stride_waves): the grid is capped, every lane group strides over its bags (bag order), and the NEXT bag's offsets
-// are read before the current bag's rows are requested (30 fields x 4.5 ids x 128-byte rows:
-// 1.06 -> 0.84 ms).  The loop is written out in one piece on purpose: at 32 registers the form of
+// Where the chain offsets -> ids -> rows is much of a bag's time (stride_waves): the grid is capped, every
+// lane group strides over its bags (bag order), and the NEXT bag's offsets are read before the current
+// bag's rows are requested (30 fields x 4.5 ids x 128-byte rows: 1.06 -> 0.84 ms).  The loop is written out in one piece on purpose: at 32 registers the form of
 // the source decides what the compiler keeps in flight, and two tidier versions of this same loop
 // (the bag's sum in a helper, the offsets held as raw 64-bit values) measured 1.07 - 1.21 ms.
 template <int G, bool BF16>
@@ -326,7 +339,7 @@ void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_i
   } else {
     fields = 0;
   }
-  const int waves = flat && fields == 0 ? stride_waves(G, n_bags, nnz) : 0;
+  const int waves = flat && fields == 0 ? stride_waves(G, BF16, n_bags, nnz) : 0;
   if (waves > 0) {
     ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_stride_kernel<G, BF16>), (unsigned)(kNumSM * kFlatCtas * waves),
                  kFlatThreads, 0, s, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, chained);

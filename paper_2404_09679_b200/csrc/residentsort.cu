@@ -25,8 +25,8 @@
 // (up to 16 CTAs of 2048) run as one thread-block cluster: counts, pairs and barriers go through
 // distributed shared memory (a barrier 0.3 us against 1.3).
 // Measured (in brackets the kernels it replaced: sort, and merge order where a step makes it): 10 k
-// occurrences of 4 workers over 80 k rows 17 us (37 + 35); 426 k of 8 over 26 M 60 us (75 + 62);
-// 1.2 M of one worker over 1 M 74 us (113).
+// occurrences of 4 workers over 80 k rows 17 us (37 + 35); 426 k of 8 over 26 M 58 us, 70 with a step's forward
+// beside it (75 + 62); 1.2 M of one worker over 1 M 66 - 70 us (113).
 //
 // The CTAs wait for one another, so the launch is a cluster or a cooperative one (all CTAs resident
 // or none started).  A wait through memory is bounded all the same (kSpinLimit) and raises

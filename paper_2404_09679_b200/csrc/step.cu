@@ -1,4 +1,5 @@
-// One whole BSP step from host buffers: stage in, run the four device calls, stage out.
+// One whole BSP step: from host buffers (stage in, run the four device calls, stage out), from device
+// buffers, and replayed as a CUDA graph.
 #include <string.h>
 
 #include <mutex>

@@ -1,6 +1,6 @@
 """The forward whose lane groups stride over the bags: bag counts on both sides of the wave counts where it
-starts and where it takes a second wave, for long bags of wide rows (always strided) and for bags just below
-and at the length where narrow rows stop striding; against the CPU checker."""
+starts and where it takes a second wave, for bags just below and at the length where each row width stops
+striding; against the CPU checker."""
 import numpy as np
 import pytest
 
@@ -16,7 +16,11 @@ PER_WAVE = 148 * 8 * 256                      # lanes of one resident wave
 @pytest.mark.parametrize("D,bf16,lanes,waves,off_by,lo,hi", [
     (128, False, 32, 8, -1, 6, 14), (128, False, 32, 8, 0, 6, 14), (96, False, 32, 15, 1, 0, 20),
     (64, False, 16, 8, 0, 4, 16), (128, True, 16, 8, 3, 0, 9), (32, False, 8, 8, 1, 5, 10),
-    (32, False, 8, 8, 1, 6, 10), (8, True, 1, 8, 0, 1, 1)])
+    (32, False, 8, 8, 1, 6, 10), (8, True, 1, 8, 0, 1, 1),
+    (128, False, 32, 8, 0, 14, 16), (128, False, 32, 8, 0, 16, 16), (64, False, 16, 8, 2, 13, 18),
+    (32, False, 8, 8, 1, 3, 8), (16, False, 4, 8, 0, 1, 4), (16, False, 4, 8, 0, 3, 3), (8, False, 2, 8, 0, 1, 2),
+    (256, True, 32, 8, 1, 2, 12), (128, True, 16, 8, 0, 4, 6), (64, True, 8, 15, 1, 1, 6), (64, True, 8, 8, 0, 4, 4),
+    (32, True, 4, 8, 0, 1, 3)])
 def test_strided_bags(D, bf16, lanes, waves, off_by, lo, hi):
     n_bags = waves * (PER_WAVE // lanes) + off_by
     rng = np.random.default_rng(D + hi + off_by)
