@@ -3,7 +3,7 @@
 //
 // Work decomposition: every segment is cut into chunks of chunk_elems consecutive elements
 // (about kSortChunksTarget chunks in all, one CTA each, so a pass is a single wave on 148 SMs
-// at 4 CTAs per SM).  One pass = histogram per chunk -> exclusive scan over (bin, chunk) inside
+// at kSortCtasPerSM CTAs per SM).  One pass = histogram per chunk -> exclusive scan over (bin, chunk) inside
 // each segment -> scatter.  The scatter ranks a 4096-pair tile with warp votes or match
 // (stable: tile order is warp-striped), reorders the tile in shared memory by bin and writes
 // each bin's run with consecutive threads, so global stores are as coalesced as the digit
@@ -433,7 +433,7 @@ radix_scatter_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __res
         const bool valid = wbase + i * 32 < tile_n;
         const uint32_t d = (k[i] >> shift) & mask;
         const unsigned m = pm[i];
-          const uint32_t old = valid ? my_wh[d] : 0u;
+        const uint32_t old = valid ? my_wh[d] : 0u;
         __syncwarp();
         if (valid && (m & lt) == 0) my_wh[d] = (unsigned short)(old + __popc(m));
         __syncwarp();
