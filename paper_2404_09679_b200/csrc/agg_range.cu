@@ -27,43 +27,38 @@ struct WeightBlob { float w[kRangeMaxWorkers]; };  // the workers' weights, a ke
 
 __global__ void __launch_bounds__(kRaThreads)
 range_split_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ wuo_in, int K,
-                   int64_t in_cap, int r_log2, int64_t P, uint32_t dropped,
-                   int64_t* __restrict__ wuo_out, int64_t* __restrict__ n_entries,
-                   int32_t* __restrict__ bnd, const WeightBlob weights, float* __restrict__ weights_out,
-                   int32_t* status) {
+                   int64_t in_cap, int r_log2, int64_t P, int64_t n_rows, uint32_t dropped,
+                   int64_t* __restrict__ wuo_out, int32_t* __restrict__ bnd, const WeightBlob weights,
+                   float* __restrict__ weights_out, int32_t* status) {
   pdl_sync();
   __shared__ int64_t s_wuo[kRangeMaxWorkers + 1];
   if (blockIdx.x == 0 && weights_out && threadIdx.x < K) weights_out[threadIdx.x] = weights.w[threadIdx.x];
   if (threadIdx.x == 0) {  // ascending and inside [0, in_cap], whatever came in
-    int64_t prev = 0, kept = 0;
+    int64_t prev = 0;
     for (int i = 0; i <= K; ++i) {
       int64_t v = wuo_in[i];
       v = v < prev ? prev : v;
       v = v > in_cap ? in_cap : v;
       s_wuo[i] = v;
-      if (i > 0 && !((dropped >> (i - 1)) & 1u)) kept += v - prev;
       prev = v;
       if (blockIdx.x == 0) wuo_out[i] = v;
     }
-    if (blockIdx.x == 0) {
-      n_entries[0] = 0;   // read as [begin, end) of the merged entries by the reduction
-      n_entries[1] = kept;
-      if (wuo_in[K] < 0 || wuo_in[K] > in_cap) set_status(status, ANTDT_ERR_CAPACITY);
-    }
+    if (blockIdx.x == 0 && (wuo_in[K] < 0 || wuo_in[K] > in_cap)) set_status(status, ANTDT_ERR_CAPACITY);
   }
   __syncthreads();
   const int64_t idx = (int64_t)blockIdx.x * kRaThreads + threadIdx.x;
   if (idx >= (int64_t)K * (P + 1)) return;
   const int w = (int)(idx / (P + 1));
   const int64_t b = idx % (P + 1);
-  const uint64_t key = (uint64_t)b << r_log2;  // b == P: past the last row id
+  const uint64_t key = b < P ? (uint64_t)b << r_log2 : (uint64_t)n_rows;  // b == P: past the last row id
   int64_t lo = s_wuo[w], hi = s_wuo[w + 1];
   while (lo < hi) {
     const int64_t mid = (lo + hi) >> 1;
     if ((uint64_t)(uint32_t)__ldg(ids + mid) < key) lo = mid + 1; else hi = mid;
   }
   bnd[(size_t)w * (P + 1) + b] = (int32_t)lo;
-  if (b == P && lo < s_wuo[w + 1]) set_status(status, ANTDT_ERR_ID_OUT_OF_RANGE);  // ids past the table
+  if (b == P && lo < s_wuo[w + 1] && !((dropped >> w) & 1u))
+    set_status(status, ANTDT_ERR_ID_OUT_OF_RANGE);  // ids past the table
 }
 
 // The pieces of range b: worker w's entries [s_beg[w], s_beg[w] + size) with s_off[w] entries of
@@ -196,13 +191,28 @@ range_count_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ 
 }
 
 // Exclusive scan of distinct[P] -> base[P+1]; one CTA of 1024 threads, consecutive ranges per
-// thread.
+// thread.  Its last warp counts the entries that get a merge slot: those of the workers that count, up to the
+// first id outside the table (ids past it, at the end of a list, have no slot; what a slot's place holds from
+// before must not be read as one).
 __global__ void __launch_bounds__(1024)
 range_scan_kernel(const int32_t* __restrict__ distinct, int64_t P, int64_t* __restrict__ base,
-                  int64_t* __restrict__ n_agg, int64_t out_cap, int32_t* status) {
+                  int64_t* __restrict__ n_agg, int64_t out_cap, const int32_t* __restrict__ bnd,
+                  const int64_t* __restrict__ wuo, int K, uint32_t dropped, int64_t* __restrict__ n_entries,
+                  int32_t* status) {
   pdl_sync();
   __shared__ int64_t warp_tot[32];
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  if (wp == 31) {
+    int64_t kept = 0;
+    if (lane < K && !((dropped >> lane) & 1u))
+      kept = max((int64_t)0, (int64_t)__ldg(bnd + (size_t)lane * (P + 1) + P) - __ldg(wuo + lane));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, o);
+    if (lane == 0) {
+      n_entries[0] = 0;  // read as [begin, end) of the merged entries by the reduction
+      n_entries[1] = kept;
+    }
+  }
   const int64_t per = (P + 1023) / 1024;
   const int64_t c0 = (int64_t)tid * per, c1 = min(P, c0 + per);
   int64_t mine = 0;
@@ -414,12 +424,12 @@ void range_merge_order(const int32_t* uniq_ids, const int64_t* wuo_in, int64_t i
   while ((1 << tile_shift) < tile) ++tile_shift;
   const int64_t n_search = (int64_t)K * (P + 1);
   ANTDT_LAUNCH("agg_range_split", range_split_kernel, (unsigned)((n_search + kRaThreads - 1) / kRaThreads),
-               kRaThreads, 0, s, uniq_ids, wuo_in, K, in_cap, r_log2, P, dropped_bits, wuo_out, n_entries,
-               bnd, wb, weights_host ? weights_dev : nullptr, status);
+               kRaThreads, 0, s, uniq_ids, wuo_in, K, in_cap, r_log2, P, n_rows, dropped_bits, wuo_out, bnd, wb,
+               weights_host ? weights_dev : nullptr, status);
   ANTDT_LAUNCH("agg_range_count", range_count_kernel, (unsigned)P, kRaThreads, 0, s,
                uniq_ids, bnd, wuo_out, K, P, r_log2, n_rows, dropped_bits, distinct, status);
   ANTDT_LAUNCH("agg_range_scan", range_scan_kernel, 1, 1024, 0, s, distinct, P, base, n_agg, out_cap,
-               status);
+               bnd, wuo_out, K, dropped_bits, n_entries, status);
   if (head_bits) cudaMemsetAsync(head_bits, 0, head_bits_words(in_cap) * 4, s);
   // every tile's entry is written unless ids were skipped as invalid: start from a valid index
   if (tile_first) cudaMemsetAsync(tile_first, 0, 4 * ((size_t)((in_cap + tile - 1) >> tile_shift) + 1), s);

@@ -42,7 +42,7 @@ void range_prepare_device();
 // Merge order of the workers' lists, ready for the tile reduction (tile_reduce.cuh):
 //   wuo_in [K+1] raw offsets (clamped to in_cap into wuo_out), dropped_bits: bit w = ignore worker w
 //   agg_ids [out_cap]   distinct row ids ascending;  n_agg = their number
-//   n_entries [2]       {0, entries of the workers that count}
+//   n_entries [2]       {0, entries of the workers that count whose ids lie in the table}
 //   src [in_cap]        position (in the concatenated lists) of the entry at each merge slot;
 //                       slots ordered by (row id, worker)
 //   head_bits           bit i set iff slot i is the first contribution of its row (zeroed here)
