@@ -312,7 +312,7 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 constexpr int kFusedRows = 1;
 constexpr int kFusedWaves = 16, kFusedWavesAdam = 64;
 constexpr int kFusedCtas = 8;
-template <int G, int VPL, bool UPDATE, bool ADAM, bool BF16>
+template <int G, int VPL, bool UPDATE, bool ADAM, bool BF16, bool PACKED>
 __global__ void __launch_bounds__(256, (VPL == 1 ? kFusedCtas : 1))
 agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __restrict__ src,
                   const int32_t* __restrict__ agg_ids, const int64_t* __restrict__ n_agg_dev,
@@ -326,8 +326,10 @@ agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __rest
   for (int i = threadIdx.x; i < K; i += blockDim.x) s_w[i] = weights[i];
   __syncthreads();
   constexpr int R = VPL == 1 ? kFusedRows : 1;  // rows a lane group has in flight
-  const int lg = threadIdx.x & (G - 1);
   const int nvec = dim / 4;
+  const RowLanes<256, G, PACKED> lanes(nvec);
+  const int lg = lanes.lg;
+  if (!lanes.on()) return;
   // 32-bit row numbers and slots (fewer than 2^31 of each): the kernel is bound by its instruction
   // stream and by the registers that live across the chain of loads
   const uint32_t n = (uint32_t)min(*n_agg_dev, out_cap);
@@ -335,8 +337,8 @@ agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __rest
   // result is flagged then, does without: it has no register to spare)
   const uint32_t n_starts = UPDATE ? n : (uint32_t)*n_agg_dev;
   const uint32_t total = (uint32_t)min(n_entries[1], in_cap);
-  const uint32_t stride = gridDim.x * (256 / G);
-  for (uint32_t u0 = blockIdx.x * (256 / G) + threadIdx.x / G; u0 < n; u0 += R * stride) {
+  const uint32_t stride = gridDim.x * lanes.groups;
+  for (uint32_t u0 = blockIdx.x * lanes.groups + lanes.grp; u0 < n; u0 += R * stride) {
     uint32_t s0[R], s1[R];
     int32_t row[R];
     bool ok[R];
@@ -432,24 +434,24 @@ agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __rest
   }
 }
 
-template <int G, int VPL>
+template <int G, int VPL, bool PACKED>
 void launch_agg_update(const FusedUpdate& fu, const uint32_t* row_start, const uint32_t* src,
                        const antdt_sparse_part* sp, int64_t out_cap, const int64_t* n_entries,
                        const uint8_t* src_worker, const float* weights, int K, cudaStream_t s) {
-  const int64_t gpb = 256 / G;
+  const int64_t gpb = row_groups(256, sp->dim / 4, G, PACKED);
   const int64_t want = (out_cap + gpb - 1) / gpb;
   const size_t smem = 4 * (size_t)K;
   const bool adam = fu.opt == ANTDT_OPT_ADAM, bf16 = fu.dtype == ANTDT_BF16;
   const int64_t cap = (int64_t)kNumSM * kFusedCtas * (adam ? kFusedWavesAdam : kFusedWaves);
   const unsigned grid = (unsigned)(want > cap ? cap : (want < 1 ? 1 : want));
   if (!fu.table) {  // the sums alone
-    ANTDT_LAUNCH("agg_reduce", (agg_update_kernel<G, VPL, false, false, false>), grid, 256, smem, s, row_start, src,
+    ANTDT_LAUNCH("agg_reduce", (agg_update_kernel<G, VPL, false, false, false, PACKED>), grid, 256, smem, s, row_start, src,
                  sp->agg_ids, sp->n_agg, out_cap, n_entries, sp->uniq_grads, sp->in_cap, src_worker, weights, K,
                  nullptr, sp->n_rows, sp->dim, fu.p, nullptr, nullptr, fu.agg_out);
     return;
   }
 #define FU_GO(A, B)                                                                              \
-  ANTDT_LAUNCH("agg_update", (agg_update_kernel<G, VPL, true, A, B>), grid, 256, smem, s, row_start, src, \
+  ANTDT_LAUNCH("agg_update", (agg_update_kernel<G, VPL, true, A, B, PACKED>), grid, 256, smem, s, row_start, src, \
                sp->agg_ids, sp->n_agg, out_cap, n_entries, sp->uniq_grads, sp->in_cap, src_worker, weights, K, \
                fu.table, sp->n_rows, sp->dim, fu.p, fu.state0, fu.state1, fu.agg_out)
   if (adam) { if (bf16) FU_GO(true, true); else FU_GO(true, false); }
@@ -655,7 +657,13 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
       const uint8_t* sw = (const uint8_t*)(w8 + L.src_worker);
       const float* wts = (const float*)(w8 + L.weights);
       const int nvec = sp->dim / 4;
-#define FU_CASE(G, VPL) launch_agg_update<G, VPL>(f, rs, src, sp, agg_cap, bounds, sw, wts, K, s)
+#define FU_CASE(G, VPL)                                                                                \
+  do {                                                                                                 \
+    if (VPL == 1 && (f.opt == ANTDT_OPT_ADAM ? row_packs_narrow(nvec, G) : row_packs(256, nvec, G)))   \
+      launch_agg_update<G, VPL, (VPL == 1 && G > 2)>(f, rs, src, sp, agg_cap, bounds, sw, wts, K, s);  \
+    else                                                                                               \
+      launch_agg_update<G, VPL, false>(f, rs, src, sp, agg_cap, bounds, sw, wts, K, s);                \
+  } while (0)
       if (nvec <= 1) FU_CASE(1, 1);
       else if (nvec <= 2) FU_CASE(2, 1);
       else if (nvec <= 4) FU_CASE(4, 1);

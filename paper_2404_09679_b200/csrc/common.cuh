@@ -164,6 +164,32 @@ __device__ __forceinline__ unsigned group_mask() {
   return ((1u << G) - 1u) << (lane & ~(unsigned)(G - 1));
 }
 
+// How a CTA's threads share out rows of nvec 16-byte vectors.  G lanes to a row (a power of two), or PACKED: nvec
+// lanes to a row, whatever nvec is, rows running on from warp to warp (24 vectors on 32 lanes leave a quarter of
+// every load, add and store unused, 5 on 8 three eighths).  Only for kernels in which the lanes of a row exchange
+// nothing.  What it costs is that a warp's rows are more, and it takes as many turns as the longest of them:
+//   gathers of bags      worth it up to 5/8 of the lanes: 20 floats 13.3 -> 10.9 us and 151 -> 120, 40 floats
+//                        22.3 -> 18.4 and 241 -> 230; but 48 floats 245 -> 256, 96 floats 405 -> 452, 24 bf16 21 -> 24
+//   Adagrad server pass  always: step of 720 k occurrences, 20 / 24 / 40 / 48 / 96 floats 384 -> 374, 389 -> 385,
+//                        505 -> 481, 520 -> 511, 743 -> 729 (20 and 40 with the forward's gain)
+//   Adam server pass     up to 5/8: step of 5.2 M, 40 floats 1027 -> 998; 24 and 96 floats 774 -> 789, 1630 -> 1664
+//   sparse update        always: server of 20 / 24 / 40 / 48 / 96 floats, Adam 219 -> 218, 227 -> 226, 316 -> 310,
+//                        330 -> 331, 514 -> 494, Adagrad 178 -> 177, 184 -> 183, 258 -> 252, 271 -> 267, 407 -> 396
+//   backward's walk      not at all (does not use it): 5 / 6 vectors 258 -> 268, 260 -> 268; 10, 12, 24 the same.
+inline int row_groups(int threads, int nvec, int G, bool packed) { return threads / (packed ? nvec : G); }
+inline bool row_packs(int threads, int nvec, int G) { return nvec <= 32 && row_groups(threads, nvec, G, true) > threads / G; }
+inline bool row_packs_narrow(int nvec, int G) { return G > 2 && nvec * 8 <= G * 5; }
+template <int THREADS, int G, bool PACKED>
+struct RowLanes {
+  int lg, grp, groups;  // vector of the row, row of the CTA, rows per CTA; grp >= groups: a thread left over
+  __device__ __forceinline__ explicit RowLanes(int nvec) {
+    lg = PACKED ? (int)threadIdx.x % nvec : (int)threadIdx.x & (G - 1);
+    grp = PACKED ? (int)threadIdx.x / nvec : (int)threadIdx.x / G;
+    groups = PACKED ? THREADS / nvec : THREADS / G;
+  }
+  __device__ __forceinline__ bool on() const { return !PACKED || grp < groups; }
+};
+
 __device__ __forceinline__ float4 ldg_f4(const float* p) {
   return __ldg(reinterpret_cast<const float4*>(p));
 }

@@ -147,8 +147,8 @@ inline int stride_below(int G, bool bf16) {  // ids per bag
   if (bf16) return G >= 32 ? 8 : (G == 16 ? 5 : (G == 8 ? 4 : 0));
   return G >= 16 ? 16 : (G == 8 ? 6 : (G == 4 ? 3 : 0));
 }
-inline int stride_waves(int G, bool bf16, int64_t n_bags, int64_t nnz) {
-  const int64_t per_wave = (int64_t)kNumSM * kFlatCtas * (kFlatThreads / G);
+inline int stride_waves(int G, int64_t bags_per_cta, bool bf16, int64_t n_bags, int64_t nnz) {
+  const int64_t per_wave = (int64_t)kNumSM * kFlatCtas * bags_per_cta;
   const int64_t W = n_bags / per_wave;
   if (W < 8 || nnz >= stride_below(G, bf16) * n_bags) return 0;
   const int64_t waves = (W + 5) / 10;
@@ -214,7 +214,7 @@ __device__ __forceinline__ void flat_range(const int64_t* __restrict__ bag_offse
 // One bag per lane group.  BY_FIELD: a CTA takes the bags of ONE field of consecutive samples and
 // consecutive CTAs stay on that field (bag = sample * fields + field), so that what is resident
 // on an SM and in L2 at one time draws from one field's hot rows.
-template <int G, bool BF16, bool BY_FIELD>
+template <int G, bool BF16, bool BY_FIELD, bool PACKED>
 __global__ void __launch_bounds__(kFlatThreads, kFlatCtas)
 embbag_fwd_flat_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
                        const int32_t* __restrict__ row_ids, int64_t nnz,
@@ -222,16 +222,17 @@ embbag_fwd_flat_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
                        float* __restrict__ pooled, int32_t* status, int fields, int64_t sample_blocks, bool chained) {
   if (chained) pdl_sync();  // (beside a kernel that it depends on the start of, it must not wait for its end)
   constexpr int EPV = BF16 ? 8 : 4;
-  const int lg = threadIdx.x & (G - 1);
+  const int nvec = dim / EPV;
+  const RowLanes<kFlatThreads, G, PACKED> lanes(nvec);
+  const int lg = lanes.lg;
   int64_t bag;
   if (BY_FIELD) {
     const int64_t f = blockIdx.x / sample_blocks, sb = blockIdx.x % sample_blocks;
-    bag = (sb * (kFlatThreads / G) + (threadIdx.x / G)) * fields + f;
+    bag = (sb * lanes.groups + lanes.grp) * fields + f;
   } else {
-    bag = (int64_t)blockIdx.x * (kFlatThreads / G) + (threadIdx.x / G);
+    bag = (int64_t)blockIdx.x * lanes.groups + lanes.grp;
   }
-  if (bag >= n_bags) return;
-  const int nvec = dim / EPV;
+  if (!lanes.on() || bag >= n_bags) return;
   int32_t begin, len;
   flat_range(bag_offsets, bag, nnz, lg, status, begin, len);
   bool bad = false;
@@ -247,7 +248,7 @@ embbag_fwd_flat_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
 // bag's rows are requested (30 fields x 4.5 ids x 128-byte rows: 1.06 -> 0.84 ms).  The loop is written out in one piece on purpose: at 32 registers the form of
 // the source decides what the compiler keeps in flight, and two tidier versions of this same loop
 // (the bag's sum in a helper, the offsets held as raw 64-bit values) measured 1.07 - 1.21 ms.
-template <int G, bool BF16>
+template <int G, bool BF16, bool PACKED>
 __global__ void __launch_bounds__(kFlatThreads, kFlatCtas)
 embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
                          const int32_t* __restrict__ row_ids, int64_t nnz,
@@ -256,9 +257,11 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
   if (chained) pdl_sync();  // (beside a kernel that it depends on the start of, it must not wait for its end)
   constexpr int EPV = BF16 ? 8 : 4;
   constexpr int PAIRS = EPV / 2;
-  constexpr int GPB = kFlatThreads / G;  // groups (bags) per CTA and turn
-  const int lg = threadIdx.x & (G - 1);
   const int nvec = dim / EPV;
+  const RowLanes<kFlatThreads, G, PACKED> lanes(nvec);
+  if (!lanes.on()) return;
+  const int GPB = lanes.groups;  // groups (bags) per CTA and turn
+  const int lg = lanes.lg;
   const uint32_t limit = (uint32_t)n_rows;
   const bool lane_on = lg < nvec;
   const uint4* tbl = static_cast<const uint4*>(table);
@@ -278,7 +281,7 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
     b0 = (int32_t)begin;  // nnz < 2^31
     ln = (int32_t)(end - begin);
   };
-  uint32_t q = blockIdx.x * GPB + threadIdx.x / G;
+  uint32_t q = blockIdx.x * GPB + lanes.grp;
   int32_t bag, begin, len;
   range_of(q, bag, begin, len);
   bool bad = false;
@@ -326,12 +329,12 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
   if (bad) set_status(status, ANTDT_ERR_ID_OUT_OF_RANGE);
 }
 
-template <int G, int VPL, bool BF16>
+template <int G, int VPL, bool BF16, bool PACKED>
 void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_ids, int64_t nnz,
                 const int64_t* bag_offsets, int64_t n_bags, float* pooled, int32_t* status,
                 cudaStream_t s, int fields, bool chained) {
   constexpr bool flat = VPL == 1;  // rows of up to 512 bytes
-  const int64_t gpb = (flat ? kFlatThreads : kFwdThreads) / G;
+  const int64_t gpb = row_groups(flat ? kFlatThreads : kFwdThreads, dim / (BF16 ? 8 : 4), G, PACKED);
   int64_t grid = (n_bags + gpb - 1) / gpb, sample_blocks = 0;
   if (fields > 0 && n_bags % fields == 0) {
     sample_blocks = (n_bags / fields + gpb - 1) / gpb;
@@ -339,15 +342,15 @@ void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_i
   } else {
     fields = 0;
   }
-  const int waves = flat && fields == 0 ? stride_waves(G, BF16, n_bags, nnz) : 0;
+  const int waves = flat && fields == 0 ? stride_waves(G, gpb, BF16, n_bags, nnz) : 0;
   if (waves > 0) {
-    ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_stride_kernel<G, BF16>), (unsigned)(kNumSM * kFlatCtas * waves),
+    ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_stride_kernel<G, BF16, PACKED>), (unsigned)(kNumSM * kFlatCtas * waves),
                  kFlatThreads, 0, s, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, chained);
   } else if (flat && fields > 0) {
-    ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_flat_kernel<G, BF16, true>), (unsigned)grid, kFlatThreads, 0, s,
+    ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_flat_kernel<G, BF16, true, PACKED>), (unsigned)grid, kFlatThreads, 0, s,
                  table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, fields, sample_blocks, chained);
   } else if (flat) {
-    ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_flat_kernel<G, BF16, false>), (unsigned)grid, kFlatThreads, 0, s,
+    ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_flat_kernel<G, BF16, false, PACKED>), (unsigned)grid, kFlatThreads, 0, s,
                  table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, fields, sample_blocks, chained);
   } else if (fields > 0) {
     ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_kernel<G, VPL, BF16, true>), (unsigned)grid, kFwdThreads, 0, s,
@@ -363,7 +366,11 @@ int32_t dispatch_fwd(int nvec, const void* table, int64_t n_rows, int dim, const
                      int64_t nnz, const int64_t* bag_offsets, int64_t n_bags, float* pooled,
                      int32_t* status, cudaStream_t s, int fields, bool chained) {
 #define FWD_CASE(G, VPL)                                                                      \
-  launch_fwd<G, VPL, BF16>(table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled,     \
+  if (VPL == 1 && row_packs_narrow(nvec, G))                                                  \
+    launch_fwd<G, VPL, BF16, (VPL == 1 && G > 2)>(table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, \
+                                                  s, fields, chained);                        \
+  else                                                                                        \
+  launch_fwd<G, VPL, BF16, false>(table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled,     \
                            status, s, fields, chained);                                       \
   return ANTDT_OK;
   if (nvec <= 1) { FWD_CASE(1, 1) }

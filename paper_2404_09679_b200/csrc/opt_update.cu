@@ -16,18 +16,20 @@ constexpr int kOptThreads = 256;
 // from two rows a stride apart; Adagrad is faster with one row and the higher occupancy.
 constexpr int kOptRowsAdam = 2;
 
-template <int G, int VPL, bool ADAM, bool BF16>
+template <int G, int VPL, bool ADAM, bool BF16, bool PACKED>
 __global__ void __launch_bounds__(kOptThreads)
 sparse_opt_kernel(void* table, int64_t n_rows, int dim, const int32_t* __restrict__ ids,
                   const float* __restrict__ grads, const int64_t* __restrict__ n_ids_dev,
                   int64_t max_ids, OptParams p, float* state0, float* state1, int32_t* status) {
   pdl_sync();
-  const int lg = threadIdx.x & (G - 1);
   const int nvec = dim / 4;
+  const RowLanes<kOptThreads, G, PACKED> lanes(nvec);
+  if (!lanes.on()) return;
+  const int lg = lanes.lg;
   const int64_t n = min(*n_ids_dev, max_ids);
-  const int64_t stride = (int64_t)gridDim.x * (kOptThreads / G);
+  const int64_t stride = (int64_t)gridDim.x * lanes.groups;
   constexpr int R = (ADAM && VPL == 1) ? kOptRowsAdam : 1;
-  for (int64_t k0 = (int64_t)blockIdx.x * (kOptThreads / G) + threadIdx.x / G; k0 < n; k0 += R * stride) {
+  for (int64_t k0 = (int64_t)blockIdx.x * lanes.groups + lanes.grp; k0 < n; k0 += R * stride) {
     int64_t row[R];
     bool ok[R];
 #pragma unroll
@@ -162,16 +164,16 @@ void launch_rowwise(bool bf16, void* table, int64_t n_rows, int dim, const int32
                  0, s, table, n_rows, dim, ids, grads, n_ids_dev, max_ids, p, state0, status);
 }
 
-template <int G, int VPL>
+template <int G, int VPL, bool PACKED>
 void launch_opt(bool adam, bool bf16, void* table, int64_t n_rows, int dim, const int32_t* ids,
                 const float* grads, const int64_t* n_ids_dev, int64_t max_ids, const OptParams& p,
                 float* state0, float* state1, int32_t* status, cudaStream_t s) {
-  const int64_t gpb = kOptThreads / G;
+  const int64_t gpb = row_groups(kOptThreads, dim / 4, G, PACKED);
   const int64_t want = (max_ids + gpb - 1) / gpb;
   const int64_t cap = (int64_t)kNumSM * 16;
   const unsigned grid = (unsigned)(want > cap ? cap : want);
 #define OPT_GO(A, B)                                                                            \
-  ANTDT_LAUNCH(A ? "sparse_adam" : "sparse_adagrad", (sparse_opt_kernel<G, VPL, A, B>), grid,   \
+  ANTDT_LAUNCH(A ? "sparse_adam" : "sparse_adagrad", (sparse_opt_kernel<G, VPL, A, B, PACKED>), grid,   \
                kOptThreads, 0, s, table, n_rows, dim, ids, grads, n_ids_dev, max_ids, p, state0, \
                state1, status)
   if (adam) { if (bf16) OPT_GO(true, true); else OPT_GO(true, false); }
@@ -222,8 +224,12 @@ extern "C" int32_t antdt_sparse_opt_update(void* table, int32_t dtype, int64_t n
     return cuda_ok();
   }
 #define OPT_CASE(G, VPL)                                                                       \
-  launch_opt<G, VPL>(adam, bf16, table, n_rows, dim, ids, grads, n_ids_dev, max_ids, p, state0, \
-                     state1, dev_status, s);
+  if (VPL == 1 && G > 2 && row_packs(kOptThreads, nvec, G))                                    \
+    launch_opt<G, VPL, (VPL == 1 && G > 2)>(adam, bf16, table, n_rows, dim, ids, grads, n_ids_dev, max_ids, p, state0, \
+                                            state1, dev_status, s);                            \
+  else                                                                                         \
+    launch_opt<G, VPL, false>(adam, bf16, table, n_rows, dim, ids, grads, n_ids_dev, max_ids, p, state0, state1,       \
+                              dev_status, s);
   if (nvec <= 1) { OPT_CASE(1, 1) }
   else if (nvec <= 2) { OPT_CASE(2, 1) }
   else if (nvec <= 4) { OPT_CASE(4, 1) }
