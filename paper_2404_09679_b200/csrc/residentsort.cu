@@ -20,13 +20,14 @@
 // ascending order: those runs ARE the aggregation's merge order.  In a step it is written on the way
 // and the merge's four kernels (agg_range.cu) are not needed.
 //
-// What a pass costs is the latency of its steps, 7 us for up to 1500 pairs a CTA, 25 us for 12288; the
-// cost that grows with the square of the CTAs (reading everybody's counts) keeps them to one per SM.  Small inputs
-// (up to 16 CTAs of 2048) run as one thread-block cluster: counts, pairs and barriers go through
-// distributed shared memory (a barrier 0.3 us against 1.3).
+// What a pass costs is the latency of its steps, 4 us in a cluster, 9 to 13 us with one CTA per SM; the
+// cost that grows with the square of the CTAs (reading everybody's counts, 2 to 5 us) keeps them to one per SM.  Small
+// inputs (up to 16 CTAs of 2048) run as one thread-block cluster: counts, pairs and barriers go through
+// distributed shared memory (a barrier 0.7 us against 1.6).  Twice the threads in the one-CTA-per-SM form: the sort
+// 2 us faster, a forward beside it 22 us slower.
 // Measured (in brackets the kernels it replaced: sort, and merge order where a step makes it): 10 k
-// occurrences of 4 workers over 80 k rows 17 us (37 + 35); 426 k of 8 over 26 M 58 us, 70 with a step's forward
-// beside it (75 + 62); 1.2 M of one worker over 1 M 66 - 70 us (113).
+// occurrences of 4 workers over 80 k rows 14 us (37 + 35); 426 k of 8 over 26 M 47 us, 64 with a step's forward
+// beside it (75 + 62); 1.2 M of one worker over 1 M 59 us (113).
 //
 // The CTAs wait for one another, so the launch is a cluster or a cooperative one (all CTAs resident
 // or none started).  A wait through memory is bounded all the same (kSpinLimit) and raises
@@ -101,12 +102,6 @@ __device__ __forceinline__ uint32_t ld_remote(uint32_t addr) {
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
   return v;
 }
-__device__ __forceinline__ uint4 ld_remote4(uint32_t addr) {
-  uint4 v;
-  asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-  return v;
-}
 __device__ __forceinline__ void st_remote2(uint32_t addr, uint32_t x, uint32_t y) {
   asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(x), "r"(y) : "memory");
 }
@@ -123,15 +118,9 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* warp_tot, u
   __syncthreads();  // an earlier scan's readers are done
   if (lane == 31) warp_tot[w] = incl;
   __syncthreads();
-  uint32_t pre = 0, tot = 0;
-#pragma unroll
-  for (int i = 0; i < kWarps; ++i) {
-    const uint32_t t = warp_tot[i];
-    pre += i < w ? t : 0u;
-    tot += t;
-  }
-  if (total) *total = tot;
-  return incl - v + pre;
+  const uint32_t x = lane < kWarps ? warp_tot[lane] : 0u;
+  if (total) *total = __reduce_add_sync(0xffffffffu, x);
+  return incl - v + __reduce_add_sync(0xffffffffu, lane < w ? x : 0u);
 }
 
 // Stable rank of every valid item among the items of its warp with the same digit; leaves the
@@ -204,12 +193,37 @@ __device__ __forceinline__ void all_barrier(uint32_t* counter, uint32_t target, 
 
 // Sums of the C published rows of counters and of those before `rank`, per counter (the
 // returned values are those of counter threadIdx.x).  rows: 16-bit counters, kBins to a row, of
-// which the first nb are used.  A thread takes eight counters (one 16-byte load) of every 64th (or
-// 32nd, ...) part of the rows: this is the one step whose cost grows with the square of the CTAs.
+// which the first nb are used.
+//   grid      a thread takes eight counters (one 16-byte load) of every 64th (or 32nd, ...) part of the
+//             rows: this is the one step whose cost grows with the square of the CTAs
+//   cluster   a thread takes two counters of every row, all rows requested at once, and adds them up as
+//             they are packed (there are at most 2^15 pairs): no sums to meet in shared memory.  With the
+//             grid's way a pass of 10 k pairs had 1.6 - 1.9 us of its 4.6 here; step 34.1 -> 30.7 us
 template <bool CLUSTER>
 __device__ __forceinline__ void sum_rows(Smem& S, const uint16_t* rows, uint32_t nb, int rank, int C,
                                          uint32_t& total, uint32_t& before) {
   const int tid = threadIdx.x;
+  if (CLUSTER) {
+    static_assert((int64_t)kResMaxCluster * kClusterItems * kThreads < 65536, "packed sums");
+    if (2u * tid < nb) {
+      uint32_t x[kResMaxCluster];
+#pragma unroll
+      for (int c = 0; c < kResMaxCluster; ++c)
+        x[c] = c < C ? ld_remote(remote(reinterpret_cast<const uint32_t*>(S.row) + tid, (uint32_t)c)) : 0u;
+      uint32_t t = 0, b = 0;
+#pragma unroll
+      for (int c = 0; c < kResMaxCluster; ++c) {
+        t += x[c];
+        b += c < rank ? x[c] : 0u;
+      }
+      S.cnt[2 * tid] = t & 0xffffu; S.cnt[2 * tid + 1] = t >> 16;
+      S.base[2 * tid] = b & 0xffffu; S.base[2 * tid + 1] = b >> 16;
+    }
+    __syncthreads();
+    total = tid < (int)nb ? S.cnt[tid] : 0u;
+    before = tid < (int)nb ? S.base[tid] : 0u;
+    return;
+  }
   const int q = nb >= 16 ? (int)(nb >> 3) : 2;  // a power of two: 16-byte columns of a row
   const int col = tid & (q - 1), grp = tid / q, groups = kThreads / q;
   S.cnt[tid] = 0u;
@@ -224,9 +238,7 @@ __device__ __forceinline__ void sum_rows(Smem& S, const uint16_t* rows, uint32_t
     uint4 x[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      x[i] = c0 + i * groups >= C ? make_uint4(0u, 0u, 0u, 0u)
-             : CLUSTER ? ld_remote4(remote(S.row, (uint32_t)(c0 + i * groups)) + 16u * col)
-                       : __ldcg(p + (size_t)(c0 + i * groups) * kRow);
+      x[i] = c0 + i * groups >= C ? make_uint4(0u, 0u, 0u, 0u) : __ldcg(p + (size_t)(c0 + i * groups) * kRow);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const uint32_t on = c0 + i * groups < rank ? 0xffffffffu : 0u;
@@ -250,13 +262,14 @@ __device__ __forceinline__ void sum_rows(Smem& S, const uint16_t* rows, uint32_t
 }
 
 // First slot of every digit for this CTA: everybody's counts of smaller digits, then those of this
-// digit in CTAs of smaller rank.
+// digit in CTAs of smaller rank.  Grid: less the place of the digit's first pair among the CTA's own (S.loc).
 template <bool CLUSTER>
 __device__ __forceinline__ void digit_bases(Smem& S, const uint16_t* rows, uint32_t nb, int rank, int C) {
   uint32_t total, before;
   sum_rows<CLUSTER>(S, rows, nb, rank, C, total, before);
   const uint32_t ex = block_scan(threadIdx.x < nb ? total : 0u, S.warp_tot, nullptr);  // barriers inside
-  S.base[threadIdx.x] = ex + before;
+  if (threadIdx.x < nb) S.base[threadIdx.x] = ex + before - (CLUSTER ? 0u : S.loc[threadIdx.x]);
+  __syncthreads();
 }
 
 // What a CTA asks for before it knows the workers' ranges: the offsets of kWindow bags around the
@@ -356,9 +369,7 @@ __device__ __forceinline__ void chunk_bags(Smem& S, const ResidentSortArgs& a, c
     }
     if (lane == 0) S.warp_tot[wp] = carry;
     __syncthreads();
-    uint32_t pre = 1;
-#pragma unroll
-    for (int i = 0; i < kWarps; ++i) pre = max(pre, i < wp ? S.warp_tot[i] : 0u);
+    const uint32_t pre = max(1u, __reduce_max_sync(0xffffffffu, lane < wp ? S.warp_tot[lane] : 0u));
 #pragma unroll
     for (int i = 0; i < IPT; ++i) {
       if (IPT > 4 && i % 4 == 0 && i * 32 >= valid) break;
@@ -368,29 +379,34 @@ __device__ __forceinline__ void chunk_bags(Smem& S, const ResidentSortArgs& a, c
 }
 
 // Ranks of the CTA's items among those of equal digit: inside the warp (rk), the prefix over the
-// warps (S.wh), and the CTA's count of every digit, stored to my_row and returned (thread's digit).
+// warps (S.wh), and the CTA's count of every digit, stored to my_row; returned: those of digits 2 tid (low
+// half) and 2 tid + 1.  clear: the masks have to be cleared (the ranking leaves them cleared).
 template <int IPT>
 __device__ __forceinline__ uint32_t rank_and_publish(Smem& S, const uint32_t (&k)[IPT], int valid, int shift, uint32_t nb,
-                                                 uint16_t* my_row, unsigned short (&rk)[IPT]) {
+                                                 uint16_t* my_row, unsigned short (&rk)[IPT], bool clear) {
   const int tid = threadIdx.x, wp = tid >> 5;
   __syncthreads();  // marks, counters and bases of the step before have been read
-  for (uint32_t i = tid; i < kWarps * nb / 2; i += kThreads) reinterpret_cast<uint32_t*>(S.wh)[i] = 0u;
-  for (uint32_t i = tid; i < kWarps * nb; i += kThreads) S.mm()[i] = 0u;
+  const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+  for (uint32_t i = tid; i < kWarps * nb / 8; i += kThreads) reinterpret_cast<uint4*>(S.wh)[i] = none;
+  if (clear)
+    for (uint32_t i = tid; i < kWarps * nb / 4; i += kThreads) reinterpret_cast<uint4*>(S.mm())[i] = none;
   __syncthreads();
   warp_rank<IPT>(k, valid, shift, nb - 1u, S.wh + wp * nb, S.mm() + wp * nb, rk);
   __syncthreads();
+  // two digits to a thread, as they are packed: a CTA holds fewer than 2^16 pairs
   uint32_t sum = 0;
-  if (tid < nb) {
+  if (2u * tid < nb) {
+    uint32_t* const wh2 = reinterpret_cast<uint32_t*>(S.wh) + tid;
     uint32_t t[kWarps];
 #pragma unroll
-    for (int i = 0; i < kWarps; ++i) t[i] = S.wh[i * nb + tid];
+    for (int i = 0; i < kWarps; ++i) t[i] = wh2[i * (nb / 2)];
 #pragma unroll
     for (int i = 0; i < kWarps; ++i) {
-      S.wh[i * nb + tid] = (unsigned short)sum;
+      wh2[i * (nb / 2)] = sum;
       sum += t[i];
     }
   }
-  my_row[tid] = (uint16_t)sum;
+  if (tid < kBins / 2) reinterpret_cast<uint32_t*>(my_row)[tid] = sum;
   return sum;
 }
 
@@ -413,12 +429,11 @@ __device__ __forceinline__ uint32_t sort_passes_by_row(Smem& S, uint32_t (&k)[IP
     const int bits = (key_bits - shift + (P - p) - 1) / (P - p);
     const uint32_t nb = 1u << bits, dmask = nb - 1u;
     unsigned short rk[IPT];
-    const uint32_t count = rank_and_publish<IPT>(S, k, valid, shift, nb, my_row, rk);
+    const uint32_t count = rank_and_publish<IPT>(S, k, valid, shift, nb, my_row, rk, !CLUSTER || p == 0);
     arrivals += C;
     if (CLUSTER) {
       all_barrier<CLUSTER>(counter, arrivals, status);
       digit_bases<CLUSTER>(S, hist, nb, cta, C);
-      __syncthreads();
 #pragma unroll
       for (int i = 0; i < IPT; ++i) {
         if (IPT > 4 && i % 4 == 0 && i * 32 >= valid) break;
@@ -434,8 +449,11 @@ __device__ __forceinline__ uint32_t sort_passes_by_row(Smem& S, uint32_t (&k)[IP
       // memory, so that consecutive threads store to consecutive slots: a store of a warp touches the
       // lines of a few digits instead of 32.
       grid_arrive(counter);
-      const uint32_t loc = block_scan(tid < (int)nb ? count : 0u, S.warp_tot, nullptr);
-      S.loc[tid] = loc;
+      const uint32_t loc = block_scan((count & 0xffffu) + (count >> 16), S.warp_tot, nullptr);
+      if (tid < kBins / 2) {
+        S.loc[2 * tid] = loc;
+        S.loc[2 * tid + 1] = loc + (count & 0xffffu);
+      }
       __syncthreads();
       uint2* const stage = S.stage();
 #pragma unroll
@@ -448,8 +466,6 @@ __device__ __forceinline__ uint32_t sort_passes_by_row(Smem& S, uint32_t (&k)[IP
       }
       grid_wait(counter, arrivals, status);
       digit_bases<CLUSTER>(S, hist, nb, cta, C);
-      S.base[tid] -= loc;
-      __syncthreads();
 #pragma unroll 4
       for (int j = tid; j < n_mine; j += kThreads) {
         const uint2 kv = stage[j];
@@ -519,7 +535,7 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
     const int64_t share = (a.n_bags + gridDim.x - 1) / gridDim.x;
     const int64_t b_end = min(a.n_bags, (cta + 1) * share);
     bool bad = false;
-#pragma unroll 4
+#pragma unroll 8
     for (int64_t b = cta * share + tid; b < b_end; b += kThreads) {
       const int64_t lo = __ldg(a.bag_offsets + b), hi = __ldg(a.bag_offsets + b + 1);
       bad |= lo < 0 || hi < lo || hi > a.nnz;
@@ -635,11 +651,13 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
       const unsigned heads = __ballot_sync(0xffffffffu, h), all = __ballot_sync(0xffffffffu, ok);
       heads_warp += __popc(heads);
       rows_warp += __popc(__ballot_sync(0xffffffffu, r));
+      if (K == 1) {  // a pair's rank is its place, a run's the heads so far
+        if (ok) ranks[j] = (uint32_t)(i * 32 + lane) | (heads_warp - __popc(heads) + __popc(heads & lt) + (h ? 1u : 0u)) << 16;
+        continue;
+      }
       unsigned peers = 0;
       uint32_t old = 0, old_h = 0;
-      if (K == 1) {
-        peers = all;
-      } else if (K <= kMatchWorkers) {
+      if (K <= kMatchWorkers) {
         if (ok) peers = __match_any_sync(all, d);
       } else {
         if (ok) atomicOr(mm + d, 1u << lane);
@@ -661,14 +679,18 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
       if (ok) ranks[j] = (old + __popc(peers & lt)) | (old_h + __popc(peers & heads & lt) + (h ? 1u : 0u)) << 16;
     }
   }
-  if (lane == 0) { S.warp_a[wp] = heads_warp; S.warp_b[wp] = rows_warp; }
-  __syncthreads();
-  uint32_t heads_pre = 0, rows_pre = 0, heads_cta = 0, rows_cta = 0;
-#pragma unroll
-  for (int i = 0; i < kWarps; ++i) {
-    heads_pre += i < wp ? S.warp_a[i] : 0u; heads_cta += S.warp_a[i];
-    rows_pre += i < wp ? S.warp_b[i] : 0u; rows_cta += S.warp_b[i];
+  if (lane == 0) {
+    S.warp_a[wp] = heads_warp;
+    S.warp_b[wp] = rows_warp;
+    if (K == 1) {
+      S.wh[wp * kB] = (unsigned short)valid;
+      S.wh[wp * kB + Kp] = (unsigned short)heads_warp;
+    }
   }
+  __syncthreads();
+  const uint32_t wa = lane < kWarps ? S.warp_a[lane] : 0u, wb = lane < kWarps ? S.warp_b[lane] : 0u;
+  const uint32_t heads_cta = __reduce_add_sync(0xffffffffu, wa), heads_pre = __reduce_add_sync(0xffffffffu, lane < wp ? wa : 0u);
+  const uint32_t rows_cta = __reduce_add_sync(0xffffffffu, wb), rows_pre = __reduce_add_sync(0xffffffffu, lane < wp ? wb : 0u);
   if (tid < (int)kB) {
     uint32_t sum = 0;
     uint32_t t[kWarps];
@@ -851,13 +873,9 @@ resident_merge_kernel(const __grid_constant__ ResidentMergeArgs a) {
   }
   if (lane == 0) { S.warp_a[wp] = kept_warp; S.warp_b[wp] = rows_warp; }
   __syncthreads();
-  uint32_t rows_pre = 0, kept_cta = 0, rows_cta = 0;
-#pragma unroll
-  for (int i = 0; i < kWarps; ++i) {
-    kept_cta += S.warp_a[i];
-    rows_pre += i < wp ? S.warp_b[i] : 0u;
-    rows_cta += S.warp_b[i];
-  }
+  const uint32_t wb = lane < kWarps ? S.warp_b[lane] : 0u;
+  const uint32_t kept_cta = __reduce_add_sync(0xffffffffu, lane < kWarps ? S.warp_a[lane] : 0u);
+  const uint32_t rows_cta = __reduce_add_sync(0xffffffffu, wb), rows_pre = __reduce_add_sync(0xffffffffu, lane < wp ? wb : 0u);
   uint16_t* const my_row = CLUSTER ? S.row : a.hist + (size_t)cta * kBins;
   if (tid < 16) my_row[tid] = (uint16_t)(tid == 0 ? kept_cta : (tid == 1 ? rows_cta : 0u));
   arrivals += C;
