@@ -301,15 +301,19 @@ constexpr int kScatItems = kSortTile / kScatThreads;  // 8
 constexpr int kScatWarps = kScatThreads / 32;         // 16
 constexpr size_t kScatSmem = 3 * kSortMaxBins * 4 + kScatWarps * kSortMaxBins * 2 + 2 * kSortTile * 4 + 64;
 
-// Lanes of the warp whose digit (BITS wide) equals this lane's: one vote per bit.
+// Lanes of the warp whose digit (BITS wide) equals this lane's: one vote per bit.  Four instructions a bit (bit
+// to predicate, vote, complement where the bit is 0, and): the ALU is the pipe that this kernel keeps busiest, and a
+// mask formed from the bit's value takes two more (three passes of 52 M pairs 1209 -> 1183 us, of 33 M 786 -> 768, of
+// 2.4 M in 90 segments 74 -> 69, of 4.2 M 103 -> 96).
 template <int BITS>
 __device__ __forceinline__ unsigned digit_peers(uint32_t d) {
   unsigned m = 0xffffffffu;
 #pragma unroll
-  for (int b = 0; b < BITS; ++b) {
-    const unsigned one = (d >> b) & 1u;
-    m &= __ballot_sync(0xffffffffu, one != 0u) ^ (one - 1u);
-  }
+  for (int b = 0; b < BITS; ++b)
+    asm volatile(
+        "{\n.reg .pred p;\n.reg .b32 t, x;\nand.b32 t, %1, %2;\nsetp.ne.u32 p, t, 0;\n"
+        "vote.sync.ballot.b32 x, p, -1;\n@!p not.b32 x, x;\nand.b32 %0, %0, x;\n}"
+        : "+r"(m) : "r"(d), "r"(1u << b));
   return m;
 }
 
