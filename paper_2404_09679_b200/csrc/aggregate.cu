@@ -323,6 +323,9 @@ agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __rest
                   float* __restrict__ agg_out) {
   pdl_sync();
   extern __shared__ float s_w[];  // the K weights
+  // requested with the weights, not behind them
+  const uint32_t rows_all = (uint32_t)*n_agg_dev;
+  const uint32_t total = (uint32_t)min(n_entries[1], in_cap);
   for (int i = threadIdx.x; i < K; i += blockDim.x) s_w[i] = weights[i];
   __syncthreads();
   constexpr int R = VPL == 1 ? kFusedRows : 1;  // rows a lane group has in flight
@@ -332,11 +335,10 @@ agg_update_kernel(const uint32_t* __restrict__ row_start, const uint32_t* __rest
   if (!lanes.on()) return;
   // 32-bit row numbers and slots (fewer than 2^31 of each): the kernel is bound by its instruction
   // stream and by the registers that live across the chain of loads
-  const uint32_t n = (uint32_t)min(*n_agg_dev, out_cap);
+  const uint32_t n = (uint32_t)min((int64_t)rows_all, out_cap);
   // where the capacity cuts rows off, the next row's start still ends the last one (the update, whose
   // result is flagged then, does without: it has no register to spare)
-  const uint32_t n_starts = UPDATE ? n : (uint32_t)*n_agg_dev;
-  const uint32_t total = (uint32_t)min(n_entries[1], in_cap);
+  const uint32_t n_starts = UPDATE ? n : rows_all;
   const uint32_t stride = gridDim.x * lanes.groups;
   for (uint32_t u0 = blockIdx.x * lanes.groups + lanes.grp; u0 < n; u0 += R * stride) {
     uint32_t s0[R], s1[R];

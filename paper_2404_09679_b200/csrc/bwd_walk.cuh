@@ -168,9 +168,8 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
   float* s_headp = reinterpret_cast<float*>(walk_smem);   // [TPS][dim] sum before the first run end
   float* s_carry = s_headp + (size_t)TPS * dim;           // [TPS][dim] sum after the last run end
   int64_t* s_bounds = reinterpret_cast<int64_t*>(s_carry + (size_t)TPS * dim);  // [K+1]
-  uint8_t* s_flag = reinterpret_cast<uint8_t*>(s_bounds + (K + 1));             // [TPS]
-  for (int i = threadIdx.x; i <= K; i += blockDim.x) s_bounds[i] = a.bounds[i];
-  __syncthreads();
+  float* s_scale = reinterpret_cast<float*>(s_bounds + (K + 1));                // [K]
+  uint8_t* s_flag = reinterpret_cast<uint8_t*>(s_scale + K);                    // [TPS]
   const int64_t n = a.n_host;
   const int lg = threadIdx.x & (G - 1);
   const int grp = threadIdx.x / G;
@@ -184,29 +183,52 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
   const uint32_t last_row = (uint32_t)(a.payload_limit - 1);
   float* my_headp = s_headp + (size_t)grp * dim;
 
+  // Everything that is found by the tile's number alone is requested before the first wait: a small input's walk is
+  // a chain of round trips to memory.
+  const int nv = in_range ? (int)min((int64_t)TILE, n - o_begin) : 0;
+  const uint32_t* pp = payload + (in_range ? o_begin : 0);
+  uint32_t cur[kRegs], ahead[kRegs];
+  auto ask = [&](uint32_t (&to)[kRegs], int block) {
+#pragma unroll
+    for (int i = 0; i < kRegs; ++i)
+      to[i] = __ldg(pp + min(block * kBlock + min(i * G + lg, kBlock - 1), max(nv - 1, 0)));
+  };
+  if (SHARED) ask(ahead, 0);
+  uint32_t h0 = 0, h1 = 0, h2 = 0;  // head bits from o_begin (TILE 16: from the word that holds it)
+  int32_t first_run = 0;
+  if (in_range) {
+    const uint32_t* hw = head_bits + (o_begin >> 5);
+    h0 = __ldg(hw);
+    h1 = __ldg(hw + 1);
+    if (TILE == 64) h2 = __ldg(hw + 2);
+    first_run = tile_first[tile];
+  }
+  for (int i = threadIdx.x; i <= K; i += blockDim.x) {
+    s_bounds[i] = a.bounds[i];
+    if (i < K) s_scale[i] = a.scales[i];
+  }
+  __syncthreads();
+
   // run heads of positions o_begin .. o_begin+TILE; entry r closes its run iff r+1 is a head
   uint64_t ends = 0;
   bool open_tail = false, started = false, last_tile = false;
-  int nv = 0, w = 0;
+  int w = 0;
   int32_t u = 0;  // run index (fewer than 2^31 occurrences, so fewer runs)
   if (in_range) {
-    nv = (int)min((int64_t)TILE, n - o_begin);
-    const uint32_t* hw = head_bits + (o_begin >> 5);
     last_tile = o_begin + TILE >= n;
     if (TILE == 64) {
-      const uint32_t h0 = __ldg(hw), h1 = __ldg(hw + 1), h2 = __ldg(hw + 2);
       const uint64_t heads = (uint64_t)h0 | ((uint64_t)h1 << 32);
       ends = (heads >> 1) | ((uint64_t)(h2 & 1u) << 63);
       open_tail = !last_tile && !(h2 & 1u);
       started = (h0 & 1u) != 0;
     } else {  // TILE < 32 and a power of two: the tile's bits and the next one lie in two words
-      const uint64_t heads = ((uint64_t)__ldg(hw) | ((uint64_t)__ldg(hw + 1) << 32)) >> (o_begin & 31);
+      const uint64_t heads = ((uint64_t)h0 | ((uint64_t)h1 << 32)) >> (o_begin & 31);
       ends = (heads >> 1) & ((1ull << (TILE & 63)) - 1ull);
       open_tail = !last_tile && !((heads >> (TILE & 63)) & 1ull);
       started = (heads & 1ull) != 0;
     }
     if (last_tile) ends = (ends & ((1ull << (nv - 1)) - 1ull)) | (1ull << (nv - 1));  // array end closes
-    u = run_index(tile_first[tile], o_begin);
+    u = run_index(first_run, o_begin);
     w = interval_of(s_bounds, K + 1, o_begin);
     if (w > K - 1) w = K - 1;
   }
@@ -221,7 +243,7 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
   float4 acc[VPL];
 #pragma unroll
   for (int k = 0; k < VPL; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-  float inv = in_range ? a.scales[w] : 0.f;
+  float inv = in_range ? s_scale[w] : 0.f;
 
   if (__all_sync(kFull, !in_range)) {
     // nothing to walk in this warp; it still joins the stretch's barrier below
@@ -232,13 +254,6 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
     // where the run that is open now goes when it closes; where the one after it goes
     float* dst = started ? out + (size_t)u * row_stride : my_headp;
     float* nxt = out + (size_t)(u + 1) * row_stride;
-    const uint32_t* pp = payload + (in_range ? o_begin : 0);
-    uint32_t cur[kRegs], ahead[kRegs];
-    auto ask = [&](uint32_t (&to)[kRegs], int block) {
-#pragma unroll
-      for (int i = 0; i < kRegs; ++i) to[i] = __ldg(pp + block * kBlock + min(i * G + lg, kBlock - 1));
-    };
-    if (SHARED) ask(ahead, 0);
 #pragma unroll 1
     for (int c = 0; c < TILE / CH; ++c) {
       uint32_t p[CH];
@@ -330,7 +345,7 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
         if (started || closed_any) {
           const int64_t o = o_begin + r;  // the run's worker is the worker of any of its entries
           while (w < K - 1 && o >= s_bounds[w + 1]) ++w;
-          if (u < a.out_cap) put_row<G, VPL>(out + (size_t)u * row_stride, acc, a.scales[w], lg, nvec);
+          if (u < a.out_cap) put_row<G, VPL>(out + (size_t)u * row_stride, acc, s_scale[w], lg, nvec);
         } else {
           put_row<G, VPL>(my_headp, acc, 1.f, lg, nvec);
         }
@@ -343,7 +358,7 @@ bwd_walk_kernel(const TileArgs a, const uint32_t* __restrict__ payload,
     if (open_tail) {  // the worker of the run that stays open: that of the tile's last entry
       const int64_t o = o_begin + nv - 1;
       while (w < K - 1 && o >= s_bounds[w + 1]) ++w;
-      inv = a.scales[w];
+      inv = s_scale[w];
     }
   }
 
@@ -423,14 +438,14 @@ void launch_bwd_walk_t(const TileArgs& a_in, const WalkScratch& ws_in, const cha
   // the tasks as the launch, at 256 it takes 5 us longer.
   ws.inline_fixup = TILE == kRedTileSmall && a.walk && a.fixup && a.tile_begin == 0 && a.tile_end == n_tiles && n_tiles > TPS &&
                     n_tiles <= kInlineFixStretches * TPS;
-  const size_t smem = 2 * (size_t)TPS * a.dim * 4 + 8 * ((size_t)a.K + 1) + TPS;
+  const size_t smem = 2 * (size_t)TPS * a.dim * 4 + 8 * ((size_t)a.K + 1) + 4 * (size_t)a.K + TPS;
   if (smem > 48 * 1024) {  // rows of 1024 floats: more than the default dynamic shared memory
     static bool attr_set[64] = {};
     int dev_id = 0;
     cudaGetDevice(&dev_id);
     if (!attr_set[dev_id & 63]) {
       cudaFuncSetAttribute(bwd_walk_kernel<G, VPL, TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(2 * (size_t)TPS * 1024 * 4 + 8 * ((size_t)kMaxSegments + 1) + TPS));
+                           (int)(2 * (size_t)TPS * 1024 * 4 + 8 * ((size_t)kMaxSegments + 1) + 4 * (size_t)kMaxSegments + TPS));
       attr_set[dev_id & 63] = true;
     }
   }

@@ -530,6 +530,7 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
   }
   BagWindow win;
   request_window(win, a, g0);
+  const int64_t raw0 = wp == 0 && lane <= K ? __ldg(a.bag_offsets + wso.v[lane] * (int64_t)F) : 0;
   // the offsets ascend inside [0, nnz]: each CTA checks a share
   {
     const int64_t share = (a.n_bags + gridDim.x - 1) / gridDim.x;
@@ -551,7 +552,7 @@ resident_sort_kernel(const __grid_constant__ ResidentSortArgs a, const __grid_co
       int64_t carry = 0;
       for (int i0 = 0; i0 <= K; i0 += 32) {
         const int i = i0 + lane;
-        const int64_t raw = i <= K ? __ldg(a.bag_offsets + wso.v[i] * (int64_t)F) : 0;
+        const int64_t raw = i0 == 0 ? raw0 : (i <= K ? __ldg(a.bag_offsets + wso.v[i] * (int64_t)F) : 0);
         if (cta == 0 && ((i == 0 && raw != 0) || (i == K && raw != a.nnz)))
           set_status(a.status, ANTDT_ERR_BAD_OFFSETS);
         int64_t x = max(raw, carry);
