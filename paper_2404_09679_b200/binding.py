@@ -24,6 +24,7 @@ OPTS = {"adagrad": OPT_ADAGRAD, "adam": OPT_ADAM, "rowwise_adagrad": OPT_ROWWISE
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libantdt.so")
 _lib = None
+_fwd = None  # _marshal.embbag_fwd, once the library is loaded
 
 EXPORTS = [
     "antdt_dds_create", "antdt_dds_destroy", "antdt_batch_sizes", "antdt_shard_plan",
@@ -92,7 +93,7 @@ class StepDesc(C.Structure):
 def lib() -> C.CDLL:
     """Loads libantdt.so (once).  A missing library is an error: build it with
     `python -m paper_2404_09679_b200.build`."""
-    global _lib
+    global _lib, _fwd
     if _lib is None:
         if not os.path.exists(_LIB_PATH):
             raise AntdtError(ERR_STATE, f"{_LIB_PATH} is not built (python -m paper_2404_09679_b200.build)")
@@ -164,6 +165,12 @@ def lib() -> C.CDLL:
                    "antdt_read_status", "antdt_profile_enable", "antdt_profile_kernels",
                    "antdt_profile_get"):
             getattr(L, fn).restype = I32
+        try:
+            from . import _marshal
+        except ImportError as e:
+            raise AntdtError(ERR_STATE, f"_marshal.so is not built (python -m paper_2404_09679_b200.build): {e}")
+        _marshal.bind(C.cast(L.antdt_embbag_fwd, P).value)
+        _fwd = _marshal.embbag_fwd
         _lib = L
     return _lib
 
@@ -339,6 +346,14 @@ def antdt_dd_solve(n_devices, speeds, global_batch: int, batch_min, batch_max, a
 
 # ---- device path ---------------------------------------------------------------------------
 def antdt_embbag_fwd(table, row_ids, bag_offsets, pooled, dev_status=None, stream=None):
+    if _fwd is None:
+        lib()
+    rc = _fwd(table, row_ids, bag_offsets, pooled, dev_status, stream)
+    if rc == OK:
+        return
+    if rc > 0:
+        raise AntdtError(rc, "antdt_embbag_fwd")
+    # an argument that is not a plain contiguous tensor
     V, D = table.shape
     n_bags = bag_offsets.numel() - 1
     _check(lib().antdt_embbag_fwd(_dp(table), _dtype_code(table), V, D, _dp(row_ids),

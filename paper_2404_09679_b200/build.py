@@ -7,12 +7,14 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INC = os.path.join(os.path.dirname(HERE), "include")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libantdt.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")  # Python objects -> the entry points' arguments
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INC, "-I", CSRC]
@@ -28,8 +30,18 @@ def _newest_dep():
     return max(os.path.getmtime(p) for p in deps)
 
 
+def _marshal_command():
+    import torch  # its headers and libraries
+    root = os.path.dirname(torch.__file__)
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], "/usr/local/cuda/include", INC]
+    return (["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+            + [x for i in inc for x in ("-isystem", i)] + [os.path.join(CSRC, "marshal.cpp"), "-o", MARSHAL, "-L", os.path.join(root, "lib"),
+               "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
+
+
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) -> str:
-    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_dep():
+    if not force and all(os.path.exists(p) and os.path.getmtime(p) >= _newest_dep() for p in (LIB, MARSHAL)):
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     os.makedirs(OBJ, exist_ok=True)
@@ -50,6 +62,12 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
         if verbose:
             print(" ".join(cmd), flush=True)
         procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))
+    src = os.path.join(CSRC, "marshal.cpp")
+    stale = not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL) < max(os.path.getmtime(src), os.path.getmtime(os.path.join(INC, "antdt.h")))
+    if force or stale:
+        procs.append((src, subprocess.Popen(_marshal_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))
+    else:
+        os.utime(MARSHAL)
     failed = False
     for src, p in procs:
         out = p.communicate()[0].decode()
