@@ -25,39 +25,68 @@ size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 // ---------------------------------------------------------------------------------------
 struct WeightBlob { float w[kRangeMaxWorkers]; };  // the workers' weights, a kernel parameter
 
+// G lanes look for a boundary together: G probes a step, so a list of 10^5 entries takes 6 round trips with 8 lanes and
+// 17 with one (1.7 k boundaries 9 -> 6 us, 7.8 k 10 -> 6, 39 k 14 -> 13).  Where the boundaries are many, one lane each
+// keeps the machine as busy with less to read (78 k: 16 us against 19).  Every entry comparing itself with the one before,
+// without any search, took 4 us for 134 k entries but 60 for 27 M, where the searches take 16.
+constexpr int64_t kSplitTogether = 50000;  // boundaries up to which eight lanes look for one
+// On the way: what the later kernels want cleared (head bits, tile_first) instead of by two memsets, behind which a
+// dependent launch waits.
+template <int G>
 __global__ void __launch_bounds__(kRaThreads)
 range_split_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ wuo_in, int K,
                    int64_t in_cap, int r_log2, int64_t P, int64_t n_rows, uint32_t dropped,
                    int64_t* __restrict__ wuo_out, int32_t* __restrict__ bnd, const WeightBlob weights,
-                   float* __restrict__ weights_out, int32_t* status) {
+                   float* __restrict__ weights_out, uint32_t* __restrict__ zero_a, int64_t n_a,
+                   uint32_t* __restrict__ zero_b, int64_t n_b, int32_t* status) {
   pdl_sync();
   __shared__ int64_t s_wuo[kRangeMaxWorkers + 1];
   if (blockIdx.x == 0 && weights_out && threadIdx.x < K) weights_out[threadIdx.x] = weights.w[threadIdx.x];
-  if (threadIdx.x == 0) {  // ascending and inside [0, in_cap], whatever came in
-    int64_t prev = 0;
-    for (int i = 0; i <= K; ++i) {
-      int64_t v = wuo_in[i];
-      v = v < prev ? prev : v;
-      v = v > in_cap ? in_cap : v;
-      s_wuo[i] = v;
-      prev = v;
-      if (blockIdx.x == 0) wuo_out[i] = v;
+  if (threadIdx.x < 32) {  // ascending and inside [0, in_cap], whatever came in
+    const int lane = threadIdx.x;
+    const int64_t raw_k = __ldg(wuo_in + K);
+    int64_t x = lane <= K ? max((int64_t)0, __ldg(wuo_in + lane)) : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x = max(x, y);
     }
-    if (blockIdx.x == 0 && (wuo_in[K] < 0 || wuo_in[K] > in_cap)) set_status(status, ANTDT_ERR_CAPACITY);
+    const int64_t most = __shfl_sync(0xffffffffu, x, 31);
+    if (lane <= K) s_wuo[lane] = min(x, in_cap);
+    if (lane == 0 && K == 32) s_wuo[32] = min(max(most, raw_k), in_cap);
+    if (lane == 0 && blockIdx.x == 0 && (raw_k < 0 || raw_k > in_cap)) set_status(status, ANTDT_ERR_CAPACITY);
   }
+  const int64_t thread = (int64_t)blockIdx.x * kRaThreads + threadIdx.x, threads = (int64_t)gridDim.x * kRaThreads;
+  for (int64_t i = thread; i < n_a; i += threads) zero_a[i] = 0u;
+  for (int64_t i = thread; i < n_b; i += threads) zero_b[i] = 0u;
   __syncthreads();
-  const int64_t idx = (int64_t)blockIdx.x * kRaThreads + threadIdx.x;
-  if (idx >= (int64_t)K * (P + 1)) return;
-  const int w = (int)(idx / (P + 1));
-  const int64_t b = idx % (P + 1);
+  if (blockIdx.x == 0 && threadIdx.x <= K) wuo_out[threadIdx.x] = s_wuo[threadIdx.x];
+  const int64_t idx = thread / G;
+  if (idx >= (int64_t)K * (P + 1)) return;  // a whole lane group
+  const int w = (int)((uint32_t)idx / (uint32_t)(P + 1));
+  const int64_t b = (uint32_t)idx % (uint32_t)(P + 1);
   const uint64_t key = b < P ? (uint64_t)b << r_log2 : (uint64_t)n_rows;  // b == P: past the last row id
-  int64_t lo = s_wuo[w], hi = s_wuo[w + 1];
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if ((uint64_t)(uint32_t)__ldg(ids + mid) < key) lo = mid + 1; else hi = mid;
+  uint32_t lo = (uint32_t)s_wuo[w], hi = (uint32_t)s_wuo[w + 1];  // the boundary lies in [lo, hi]
+  if (G == 1) {
+    while (lo < hi) {
+      const uint32_t mid = (lo + hi) >> 1;
+      if ((uint64_t)(uint32_t)__ldg(ids + mid) < key) lo = mid + 1; else hi = mid;
+    }
+  } else {
+    const int lg = threadIdx.x & (G - 1), lane0 = (threadIdx.x & 31) - lg;
+    while (lo < hi) {
+      // probes lo + step - 1, lo + 2 step - 1, ...: as many of them below the key as lanes say so, from the left
+      const uint32_t step = (hi - lo + G) / (G + 1), at = lo + (uint32_t)(lg + 1) * step - 1u;
+      const bool below = at < hi && (uint64_t)(uint32_t)__ldg(ids + at) < key;
+      const unsigned v = __ballot_sync(group_mask<G>(), below) >> lane0 & ((1u << (G & 31)) - 1u);
+      const uint32_t c = (uint32_t)__ffs((int)~v) - 1u;
+      lo += c * step;
+      if (c < G) hi = min(hi, lo + step - 1u);  // (behind the last probe nothing is known)
+    }
+    if (lg) return;
   }
   bnd[(size_t)w * (P + 1) + b] = (int32_t)lo;
-  if (b == P && lo < s_wuo[w + 1] && !((dropped >> w) & 1u))
+  if (b == P && (int64_t)lo < s_wuo[w + 1] && !((dropped >> w) & 1u))
     set_status(status, ANTDT_ERR_ID_OUT_OF_RANGE);  // ids past the table
 }
 
@@ -423,16 +452,20 @@ void range_merge_order(const int32_t* uniq_ids, const int64_t* wuo_in, int64_t i
   int tile_shift = 0;
   while ((1 << tile_shift) < tile) ++tile_shift;
   const int64_t n_search = (int64_t)K * (P + 1);
-  ANTDT_LAUNCH("agg_range_split", range_split_kernel, (unsigned)((n_search + kRaThreads - 1) / kRaThreads),
-               kRaThreads, 0, s, uniq_ids, wuo_in, K, in_cap, r_log2, P, n_rows, dropped_bits, wuo_out, bnd, wb,
-               weights_host ? weights_dev : nullptr, status);
+  // every tile's entry is written unless ids were skipped as invalid: start from a valid index
+  const int64_t n_tiles = tile_first ? ((in_cap + tile - 1) >> tile_shift) + 1 : 0;
+  const int64_t n_words = head_bits ? (int64_t)head_bits_words(in_cap) : 0;
+#define SPLIT_GO(G)                                                                                                     \
+  ANTDT_LAUNCH("agg_range_split", range_split_kernel<G>, (unsigned)((n_search * G + kRaThreads - 1) / kRaThreads),       \
+               kRaThreads, 0, s, uniq_ids, wuo_in, K, in_cap, r_log2, P, n_rows, dropped_bits, wuo_out, bnd, wb,        \
+               weights_host ? weights_dev : nullptr, head_bits, n_words, reinterpret_cast<uint32_t*>(tile_first), n_tiles, \
+               status)
+  if (n_search <= kSplitTogether) SPLIT_GO(8); else SPLIT_GO(1);
+#undef SPLIT_GO
   ANTDT_LAUNCH("agg_range_count", range_count_kernel, (unsigned)P, kRaThreads, 0, s,
                uniq_ids, bnd, wuo_out, K, P, r_log2, n_rows, dropped_bits, distinct, status);
   ANTDT_LAUNCH("agg_range_scan", range_scan_kernel, 1, 1024, 0, s, distinct, P, base, n_agg, out_cap,
                bnd, wuo_out, K, dropped_bits, n_entries, status);
-  if (head_bits) cudaMemsetAsync(head_bits, 0, head_bits_words(in_cap) * 4, s);
-  // every tile's entry is written unless ids were skipped as invalid: start from a valid index
-  if (tile_first) cudaMemsetAsync(tile_first, 0, 4 * ((size_t)((in_cap + tile - 1) >> tile_shift) + 1), s);
   ANTDT_LAUNCH("agg_range_emit", range_emit_kernel, (unsigned)P, kRaThreads,
                emit_smem(r_log2, K, head_bits != nullptr), s,
                uniq_ids, bnd, wuo_out, K, P, r_log2, n_rows, dropped_bits, base, agg_ids, out_cap, src,

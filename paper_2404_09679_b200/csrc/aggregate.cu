@@ -288,8 +288,7 @@ dense_wsum_bulk_kernel(const float* __restrict__ grads, uint32_t n, int64_t stri
 // aggregated gradient is never written to or read back from memory (agg_out, if given, receives
 // it all the same).  No partial sums, no second pass: a row has at most K contributions.
 // Without a table (UPDATE false) it forms the sums alone, for lists so short that the tile reduction's
-// second launch counts: 9 k entries of 5 workers 64.5 -> 57 us for a step of four calls.  (For long ones the
-// tile reduction is faster, 129 against 170 us on 1.9 M entries x 64.)
+// second launch counts (sum_by_rows, and what the resident merge takes as a cluster).
 struct FusedUpdate {
   void* table; int dtype; int opt; OptParams p; float* state0; float* state1; float* agg_out;
 };
@@ -473,6 +472,12 @@ extern "C" size_t antdt_weighted_aggregate_workspace_bytes(int64_t in_cap, int32
 
 namespace antdt {
 namespace {
+// Lists of up to 32 workers that are summed row by row (agg_update_kernel without a table) instead of by tiles: one
+// launch for two and no head bits, while a tile's walk keeps more gradient rows in flight.  Server of two kernels, by
+// tiles -> by rows: 63 k entries x 32 floats 31 -> 25 us, 108 k x 20 32 -> 26, 312 k x 16 51 -> 43, 133 k x 64 43 -> 42;
+// but 1.2 M x 16 93 -> 101, 624 k x 64 of 4 workers 79 -> 85, and where many workers list a row (a lane group takes its
+// contributions in turn) 312 k x 64 over 50 k rows 86 -> 101, 624 k x 32 of 32 workers over 400 k 73 -> 78.
+bool sum_by_rows(int64_t in_cap, int dim, int64_t n_rows) { return in_cap * dim <= (int64_t)1 << 23 && in_cap <= 2 * n_rows; }
 constexpr int64_t kDenseBesideBytes = 8 << 20;  // below, the fork and join cost what they hide
 enum { kDenseStart = 0, kDenseDone = 1 };  // events of the dense part's side set
 constexpr int kBulkSmem = 4 * kBulkSlots * kBulkGroup * kBulkElems;
@@ -579,7 +584,8 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
   bool resident = sp && !merged && resident_merge_wanted(K, in_cap, sp->n_rows);
   const bool by_ranges = sp && K <= kRangeMaxWorkers && in_cap > 0;
   // a lane group per row: the one-pass update, and the sums of short lists
-  bool by_rows = sp && in_cap > 0 && ((fu && K <= kRangeMaxWorkers) || (!fu && resident && resident_sort_clears(in_cap)));
+  const bool few = sp && !fu && K <= kRangeMaxWorkers && sum_by_rows(in_cap, sp->dim, sp->n_rows);
+  bool by_rows = sp && in_cap > 0 && ((fu && K <= kRangeMaxWorkers) || (!fu && resident && resident_sort_clears(in_cap)) || few);
   auto upload_weights = [&] { upload_small(hw, 4 * (size_t)K, w8 + L.weights, s); };
   if (!by_ranges && !resident) upload_weights();
   // the dense part runs beside the sparse one where there is enough of it
@@ -623,7 +629,7 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
         return ANTDT_ERR_CUDA;
       if (rc == kResidentRefused) {
         resident = false;
-        by_rows = fu && K <= kRangeMaxWorkers;
+        by_rows = (fu && K <= kRangeMaxWorkers) || few;
         if (!by_ranges) upload_weights();
       }
     }
@@ -639,10 +645,10 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
       if (fork && cudaStreamWaitEvent(so, fork->ids_ready, 0) != cudaSuccess) return ANTDT_ERR_CUDA;
       range_merge_order(sp->uniq_ids, sp->worker_uniq_offsets, in_cap, sp->n_rows, K, dropped_bits,
                         sp->agg_ids, sp->n_agg, agg_cap, (int64_t*)(w8 + L.wuo), bounds,
-                        (uint32_t*)(w8 + L.src), fu ? nullptr : (uint32_t*)(w8 + L.head_bits),
-                        fu ? nullptr : (int32_t*)(w8 + L.tile_first), red_tile_for(in_cap, sp->dim),
-                        fu ? (uint32_t*)(w8 + L.row_start) : nullptr,
-                        fu ? (uint8_t*)(w8 + L.src_worker) : nullptr, hw, (float*)(w8 + L.weights),
+                        (uint32_t*)(w8 + L.src), by_rows ? nullptr : (uint32_t*)(w8 + L.head_bits),
+                        by_rows ? nullptr : (int32_t*)(w8 + L.tile_first), red_tile_for(in_cap, sp->dim),
+                        by_rows ? (uint32_t*)(w8 + L.row_start) : nullptr,
+                        by_rows ? (uint8_t*)(w8 + L.src_worker) : nullptr, hw, (float*)(w8 + L.weights),
                         w8 + L.range_ws, L.range, dev_status, so);
       if (fork && (cudaEventRecord(fork->order_done, so) != cudaSuccess ||
                    cudaStreamWaitEvent(s, fork->order_done, 0) != cudaSuccess))

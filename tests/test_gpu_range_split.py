@@ -1,0 +1,42 @@
+"""The range merge's boundaries: lists on both sides of the count from which one lane looks for a boundary instead of
+eight, list lengths around powers of nine (probes of eight lanes), empty lists, dense and sparse ones, a table whose last
+range is a part of one, ids at the ends of the table; and sums by rows on both sides of their rule.  Against the CPU checker."""
+import numpy as np
+import pytest
+
+import oracle
+from tests import gpu_util as G
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(rng, V, sizes, D, ends=True):
+    parts = []
+    for n in sizes:
+        p = np.sort(rng.choice(V, size=min(n, V), replace=False)).astype(np.int32) if n else np.zeros(0, np.int32)
+        if ends and len(p) > 2:
+            p[0], p[-1] = 0, V - 1
+            p = np.unique(p)
+        parts.append(p)
+    uid = np.concatenate(parts)
+    wuo = np.concatenate([[0], np.cumsum([len(p) for p in parts])]).astype(np.int64)
+    g = rng.normal(size=(len(uid), D)).astype(np.float32)
+    bsz = rng.integers(1, 50, size=len(sizes))
+    want_ids, want = oracle.aggregate_sparse(uid, wuo, g, bsz.astype(np.int64))
+    ids, agg, n, _, code = G.gpu_aggregate(uid, wuo, g, bsz, V)
+    assert code == 0 and n == len(want_ids) and np.array_equal(ids, want_ids)
+    G.close(agg, want)
+
+
+@pytest.mark.parametrize("V", [700_000, 4096 * 190, 4096 * 3200, 4096 * 4000 + 1])
+def test_boundaries(V):
+    rng = np.random.default_rng(V % 1000)
+    # 16 workers: 4096 * 3200 rows have 51 k boundaries, more than eight lanes look for together
+    _check(rng, V, [0, 1, 2, 8, 9, 10, 80, 81, 82, 729, 6561, 6560, 59_049, 0, 70_001, 0], 4)
+
+
+@pytest.mark.parametrize("K,n,D,V", [(32, 1200, 4, 9000), (2, 65_536, 64, 65_536), (2, 65_537, 64, 70_000), (3, 30_000, 20, 45_000),
+                                     (3, 30_001, 20, 45_000), (1, 40_000, 200, 2_000_000), (32, 2600, 100, 300_000)])
+def test_sums_by_rows_and_by_tiles(K, n, D, V):
+    rng = np.random.default_rng(K * n)
+    _check(rng, V, [n] * K, D, ends=False)
