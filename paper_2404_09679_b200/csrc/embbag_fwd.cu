@@ -3,11 +3,13 @@
 // One group of G lanes owns one bag; a row is read as G (x VPL) 16-byte vectors, so a warp
 // issues fully coalesced 128-bit loads over 32/G rows at once.  The path is a random gather bound
 // by the latency of its chain of dependent loads (offsets -> ids -> rows) and by HBM / L2 for the
-// rows; there is no contraction here and so no tensor-core work.  Three kernels:
+// rows; there is no contraction here and so no tensor-core work.  Four kernels:
 //   embbag_fwd_flat_kernel    rows of up to 512 bytes, one bag per group: every lane reads the ids
 //                             itself, four rows in flight, 32 registers -> 64 warps per SM
 //   embbag_fwd_stride_kernel  the same for many bags: capped grid, groups stride over the bags
 //                             and read the next bag's offsets ahead
+//   embbag_fwd_ahead_kernel   the same with the next bag's ids asked for ahead and more rows in flight, for
+//                             longer bags
 //   embbag_fwd_kernel         wider rows (VPL vectors per lane): ids staged through the group's
 //                             registers G at a time (one coalesced load, then shuffles)
 #include "common.cuh"
@@ -329,6 +331,131 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
   if (bad) set_status(status, ANTDT_ERR_ID_OUT_OF_RANGE);
 }
 
+// Which bags are read ahead of (embbag_fwd_ahead_kernel), with how many rows requested at once per lane (0: not),
+// and whether in field-major order.  More rows in flight per lane mean fewer warps (eight: 4 CTAs per SM, four: 5),
+// which pays once a bag has ids enough to fill them; a grid of one wave (2 waves 1 - 5% slower, 8 CTAs per SM no faster
+// than the other kernels).  us before -> reading ahead, by ids per bag, one resident wave of bags (W 1) and many:
+//   fp32, 32 vectors   3: 368 -> 503   10, W 1 / 3 / 24: 13.2 / 25.1 / 122 -> 11.4 / 22.0 / 107   25: 782 -> 693
+//         16 vectors   2: 190 -> 235   6, W 1 / 24: 11.1 / 100 -> 10.3 / 95   15, W 3 / 24: 33 / 178 -> 28 / 151
+//          8 vectors   four rows: 4: 153 -> 146, but 35 M ids over 50 M rows 839 -> 883   10, W 24: 153 -> 145
+//          4 vectors   3, W 24: 99 -> 91   8: 148 -> 140   15: 205 -> 185
+//   bf16, 32 vectors   12, W 6 / 24: 52 / 169 -> 52 / 171   25: 281 -> 247
+//         16 vectors   4: 331 -> 337   9, W 1 / 24: 14.5 / 160 -> 12.9 / 144   12: 634 -> 567
+//          8 vectors   four rows: 2, W 24: 91 -> 85   eight: 5, W 24: 136 -> 116   15: 248 -> 214   20: 531 -> 461
+//          4 vectors   four rows: 4, W 24: 136 -> 122   15: 258 -> 234
+// Inside a step, with bags of eight ids and more: one field at a time, not read ahead | bag order | field order:
+//   fp32, 32 / 8 / 4 vectors, 10 ids: 574 | 590 | 612, 400 | 423 | 405, 422 | 503 | 455
+//         16 vectors, 10 and 20 ids: 670 | 612 | 673, 705 | 691 | 680; 65 M ids over 10 M rows 1863 | 1791 | 1885
+//   bf16, 32 vectors, 20 ids: 490 | 459 | 481; 16, 12 ids: 667 | 596 | 649; 4, 12 ids: 619 | 622 | 555
+//          8 vectors, 10 ids: 534 | 455 | 478, 105 M of 20 ids over 20 M rows 1667 | 1710 | 1509
+__host__ __device__ constexpr int ahead_ctas(int rows) { return rows == 8 ? 4 : 5; }  // per SM
+struct Ahead { int rows; bool by_field; };
+inline Ahead ahead_of(int G, bool bf16, bool fields_known, int64_t bags_per_cta, int64_t n_bags, int64_t nnz) {
+  const Ahead no = {0, false};
+  if (n_bags < (int64_t)kNumSM * kFlatCtas * bags_per_cta) return no;
+  auto ids = [&](int64_t per_bag) { return nnz >= per_bag * n_bags; };
+  if (!bf16) {
+    if (G == 16) return ids(6) ? Ahead{8, fields_known && ids(16)} : no;
+    if (fields_known) return no;
+    return G == 32 && ids(8) ? Ahead{8, false} : G == 8 && ids(8) ? Ahead{4, false} : G == 4 && ids(3) ? Ahead{8, false} : no;
+  }
+  if (G == 32) return ids(16) ? Ahead{8, false} : no;
+  if (G == 16) return ids(8) ? Ahead{8, false} : no;
+  if (G == 8) return ids(4) ? Ahead{8, fields_known && ids(16)} : ids(2) ? Ahead{4, false} : no;
+  return ids(3) ? Ahead{4, fields_known} : no;
+}
+
+// The same with a bag's ids held by the lanes of its group, one each, and everything asked for ahead: while a bag's
+// rows are on their way, so are the next bag's ids and the offsets of the one after it.  What is left of the chain
+// offsets -> ids -> rows is the last step.  Lanes of a warp go through their bags together, to the longest of them
+// (the ids are handed round by shuffles).  BY_FIELD: bags in field-major order.
+template <int G, bool BF16, bool BY_FIELD, int U>
+__global__ void __launch_bounds__(kFlatThreads, ahead_ctas(U))
+embbag_fwd_ahead_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
+                        const int32_t* __restrict__ row_ids, int64_t nnz,
+                        const int64_t* __restrict__ bag_offsets, int64_t n_bags,
+                        float* __restrict__ pooled, int32_t* status, uint32_t fields, uint32_t samples, bool chained) {
+  if (chained) pdl_sync();
+  constexpr int EPV = BF16 ? 8 : 4;
+  constexpr int PAIRS = EPV / 2;
+  constexpr int GPB = kFlatThreads / G;
+  constexpr int kStep = U < G ? U : G;  // rows requested at once
+  constexpr unsigned kFull = 0xffffffffu;
+  constexpr uint32_t kNone = 0xffffffffu;
+  const int lg = threadIdx.x & (G - 1);
+  const int nvec = dim / EPV;
+  const uint32_t limit = (uint32_t)n_rows, row_vecs = (uint32_t)nvec, n_slots = (uint32_t)n_bags;
+  const bool lane_on = lg < nvec;
+  const uint4* const tbl = static_cast<const uint4*>(table);
+  const uint32_t stride = gridDim.x * GPB;
+  bool bad = false;
+  auto bag_of = [&](uint32_t q) { return BY_FIELD ? q % samples * fields + q / samples : q; };
+  // a slot's id range; behind the last slot, and for bad offsets, an empty one
+  auto range_of = [&](uint32_t q, uint32_t& begin, uint32_t& len) {
+    begin = len = 0;
+    if (q >= n_slots) return;
+    const uint32_t bag = bag_of(q);
+    const int64_t b = bag_offsets[bag], e = bag_offsets[bag + 1];
+    if (b < 0 || e < b || e > nnz) {
+      if (lg == 0) set_status(status, ANTDT_ERR_BAD_OFFSETS);
+      return;
+    }
+    begin = (uint32_t)b;  // nnz < 2^31
+    len = (uint32_t)(e - b);
+  };
+  auto id_at = [&](uint32_t begin, uint32_t len, uint32_t j) {  // kNone: no row
+    return j < len ? (uint32_t)__ldg(row_ids + begin + j) : kNone;
+  };
+  uint32_t q = blockIdx.x * GPB + threadIdx.x / G;
+  uint32_t begin, len, nbegin, nlen;
+  range_of(q, begin, len);
+  uint32_t id = id_at(begin, len, lg);
+  range_of(q + stride, nbegin, nlen);  // fewer than 2^31 slots and three strides below 2^20: no slot number wraps
+  while (__any_sync(kFull, q < n_slots)) {
+    const uint32_t next_id = id_at(nbegin, nlen, lg);
+    uint32_t fbegin, flen;
+    range_of(q + 2 * stride, fbegin, flen);
+    const uint32_t longest = __reduce_max_sync(kFull, len);
+    uint64_t acc[PAIRS];
+#pragma unroll
+    for (int e = 0; e < PAIRS; ++e) acc[e] = 0ull;
+    for (uint32_t base = 0; base < longest; base += G) {
+      if (base > 0) id = id_at(begin, len, base + lg);
+      bad |= id >= limit && base + lg < len;
+      if (id >= limit) id = kNone;
+#pragma unroll 1
+      for (uint32_t j0 = 0; j0 < G && base + j0 < longest; j0 += kStep) {
+        uint4 v[kStep];
+#pragma unroll
+        for (int t = 0; t < kStep; ++t) {
+          const uint32_t x = __shfl_sync(kFull, id, j0 + t, G);
+          v[t] = x != kNone && lane_on ? __ldg(tbl + (size_t)x * row_vecs + lg) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int t = 0; t < kStep; ++t) {
+          if (BF16) {
+            acc[0] = f32x2_add(acc[0], f32x2_pack(v[t].x << 16, v[t].x & 0xffff0000u));
+            acc[1] = f32x2_add(acc[1], f32x2_pack(v[t].y << 16, v[t].y & 0xffff0000u));
+            acc[2] = f32x2_add(acc[2], f32x2_pack(v[t].z << 16, v[t].z & 0xffff0000u));
+            acc[3] = f32x2_add(acc[3], f32x2_pack(v[t].w << 16, v[t].w & 0xffff0000u));
+          } else {
+            acc[0] = f32x2_add(acc[0], f32x2_pack(v[t].x, v[t].y));
+            acc[1] = f32x2_add(acc[1], f32x2_pack(v[t].z, v[t].w));
+          }
+        }
+      }
+    }
+    if (q < n_slots && lane_on) {
+      ulonglong2* o = reinterpret_cast<ulonglong2*>(pooled + (size_t)bag_of(q) * dim + (size_t)lg * EPV);
+      o[0] = make_ulonglong2(acc[0], acc[1]);
+      if (BF16) o[1] = make_ulonglong2(acc[2], acc[3]);
+    }
+    q += stride;
+    id = next_id; begin = nbegin; len = nlen; nbegin = fbegin; nlen = flen;
+  }
+  if (bad) set_status(status, ANTDT_ERR_ID_OUT_OF_RANGE);
+}
+
 template <int G, int VPL, bool BF16, bool PACKED>
 void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_ids, int64_t nnz,
                 const int64_t* bag_offsets, int64_t n_bags, float* pooled, int32_t* status,
@@ -343,7 +470,19 @@ void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_i
     fields = 0;
   }
   const int waves = flat && fields == 0 ? stride_waves(G, gpb, BF16, n_bags, nnz) : 0;
-  if (waves > 0) {
+  const Ahead ahead = flat && !PACKED && G >= 4 ? ahead_of(G, BF16, fields > 0, gpb, n_bags, nnz) : Ahead{0, false};
+#define AHEAD_GO(U, FIELD)                                                                                                \
+  {                                                                                                                       \
+    const int64_t cap = (int64_t)kNumSM * ahead_ctas(U), want = (n_bags + gpb - 1) / gpb;                                 \
+    ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_ahead_kernel<(G < 4 ? 4 : G), BF16, FIELD, U>), (unsigned)(want < cap ? want : cap), \
+                 kFlatThreads, 0, s, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status,              \
+                 (uint32_t)(FIELD ? fields : 1), (uint32_t)(FIELD ? n_bags / fields : n_bags), chained);                  \
+  }
+  if (ahead.rows == 8 && ahead.by_field) AHEAD_GO(8, true)
+  else if (ahead.rows == 8) AHEAD_GO(8, false)
+  else if (ahead.rows == 4 && ahead.by_field) AHEAD_GO(4, true)
+  else if (ahead.rows == 4) AHEAD_GO(4, false)
+  else if (waves > 0) {
     ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_stride_kernel<G, BF16, PACKED>), (unsigned)(kNumSM * kFlatCtas * waves),
                  kFlatThreads, 0, s, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, chained);
   } else if (flat && fields > 0) {
