@@ -415,13 +415,19 @@ __host__ __device__ inline EmitShape emit_shape(int r_log2, int K) {
   return e;
 }
 
+// A range of few entries (KEPT to a thread) is searched and read once, its entries stay in registers; with more than 16
+// workers (whose wide sets leave room for five CTAs to an SM only) KEPT is 8, and the first slots are put in order in shared
+// memory and stored by consecutive threads.  16.2 M entries of 32 workers over 50 M rows 241 -> 186 us; 2.6 M of 14 over 20 M
+// 42 -> 36; of 16 workers, 17 M over 20 M rows 167 -> 167 (most ranges hold more).  Reading the other entries in batches in
+// the order that ends with those kept: 186 - 275; the staged slots with up to 16 workers: 167 -> 174.
+template <int KEPT>
 __global__ void __launch_bounds__(kRaThreads)
 range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ bnd,
                   const int64_t* __restrict__ wuo, int K, int64_t P, int r_log2, int64_t n_rows,
                   const RangeDropped dropped, const int64_t* __restrict__ base, int32_t* __restrict__ agg_ids,
                   int64_t out_cap, uint32_t* __restrict__ src, uint32_t* head_bits,
                   int32_t* __restrict__ tile_first, int tile_shift, uint32_t* __restrict__ row_start,
-                  uint8_t* __restrict__ src_worker, int32_t* status) {
+                  uint8_t* __restrict__ src_worker, int staged, int32_t* status) {
   pdl_sync();
   extern __shared__ __align__(16) unsigned char ra_smem[];
   const int R = 1 << r_log2;
@@ -439,7 +445,9 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
   int32_t* s_beg = wrank + 256;  // [32]
   int32_t* s_off = s_beg + 32;   // [33]
   int32_t* s_tmp = s_off + 33;   // [16]
-  uint32_t* hb = reinterpret_cast<uint32_t*>(s_tmp + 16);  // head bits of this range's slots
+  uint32_t* st_src = reinterpret_cast<uint32_t*>(s_tmp + 16);            // [staged] the range's first slots
+  uint8_t* st_worker = reinterpret_cast<uint8_t*>(st_src + staged);      // [staged] where src_worker is wanted
+  uint32_t* hb = st_src + staged + (src_worker ? staged / 4 : 0);  // head bits of this range's slots
   const int64_t b = blockIdx.x;
   const int tid = threadIdx.x;
   const int64_t u0 = __ldg(base + b);  // requested now: every global round trip here is serial
@@ -464,11 +472,48 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
   }
   __syncthreads();
   const uint32_t base_key = (uint32_t)(b << r_log2);
-  for_each_entry<1>(ids, pc.entries, R, base_key, n_rows, s_beg, s_off, status,
-                 [&](int w, int, uint32_t, uint32_t kl) {
-                   atomicOr(&mask[kl >> lg], (1u << w) << ((kl & sub) << sub_sh));
-                   atomicOr(&pres[kl >> 5], 1u << (kl & 31));
-                 });
+  constexpr uint32_t kNone = 0xffffffffu;
+  auto fill = [&](int w, uint32_t kl) {
+    atomicOr(&mask[kl >> lg], (1u << w) << ((kl & sub) << sub_sh));
+    atomicOr(&pres[kl >> 5], 1u << (kl & 31));
+  };
+  // few entries stay in registers from here to the end: position, and id inside the range << 8 | worker
+  const bool keep = pc.entries <= KEPT * kRaThreads;
+  uint32_t kept_j[KEPT], kept[KEPT];
+  if (keep) {
+#pragma unroll
+    for (int g = 0; g < KEPT; g += kRaBatch) {
+#pragma unroll
+      for (int t = g; t < g + kRaBatch; ++t) kept[t] = kNone;
+      if (g * kRaThreads >= pc.entries) continue;  // no thread has one
+      uint32_t id[kRaBatch];
+      int w[kRaBatch];
+#pragma unroll
+      for (int t = 0; t < kRaBatch; ++t) {
+        const int e = (g + t) * kRaThreads + tid;
+        int j;
+        entry_of<1>(e < pc.entries ? e : 0, s_beg, s_off, w[t], j);
+        kept_j[g + t] = (uint32_t)j;
+        id[t] = (uint32_t)__ldg(ids + j);
+      }
+#pragma unroll
+      for (int t = 0; t < kRaBatch; ++t) {
+        const uint32_t kl = id[t] - base_key;
+        if ((g + t) * kRaThreads + tid >= pc.entries) continue;
+        if (kl < (uint32_t)R && (int64_t)id[t] < n_rows) {
+          kept[g + t] = kl << 8 | (uint32_t)w[t];
+          fill(w[t], kl);
+        } else {
+          set_status(status, ANTDT_ERR_ID_OUT_OF_RANGE);
+        }
+      }
+    }
+  } else {
+    for_each_entry<1>(ids, pc.entries, R, base_key, n_rows, s_beg, s_off, status,
+                      [&](int w, int, uint32_t, uint32_t kl) { fill(w, kl); });
+  }
+  if (KEPT > 4)
+    for (int i = tid; i < min(staged, pc.entries); i += kRaThreads) st_src[i] = kNone;  // (a list that repeats ids leaves slots out)
   __syncthreads();
 
   // thread q owns presence word q: present ids and contributions in it, prefix sums over the words
@@ -481,10 +526,11 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
     wrank[tid] = n_ids;
     int t = n_ids, first = n_con;
     for (uint32_t rest = pw; rest; rest &= rest - 1u) {
+      const int kl = tid * 32 + __ffs((int)rest) - 1;
       if (shp.fc16) first_c16[t++] = (unsigned short)first;
       else first_c[t++] = (uint32_t)first;
       if (head_bits) atomicOr(&hb[(hb_shift + first) >> 5], 1u << ((hb_shift + first) & 31));
-      first += __popc(workers_of(tid * 32 + __ffs((int)rest) - 1));
+      first += __popc(workers_of(kl));
     }
   }
   __syncthreads();
@@ -498,21 +544,38 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
     else atomicOr(&head_bits[g], word);
   }
   const int64_t tile_mask = ((int64_t)1 << tile_shift) - 1;
-  for_each_entry<1>(ids, pc.entries, R, base_key, n_rows, s_beg, s_off, nullptr,
-                 [&](int w, int j, uint32_t id, uint32_t kl) {
-                   const int t = wrank[kl >> 5] + __popc(pres[kl >> 5] & ((1u << (kl & 31)) - 1u));
-                   const int slot = __popc(workers_of((int)kl) & ((1u << w) - 1u));
-                   const int64_t dest = pc.before + (int64_t)(shp.fc16 ? first_c16[t] : first_c[t]) + slot;
-                   const int64_t u = u0 + t;
-                   src[dest] = (uint32_t)j;
-                   if (src_worker) src_worker[dest] = (uint8_t)w;  // saves the reader a search
-                   if (slot == 0) {
-                     if (u < out_cap) agg_ids[u] = (int32_t)id;
-                     // the row's first merge slot (one more than rows: it ends the last one)
-                     if (row_start && u <= out_cap) row_start[u] = (uint32_t)dest;
-                   }
-                   if (tile_first && (dest & tile_mask) == 0) tile_first[dest >> tile_shift] = (int32_t)u;
-                 });
+  auto place = [&](int w, uint32_t j, int kl) {
+    const int t = wrank[kl >> 5] + __popc(pres[kl >> 5] & ((1u << (kl & 31)) - 1u));
+    const int slot = __popc(workers_of(kl) & ((1u << w) - 1u)), at = (int)(shp.fc16 ? first_c16[t] : first_c[t]) + slot;
+    const int64_t dest = pc.before + at, u = u0 + t;
+    if (KEPT > 4 && at < staged) {
+      st_src[at] = j;
+      if (src_worker) st_worker[at] = (uint8_t)w;
+    } else {
+      src[dest] = j;
+      if (src_worker) src_worker[dest] = (uint8_t)w;  // saves the reader a search
+    }
+    if (slot == 0) {
+      if (u < out_cap) agg_ids[u] = (int32_t)(base_key + (uint32_t)kl);
+      // the row's first merge slot (one more than rows: it ends the last one)
+      if (row_start && u <= out_cap) row_start[u] = (uint32_t)dest;
+    }
+    if (tile_first && (dest & tile_mask) == 0) tile_first[dest >> tile_shift] = (int32_t)u;
+  };
+  if (keep) {
+#pragma unroll
+    for (int t = 0; t < KEPT; ++t)
+      if (kept[t] != kNone) place((int)(kept[t] & 31u), kept_j[t], (int)(kept[t] >> 8));
+  } else {
+    for_each_entry<1>(ids, pc.entries, R, base_key, n_rows, s_beg, s_off, nullptr,
+                      [&](int w, int j, uint32_t, uint32_t kl) { place(w, (uint32_t)j, (int)kl); });
+  }
+  if (KEPT == 4) return;
+  __syncthreads();
+  for (int i = tid; i < min(staged, pc.entries); i += kRaThreads) {
+    src[pc.before + i] = st_src[i];
+    if (src_worker) src_worker[pc.before + i] = st_worker[i];
+  }
 }
 
 // The same for more than 32 workers: NW words to a worker set, word-major.  Ranges are many and short here (some 100
@@ -621,12 +684,20 @@ range_emit_wide_kernel(const int32_t* __restrict__ ids, const int32_t* __restric
 }
 size_t emit_wide_smem(int r_log2, int words) { return ((size_t)4 * words + 6) << r_log2; }
 
-// Tables, small arrays, and the head bits of up to R*K slots for a reader that wants them (without
+// Slots of a range that are put in order in shared memory: those of an average range and a quarter more (the others are
+// stored where they are found).
+int emit_staged(int K, int64_t in_cap, int64_t P) {
+  if (K <= 16) return 0;
+  const int64_t n = (in_cap / P * 5 / 4 + 255) & ~(int64_t)255;
+  return (int)(n < 512 ? 512 : (n > 4096 ? 4096 : n));
+}
+
+// Tables, small arrays, staged slots, and the head bits of up to R*K slots for a reader that wants them (without
 // them an SM works on 6 ranges of 32 workers at once instead of 4: 278 -> 249 us on 16.2 M entries).
-size_t emit_smem(int r_log2, int K, bool head_bits) {
+size_t emit_smem(int r_log2, int K, int staged, bool src_worker, bool head_bits) {
   const size_t R = (size_t)1 << r_log2;
   const EmitShape e = emit_shape(r_log2, K);
-  return 4 * (R >> e.mask_lg) + (e.fc16 ? 2 : 4) * R + 8 + 4 * (256 + 256 + 32 + 33 + 16) +
+  return 4 * (R >> e.mask_lg) + (e.fc16 ? 2 : 4) * R + 8 + 4 * (256 + 256 + 32 + 33 + 16) + (src_worker ? 5 : 4) * (size_t)staged +
          (head_bits ? 4 * (R * (size_t)K / 32 + 2) : 0) + 12;
 }
 
@@ -649,8 +720,10 @@ void range_prepare_device() {
   cudaGetDevice(&dev_id);
   bool& done = attr_set[dev_id & 63];
   if (done) return;
-  cudaFuncSetAttribute(range_emit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)emit_smem(kRangeMaxLog2, kRangeMaxWorkers, true));
+  cudaFuncSetAttribute(range_emit_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)emit_smem(kRangeMaxLog2, 16, 0, true, true));
+  cudaFuncSetAttribute(range_emit_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)emit_smem(kRangeMaxLog2, kRangeMaxWorkers, 4096, true, true));
   done = true;
 }
 
@@ -701,17 +774,21 @@ void range_merge_order(const int32_t* uniq_ids, const int64_t* wuo_in, int64_t i
   ANTDT_LAUNCH("agg_range_emit", (range_emit_wide_kernel<NW, PER>), (unsigned)P, kRaThreads, emit_wide_smem(r_log2, NW), s, \
                uniq_ids, bnd, wuo_out, K, P, n_rows, dropped, base, agg_ids, out_cap, src, head_bits, tile_first,    \
                tile_shift, status)
-  if (!wide)
-    ANTDT_LAUNCH("agg_range_emit", range_emit_kernel, (unsigned)P, kRaThreads,
-                 emit_smem(r_log2, K, head_bits != nullptr), s,
-                 uniq_ids, bnd, wuo_out, K, P, r_log2, n_rows, dropped, base, agg_ids, out_cap, src,
-                 head_bits, tile_first, tile_shift, row_start, src_worker, status);
-  else if (r_log2 == kRangeWideLog2) {
+  const int staged = emit_staged(K, in_cap, P);
+#define EMIT_GO(KEPT)                                                                                                 \
+  ANTDT_LAUNCH("agg_range_emit", range_emit_kernel<KEPT>, (unsigned)P, kRaThreads,                                    \
+               emit_smem(r_log2, K, staged, src_worker != nullptr, head_bits != nullptr), s,                          \
+               uniq_ids, bnd, wuo_out, K, P, r_log2, n_rows, dropped, base, agg_ids, out_cap, src,                    \
+               head_bits, tile_first, tile_shift, row_start, src_worker, staged, status)
+  if (!wide) {
+    if (staged) EMIT_GO(8); else EMIT_GO(4);
+  } else if (r_log2 == kRangeWideLog2) {
     if (K <= 64) WIDE_GO(2, 4); else if (K <= 96) WIDE_GO(3, 4); else WIDE_GO(4, 4);
   } else {
     if (K <= 64) WIDE_GO(2, 8); else if (K <= 96) WIDE_GO(3, 8); else WIDE_GO(4, 8);
   }
 #undef WIDE_GO
+#undef EMIT_GO
 }
 
 }  // namespace antdt

@@ -1,6 +1,7 @@
 """The range merge's boundaries: lists on both sides of the count from which one lane looks for a boundary instead of
 eight, list lengths around powers of nine (probes of eight lanes), empty lists, dense and sparse ones, a table whose last
-range is a part of one, ids at the ends of the table; and sums by rows on both sides of their rule.  Against the CPU checker."""
+range is a part of one, ids at the ends of the table; sums by rows on both sides of their rule; and ranges of as many entries as the emit kernel's CTA keeps in registers or puts
+in order in shared memory.  Against the CPU checker."""
 import numpy as np
 import pytest
 
@@ -40,3 +41,25 @@ def test_boundaries(V):
 def test_sums_by_rows_and_by_tiles(K, n, D, V):
     rng = np.random.default_rng(K * n)
     _check(rng, V, [n] * K, D, ends=False)
+
+
+# entries of the first range around 4 and 8 per thread; more than the staged slots (1536 here) in the last three
+@pytest.mark.parametrize("D", [4, 132])
+@pytest.mark.parametrize("K", [16, 17, 32])
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 2048, 2049, 4097, 30_000])
+def test_entries_per_range(n, K, D):
+    rng = np.random.default_rng(n + K)
+    V = 4096 * 60 + 7
+    parts = []
+    for w in range(K):
+        k = min(4096, n // K + (w < n % K))
+        parts.append(np.sort(np.concatenate([rng.choice(4096, size=k, replace=False),
+                                             4096 + rng.choice(V - 4096, size=66_000 // K, replace=False)])).astype(np.int32))
+    uid = np.concatenate(parts)
+    wuo = np.concatenate([[0], np.cumsum([len(p) for p in parts])]).astype(np.int64)
+    g = rng.normal(size=(len(uid), D)).astype(np.float32)
+    bsz = rng.integers(1, 50, size=K)
+    want_ids, want = oracle.aggregate_sparse(uid, wuo, g, bsz.astype(np.int64))
+    ids, agg, m, _, code = G.gpu_aggregate(uid, wuo, g, bsz, V)
+    assert code == 0 and m == len(want_ids) and np.array_equal(ids, want_ids)
+    G.close(agg, want)
