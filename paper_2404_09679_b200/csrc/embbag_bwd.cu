@@ -74,13 +74,15 @@ bwd_prep_kernel(const int64_t* __restrict__ wso, int K, int F, const int64_t* __
 
 // One warp expands kExpandGroups x 32 consecutive bags: lane l holds the end offset of bag l of every
 // group, all requested at once (the kernel is one dependent load and a stream of stores).
-// A lane finds the bag of one occurrence by a 5-step search over the lanes' ends and walks on from
-// there for the three that follow: one 16-byte store (the first and last few occurrences of a group,
-// off the 16-byte grid, go one by one).
-// 5.2 M bags, 105 M occurrences: 129 us, were 162 with one group per warp and a search and a 4-byte
-// store per occurrence.
+// The bags mark the slots that they begin in a window of shared memory, and a lane has the bags of four slots from a
+// running maximum over the marks: one 16-byte store (the first and last few occurrences, off the 16-byte grid, go one by
+// one).  The groups of a warp are one span, so the last turn of 128 slots is not spent on every group.
+// Searching each four slots' bag among the lanes' ends, group by group, was bound by its instructions: 5.2 M bags, 105 M
+// occurrences 130 -> 83 us, 6.6 M and 65 M 114 -> 76, 7.9 M and 35 M 99 -> 56.
 constexpr int kExpandGroups = 4;
-__global__ void __launch_bounds__(256)
+constexpr uint32_t kExpandWindow = 1024;
+static_assert(32 * kExpandGroups < 256, "a mark is a byte");
+__global__ void __launch_bounds__(256, 6)
 expand_bags_kernel(const int64_t* __restrict__ bag_offsets, int64_t n_bags, int64_t nnz,
                    uint32_t* __restrict__ occ_bag, int32_t* status, uint32_t* __restrict__ zero_words,
                    int64_t n_zero_words, int32_t* __restrict__ zero_pair) {
@@ -98,51 +100,80 @@ expand_bags_kernel(const int64_t* __restrict__ bag_offsets, int64_t n_bags, int6
        i += (int64_t)gridDim.x * blockDim.x)
     zero_words[i] = 0u;
   if (blockIdx.x == 0 && threadIdx.x < 2 && zero_pair) zero_pair[threadIdx.x] = 0;
+  uint32_t begin[kExpandGroups], end[kExpandGroups];  // of this lane's bag, where the group is not bad
+  unsigned bad_groups = 0;
 #pragma unroll
   for (int g = 0; g < kExpandGroups; ++g) {
-    const int64_t b0 = first_bag + 32 * g;
-    if (b0 >= n_bags) return;
-    const int64_t lo = at[g], next = __shfl_sync(0xffffffffu, at[g + 1], 0);
-    int64_t hi = __shfl_down_sync(0xffffffffu, lo, 1);
+    const int64_t next = __shfl_sync(0xffffffffu, at[g + 1], 0);
+    int64_t hi = __shfl_down_sync(0xffffffffu, at[g], 1);
     if (lane == 31) hi = next;
-    const bool bad = lo < 0 || hi < lo || hi > nnz;
-    if (__any_sync(0xffffffffu, bad)) {  // skip the whole group; readers bound-check bag indices
-      if (lane == 0) set_status(status, ANTDT_ERR_BAD_OFFSETS);
-      continue;
+    // skip the whole group; readers bound-check bag indices
+    if (__any_sync(0xffffffffu, at[g] < 0 || hi < at[g] || hi > nnz)) bad_groups |= 1u << g;
+    begin[g] = (uint32_t)at[g];
+    end[g] = (uint32_t)hi;
+  }
+  if (bad_groups && lane == 0) set_status(status, ANTDT_ERR_BAD_OFFSETS);
+  __shared__ __align__(16) uint8_t s_marks[8][kExpandWindow];
+  uint8_t* const marks = s_marks[threadIdx.x >> 5];
+  // the groups that `groups` has a bit for (a row of them, none bad)
+  auto expand = [&](unsigned groups) {
+    uint32_t first = 0, last = 0;
+#pragma unroll
+    for (int g = kExpandGroups - 1; g >= 0; --g) {
+      const uint32_t lo = __shfl_sync(0xffffffffu, begin[g], 0), hi = __shfl_sync(0xffffffffu, end[g], 31);
+      if (!((groups >> g) & 1u)) continue;
+      first = lo;
+      if (!((groups >> g) >> 1)) last = hi;
     }
-    const int64_t first = __shfl_sync(0xffffffffu, lo, 0);
-    // the group's range starts this far into an aligned group of four; slots are counted from there
-    const uint32_t skew = (uint32_t)(((reinterpret_cast<uintptr_t>(occ_bag) >> 2) + (uint64_t)first) & 3);
-    const BagSpan span((uint32_t)(next - first), skew);         // offsets lie in [0, nnz]
-    const uint32_t my_end = (uint32_t)(hi - first) + span.skew;  // ascending over the lanes
-    uint32_t* const out = occ_bag + (first - (int64_t)skew);     // slot 0, on the 16-byte grid
-    for (uint32_t base = 0; base < span.total; base += kSpanTurn) {
-      const uint32_t x = base + 4 * lane;
-      int l = 0;  // first lane whose end is > max(x, skew)
+    // the range starts this far into an aligned group of four; slots are counted from there
+    const uint32_t skew = (uint32_t)(((reinterpret_cast<uintptr_t>(occ_bag) >> 2) + first) & 3);
+    const BagSpan span(last - first, skew);                            // offsets lie in [0, nnz]
+    uint32_t* const out = occ_bag + ((int64_t)first - (int64_t)skew);  // slot 0, on the 16-byte grid
+    uint32_t carry = 0;                                                // mark of the bag that goes on
+    for (uint32_t base = 0; base < span.total; base += kExpandWindow) {
+      __syncwarp();
 #pragma unroll
-      for (int step = 16; step > 0; step >>= 1) {
-        const uint32_t e = __shfl_sync(0xffffffffu, my_end, l + step - 1);
-        if (e <= max(x, span.skew)) l += step;
+      for (uint32_t i = 0; i < kExpandWindow / 512; ++i)
+        reinterpret_cast<uint4*>(marks)[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+      __syncwarp();
+#pragma unroll
+      for (int g = 0; g < kExpandGroups; ++g) {
+        const uint32_t x = begin[g] - first + skew - base;  // from this window's start
+        if (((groups >> g) & 1u) && end[g] > begin[g] && x < kExpandWindow) marks[x] = (uint8_t)(32 * g + lane + 1);
       }
-      uint32_t q[4];
-      uint32_t end = __shfl_sync(0xffffffffu, my_end, l & 31);
+      __syncwarp();
+      for (uint32_t t = 0; t < kExpandWindow && base + t < span.total; t += kSpanTurn) {
+        const uint32_t x = base + t + 4 * lane, q = *reinterpret_cast<const uint32_t*>(marks + t + 4 * lane);
+        uint32_t m[4];
+        m[0] = q & 255u; m[1] = max(m[0], q >> 8 & 255u); m[2] = max(m[1], q >> 16 & 255u); m[3] = max(m[2], q >> 24);
+        uint32_t incl = m[3];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        // on to the bag that holds x + j (empty bags are stepped over; the vote keeps the lanes together)
-        while (__any_sync(0xffffffffu, x + j >= end && l < 31)) {
-          if (x + j >= end && l < 31) ++l;
-          end = __shfl_sync(0xffffffffu, my_end, l & 31);
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl = max(incl, y);
         }
-        q[j] = (uint32_t)min(b0 + l, n_bags - 1);
-      }
-      if (span.whole(x)) {
-        *reinterpret_cast<uint4*>(out + x) = make_uint4(q[0], q[1], q[2], q[3]);
-      } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (span.holds(x + j)) out[x + j] = q[j];
+        uint32_t before = __shfl_up_sync(0xffffffffu, incl, 1);
+        before = lane ? max(before, carry) : carry;
+        carry = max(carry, __shfl_sync(0xffffffffu, incl, 31));
+        const uint32_t b0 = (uint32_t)first_bag - 1u;
+        const uint4 bags = make_uint4(b0 + max(m[0], before), b0 + max(m[1], before), b0 + max(m[2], before), b0 + max(m[3], before));
+        if (span.whole(x)) {
+          *reinterpret_cast<uint4*>(out + x) = bags;
+        } else {
+          if (span.holds(x)) out[x] = bags.x;
+          if (span.holds(x + 1)) out[x + 1] = bags.y;
+          if (span.holds(x + 2)) out[x + 2] = bags.z;
+          if (span.holds(x + 3)) out[x + 3] = bags.w;
+        }
       }
     }
+  };
+  constexpr unsigned kAll = (1u << kExpandGroups) - 1u;
+#pragma unroll 1
+  for (unsigned g = 0; g < kExpandGroups; ++g) {  // one span, or the good groups one by one
+    if ((bad_groups >> g) & 1u) continue;
+    expand(bad_groups ? 1u << g : kAll);
+    if (!bad_groups) return;
   }
 }
 
