@@ -224,8 +224,7 @@ embbag_fwd_flat_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
                        float* __restrict__ pooled, int32_t* status, int fields, int64_t sample_blocks, bool chained) {
   if (chained) pdl_sync();  // (beside a kernel that it depends on the start of, it must not wait for its end)
   constexpr int EPV = BF16 ? 8 : 4;
-  const int nvec = dim / EPV;
-  const RowLanes<kFlatThreads, G, PACKED> lanes(nvec);
+  const RowLanes<kFlatThreads, G, PACKED> lanes(PACKED ? dim / EPV : G);
   const int lg = lanes.lg;
   int64_t bag;
   if (BY_FIELD) {
@@ -235,6 +234,7 @@ embbag_fwd_flat_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
     bag = (int64_t)blockIdx.x * lanes.groups + lanes.grp;
   }
   if (!lanes.on() || bag >= n_bags) return;
+  const int nvec = dim / EPV;
   int32_t begin, len;
   flat_range(bag_offsets, bag, nnz, lg, status, begin, len);
   bool bad = false;
@@ -335,12 +335,12 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
 // and whether in field-major order.  More rows in flight per lane mean fewer warps (eight: 4 CTAs per SM, four: 5),
 // which pays once a bag has ids enough to fill them; a grid of one wave (2 waves 1 - 5% slower, 8 CTAs per SM no faster
 // than the other kernels).  us before -> reading ahead, by ids per bag, one resident wave of bags (W 1) and many:
-//   fp32, 32 vectors   3: 368 -> 503   10, W 1 / 3 / 24: 13.2 / 25.1 / 122 -> 11.4 / 22.0 / 107   25: 782 -> 693
+//   fp32, 32 vectors   3: 368 -> 503   5.5: 257 -> 264   10, W 1 / 3 / 24: 13.2 / 25.1 / 122 -> 11.4 / 22.0 / 107   25: 782 -> 693
 //         16 vectors   2: 190 -> 235   6, W 1 / 24: 11.1 / 100 -> 10.3 / 95   15, W 3 / 24: 33 / 178 -> 28 / 151
 //          8 vectors   four rows: 4: 153 -> 146, but 35 M ids over 50 M rows 839 -> 883   10, W 24: 153 -> 145
 //          4 vectors   3, W 24: 99 -> 91   8: 148 -> 140   15: 205 -> 185
 //   bf16, 32 vectors   12, W 6 / 24: 52 / 169 -> 52 / 171   25: 281 -> 247
-//         16 vectors   4: 331 -> 337   9, W 1 / 24: 14.5 / 160 -> 12.9 / 144   12: 634 -> 567
+//         16 vectors   4: 331 -> 337   5.5, W 1 / 24: 30.8 / 195 -> 27.1 / 182   9, W 1 / 24: 14.5 / 160 -> 12.9 / 144   12: 634 -> 567
 //          8 vectors   four rows: 2, W 24: 91 -> 85   eight: 5, W 24: 136 -> 116   15: 248 -> 214   20: 531 -> 461
 //          4 vectors   four rows: 4, W 24: 136 -> 122   15: 258 -> 234
 // Inside a step, with bags of eight ids and more: one field at a time, not read ahead | bag order | field order:
@@ -360,7 +360,7 @@ inline Ahead ahead_of(int G, bool bf16, bool fields_known, int64_t bags_per_cta,
     return G == 32 && ids(8) ? Ahead{8, false} : G == 8 && ids(8) ? Ahead{4, false} : G == 4 && ids(3) ? Ahead{8, false} : no;
   }
   if (G == 32) return ids(16) ? Ahead{8, false} : no;
-  if (G == 16) return ids(8) ? Ahead{8, false} : no;
+  if (G == 16) return ids(fields_known ? 8 : 5) ? Ahead{8, false} : no;
   if (G == 8) return ids(4) ? Ahead{8, fields_known && ids(16)} : ids(2) ? Ahead{4, false} : no;
   return ids(3) ? Ahead{4, fields_known} : no;
 }
