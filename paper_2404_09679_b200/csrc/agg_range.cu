@@ -11,6 +11,8 @@
 // A direct gather-and-sum per distinct id inside the range CTA was measured first: 2.5 ms on the
 // 100M-row workload against 1.06 ms for the tile reduction on the merge order, whose walk keeps
 // four row loads in flight per lane and has no per-row search.
+#include <algorithm>
+
 #include "agg_range.cuh"
 #include "segsort.cuh"
 
@@ -756,8 +758,12 @@ void range_merge_order(const int32_t* uniq_ids, const int64_t* wuo_in, int64_t i
     WeightBlob wb = {};
     for (int i = 0; weights_host && i < K; ++i) wb.w[i] = weights_host[i];
     const int64_t n_search = (int64_t)K * (P + 1);
+    // CTAs for the searches, or for the clearing (16 words a thread, up to a wave) where the lists' capacity is large beside
+    // the table: 7.1 M entries of room over 34 k rows 101 -> 58 us
+    const int64_t n_clear = std::min((n_words + n_tiles + 16 * kRaThreads - 1) / (16 * kRaThreads), (int64_t)8 * kNumSM);
 #define SPLIT_GO(G)                                                                                                     \
-  ANTDT_LAUNCH("agg_range_split", range_split_kernel<G>, (unsigned)((n_search * G + kRaThreads - 1) / kRaThreads),       \
+  ANTDT_LAUNCH("agg_range_split", range_split_kernel<G>,                                                               \
+               (unsigned)std::max((n_search * G + kRaThreads - 1) / kRaThreads, n_clear),                               \
                kRaThreads, 0, s, uniq_ids, wuo_in, K, in_cap, r_log2, P, n_rows, dropped, wuo_out, bnd, wb,             \
                w_out, head_bits, n_words, tiles, n_tiles, status)
     if (n_search <= kSplitTogether) SPLIT_GO(8); else SPLIT_GO(1);
