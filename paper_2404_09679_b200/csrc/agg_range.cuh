@@ -33,10 +33,12 @@ inline int range_log2(int64_t n_rows, int64_t in_cap) {
 // entries per range: 234 k of 90 workers over 1 M rows (240, one wave) 64 -> 56 us, 936 k of 64 over 2 M (480) 109 -> 82, of
 // 90 over 2.5 M (383) 113 -> 94, 2.3 M of 40 over 5 M (480) 193 -> 168, 2.5 M of 64 over 10 M (260) 398 -> 389, 4.7 M of
 // 100 over 5 M (960) 297 -> 295; but 936 k of 90 over 5 M (192) 118 -> 119, 2.7 M of 100 over 20 M (140) 592 -> 639.
+// Above 10000 entries of room to a range (8 ns each in its one CTA) the sort is faster: 2.3 M of 57 over 110 k rows
+// (22 k) 115 -> 190, where 73 workers' lists with room for 9.7 k go 144 -> 95.
 // The boundaries cost K (P + 1) words, in the scratch of the sort (8 bytes an entry).
 constexpr int kRangeWideWorkers = 128;
 constexpr int kRangeWideLog2 = 10, kRangeWideMaxLog2 = 11;
-constexpr int64_t kRangeWideWave = 8 * kNumSM, kRangeWideEntries = 250;
+constexpr int64_t kRangeWideWave = 8 * kNumSM, kRangeWideEntries = 250, kRangeWideMost = 10000;
 inline int64_t ranges_of(int64_t n_rows, int log2) { return (n_rows + ((int64_t)1 << log2) - 1) >> log2; }
 // Ranges twice as wide where a worker has fewer than two entries in one.
 inline int range_wide_log2(int K, int64_t n_rows, int64_t in_cap) {
@@ -45,7 +47,7 @@ inline int range_wide_log2(int K, int64_t n_rows, int64_t in_cap) {
 inline bool range_wide_wanted(int K, int64_t n_rows, int64_t in_cap) {
   if (K <= kRangeMaxWorkers || K > kRangeWideWorkers) return false;
   const int64_t P = ranges_of(n_rows, kRangeWideLog2);
-  return (P <= kRangeWideWave || in_cap >= kRangeWideEntries * P) &&
+  return (P <= kRangeWideWave || in_cap >= kRangeWideEntries * P) && in_cap <= kRangeWideMost * P &&
          2 * in_cap >= K * (ranges_of(n_rows, range_wide_log2(K, n_rows, in_cap)) + 1);
 }
 
