@@ -278,8 +278,7 @@ int32_t antdt_embbag_bwd_dedup_static(const int32_t* row_ids, int64_t nnz,
  * strictly (what antdt_embbag_bwd_dedup writes does); a list of up to 32 workers that repeats
  * ids so often that a stretch of 4096 consecutive row ids (8192 for tables beyond 2^30 rows or
  * inputs that hit the table sparsely) holds more entries than K times its width raises
- * BAD_OFFSETS in dev_status and that stretch is left out of the result; a list of more workers
- * that does not strictly ascend may raise BAD_OFFSETS too (where they are merged without a sort).
+ * BAD_OFFSETS in dev_status and that stretch is left out of the result.
  *   batch_sizes host [K] int64: the b_i actually served this step (counts), sum > 0. */
 typedef struct {
   int32_t dim;

@@ -1,7 +1,6 @@
 // Range-partitioned merge of the workers' row lists (see agg_range.cuh).
 //
-//   split    first entry of every worker's list at or after each range boundary (binary search; for more than 32
-//            workers every entry compares itself with the one before)
+//   split    first entry of every worker's list at or after each range boundary (binary search)
 //   count    per range: worker-set table in shared memory -> number of distinct row ids
 //   scan     distinct ids before each range; total = n_agg; capacity check
 //   emit     per range: the table again, prefix sums over it, then every entry's slot in the
@@ -38,7 +37,7 @@ constexpr int64_t kSplitTogether = 50000;  // boundaries up to which eight lanes
 template <int G>
 __global__ void __launch_bounds__(kRaThreads)
 range_split_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ wuo_in, int K,
-                   int64_t in_cap, int r_log2, int64_t P, int64_t n_rows, const RangeDropped dropped,
+                   int64_t in_cap, int r_log2, int64_t P, int64_t n_rows, uint32_t dropped,
                    int64_t* __restrict__ wuo_out, int32_t* __restrict__ bnd, const WeightBlob weights,
                    float* __restrict__ weights_out, uint32_t* __restrict__ zero_a, int64_t n_a,
                    uint32_t* __restrict__ zero_b, int64_t n_b, int32_t* status) {
@@ -89,166 +88,55 @@ range_split_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ 
     if (lg) return;
   }
   bnd[(size_t)w * (P + 1) + b] = (int32_t)lo;
-  if (b == P && (int64_t)lo < s_wuo[w + 1] && !dropped.has(w))
+  if (b == P && (int64_t)lo < s_wuo[w + 1] && !((dropped >> w) & 1u))
     set_status(status, ANTDT_ERR_ID_OUT_OF_RANGE);  // ids past the table
 }
 
-// The same for more than 32 workers, boundaries range by range: every entry compares its range with that of the one
-// before and writes the boundaries between them; a warp writes wide gaps together.  An entry that is not above the one
-// before raises BAD_OFFSETS.
-constexpr int kSplitItems = 4;
-struct WideWeights { float w[kRangeWideWorkers]; };
-__global__ void __launch_bounds__(kRaThreads)
-range_split_wide_kernel(const int32_t* __restrict__ ids, const int64_t* __restrict__ wuo_in, int K, int64_t in_cap,
-                        int r_log2, int32_t P, int64_t n_rows, const RangeDropped dropped, int64_t* __restrict__ wuo_out,
-                        int32_t* __restrict__ bnd, const WideWeights weights, float* __restrict__ weights_out,
-                        uint32_t* __restrict__ zero_a, int64_t n_a, uint32_t* __restrict__ zero_b, int64_t n_b,
-                        int32_t* status) {
-  pdl_sync();
-  constexpr unsigned kFull = 0xffffffffu;
-  __shared__ uint32_t s_wuo[kRangeWideWorkers + 1];
-  const int tid = threadIdx.x, lane = tid & 31;
-  if (blockIdx.x == 0 && weights_out && tid < K) weights_out[tid] = weights.w[tid];
-  if (tid < 32) {  // ascending and inside [0, in_cap], whatever came in
-    int64_t carry = 0;
-    for (int i0 = 0; i0 <= K; i0 += 32) {
-      const int i = i0 + lane;
-      const int64_t raw = i <= K ? __ldg(wuo_in + i) : 0;
-      if (i == K && blockIdx.x == 0 && (raw < 0 || raw > in_cap)) set_status(status, ANTDT_ERR_CAPACITY);
-      int64_t x = max(raw, carry);
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int64_t y = __shfl_up_sync(kFull, x, o);
-        if (lane >= o) x = max(x, y);
-      }
-      carry = __shfl_sync(kFull, x, 31);
-      if (i <= K) s_wuo[i] = (uint32_t)min(x, in_cap);
-    }
-  }
-  const int64_t thread = (int64_t)blockIdx.x * kRaThreads + tid, threads = (int64_t)gridDim.x * kRaThreads;
-  for (int64_t i = thread; i < n_a; i += threads) zero_a[i] = 0u;
-  for (int64_t i = thread; i < n_b; i += threads) zero_b[i] = 0u;
-  __syncthreads();
-  if (blockIdx.x == 0)
-    for (int i = tid; i <= K; i += kRaThreads) wuo_out[i] = s_wuo[i];
-  for (int w = blockIdx.x; w < K; w += gridDim.x)  // empty lists have no entry to write their boundaries
-    if (s_wuo[w] == s_wuo[w + 1])
-      for (int32_t b = tid; b <= P; b += kRaThreads) bnd[(size_t)b * K + w] = (int32_t)s_wuo[w];
-  const uint32_t n0 = s_wuo[0], n = s_wuo[K];
-  auto range_of = [&](uint32_t id) { return (int64_t)id < n_rows ? (int32_t)(id >> r_log2) : P; };  // P: past the table
-  // boundaries first .. last of worker w (none if last < first) lie at entry `at`; every lane of a warp calls this
-  auto put = [&](int32_t first, int32_t last, int w, uint32_t at) {
-    const bool wide = last - first >= 8;
-    if (!wide)
-      for (int32_t b = first; b <= last; ++b) bnd[(size_t)b * K + w] = (int32_t)at;
-    for (unsigned v = __ballot_sync(kFull, wide); v; v &= v - 1u) {
-      const int l = __ffs((int)v) - 1;
-      const int32_t f = __shfl_sync(kFull, first, l), e = __shfl_sync(kFull, last, l);
-      const int wl = __shfl_sync(kFull, w, l);
-      const uint32_t a = __shfl_sync(kFull, at, l);
-      for (int32_t b = f + lane; b <= e; b += 32) bnd[(size_t)b * K + wl] = (int32_t)a;
-    }
-  };
-  uint32_t id[kSplitItems], before[kSplitItems];
-  const uint32_t e0 = n0 + (uint32_t)blockIdx.x * (kRaThreads * kSplitItems) + tid;
-#pragma unroll
-  for (int t = 0; t < kSplitItems; ++t) {
-    const uint32_t e = e0 + t * kRaThreads;
-    id[t] = e < n ? (uint32_t)__ldg(ids + e) : 0u;
-    before[t] = e < n && e > 0 ? (uint32_t)__ldg(ids + e - 1) : 0u;
-  }
-#pragma unroll
-  for (int t = 0; t < kSplitItems; ++t) {
-    const uint32_t e = e0 + t * kRaThreads;
-    const bool on = e < n;
-    int w = 0;  // last w with s_wuo[w] <= e: the list that holds e
-#pragma unroll
-    for (int step = kRangeWideWorkers / 2; step > 0; step >>= 1)
-      if (w + step < K && s_wuo[w + step] <= e) w += step;
-    const bool first = on && e == s_wuo[w], last = on && e + 1 == s_wuo[w + 1];
-    const int32_t r = range_of(id[t]), rb = first ? -1 : range_of(before[t]);
-    if (on && !dropped.has(w)) {
-      if (!first && id[t] <= before[t]) set_status(status, ANTDT_ERR_BAD_OFFSETS);
-      if (r == P) set_status(status, ANTDT_ERR_ID_OUT_OF_RANGE);
-    }
-    put(on ? rb + 1 : 0, on ? r : -1, w, e);
-    put(last ? r + 1 : 0, last ? P : -1, w, e + 1);
-  }
-}
-
-// Workers that a set of NW words has room for, rounded up to a power of two (the search among pieces).
-template <int NW> constexpr int kSlots = NW == 3 ? 128 : 32 * NW;
-
 // The pieces of range b: worker w's entries [s_beg[w], s_beg[w] + size) with s_off[w] entries of
-// earlier workers before them (s_off[kSlots] = entries in the range; a dropped worker's piece is
+// earlier workers before them (s_off[K] = entries in the range; a dropped worker's piece is
 // empty).  Also the number of entries of all earlier ranges.  One barrier inside.
-// Up to 32 workers (NW 1) the boundaries lie worker by worker, above range by range: a lane holds kSlots / 32
-// workers in a row.  There they were not searched for, so a list that does not ascend has left some unwritten: whatever
-// is read is held inside its worker's list.
 struct Pieces { int entries; int64_t before; };
-template <int NW>
 __device__ __forceinline__ Pieces range_pieces(const int32_t* __restrict__ bnd,
                                                const int64_t* __restrict__ wuo, int K, int64_t P,
-                                               int64_t b, const RangeDropped& dropped, int32_t* s_beg,
+                                               int64_t b, uint32_t dropped, int32_t* s_beg,
                                                int32_t* s_off, int64_t* s_before) {
   if (threadIdx.x < 32) {
-    constexpr int PER = kSlots<NW> / 32;
-    const int lane = threadIdx.x;
-    int beg[PER], size[PER], sum = 0;
+    const int w = threadIdx.x;
+    int beg = 0, size = 0;
     int64_t before = 0;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      const int w = lane * PER + i;
-      beg[i] = 0;
-      size[i] = 0;
-      if (w < K && !dropped.has(w)) {
-        const int32_t* at = NW == 1 ? bnd + (size_t)w * (P + 1) + b : bnd + (size_t)b * K + w;
-        int64_t lo = __ldg(at), hi = __ldg(at + (NW == 1 ? 1 : K));
-        const int64_t first = __ldg(wuo + w);
-        if (NW > 1) {
-          const int64_t end = __ldg(wuo + w + 1);
-          lo = min(max(lo, first), end);
-          hi = min(max(hi, first), end);
-        }
-        beg[i] = (int)lo;
-        size[i] = hi > lo ? (int)(hi - lo) : 0;  // a list that does not ascend: treated as empty here
-        before += lo - first;
-      }
-      sum += size[i];
+    if (w < K && !((dropped >> w) & 1u)) {
+      beg = __ldg(bnd + (size_t)w * (P + 1) + b);
+      const int end = __ldg(bnd + (size_t)w * (P + 1) + b + 1);
+      size = end > beg ? end - beg : 0;  // a list that does not ascend: treated as empty here
+      before = (int64_t)beg - __ldg(wuo + w);
     }
-    int incl = sum;
+    int incl = size;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
+      if (w >= o) incl += t;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
-    int off = incl - sum;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-      s_beg[lane * PER + i] = beg[i];
-      s_off[lane * PER + i] = off;
-      off += size[i];
-    }
-    if (lane == 31) s_off[kSlots<NW>] = incl;
-    if (lane == 0) *s_before = before;
+    s_beg[w] = beg;
+    s_off[w] = incl - size;
+    if (w == 31) s_off[32] = incl;
+    if (w == 0) *s_before = before;
   }
   __syncthreads();
   Pieces p;
-  p.entries = s_off[kSlots<NW>];
+  p.entries = s_off[32];
   p.before = *s_before;
   return p;
 }
 
 // Entry e of the range (entries numbered worker by worker): its worker and its position in the
 // concatenated lists.
-template <int NW>
 __device__ __forceinline__ void entry_of(int e, const int32_t* s_beg, const int32_t* s_off, int& w,
                                          int& j) {
   int lo = 0;  // last w with s_off[w] <= e: the non-empty piece that holds e
 #pragma unroll
-  for (int step = kSlots<NW> / 2; step > 0; step >>= 1)
+  for (int step = 16; step > 0; step >>= 1)
     if (s_off[lo + step] <= e) lo += step;
   w = lo;
   j = s_beg[lo] + (e - s_off[lo]);
@@ -257,7 +145,7 @@ __device__ __forceinline__ void entry_of(int e, const int32_t* s_beg, const int3
 // One pass over the range's entries, a batch of loads in flight per thread.  f(w, j, id, kl)
 // for the entries whose row id lies in the range and in the table; the others raise
 // ID_OUT_OF_RANGE and are skipped.
-template <int NW, typename F>
+template <typename F>
 __device__ __forceinline__ void for_each_entry(const int32_t* __restrict__ ids, int entries, int R,
                                                uint32_t base_key, int64_t n_rows, const int32_t* s_beg,
                                                const int32_t* s_off, int32_t* status, F f) {
@@ -267,7 +155,7 @@ __device__ __forceinline__ void for_each_entry(const int32_t* __restrict__ ids, 
 #pragma unroll
     for (int t = 0; t < kRaBatch; ++t) {
       const int e = e0 + t * kRaThreads;
-      entry_of<NW>(e < entries ? e : e0, s_beg, s_off, w[t], j[t]);
+      entry_of(e < entries ? e : e0, s_beg, s_off, w[t], j[t]);
       id[t] = (uint32_t)__ldg(ids + j[t]);
     }
 #pragma unroll
@@ -306,24 +194,23 @@ __device__ __forceinline__ void block_scan2(int& a, int& b, int& tot_a, int& tot
 }
 
 // Distinct row ids of range b: one presence bit per row id of the range.
-template <int NW>
 __global__ void __launch_bounds__(kRaThreads)
 range_count_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ bnd,
                    const int64_t* __restrict__ wuo, int K, int64_t P, int r_log2, int64_t n_rows,
-                   const RangeDropped dropped, int32_t* __restrict__ distinct, int32_t* status) {
+                   uint32_t dropped, int32_t* __restrict__ distinct, int32_t* status) {
   pdl_sync();
   __shared__ uint32_t pres[(1 << kRangeMaxLog2) / 32];
   __shared__ int64_t s_before;
-  __shared__ int32_t s_beg[kSlots<NW>], s_off[kSlots<NW> + 1], s_tmp[2 * kRaWarps];
+  __shared__ int32_t s_beg[32], s_off[33], s_tmp[2 * kRaWarps];
   const int R = 1 << r_log2;
   const int64_t b = blockIdx.x;
   if (threadIdx.x < R / 32) pres[threadIdx.x] = 0u;
-  const Pieces pc = range_pieces<NW>(bnd, wuo, K, P, b, dropped, s_beg, s_off, &s_before);
+  const Pieces pc = range_pieces(bnd, wuo, K, P, b, dropped, s_beg, s_off, &s_before);
   if (pc.entries == 0) {
     if (threadIdx.x == 0) distinct[b] = 0;
     return;
   }
-  for_each_entry<NW>(ids, pc.entries, R, (uint32_t)(b << r_log2), n_rows, s_beg, s_off, status,
+  for_each_entry(ids, pc.entries, R, (uint32_t)(b << r_log2), n_rows, s_beg, s_off, status,
                  [&](int, int, uint32_t, uint32_t kl) { atomicOr(&pres[kl >> 5], 1u << (kl & 31)); });
   __syncthreads();
   int cnt = threadIdx.x < R / 32 ? __popc(pres[threadIdx.x]) : 0, zero = 0, tot, tz;
@@ -338,19 +225,15 @@ range_count_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ 
 __global__ void __launch_bounds__(1024)
 range_scan_kernel(const int32_t* __restrict__ distinct, int64_t P, int64_t* __restrict__ base,
                   int64_t* __restrict__ n_agg, int64_t out_cap, const int32_t* __restrict__ bnd,
-                  const int64_t* __restrict__ wuo, int K, int64_t bnd_step, int64_t bnd_last,
-                  const RangeDropped dropped, int64_t* __restrict__ n_entries,
+                  const int64_t* __restrict__ wuo, int K, uint32_t dropped, int64_t* __restrict__ n_entries,
                   int32_t* status) {
   pdl_sync();
   __shared__ int64_t warp_tot[32];
   const int tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   if (wp == 31) {
     int64_t kept = 0;
-    for (int w = lane; w < K; w += 32)  // bnd_last: where the list of worker 0 ends among the boundaries
-      if (!dropped.has(w)) {
-        const int64_t first = __ldg(wuo + w), end = __ldg(wuo + w + 1);
-        kept += max((int64_t)0, min((int64_t)__ldg(bnd + w * bnd_step + bnd_last), end) - first);
-      }
+    if (lane < K && !((dropped >> lane) & 1u))
+      kept = max((int64_t)0, (int64_t)__ldg(bnd + (size_t)lane * (P + 1) + P) - __ldg(wuo + lane));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) kept += __shfl_xor_sync(0xffffffffu, kept, o);
     if (lane == 0) {
@@ -426,7 +309,7 @@ template <int KEPT>
 __global__ void __launch_bounds__(kRaThreads)
 range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ bnd,
                   const int64_t* __restrict__ wuo, int K, int64_t P, int r_log2, int64_t n_rows,
-                  const RangeDropped dropped, const int64_t* __restrict__ base, int32_t* __restrict__ agg_ids,
+                  uint32_t dropped, const int64_t* __restrict__ base, int32_t* __restrict__ agg_ids,
                   int64_t out_cap, uint32_t* __restrict__ src, uint32_t* head_bits,
                   int32_t* __restrict__ tile_first, int tile_shift, uint32_t* __restrict__ row_start,
                   uint8_t* __restrict__ src_worker, int staged, int32_t* status) {
@@ -453,7 +336,7 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
   const int64_t b = blockIdx.x;
   const int tid = threadIdx.x;
   const int64_t u0 = __ldg(base + b);  // requested now: every global round trip here is serial
-  const Pieces pc = range_pieces<1>(bnd, wuo, K, P, b, dropped, s_beg, s_off, s_before);
+  const Pieces pc = range_pieces(bnd, wuo, K, P, b, dropped, s_beg, s_off, s_before);
   if (pc.entries == 0) return;
   // A worker lists a row id at most once, so a range holds at most R*K entries and the arrays
   // below are sized for that.  More means a list that does not strictly ascend: flag it and
@@ -494,7 +377,7 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
       for (int t = 0; t < kRaBatch; ++t) {
         const int e = (g + t) * kRaThreads + tid;
         int j;
-        entry_of<1>(e < pc.entries ? e : 0, s_beg, s_off, w[t], j);
+        entry_of(e < pc.entries ? e : 0, s_beg, s_off, w[t], j);
         kept_j[g + t] = (uint32_t)j;
         id[t] = (uint32_t)__ldg(ids + j);
       }
@@ -511,7 +394,7 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
       }
     }
   } else {
-    for_each_entry<1>(ids, pc.entries, R, base_key, n_rows, s_beg, s_off, status,
+    for_each_entry(ids, pc.entries, R, base_key, n_rows, s_beg, s_off, status,
                       [&](int w, int, uint32_t, uint32_t kl) { fill(w, kl); });
   }
   if (KEPT > 4)
@@ -569,7 +452,7 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
     for (int t = 0; t < KEPT; ++t)
       if (kept[t] != kNone) place((int)(kept[t] & 31u), kept_j[t], (int)(kept[t] >> 8));
   } else {
-    for_each_entry<1>(ids, pc.entries, R, base_key, n_rows, s_beg, s_off, nullptr,
+    for_each_entry(ids, pc.entries, R, base_key, n_rows, s_beg, s_off, nullptr,
                       [&](int w, int j, uint32_t, uint32_t kl) { place(w, (uint32_t)j, (int)kl); });
   }
   if (KEPT == 4) return;
@@ -579,112 +462,6 @@ range_emit_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ b
     if (src_worker) src_worker[pc.before + i] = st_worker[i];
   }
 }
-
-// The same for more than 32 workers: NW words to a worker set, word-major.  Ranges are many and short here (some 100
-// to 1000 entries), so a CTA is a chain of latencies: every thread sums up R / 256 ids that lie side by side instead of
-// walking the bits of a presence word, and keeps its first entries in registers from the fill to the end.
-constexpr int kWideHeadSlots = 4096;  // slots of a range whose head bits are collected in shared memory first
-template <int NW, int PER>  // PER: ids per thread, the range's width / 256
-__global__ void __launch_bounds__(kRaThreads)
-range_emit_wide_kernel(const int32_t* __restrict__ ids, const int32_t* __restrict__ bnd,
-                       const int64_t* __restrict__ wuo, int K, int64_t P, int64_t n_rows,
-                       const RangeDropped dropped, const int64_t* __restrict__ base, int32_t* __restrict__ agg_ids,
-                       int64_t out_cap, uint32_t* __restrict__ src, uint32_t* head_bits,
-                       int32_t* __restrict__ tile_first, int tile_shift, int32_t* status) {
-  pdl_sync();
-  constexpr int R = PER * kRaThreads;
-  constexpr int kHeadWords = kWideHeadSlots / 32 + 1;
-  extern __shared__ __align__(16) unsigned char ra_smem[];
-  uint32_t* const mask = reinterpret_cast<uint32_t*>(ra_smem);       // [NW][R]
-  uint32_t* const first_c = mask + NW * R;                           // [R] contributions of smaller ids
-  uint16_t* const rank = reinterpret_cast<uint16_t*>(first_c + R);   // [R] smaller ids
-  __shared__ int64_t s_before;
-  __shared__ int32_t s_beg[kSlots<NW>], s_off[kSlots<NW> + 1], s_tmp[2 * kRaWarps];
-  __shared__ uint32_t hb[kHeadWords];
-  const int64_t b = blockIdx.x;
-  const int tid = threadIdx.x;
-  const int64_t u0 = __ldg(base + b);  // requested now: every global round trip here is serial
-  for (int i = tid; i < NW * R / 4; i += kRaThreads) reinterpret_cast<uint4*>(mask)[i] = make_uint4(0u, 0u, 0u, 0u);
-  if (tid < kHeadWords) hb[tid] = 0u;
-  const Pieces pc = range_pieces<NW>(bnd, wuo, K, P, b, dropped, s_beg, s_off, &s_before);
-  if (pc.entries == 0) return;
-  if (pc.entries > K * R) {  // lists that do not strictly ascend: as above
-    if (tid == 0) set_status(status, ANTDT_ERR_BAD_OFFSETS);
-    return;
-  }
-  const uint32_t base_key = (uint32_t)b * (uint32_t)R;
-  uint32_t kept_j[kRaBatch], kept[kRaBatch];  // position, and id inside the range << 8 | worker
-  auto load = [&](int e0) {
-#pragma unroll
-    for (int t = 0; t < kRaBatch; ++t) {
-      const int e = e0 + t * kRaThreads;
-      int w, j;
-      entry_of<NW>(e < pc.entries ? e : 0, s_beg, s_off, w, j);
-      const uint32_t id = (uint32_t)__ldg(ids + j), kl = id - base_key;
-      kept_j[t] = (uint32_t)j;
-      kept[t] = e < pc.entries && kl < (uint32_t)R && (int64_t)id < n_rows ? kl << 8 | (uint32_t)w : 0xffffffffu;
-      if (e < pc.entries && kept[t] == 0xffffffffu) set_status(status, ANTDT_ERR_ID_OUT_OF_RANGE);
-    }
-  };
-  const int last = (pc.entries - 1) / (kRaBatch * kRaThreads) * (kRaBatch * kRaThreads);
-  for (int e0 = 0; e0 <= last; e0 += kRaBatch * kRaThreads) {
-    load(e0 + tid);
-#pragma unroll
-    for (int t = 0; t < kRaBatch; ++t)
-      if (kept[t] != 0xffffffffu) atomicOr(&mask[(kept[t] >> 5 & 7u) * R + (kept[t] >> 8)], 1u << (kept[t] & 31u));
-  }
-  __syncthreads();
-  int n[PER], n_ids = 0, n_con = 0;
-#pragma unroll
-  for (int i = 0; i < PER; i += 4) {
-    n[i] = n[i + 1] = n[i + 2] = n[i + 3] = 0;
-#pragma unroll
-    for (int k = 0; k < NW; ++k) {
-      const uint4 m = *reinterpret_cast<const uint4*>(mask + k * R + tid * PER + i);
-      n[i] += __popc(m.x); n[i + 1] += __popc(m.y); n[i + 2] += __popc(m.z); n[i + 3] += __popc(m.w);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < PER; ++i) { n_con += n[i]; n_ids += n[i] > 0; }
-  int tot_ids, tot_con;
-  block_scan2(n_ids, n_con, tot_ids, tot_con, s_tmp);  // now exclusive prefixes
-  const int hb_shift = (int)(pc.before & 31);
-  const bool staged = hb_shift + pc.entries <= kHeadWords * 32;
-#pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    first_c[tid * PER + i] = (uint32_t)n_con;
-    rank[tid * PER + i] = (uint16_t)n_ids;
-    if (n[i] > 0) {
-      const int at = hb_shift + n_con;
-      if (staged) atomicOr(&hb[at >> 5], 1u << (at & 31));
-      else atomicOr(&head_bits[(pc.before >> 5) + (at >> 5)], 1u << (at & 31));
-      ++n_ids;
-    }
-    n_con += n[i];
-  }
-  __syncthreads();
-  if (staged && tid < kHeadWords && hb[tid]) atomicOr(&head_bits[(pc.before >> 5) + tid], hb[tid]);
-  const int64_t tile_mask = ((int64_t)1 << tile_shift) - 1;
-  for (int e0 = last; e0 >= 0; e0 -= kRaBatch * kRaThreads) {  // what is kept first
-    if (e0 < last) load(e0 + tid);
-#pragma unroll
-    for (int t = 0; t < kRaBatch; ++t) {
-      if (kept[t] == 0xffffffffu) continue;
-      const int kl = (int)(kept[t] >> 8), w = (int)(kept[t] & 255u);
-      int slot = 0;
-#pragma unroll
-      for (int k = 0; k < NW; ++k) {
-        const uint32_t m = mask[k * R + kl];
-        slot += k < (w >> 5) ? __popc(m) : (k == (w >> 5) ? __popc(m & ((1u << (w & 31)) - 1u)) : 0);
-      }
-      const int64_t dest = pc.before + (int64_t)first_c[kl] + slot, u = u0 + rank[kl];
-      src[dest] = kept_j[t];
-      if (slot == 0 && u < out_cap) agg_ids[u] = (int32_t)(base_key + (uint32_t)kl);
-      if ((dest & tile_mask) == 0) tile_first[dest >> tile_shift] = (int32_t)u;
-    }
-  }
-}
-size_t emit_wide_smem(int r_log2, int words) { return ((size_t)4 * words + 6) << r_log2; }
 
 // Slots of a range that are put in order in shared memory: those of an average range and a quarter more (the others are
 // stored where they are found).
@@ -730,70 +507,48 @@ void range_prepare_device() {
 }
 
 void range_merge_order(const int32_t* uniq_ids, const int64_t* wuo_in, int64_t in_cap, int64_t n_rows,
-                       int K, const RangeDropped& dropped, int32_t* agg_ids, int64_t* n_agg, int64_t out_cap,
+                       int K, uint32_t dropped_bits, int32_t* agg_ids, int64_t* n_agg, int64_t out_cap,
                        int64_t* wuo_out, int64_t* n_entries, uint32_t* src, uint32_t* head_bits,
                        int32_t* tile_first, int tile, uint32_t* row_start, uint8_t* src_worker,
                        const float* weights_host,
-                       float* weights_dev, int32_t* bnd, int32_t* distinct, int64_t* base, int32_t* status,
+                       float* weights_dev, char* ws, const RangeLayout& L, int32_t* status,
                        cudaStream_t s) {
   range_prepare_device();
-  const bool wide = K > kRangeMaxWorkers;
-  const int r_log2 = wide ? range_wide_log2(K, n_rows, in_cap) : range_log2(n_rows, in_cap);
-  const int64_t P = (n_rows + ((int64_t)1 << r_log2) - 1) >> r_log2;
+  WeightBlob wb;
+  for (int i = 0; i < kRangeMaxWorkers; ++i) wb.w[i] = (weights_host && i < K) ? weights_host[i] : 0.f;
+  const int r_log2 = range_log2(n_rows, in_cap);
+  const int64_t P = (n_rows + ((int64_t)1 << r_log2) - 1) >> r_log2;  // <= kRangeMaxRanges
+  int32_t* bnd = (int32_t*)(ws + L.bnd);
+  int32_t* distinct = (int32_t*)(ws + L.distinct);
+  int64_t* base = (int64_t*)(ws + L.base);
   int tile_shift = 0;
   while ((1 << tile_shift) < tile) ++tile_shift;
+  const int64_t n_search = (int64_t)K * (P + 1);
   // every tile's entry is written unless ids were skipped as invalid: start from a valid index
   const int64_t n_tiles = tile_first ? ((in_cap + tile - 1) >> tile_shift) + 1 : 0;
   const int64_t n_words = head_bits ? (int64_t)head_bits_words(in_cap) : 0;
-  uint32_t* const tiles = reinterpret_cast<uint32_t*>(tile_first);
-  float* const w_out = weights_host ? weights_dev : nullptr;
-  if (wide) {
-    WideWeights wb = {};
-    for (int i = 0; weights_host && i < K; ++i) wb.w[i] = weights_host[i];
-    ANTDT_LAUNCH("agg_range_split", range_split_wide_kernel,
-                 (unsigned)((in_cap + kRaThreads * kSplitItems - 1) / (kRaThreads * kSplitItems)), kRaThreads, 0, s, uniq_ids,
-                 wuo_in, K, in_cap, r_log2, (int32_t)P, n_rows, dropped, wuo_out, bnd, wb, w_out, head_bits, n_words, tiles,
-                 n_tiles, status);
-  } else {
-    WeightBlob wb = {};
-    for (int i = 0; weights_host && i < K; ++i) wb.w[i] = weights_host[i];
-    const int64_t n_search = (int64_t)K * (P + 1);
-    // CTAs for the searches, or for the clearing (16 words a thread, up to a wave) where the lists' capacity is large beside
-    // the table: 7.1 M entries of room over 34 k rows 101 -> 58 us
-    const int64_t n_clear = std::min((n_words + n_tiles + 16 * kRaThreads - 1) / (16 * kRaThreads), (int64_t)8 * kNumSM);
+  // CTAs for the searches, or for the clearing (16 words a thread, up to a wave) where the lists' capacity is large beside
+  // the table: 7.1 M entries of room over 34 k rows 101 -> 58 us
+  const int64_t n_clear = std::min((n_words + n_tiles + 16 * kRaThreads - 1) / (16 * kRaThreads), (int64_t)8 * kNumSM);
 #define SPLIT_GO(G)                                                                                                     \
   ANTDT_LAUNCH("agg_range_split", range_split_kernel<G>,                                                               \
                (unsigned)std::max((n_search * G + kRaThreads - 1) / kRaThreads, n_clear),                               \
-               kRaThreads, 0, s, uniq_ids, wuo_in, K, in_cap, r_log2, P, n_rows, dropped, wuo_out, bnd, wb,             \
-               w_out, head_bits, n_words, tiles, n_tiles, status)
-    if (n_search <= kSplitTogether) SPLIT_GO(8); else SPLIT_GO(1);
+               kRaThreads, 0, s, uniq_ids, wuo_in, K, in_cap, r_log2, P, n_rows, dropped_bits, wuo_out, bnd, wb,        \
+               weights_host ? weights_dev : nullptr, head_bits, n_words, reinterpret_cast<uint32_t*>(tile_first), n_tiles, \
+               status)
+  if (n_search <= kSplitTogether) SPLIT_GO(8); else SPLIT_GO(1);
 #undef SPLIT_GO
-  }
-#define COUNT_GO(NW)                                                                                                  \
-  ANTDT_LAUNCH("agg_range_count", range_count_kernel<NW>, (unsigned)P, kRaThreads, 0, s,                              \
-               uniq_ids, bnd, wuo_out, K, P, r_log2, n_rows, dropped, distinct, status)
-  if (K <= 32) COUNT_GO(1); else if (K <= 64) COUNT_GO(2); else if (K <= 96) COUNT_GO(3); else COUNT_GO(4);
-#undef COUNT_GO
+  ANTDT_LAUNCH("agg_range_count", range_count_kernel, (unsigned)P, kRaThreads, 0, s,
+               uniq_ids, bnd, wuo_out, K, P, r_log2, n_rows, dropped_bits, distinct, status);
   ANTDT_LAUNCH("agg_range_scan", range_scan_kernel, 1, 1024, 0, s, distinct, P, base, n_agg, out_cap,
-               bnd, wuo_out, K, wide ? (int64_t)1 : P + 1, wide ? P * K : P, dropped, n_entries, status);
-#define WIDE_GO(NW, PER)                                                                                              \
-  ANTDT_LAUNCH("agg_range_emit", (range_emit_wide_kernel<NW, PER>), (unsigned)P, kRaThreads, emit_wide_smem(r_log2, NW), s, \
-               uniq_ids, bnd, wuo_out, K, P, n_rows, dropped, base, agg_ids, out_cap, src, head_bits, tile_first,    \
-               tile_shift, status)
+               bnd, wuo_out, K, dropped_bits, n_entries, status);
   const int staged = emit_staged(K, in_cap, P);
 #define EMIT_GO(KEPT)                                                                                                 \
   ANTDT_LAUNCH("agg_range_emit", range_emit_kernel<KEPT>, (unsigned)P, kRaThreads,                                    \
                emit_smem(r_log2, K, staged, src_worker != nullptr, head_bits != nullptr), s,                          \
-               uniq_ids, bnd, wuo_out, K, P, r_log2, n_rows, dropped, base, agg_ids, out_cap, src,                    \
+               uniq_ids, bnd, wuo_out, K, P, r_log2, n_rows, dropped_bits, base, agg_ids, out_cap, src,               \
                head_bits, tile_first, tile_shift, row_start, src_worker, staged, status)
-  if (!wide) {
-    if (staged) EMIT_GO(8); else EMIT_GO(4);
-  } else if (r_log2 == kRangeWideLog2) {
-    if (K <= 64) WIDE_GO(2, 4); else if (K <= 96) WIDE_GO(3, 4); else WIDE_GO(4, 4);
-  } else {
-    if (K <= 64) WIDE_GO(2, 8); else if (K <= 96) WIDE_GO(3, 8); else WIDE_GO(4, 8);
-  }
-#undef WIDE_GO
+  if (staged) EMIT_GO(8); else EMIT_GO(4);
 #undef EMIT_GO
 }
 

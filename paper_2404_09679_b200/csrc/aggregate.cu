@@ -1,8 +1,7 @@
 // Server aggregation: batch-size weighted sum of the workers' mean gradients.
 //
 // Sparse part, up to 32 workers: the range-partitioned merge of agg_range.cu (no sort).
-// Sparse part, 33 to 128 workers whose lists are not too sparse in the table: the same (range_wide_wanted).
-// Sparse part, small lists and other ones of up to 1.8 M entries and 128 workers: the resident merge
+// Sparse part, small lists and up to 1.8 M entries of 33 to 128 workers: the resident merge
 // (residentsort.cu).
 // Sparse part, more: the workers' row lists (each ascending) are merged by one stable radix sort of
 // (row id, position in the concatenated list); equal rows then sit together in ascending
@@ -582,9 +581,8 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
   char* w8 = static_cast<char*>(ws);
 
   // the two merges carry the weights themselves
-  bool resident = sp && !merged && resident_merge_wanted(K, in_cap, sp->n_rows) &&
-                  !(range_wide_wanted(K, sp->n_rows, in_cap) && !resident_sort_clears(in_cap));
-  const bool by_ranges = sp && in_cap > 0 && (K <= kRangeMaxWorkers || range_wide_wanted(K, sp->n_rows, in_cap));
+  bool resident = sp && !merged && resident_merge_wanted(K, in_cap, sp->n_rows);
+  const bool by_ranges = sp && K <= kRangeMaxWorkers && in_cap > 0;
   // a lane group per row: the one-pass update, and the sums of short lists
   const bool few = sp && !fu && K <= kRangeMaxWorkers && sum_by_rows(in_cap, sp->dim, sp->n_rows);
   bool by_rows = sp && in_cap > 0 && ((fu && K <= kRangeMaxWorkers) || (!fu && resident && resident_sort_clears(in_cap)) || few);
@@ -638,25 +636,20 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
     if (merged || resident) {
       // the merge order is there: the backward's sort made it on the way, or the resident merge
     } else if (by_ranges) {
-      // the merge order comes from the range-partitioned pass, no sort
-      RangeDropped drop = {};
+      // up to 32 workers: the merge order comes from the range-partitioned pass, no sort
+      uint32_t dropped_bits = 0;
       for (int i = 0; i < K; ++i)
-        if (dropped && dropped[i]) drop.bits[i >> 5] |= 1u << (i & 31);
-      // scratch: its own, or with more than 32 workers the sort's (keys_a and keys_b lie side by side)
-      const bool wide = K > kRangeMaxWorkers;
-      int32_t* const bnd = (int32_t*)(wide ? w8 + L.keys_a : w8 + L.range_ws + L.range.bnd);
-      int64_t* const base = (int64_t*)(wide ? w8 + L.run_start : w8 + L.range_ws + L.range.base);
-      int32_t* const distinct = (int32_t*)(wide ? w8 + L.vals_t : w8 + L.range_ws + L.range.distinct);
+        if (dropped && dropped[i]) dropped_bits |= 1u << i;
       // the order needs the id lists only: on a forked step it runs beside the backward's sums
       cudaStream_t so = fork ? fork->side : s;
       if (fork && cudaStreamWaitEvent(so, fork->ids_ready, 0) != cudaSuccess) return ANTDT_ERR_CUDA;
-      range_merge_order(sp->uniq_ids, sp->worker_uniq_offsets, in_cap, sp->n_rows, K, drop,
+      range_merge_order(sp->uniq_ids, sp->worker_uniq_offsets, in_cap, sp->n_rows, K, dropped_bits,
                         sp->agg_ids, sp->n_agg, agg_cap, (int64_t*)(w8 + L.wuo), bounds,
                         (uint32_t*)(w8 + L.src), by_rows ? nullptr : (uint32_t*)(w8 + L.head_bits),
                         by_rows ? nullptr : (int32_t*)(w8 + L.tile_first), red_tile_for(in_cap, sp->dim),
                         by_rows ? (uint32_t*)(w8 + L.row_start) : nullptr,
                         by_rows ? (uint8_t*)(w8 + L.src_worker) : nullptr, hw, (float*)(w8 + L.weights),
-                        bnd, distinct, base, dev_status, so);
+                        w8 + L.range_ws, L.range, dev_status, so);
       if (fork && (cudaEventRecord(fork->order_done, so) != cudaSuccess ||
                    cudaStreamWaitEvent(s, fork->order_done, 0) != cudaSuccess))
         return ANTDT_ERR_CUDA;

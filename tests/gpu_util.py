@@ -58,6 +58,17 @@ def new_status():
     return torch.zeros(1, dtype=torch.int32, device="cuda")
 
 
+def kernels_of(fn):
+    """fn's result and the names of the library's kernels that it launched."""
+    torch.cuda.synchronize()
+    B.antdt_profile_enable(True)
+    out = fn()
+    torch.cuda.synchronize()
+    names = {k for k, (n, _) in B.antdt_profile_get().items() if n > 0}
+    B.antdt_profile_enable(False)
+    return out, names
+
+
 def gpu_fwd(table_np, ids, off, status=None):
     t = table_to_dev(table_np)
     n_bags = off.shape[0] - 1

@@ -36,14 +36,8 @@ def stream():
 
 
 def _ran(fn, stream):
-    torch.cuda.synchronize()
-    B.antdt_profile_enable(True)
     with torch.cuda.stream(stream):
-        out = fn()
-    torch.cuda.synchronize()
-    names = {k for k, (n, _) in B.antdt_profile_get().items() if n > 0}
-    B.antdt_profile_enable(False)
-    return out, names
+        return G.kernels_of(fn)
 
 
 @pytest.mark.parametrize("n,K,resident", [(60_000, 3, True), (400_000, 3, False), (1_700_000, 2, False)])
@@ -68,6 +62,8 @@ def test_merge_of_many_workers(stream):
     uid, wuo = np.concatenate(parts), np.arange(K + 1, dtype=np.int64) * 12_000
     g = rng.normal(size=(len(uid), D)).astype(np.float32)
     bsz = rng.integers(1, 50, size=K)
+    _, names = G.kernels_of(lambda: G.gpu_aggregate(uid, wuo, g, bsz, V))
+    assert "resident_merge" in names                   # where all SMs are there
     (ids, agg, n, _, code), names = _ran(lambda: G.gpu_aggregate(uid, wuo, g, bsz, V), stream)
     want_ids, want = oracle.aggregate_sparse(uid, wuo, g, bsz.astype(np.int64))
     assert code == 0 and n == len(want_ids) and np.array_equal(ids, want_ids) and "resident_merge" not in names

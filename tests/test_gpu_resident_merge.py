@@ -18,14 +18,16 @@ def _lists(rng, K, V, sizes):
 
 @pytest.mark.parametrize("K,V,total", [
     (1, 5, 1), (2, 40, 33), (3, 1000, 1500), (32, 700, 8000), (5, 1 << 20, 16 * 2048), (5, 1 << 20, 16 * 2048 + 1),
-    (33, 90, 2000), (90, 200_000, 60_000), (128, 3000, 120_000), (129, 3000, 20_000), (40, 2_000_000, 900_000)])
+    (33, 90, 2000), (90, 200_000, 60_000), (128, 3000, 120_000), (129, 3000, 20_000), (40, 2_000_000, 900_000),
+    (60, 3_000_000, 1_700_000)])  # the last two: 16 and 24 pairs a thread
 def test_merge_matches_checker(K, V, total):
     rng = np.random.default_rng(K * 7 + total)
     cuts = np.sort(rng.integers(0, total + 1, size=K - 1))
     uid, wuo = _lists(rng, K, V, np.diff(np.concatenate([[0], cuts, [total]])))
     g = rng.normal(size=(len(uid), 8)).astype(np.float32)
     bsz = rng.integers(1, 50, size=K)
-    ids, agg, n, _, code = G.gpu_aggregate(uid, wuo, g, bsz, V)
+    (ids, agg, n, _, code), names = G.kernels_of(lambda: G.gpu_aggregate(uid, wuo, g, bsz, V))
+    assert ("resident_merge" in names) == (K <= 32 and total <= 16 * 2048 or 32 < K <= 128)
     want_ids, want = oracle.aggregate_sparse(uid, wuo, g, bsz.astype(np.int64))
     assert code == 0 and n == len(want_ids) and np.array_equal(ids, want_ids)
     G.close(agg, want)
