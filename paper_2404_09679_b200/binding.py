@@ -24,7 +24,7 @@ OPTS = {"adagrad": OPT_ADAGRAD, "adam": OPT_ADAM, "rowwise_adagrad": OPT_ROWWISE
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libantdt.so")
 _lib = None
-_fwd = None  # _marshal.embbag_fwd, once the library is loaded
+_fwd = None  # once the library is loaded: _marshal.embbag_fwd, or _general_only without that module
 
 EXPORTS = [
     "antdt_dds_create", "antdt_dds_destroy", "antdt_batch_sizes", "antdt_shard_plan",
@@ -88,6 +88,22 @@ class StepDesc(C.Structure):
         ("h_pooled", C.c_void_p), ("h_dense_out", C.c_void_p), ("h_n_agg", C.c_void_p),
         ("h_status", C.c_void_p), ("staging_idle", C.c_int32), ("fuse_update", C.c_int32),
     ]
+
+
+def _general_only(*_) -> int:
+    return -1
+
+
+def _native_forward(L: C.CDLL):
+    """The forward's native marshalling, where the module is there and of the torch that runs."""
+    try:
+        from . import _marshal
+    except ImportError:
+        return _general_only
+    if str(torch.__version__) != getattr(_marshal, "torch_version", None):
+        return _general_only
+    _marshal.bind(C.cast(L.antdt_embbag_fwd, C.c_void_p).value)
+    return _marshal.embbag_fwd
 
 
 def lib() -> C.CDLL:
@@ -165,12 +181,7 @@ def lib() -> C.CDLL:
                    "antdt_read_status", "antdt_profile_enable", "antdt_profile_kernels",
                    "antdt_profile_get"):
             getattr(L, fn).restype = I32
-        try:
-            from . import _marshal
-        except ImportError as e:
-            raise AntdtError(ERR_STATE, f"_marshal.so is not built (python -m paper_2404_09679_b200.build): {e}")
-        _marshal.bind(C.cast(L.antdt_embbag_fwd, P).value)
-        _fwd = _marshal.embbag_fwd
+        _fwd = _native_forward(L)
         _lib = L
     return _lib
 
@@ -353,7 +364,7 @@ def antdt_embbag_fwd(table, row_ids, bag_offsets, pooled, dev_status=None, strea
         return
     if rc > 0:
         raise AntdtError(rc, "antdt_embbag_fwd")
-    # an argument that is not a plain contiguous tensor
+    # an argument that is not a plain contiguous tensor, or no native marshalling
     V, D = table.shape
     n_bags = bag_offsets.numel() - 1
     _check(lib().antdt_embbag_fwd(_dp(table), _dtype_code(table), V, D, _dp(row_ids),

@@ -67,4 +67,9 @@ PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, kMethods}
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__marshal() { return PyModule_Create(&kModule); }
+PyMODINIT_FUNC PyInit__marshal() {
+  PyObject* m = PyModule_Create(&kModule);
+  // the torch it was built against: with another one it is not used
+  if (m && PyModule_AddStringConstant(m, "torch_version", ANTDT_TORCH) < 0) Py_CLEAR(m);
+  return m;
+}
