@@ -369,6 +369,13 @@ inline Ahead ahead_of(int G, bool bf16, bool fields_known, int64_t bags_per_cta,
 // rows are on their way, so are the next bag's ids and the offsets of the one after it.  What is left of the chain
 // offsets -> ids -> rows is the last step.  Lanes of a warp go through their bags together, to the longest of them
 // (the ids are handed round by shuffles).  BY_FIELD: bags in field-major order.
+// A lane group has its bags beforehand, so a bag of very many ids would hold up the others of its warp, and two in one warp
+// each other: all lanes take it together, a lane group every 32 / G-th step of its rows, and the groups' sums are added up.
+// One bag in 5000 of 5000 ids, 19 ids on average, W 12, not read ahead | ahead | long bags shared: fp32 8 vectors 1074 | 1527 |
+// 664 us, 4 vectors 1054 | 1571 | 425, bf16 16 vectors 1231 | 674 | 455, 8 vectors 1270 | 1425 | 477, 4 vectors 1225 | 1602 |
+// 512; inside a step, field order, fp32 16 vectors, W 130: 2262 | 2395 | 1679.  Not with fp32 rows of 16 vectors in bag order,
+// whose ordinary bags take 3% longer with that code beside them (215 -> 221; in field order 1665 -> 1693, 1763 not read ahead).
+constexpr uint32_t kLongBag = 256;
 template <int G, bool BF16, bool BY_FIELD, int U>
 __global__ void __launch_bounds__(kFlatThreads, ahead_ctas(U))
 embbag_fwd_ahead_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
@@ -415,41 +422,76 @@ embbag_fwd_ahead_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
     const uint32_t next_id = id_at(nbegin, nlen, lg);
     uint32_t fbegin, flen;
     range_of(q + 2 * stride, fbegin, flen);
-    const uint32_t longest = __reduce_max_sync(kFull, len);
+    uint32_t longest = __reduce_max_sync(kFull, len);
     uint64_t acc[PAIRS];
+    auto clear = [&] {
 #pragma unroll
-    for (int e = 0; e < PAIRS; ++e) acc[e] = 0ull;
+      for (int e = 0; e < PAIRS; ++e) acc[e] = 0ull;
+    };
+    // kStep rows, which lanes j0 and on of the group hold in `ids`
+    auto add_rows = [&](uint32_t ids, uint32_t j0) {
+      uint4 v[kStep];
+#pragma unroll
+      for (int t = 0; t < kStep; ++t) {
+        const uint32_t x = __shfl_sync(kFull, ids, j0 + t, G);
+        v[t] = x != kNone && lane_on ? __ldg(tbl + (size_t)x * row_vecs + lg) : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int t = 0; t < kStep; ++t) {
+        if (BF16) {
+          acc[0] = f32x2_add(acc[0], f32x2_pack(v[t].x << 16, v[t].x & 0xffff0000u));
+          acc[1] = f32x2_add(acc[1], f32x2_pack(v[t].y << 16, v[t].y & 0xffff0000u));
+          acc[2] = f32x2_add(acc[2], f32x2_pack(v[t].z << 16, v[t].z & 0xffff0000u));
+          acc[3] = f32x2_add(acc[3], f32x2_pack(v[t].w << 16, v[t].w & 0xffff0000u));
+        } else {
+          acc[0] = f32x2_add(acc[0], f32x2_pack(v[t].x, v[t].y));
+          acc[1] = f32x2_add(acc[1], f32x2_pack(v[t].z, v[t].w));
+        }
+      }
+    };
+    auto store = [&] {
+      ulonglong2* o = reinterpret_cast<ulonglong2*>(pooled + (size_t)bag_of(q) * dim + (size_t)lg * EPV);
+      o[0] = make_ulonglong2(acc[0], acc[1]);
+      if (BF16) o[1] = make_ulonglong2(acc[2], acc[3]);
+    };
+    bool stored = q >= n_slots;
+    if ((BF16 || BY_FIELD ? G < 32 : G < 16) && longest >= kLongBag) {
+      const uint32_t lane = threadIdx.x & 31;
+      for (unsigned todo = __ballot_sync(kFull, lg == 0 && len >= kLongBag); todo; todo &= todo - 1u) {
+        const int from = __ffs((int)todo) - 1;
+        const uint32_t b = __shfl_sync(kFull, begin, from), l = __shfl_sync(kFull, len, from);
+        clear();
+        uint32_t mine = id_at(b, l, lane);
+        for (uint32_t base = 0; base < l; base += 32) {
+          const uint32_t later = id_at(b, l, base + 32 + lane);
+          bad |= mine >= limit && base + lane < l;
+          if (mine >= limit) mine = kNone;
+#pragma unroll 1
+          for (uint32_t j0 = 0; j0 < G; j0 += kStep) add_rows(mine, j0);
+          mine = later;
+        }
+#pragma unroll
+        for (int o = G; o < 32; o <<= 1)
+#pragma unroll
+          for (int e = 0; e < PAIRS; ++e) acc[e] = f32x2_add(acc[e], __shfl_xor_sync(kFull, acc[e], o));
+        if (lane - lg == from) {
+          if (lane_on) store();
+          stored = true;
+          len = 0;
+          id = kNone;
+        }
+      }
+      longest = __reduce_max_sync(kFull, len);
+    }
+    clear();
     for (uint32_t base = 0; base < longest; base += G) {
       if (base > 0) id = id_at(begin, len, base + lg);
       bad |= id >= limit && base + lg < len;
       if (id >= limit) id = kNone;
 #pragma unroll 1
-      for (uint32_t j0 = 0; j0 < G && base + j0 < longest; j0 += kStep) {
-        uint4 v[kStep];
-#pragma unroll
-        for (int t = 0; t < kStep; ++t) {
-          const uint32_t x = __shfl_sync(kFull, id, j0 + t, G);
-          v[t] = x != kNone && lane_on ? __ldg(tbl + (size_t)x * row_vecs + lg) : make_uint4(0u, 0u, 0u, 0u);
-        }
-#pragma unroll
-        for (int t = 0; t < kStep; ++t) {
-          if (BF16) {
-            acc[0] = f32x2_add(acc[0], f32x2_pack(v[t].x << 16, v[t].x & 0xffff0000u));
-            acc[1] = f32x2_add(acc[1], f32x2_pack(v[t].y << 16, v[t].y & 0xffff0000u));
-            acc[2] = f32x2_add(acc[2], f32x2_pack(v[t].z << 16, v[t].z & 0xffff0000u));
-            acc[3] = f32x2_add(acc[3], f32x2_pack(v[t].w << 16, v[t].w & 0xffff0000u));
-          } else {
-            acc[0] = f32x2_add(acc[0], f32x2_pack(v[t].x, v[t].y));
-            acc[1] = f32x2_add(acc[1], f32x2_pack(v[t].z, v[t].w));
-          }
-        }
-      }
+      for (uint32_t j0 = 0; j0 < G && base + j0 < longest; j0 += kStep) add_rows(id, j0);
     }
-    if (q < n_slots && lane_on) {
-      ulonglong2* o = reinterpret_cast<ulonglong2*>(pooled + (size_t)bag_of(q) * dim + (size_t)lg * EPV);
-      o[0] = make_ulonglong2(acc[0], acc[1]);
-      if (BF16) o[1] = make_ulonglong2(acc[2], acc[3]);
-    }
+    if (!stored && lane_on) store();
     q += stride;
     id = next_id; begin = nbegin; len = nlen; nbegin = fbegin; nlen = flen;
   }
