@@ -333,8 +333,8 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
 
 // Which bags are read ahead of (embbag_fwd_ahead_kernel), with how many rows requested at once per lane (0: not),
 // and whether in field-major order.  More rows in flight per lane mean fewer warps (eight: 4 CTAs per SM, four: 5),
-// which pays once a bag has ids enough to fill them; a grid of one wave (2 waves 1 - 5% slower, 8 CTAs per SM no faster
-// than the other kernels).  us before -> reading ahead, by ids per bag, one resident wave of bags (W 1) and many:
+// which pays once a bag has ids enough to fill them (8 CTAs per SM no faster than the other kernels).
+// us before -> reading ahead, by ids per bag, one resident wave of bags (W 1) and many:
 //   fp32, 32 vectors   3: 368 -> 503   5.5: 257 -> 264   10, W 1 / 3 / 24: 13.2 / 25.1 / 122 -> 11.4 / 22.0 / 107   25: 782 -> 693
 //         16 vectors   2: 190 -> 235   6, W 1 / 24: 11.1 / 100 -> 10.3 / 95   15, W 3 / 24: 33 / 178 -> 28 / 151
 //          8 vectors   four rows: 4: 153 -> 146, but 35 M ids over 50 M rows 839 -> 883   10, W 24: 153 -> 145
@@ -349,6 +349,15 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
 //   bf16, 32 vectors, 20 ids: 490 | 459 | 481; 16, 12 ids: 667 | 596 | 649; 4, 12 ids: 619 | 622 | 555
 //          8 vectors, 10 ids: 534 | 455 | 478, 105 M of 20 ids over 20 M rows 1667 | 1710 | 1509
 __host__ __device__ constexpr int ahead_ctas(int rows) { return rows == 8 ? 4 : 5; }  // per SM
+// The grid in waves of CTAs, W as above.  One wave where it leaves a lane group few turns: W 48, 9 ids in 1 / 2 / 4 waves,
+// fp32 16 and 32 vectors 215 / 232 / 234 and 197 / 215 / 212 us.  With many turns the SMs drift apart, and a warp that meets
+// several long bags ends late; 9 ids in 1 / 8 / 16 waves, without reading ahead in brackets:
+//   fp32, 32 vectors, W 70 / 130 / 346   299 / 294 / 300 (297), 560 / 526 / 520 (527), 1485 / 1371 / 1326 (1338)
+//         16 vectors                     318 / 328 / 330 (344), 589 / 589 / 580 (611), 1579 / 1538 / 1488 (1560)
+//   bf16, 16 vectors                     421 / 408 / 413 (445), 771 / 740 / 732 (814), 2046 / 1940 / 1887 (2143)
+//   one bag in 5000 of 4500 ids, fp32, 32 vectors, W 70 / 130  1492 / 698 / 707 (1264), 1751 / 1244 / 954 (1504)
+// (32 waves: W 70 322, W 346 1330.)  In field order every wave would go through all fields: 16 vectors 1667 -> 1800.
+inline int ahead_waves(int64_t W, bool by_field) { return by_field || W < 64 ? 1 : (int)(W < 128 ? W / 8 : 16); }
 struct Ahead { int rows; bool by_field; };
 inline Ahead ahead_of(int G, bool bf16, bool fields_known, int64_t bags_per_cta, int64_t n_bags, int64_t nnz) {
   const Ahead no = {0, false};
@@ -417,7 +426,7 @@ embbag_fwd_ahead_kernel(const void* __restrict__ table, int64_t n_rows, int dim,
   uint32_t begin, len, nbegin, nlen;
   range_of(q, begin, len);
   uint32_t id = id_at(begin, len, lg);
-  range_of(q + stride, nbegin, nlen);  // fewer than 2^31 slots and three strides below 2^20: no slot number wraps
+  range_of(q + stride, nbegin, nlen);  // fewer than 2^31 slots and three strides below 2^24: no slot number wraps
   while (__any_sync(kFull, q < n_slots)) {
     const uint32_t next_id = id_at(nbegin, nlen, lg);
     uint32_t fbegin, flen;
@@ -515,7 +524,7 @@ void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_i
   const Ahead ahead = flat && !PACKED && G >= 4 ? ahead_of(G, BF16, fields > 0, gpb, n_bags, nnz) : Ahead{0, false};
 #define AHEAD_GO(U, FIELD)                                                                                                \
   {                                                                                                                       \
-    const int64_t cap = (int64_t)kNumSM * ahead_ctas(U), want = (n_bags + gpb - 1) / gpb;                                 \
+    const int64_t cap = (int64_t)kNumSM * ahead_ctas(U) * ahead_waves(n_bags / (kNumSM * kFlatCtas * gpb), FIELD), want = (n_bags + gpb - 1) / gpb; \
     ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_ahead_kernel<(G < 4 ? 4 : G), BF16, FIELD, U>), (unsigned)(want < cap ? want : cap), \
                  kFlatThreads, 0, s, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status,              \
                  (uint32_t)(FIELD ? fields : 1), (uint32_t)(FIELD ? n_bags / fields : n_bags), chained);                  \

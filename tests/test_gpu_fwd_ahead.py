@@ -125,3 +125,21 @@ def test_long_bags_inside_a_step():
     for b in list(range(40)) + [S * F - 7, S * F - 6, S * F - 1]:
         want, err = _exact(W, ids[off[b]:off[b + 1]], False)
         assert (np.abs(got[b] - want) <= err).all(), b
+
+
+@pytest.mark.parametrize("D,bf16,lanes,mean,waves", [(16, False, 4, 3, 64), (128, False, 32, 8, 63), (128, False, 32, 8, 64), (128, False, 32, 8, 129)])
+def test_many_turns(D, bf16, lanes, mean, waves):
+    """Bags on both sides of the counts from which the grid is more than one wave, and not larger any more."""
+    n_bags = PER_WAVE // lanes * waves + waves
+    rng = np.random.default_rng(waves)
+    lens = rng.integers(0, 2 * mean + 2, size=n_bags)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    ids = rng.integers(0, 3000, size=int(off[-1])).astype(np.int32)
+    W = rng.normal(0, 0.01, size=(3000, D)).astype(np.float32)
+    out, st = torch.full((n_bags, D), float("nan"), device="cuda"), G.new_status()
+    B.antdt_embbag_fwd(G.dev(W), G.dev(ids), G.dev(off), out, st)
+    assert int(st) == 0 and not out.isnan().any()
+    pick = np.unique(np.concatenate([[0, n_bags - 1], rng.integers(0, n_bags, 5000)]))
+    some = np.concatenate([ids[off[b]:off[b + 1]] for b in pick])
+    cut = np.concatenate([[0], np.cumsum(off[pick + 1] - off[pick])]).astype(np.int64)
+    G.close(out[G.dev(pick)].cpu().numpy(), oracle.embbag_fwd(W, some, cut))
