@@ -341,12 +341,13 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
 //          4 vectors   3, W 24: 99 -> 91   8: 148 -> 140   15: 205 -> 185
 //   bf16, 32 vectors   12, W 6 / 24: 52 / 169 -> 52 / 171   25: 281 -> 247
 //         16 vectors   4: 331 -> 337   5.5, W 1 / 24: 30.8 / 195 -> 27.1 / 182   9, W 1 / 24: 14.5 / 160 -> 12.9 / 144   12: 634 -> 567
-//          8 vectors   four rows: 2, W 24: 91 -> 85   eight: 5, W 24: 136 -> 116   15: 248 -> 214   20: 531 -> 461
+//          8 vectors   5, W 24: 136 -> 116   15: 248 -> 214   20: 531 -> 461   (four rows: 2, W 24 / 346: 91 -> 85, 1149 -> 1245)
 //          4 vectors   four rows: 4, W 24: 136 -> 122   15: 258 -> 234
 // Inside a step, with bags of eight ids and more: one field at a time, not read ahead | bag order | field order:
 //   fp32, 32 / 8 / 4 vectors, 10 ids: 574 | 590 | 612, 400 | 423 | 405, 422 | 503 | 455
 //         16 vectors, 10 and 20 ids: 670 | 612 | 673, 705 | 691 | 680; 65 M ids over 10 M rows 1863 | 1791 | 1885
-//   bf16, 32 vectors, 20 ids: 490 | 459 | 481; 16, 12 ids: 667 | 596 | 649; 4, 12 ids: 619 | 622 | 555
+//   bf16, 32 vectors, 20 ids: 490 | 459 | 481; 16, 12 ids: 667 | 596 | 649
+//         4 vectors, 12 ids: 619 | 622 | 555, but with hashed ids 911 | - | 1020, 9 and 20 ids 732 | - | 786, 969 | - | 1115
 //          8 vectors, 10 ids: 534 | 455 | 478, 105 M of 20 ids over 20 M rows 1667 | 1710 | 1509
 __host__ __device__ constexpr int ahead_ctas(int rows) { return rows == 8 ? 4 : 5; }  // per SM
 // The grid in waves of CTAs, W as above.  One wave where it leaves a lane group few turns: W 48, 9 ids in 1 / 2 / 4 waves,
@@ -370,8 +371,8 @@ inline Ahead ahead_of(int G, bool bf16, bool fields_known, int64_t bags_per_cta,
   }
   if (G == 32) return ids(16) ? Ahead{8, false} : no;
   if (G == 16) return ids(fields_known ? 8 : 5) ? Ahead{8, false} : no;
-  if (G == 8) return ids(4) ? Ahead{8, fields_known && ids(16)} : ids(2) ? Ahead{4, false} : no;
-  return ids(3) ? Ahead{4, fields_known} : no;
+  if (G == 8) return ids(4) ? Ahead{8, fields_known && ids(16)} : no;
+  return ids(3) && !fields_known ? Ahead{4, false} : no;
 }
 
 // The same with a bag's ids held by the lanes of its group, one each, and everything asked for ahead: while a bag's
