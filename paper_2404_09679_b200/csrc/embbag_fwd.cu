@@ -375,6 +375,17 @@ inline Ahead ahead_of(int G, bool bf16, bool fields_known, int64_t bags_per_cta,
   return ids(3) && !fields_known ? Ahead{4, false} : no;
 }
 
+// Whether rows of up to 5/8 of a lane group's vectors are packed lane by lane: not where the bags are few, when a warp's
+// longer chain of bags is all there is.  Not packed -> packed, W as above, us on tables that L2 holds, at 12 ids:
+//   fp32, 5 vectors     W 0.2 / 1 / 1.3 / 2 / 3   5.1 -> 5.0, 7.9 -> 9.1, 10.3 -> 9.3, 13.3 -> 12.4, 18.9 -> 15.7
+//         10 vectors                              5.1 -> 4.8, 7.6 -> 7.9, 9.2 -> 8.1, 12.1 -> 10.5, 16.9 -> 13.9
+//   bf16, 5 vectors     W 0.2 / 1 / 1.6 / 2 / 3   5.8 -> 7.3, 10.0 -> 11.1, 14.3 -> 13.6, 16.9 -> 15.9, 24.7 -> 20.3
+//         (larger tables, W 1.6 / 2 / 2.5 / 3     26.7 -> 29.6, 30.7 -> 34.7, 35.8 -> 34.7, 41.0 -> 37.7)
+inline bool fwd_packs(int nvec, int G, bool bf16, int64_t n_bags) {
+  const int64_t per_wave = (int64_t)kNumSM * kFlatCtas * (kFlatThreads / G);
+  return row_packs_narrow(nvec, G) && 10 * n_bags >= (bf16 ? 25 : 12) * per_wave;
+}
+
 // The same with a bag's ids held by the lanes of its group, one each, and everything asked for ahead: while a bag's
 // rows are on their way, so are the next bag's ids and the offsets of the one after it.  What is left of the chain
 // offsets -> ids -> rows is the last step.  Lanes of a warp go through their bags together, to the longest of them
@@ -522,7 +533,9 @@ void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_i
     fields = 0;
   }
   const int waves = flat && fields == 0 ? stride_waves(G, gpb, BF16, n_bags, nnz) : 0;
-  const Ahead ahead = flat && !PACKED && G >= 4 ? ahead_of(G, BF16, fields > 0, gpb, n_bags, nnz) : Ahead{0, false};
+  // (fp32 rows that would be packed were the bags more: 12 ids, W 1: 7.9 -> 9.0)
+  const bool may_ahead = flat && !PACKED && G >= 4 && (BF16 || !row_packs_narrow(dim / 4, G));
+  const Ahead ahead = may_ahead ? ahead_of(G, BF16, fields > 0, gpb, n_bags, nnz) : Ahead{0, false};
 #define AHEAD_GO(U, FIELD)                                                                                                \
   {                                                                                                                       \
     const int64_t cap = (int64_t)kNumSM * ahead_ctas(U) * ahead_waves(n_bags / (kNumSM * kFlatCtas * gpb), FIELD), want = (n_bags + gpb - 1) / gpb; \
@@ -557,7 +570,7 @@ int32_t dispatch_fwd(int nvec, const void* table, int64_t n_rows, int dim, const
                      int64_t nnz, const int64_t* bag_offsets, int64_t n_bags, float* pooled,
                      int32_t* status, cudaStream_t s, int fields, bool chained) {
 #define FWD_CASE(G, VPL)                                                                      \
-  if (VPL == 1 && row_packs_narrow(nvec, G))                                                  \
+  if (VPL == 1 && fwd_packs(nvec, G, BF16, n_bags))                                           \
     launch_fwd<G, VPL, BF16, (VPL == 1 && G > 2)>(table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, \
                                                   s, fields, chained);                        \
   else                                                                                        \

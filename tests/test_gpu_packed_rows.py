@@ -3,8 +3,11 @@ lane, around CTA edges (a row that begins in one warp and ends in the next, thre
 last CTA with one row); against the CPU checker, and on every path the rows behind the last one stay untouched."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
+from paper_2404_09679_b200 import binding as B
+from paper_2404_09679_b200.step import DeviceStep, OptConfig, StepBuffers
 from tests import gpu_util as G
 from tests import test_gpu_fused_update as fused
 from tests.test_gpu_parity import _bf16_bits
@@ -18,6 +21,46 @@ pytestmark = pytest.mark.gpu
 def test_forward(D, bf16, hi, n_bags):
     if n_bags > 100_000 and D > 40:
         n_bags = 148 * 8 * (256 * (8 if bf16 else 4) // D) * 8 + 1      # the first count that is strided over
+    _check_forward(D, bf16, hi, n_bags)
+
+
+# Rows are packed from so many bags on: tenths of one resident wave of unpacked lane groups.
+def _line(D, bf16):
+    lanes = 1 << (D // (8 if bf16 else 4) - 1).bit_length()
+    return -(-148 * 8 * (256 // lanes) * (25 if bf16 else 12) // 10)
+
+
+@pytest.mark.parametrize("D,bf16,hi", [(20, False, 6), (40, False, 20), (80, False, 5), (40, True, 6), (72, True, 20), (160, True, 4)])
+@pytest.mark.parametrize("over", ["below", "at", "one row in the last CTA", "a full last CTA"])
+def test_forward_around_the_count_from_which_rows_are_packed(D, bf16, hi, over):
+    line, per = _line(D, bf16), 256 // (D // (8 if bf16 else 4))
+    full = -(-line // per) * per
+    _check_forward(D, bf16, hi, {"below": line - 1, "at": line, "one row in the last CTA": full + 1, "a full last CTA": full}[over])
+
+
+@pytest.mark.parametrize("D,bf16", [(20, False), (36, False), (80, False), (40, True), (160, True)])
+@pytest.mark.parametrize("F", [3, 7])
+def test_forward_inside_a_step(D, bf16, F):
+    """Nine ids a bag: one field at a time, CTAs of consecutive samples, the last of them with a part of its rows."""
+    rng = np.random.default_rng(D + F)
+    V, K, S = 3000, 3, _line(D, bf16) // F + 2
+    off = np.concatenate([[0], np.cumsum(rng.integers(0, 19, size=S * F) + (np.arange(S * F) % 64 == 5))]).astype(np.int64)
+    assert 8 * S * F <= off[-1]                        # the rule of field order
+    ids = rng.integers(0, V, size=off[-1]).astype(np.int32)
+    W = rng.normal(0, 0.01, size=(V, D)).astype(np.float32)
+    Wt = _bf16_bits(W) if bf16 else W
+    buf, table, s0 = StepBuffers(D, K, len(ids), S * F), G.table_to_dev(Wt), torch.ones(V, D, device="cuda")
+    ids_t, off_t, dY = G.dev(ids), G.dev(off), torch.zeros(S * F, D, device="cuda")
+    buf.pooled.fill_(float("nan"))
+    step = DeviceStep(buf, table, s0, None, OptConfig(B.OPT_ADAGRAD, 0.01), K, True)
+    cuts = [0, S // 2, S // 2 + 3, S]
+    step.run(1, ids_t, off_t, F, dY, cuts, np.diff(cuts).tolist())
+    torch.cuda.synchronize()
+    assert int(buf.status) == 0
+    G.close(buf.pooled[:S * F].cpu().numpy(), oracle.embbag_fwd(Wt, ids, off))
+
+
+def _check_forward(D, bf16, hi, n_bags):
     rng = np.random.default_rng(D + n_bags)
     V = 2000
     W = rng.normal(0, 0.01, size=(V, D)).astype(np.float32)
