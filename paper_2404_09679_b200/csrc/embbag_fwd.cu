@@ -12,6 +12,8 @@
 //                             longer bags
 //   embbag_fwd_kernel         wider rows (VPL vectors per lane): ids staged through the group's
 //                             registers G at a time (one coalesced load, then shuffles)
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace antdt {
@@ -331,8 +333,8 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
   if (bad) set_status(status, ANTDT_ERR_ID_OUT_OF_RANGE);
 }
 
-// Which bags are read ahead of (embbag_fwd_ahead_kernel), with how many rows requested at once per lane (0: not),
-// and whether in field-major order.  More rows in flight per lane mean fewer warps (eight: 4 CTAs per SM, four: 5),
+// Which bags are read ahead of (embbag_fwd_ahead_kernel, ahead_of), with how many rows requested at once per lane
+// (ahead_rows), and whether in field-major order.  More rows in flight per lane mean fewer warps (eight: 4 CTAs per SM, four: 5),
 // which pays once a bag has ids enough to fill them (8 CTAs per SM no faster than the other kernels).
 // us before -> reading ahead, by ids per bag, one resident wave of bags (W 1) and many:
 //   fp32, 32 vectors   3: 368 -> 503   5.5: 257 -> 264   10, W 1 / 3 / 24: 13.2 / 25.1 / 122 -> 11.4 / 22.0 / 107   25: 782 -> 693
@@ -359,20 +361,16 @@ __host__ __device__ constexpr int ahead_ctas(int rows) { return rows == 8 ? 4 : 
 //   one bag in 5000 of 4500 ids, fp32, 32 vectors, W 70 / 130  1492 / 698 / 707 (1264), 1751 / 1244 / 954 (1504)
 // (32 waves: W 70 322, W 346 1330.)  In field order every wave would go through all fields: 16 vectors 1667 -> 1800.
 inline int ahead_waves(int64_t W, bool by_field) { return by_field || W < 64 ? 1 : (int)(W < 128 ? W / 8 : 16); }
-struct Ahead { int rows; bool by_field; };
+constexpr int ahead_rows(int G, bool bf16) { return G == (bf16 ? 4 : 8) ? 4 : 8; }
+constexpr bool ahead_in_fields(int G, bool bf16) { return G == (bf16 ? 8 : 16); }  // at all, from 16 ids on
+enum class Ahead { kNo, kBags, kFields };
 inline Ahead ahead_of(int G, bool bf16, bool fields_known, int64_t bags_per_cta, int64_t n_bags, int64_t nnz) {
-  const Ahead no = {0, false};
-  if (n_bags < (int64_t)kNumSM * kFlatCtas * bags_per_cta) return no;
+  if (G < 4 || n_bags < (int64_t)kNumSM * kFlatCtas * bags_per_cta) return Ahead::kNo;
   auto ids = [&](int64_t per_bag) { return nnz >= per_bag * n_bags; };
-  if (!bf16) {
-    if (G == 16) return ids(6) ? Ahead{8, fields_known && ids(16)} : no;
-    if (fields_known) return no;
-    return G == 32 && ids(8) ? Ahead{8, false} : G == 8 && ids(8) ? Ahead{4, false} : G == 4 && ids(3) ? Ahead{8, false} : no;
-  }
-  if (G == 32) return ids(16) ? Ahead{8, false} : no;
-  if (G == 16) return ids(fields_known ? 8 : 5) ? Ahead{8, false} : no;
-  if (G == 8) return ids(4) ? Ahead{8, fields_known && ids(16)} : no;
-  return ids(3) && !fields_known ? Ahead{4, false} : no;
+  const bool narrow = G == 4 || (!bf16 && G != 16);  // not inside a step
+  const int64_t from = bf16 ? (G == 32 ? 16 : G == 16 ? 5 : G == 8 ? 4 : 3) : (G >= 32 || G == 8 ? 8 : G == 16 ? 6 : 3);
+  if (!ids(from) || (narrow && fields_known)) return Ahead::kNo;
+  return ahead_in_fields(G, bf16) && fields_known && ids(16) ? Ahead::kFields : Ahead::kBags;
 }
 
 // Whether rows of up to 5/8 of a lane group's vectors are packed lane by lane: not where the bags are few, when a warp's
@@ -534,20 +532,26 @@ void launch_fwd(const void* table, int64_t n_rows, int dim, const int32_t* row_i
   }
   const int waves = flat && fields == 0 ? stride_waves(G, gpb, BF16, n_bags, nnz) : 0;
   // (fp32 rows that would be packed were the bags more: 12 ids, W 1: 7.9 -> 9.0)
-  const bool may_ahead = flat && !PACKED && G >= 4 && (BF16 || !row_packs_narrow(dim / 4, G));
-  const Ahead ahead = may_ahead ? ahead_of(G, BF16, fields > 0, gpb, n_bags, nnz) : Ahead{0, false};
-#define AHEAD_GO(U, FIELD)                                                                                                \
-  {                                                                                                                       \
-    const int64_t cap = (int64_t)kNumSM * ahead_ctas(U) * ahead_waves(n_bags / (kNumSM * kFlatCtas * gpb), FIELD), want = (n_bags + gpb - 1) / gpb; \
-    ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_ahead_kernel<(G < 4 ? 4 : G), BF16, FIELD, U>), (unsigned)(want < cap ? want : cap), \
-                 kFlatThreads, 0, s, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status,              \
-                 (uint32_t)(FIELD ? fields : 1), (uint32_t)(FIELD ? n_bags / fields : n_bags), chained);                  \
+  const bool may_ahead = flat && !PACKED && (BF16 || !row_packs_narrow(dim / 4, G));
+  const Ahead ahead = may_ahead ? ahead_of(G, BF16, fields > 0, gpb, n_bags, nnz) : Ahead::kNo;
+  if constexpr (flat && !PACKED && G >= 4) {
+    constexpr int U = ahead_rows(G, BF16);
+    const int64_t cap = (int64_t)kNumSM * ahead_ctas(U) * ahead_waves(n_bags / (kNumSM * kFlatCtas * gpb), ahead == Ahead::kFields);
+    const unsigned ctas = (unsigned)std::min((n_bags + gpb - 1) / gpb, cap);
+    if constexpr (ahead_in_fields(G, BF16)) {
+      if (ahead == Ahead::kFields) {
+        ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_ahead_kernel<G, BF16, true, U>), ctas, kFlatThreads, 0, s, table, n_rows, dim,
+                     row_ids, nnz, bag_offsets, n_bags, pooled, status, (uint32_t)fields, (uint32_t)(n_bags / fields), chained);
+        return;
+      }
+    }
+    if (ahead == Ahead::kBags) {
+      ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_ahead_kernel<G, BF16, false, U>), ctas, kFlatThreads, 0, s, table, n_rows, dim,
+                   row_ids, nnz, bag_offsets, n_bags, pooled, status, 1u, (uint32_t)n_bags, chained);
+      return;
+    }
   }
-  if (ahead.rows == 8 && ahead.by_field) AHEAD_GO(8, true)
-  else if (ahead.rows == 8) AHEAD_GO(8, false)
-  else if (ahead.rows == 4 && ahead.by_field) AHEAD_GO(4, true)
-  else if (ahead.rows == 4) AHEAD_GO(4, false)
-  else if (waves > 0) {
+  if (waves > 0) {
     ANTDT_LAUNCH("embbag_fwd", (embbag_fwd_stride_kernel<G, BF16, PACKED>), (unsigned)(kNumSM * kFlatCtas * waves),
                  kFlatThreads, 0, s, table, n_rows, dim, row_ids, nnz, bag_offsets, n_bags, pooled, status, chained);
   } else if (flat && fields > 0) {
