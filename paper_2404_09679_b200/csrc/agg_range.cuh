@@ -6,8 +6,9 @@
 // a table of R words in shared memory holds, for each row id of the range, the set of workers
 // whose list contains it (one bit per worker).  Non-zero words, in order, ARE the merged list of
 // distinct ids; the set bits of a word, in order, are the contributions of that row in ascending
-// worker order.  No sort and no waiting on other CTAs, and nothing depends on how the ids are
-// distributed: a range never holds more than R * K entries.
+// worker order.  No sort and no waiting on other CTAs, and a range never holds more than R * K entries however the
+// ids lie.  The time does depend on that: a range is one CTA's work (3 ns an entry: lists of 32 workers that lie almost
+// entirely in one range, 322 k entries, 230 us where spread ones take 50).
 #pragma once
 #include "common.cuh"
 

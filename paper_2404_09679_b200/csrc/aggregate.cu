@@ -1,7 +1,7 @@
 // Server aggregation: batch-size weighted sum of the workers' mean gradients.
 //
 // Sparse part, up to 32 workers: the range-partitioned merge of agg_range.cu (no sort).
-// Sparse part, small lists and up to 1.8 M entries of 33 to 128 workers: the resident merge
+// Sparse part, small lists, and up to 1.8 M entries of 33 to 128 workers: the resident merge
 // (residentsort.cu).
 // Sparse part, more: the workers' row lists (each ascending) are merged by one stable radix sort of
 // (row id, position in the concatenated list); equal rows then sit together in ascending
@@ -476,7 +476,8 @@ namespace {
 // launch for two and no head bits, while a tile's walk keeps more gradient rows in flight.  Server of two kernels, by
 // tiles -> by rows: 63 k entries x 32 floats 31 -> 25 us, 108 k x 20 32 -> 26, 312 k x 16 51 -> 43, 133 k x 64 43 -> 42;
 // but 1.2 M x 16 93 -> 101, 624 k x 64 of 4 workers 79 -> 85, and where many workers list a row (a lane group takes its
-// contributions in turn) 312 k x 64 over 50 k rows 86 -> 101, 624 k x 32 of 32 workers over 400 k 73 -> 78.
+// contributions in turn) 312 k x 64 over 50 k rows 86 -> 101, 624 k x 32 of 32 workers over 400 k 73 -> 78, or the lists lie
+// almost entirely in one range (whose CTA stores the worker of every slot too) 322 k x 16 of 32 workers 234 -> 254.
 bool sum_by_rows(int64_t in_cap, int dim, int64_t n_rows) { return in_cap * dim <= (int64_t)1 << 23 && in_cap <= 2 * n_rows; }
 constexpr int64_t kDenseBesideBytes = 8 << 20;  // below, the fork and join cost what they hide
 enum { kDenseStart = 0, kDenseDone = 1 };  // events of the dense part's side set
@@ -509,7 +510,7 @@ void launch_dense(const antdt_dense_part* dp, const float* weights, const float*
                dp->grads, n4, dp->stride, K <= kDenseBlobWorkers ? (const float*)nullptr : weights, blob, K, dp->out);
 }
 
-// More than 32 workers: merge order by one stable radix sort of (row id, position).
+// More than 32 workers, where the resident merge does not fit: merge order by one stable radix sort of (row id, position).
 void sort_merge_order(const antdt_sparse_part* sp, const uint8_t* dropped, bool any_dropped, int K,
                       int64_t in_cap, int64_t agg_cap, char* w8, const AggLayout& L,
                       int32_t* dev_status, cudaStream_t s) {
@@ -795,7 +796,7 @@ int32_t aggregate_update_forked(const antdt_sparse_part* sp, const antdt_dense_p
   if (opt != ANTDT_OPT_ADAGRAD && opt != ANTDT_OPT_ADAM) return ANTDT_ERR_INVALID_ARG;
   if (opt == ANTDT_OPT_ADAM && !state1) return ANTDT_ERR_INVALID_ARG;
   if (!aligned16(table) || !aligned16(state0) || !aligned16(state1)) return ANTDT_ERR_INVALID_ARG;
-  if (n_workers > kRangeMaxWorkers) {  // the sort-based merge: two steps, agg_grads is needed
+  if (n_workers > kRangeMaxWorkers) {  // the merge order has no row starts there: two steps, agg_grads is needed
     if (sp->out_cap > 0 && !sp->agg_grads) return ANTDT_ERR_INVALID_ARG;
     const int32_t rc = aggregate_impl(sp, dp, batch_sizes, nullptr, n_workers, ws, ws_bytes,
                                       dev_status, stream);

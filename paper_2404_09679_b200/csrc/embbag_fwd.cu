@@ -9,7 +9,7 @@
 //   embbag_fwd_stride_kernel  the same for many bags: capped grid, groups stride over the bags
 //                             and read the next bag's offsets ahead
 //   embbag_fwd_ahead_kernel   the same with the next bag's ids asked for ahead and more rows in flight, for
-//                             longer bags
+//                             longer bags from one resident wave of them on
 //   embbag_fwd_kernel         wider rows (VPL vectors per lane): ids staged through the group's
 //                             registers G at a time (one coalesced load, then shuffles)
 #include <algorithm>
@@ -133,7 +133,8 @@ constexpr int kFlatCtas = 8;     // CTAs per SM
 // per lane group.  W: waves that one bag per lane group would make.
 // Reading the next bag's offsets ahead pays once a lane group has several turns, and the more of a bag's time
 // its offsets are: the shorter its list and the wider its rows.  Above a length that depends on both, the
-// fewer lane groups at work cost more than the offsets.  One bag per group -> striding, us, by ids per bag:
+// fewer lane groups at work cost more than the offsets.  (ahead_of is asked first: fp32 lengths above 5 ids of 16 vectors,
+// 7 of 32 and 2 of 4 are reached by packed rows only, whose lane groups are as many as rows fit a CTA.)  One bag per group -> striding, us, by ids per bag:
 //   fp32, 32 vectors, W 39    1: 93 -> 79    3: 116 -> 99    10: 200 -> 191   20: 321 -> 325   40: 560 -> 584
 //         16 vectors, W 39    1: 96 -> 82    3: 127 -> 108   10: 224 -> 217   20: 361 -> 367   40: 632 -> 688
 //          8 vectors, W 39    1: 100 -> 88   4.5: 169 -> 158   5.5: 186 -> 182   6: 194 -> 194   7: 211 -> 219
