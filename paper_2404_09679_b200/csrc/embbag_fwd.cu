@@ -351,8 +351,7 @@ embbag_fwd_stride_kernel(const void* __restrict__ table, int64_t n_rows, int dim
 //         16 vectors, 10 and 20 ids: 670 | 612 | 673, 705 | 691 | 680; 65 M ids over 10 M rows 1863 | 1791 | 1885
 //   bf16, 32 vectors, 20 ids: 490 | 459 | 481; 16, 12 ids: 667 | 596 | 649
 //         4 vectors, 12 ids: 619 | 622 | 555, but with hashed ids 911 | - | 1020, 9 and 20 ids 732 | - | 786, 969 | - | 1115
-//          8 vectors, 10 ids: 534 | 455 | 478, 105 M of 20 ids over 20 M rows 1667 | 1710 | 1509 (over 100 M rows no gain:
-//                       1675 | - | 1679)
+//          8 vectors, 10 ids: 534 | 455 | 478, 105 M of 20 ids over 20 M rows 1667 | 1710 | 1509, over 100 M rows 1675 | - | 1515
 __host__ __device__ constexpr int ahead_ctas(int rows) { return rows == 8 ? 4 : 5; }  // per SM
 // The grid in waves of CTAs, W as above.  One wave where it leaves a lane group few turns: W 48, 9 ids in 1 / 2 / 4 waves,
 // fp32 16 and 32 vectors 215 / 232 / 234 and 197 / 215 / 212 us.  With many turns the SMs drift apart, and a warp that meets
