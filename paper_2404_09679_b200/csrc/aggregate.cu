@@ -472,13 +472,19 @@ extern "C" size_t antdt_weighted_aggregate_workspace_bytes(int64_t in_cap, int32
 
 namespace antdt {
 namespace {
-// Lists of up to 32 workers that are summed row by row (agg_update_kernel without a table) instead of by tiles: one
+// Lists of up to 16 workers that are summed row by row (agg_update_kernel without a table) instead of by tiles: one
 // launch for two and no head bits, while a tile's walk keeps more gradient rows in flight.  Server of two kernels, by
 // tiles -> by rows: 63 k entries x 32 floats 31 -> 25 us, 108 k x 20 32 -> 26, 312 k x 16 51 -> 43, 133 k x 64 43 -> 42;
 // but 1.2 M x 16 93 -> 101, 624 k x 64 of 4 workers 79 -> 85, and where many workers list a row (a lane group takes its
-// contributions in turn) 312 k x 64 over 50 k rows 86 -> 101, 624 k x 32 of 32 workers over 400 k 73 -> 78, or the lists lie
-// almost entirely in one range (whose CTA stores the worker of every slot too) 322 k x 16 of 32 workers 234 -> 254.
-bool sum_by_rows(int64_t in_cap, int dim, int64_t n_rows) { return in_cap * dim <= (int64_t)1 << 23 && in_cap <= 2 * n_rows; }
+// contributions in turn) 312 k x 64 over 50 k rows 86 -> 101.  A row's lists are at most as many as there are workers; by
+// 4 / 8 / 12 / 16 / 20 / 24 / 32 of them: one field of 1 M rows, ids by frequency, 200 k occurrences x 32 77 -> 70, 95 -> 88,
+// 108 -> 104, 115 -> 115, 130 -> 133, 135 -> 143, 148 -> 165, 400 k x 16 85 -> 79, 114 -> 109, 137 -> 133, 154 -> 156, 174 -> 179,
+// 184 -> 195, 202 -> 228; 26 such fields, 426 k x 16 51 -> 44, 53 -> 47, 59 -> 51, 60 -> 56, 63 -> 63, 64 -> 66, 64 -> 73; hashed
+// ids, 213 k x 32 45 -> 39, 45 -> 40, 47 -> 42, 47 -> 43, 47 -> 47, 48 -> 48, 48 -> 51.
+constexpr int kByRowsWorkers = 16;
+bool sum_by_rows(int K, int64_t in_cap, int dim, int64_t n_rows) {
+  return K <= kByRowsWorkers && in_cap * dim <= (int64_t)1 << 23 && in_cap <= 2 * n_rows;
+}
 constexpr int64_t kDenseBesideBytes = 8 << 20;  // below, the fork and join cost what they hide
 enum { kDenseStart = 0, kDenseDone = 1 };  // events of the dense part's side set
 constexpr int kBulkSmem = 4 * kBulkSlots * kBulkGroup * kBulkElems;
@@ -585,7 +591,7 @@ int32_t aggregate_impl(const antdt_sparse_part* sp, const antdt_dense_part* dp,
   bool resident = sp && !merged && resident_merge_wanted(K, in_cap, sp->n_rows);
   const bool by_ranges = sp && K <= kRangeMaxWorkers && in_cap > 0;
   // a lane group per row: the one-pass update, and the sums of short lists
-  const bool few = sp && !fu && K <= kRangeMaxWorkers && sum_by_rows(in_cap, sp->dim, sp->n_rows);
+  const bool few = sp && !fu && sum_by_rows(K, in_cap, sp->dim, sp->n_rows);
   bool by_rows = sp && in_cap > 0 && ((fu && K <= kRangeMaxWorkers) || (!fu && resident && resident_sort_clears(in_cap)) || few);
   auto upload_weights = [&] { upload_small(hw, 4 * (size_t)K, w8 + L.weights, s); };
   if (!by_ranges && !resident) upload_weights();

@@ -43,6 +43,21 @@ def test_sums_by_rows_and_by_tiles(K, n, D, V):
     _check(rng, V, [n] * K, D, ends=False)
 
 
+# many workers that list the same rows: each row's sum would be one lane group's chain
+@pytest.mark.parametrize("K,by_rows", [(16, True), (17, False), (32, False)])
+def test_many_workers_rows_are_summed_by_tiles(K, by_rows):
+    rng = np.random.default_rng(K)
+    uid = np.concatenate([np.sort(rng.choice(6000, size=3000, replace=False)) for _ in range(K)]).astype(np.int32)
+    wuo = np.arange(K + 1, dtype=np.int64) * 3000
+    g = rng.normal(size=(len(uid), 20)).astype(np.float32)
+    bsz = rng.integers(1, 50, size=K)
+    want_ids, want = oracle.aggregate_sparse(uid, wuo, g, bsz.astype(np.int64))
+    (ids, agg, n, _, code), names = G.kernels_of(lambda: G.gpu_aggregate(uid, wuo, g, bsz, 1_000_000))
+    assert code == 0 and n == len(want_ids) and np.array_equal(ids, want_ids)
+    G.close(agg, want)
+    assert "agg_range_emit" in names and ("agg_fixup" not in names) == by_rows
+
+
 # entries of the first range around 4 and 8 per thread; more than the staged slots (1536 here) in the last three
 @pytest.mark.parametrize("D", [4, 132])
 @pytest.mark.parametrize("K", [16, 17, 32])
