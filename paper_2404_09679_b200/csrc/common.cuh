@@ -173,6 +173,7 @@ __device__ __forceinline__ unsigned group_mask() {
 //   Adagrad server pass  always: step of 720 k occurrences, 20 / 24 / 40 / 48 / 96 floats 384 -> 374, 389 -> 385,
 //                        505 -> 481, 520 -> 511, 743 -> 729 (20 and 40 with the forward's gain)
 //   Adam server pass     up to 5/8: step of 5.2 M, 40 floats 1027 -> 998; 24 and 96 floats 774 -> 789, 1630 -> 1664
+//                        (the packed fp32 instances spill 44 bytes for 16, and are faster up to there all the same)
 //   sparse update        always: server of 20 / 24 / 40 / 48 / 96 floats, Adam 219 -> 218, 227 -> 226, 316 -> 310,
 //                        330 -> 331, 514 -> 494, Adagrad 178 -> 177, 184 -> 183, 258 -> 252, 271 -> 267, 407 -> 396
 //   backward's walk      not at all (does not use it): 5 / 6 vectors 258 -> 268, 260 -> 268; 10, 12, 24 the same.
